@@ -197,17 +197,25 @@ gs::InType in_type(gs_dtype d) {
 
 // fp32 inputs go to the tensor cores (3xTF32) when the path is chosen
 // explicitly, or automatically for forward sums that the variant covers
-// and that are large enough to repay its extra operand kernels (measured
-// on a GB300 at D = 16, C = 1: 4096^2 pairs take 0.157 ms through the
-// tensor-core path and 0.136 ms through the SIMT kernel; 16384^2 pairs
-// 0.197 ms and 0.571 ms).
+// and that are large enough to repay its extra operand kernels: from 2^25
+// pairs, and single problems of few coordinates, whose squared distances
+// are cheap on the SIMT kernel (it works in register tiles of 4, 8, 16, ..
+// coordinates), from 3 x 2^25 pairs (D <= 4) or 3 x 2^24 (D <= 8).  Measured
+// on a GB300, C = 1, whole calls, SIMT / tensor cores: 5800^2 pairs D = 4
+// 24 / 40 us, D = 16 50 / 43 us; 16384^2 pairs D = 4 113 / 71 us, D = 8 172 /
+// 71 us, D = 16 296 / 76 us.
+// Batches keep 2^25 for every D: the tensor-core path runs them in one
+// launch of each kernel, the SIMT kernel problem by problem.
 constexpr int64_t kFp32TensorMinPairs = int64_t(1) << 25;
 
 bool fp32_on_tensor_cores(const Call& c) {
     if (c.opt.path == GS_PATH_TENSOR) return true;
     if (c.opt.path != GS_PATH_AUTO) return false;
+    const int64_t least = c.B > 1 || c.D > 8 ? kFp32TensorMinPairs
+                          : c.D > 4          ? kFp32TensorMinPairs / 2 * 3
+                                             : kFp32TensorMinPairs * 3;
     return !c.grad && c.C <= gs::kFmaMaxChannels && c.D <= gs::kTf32MaxDp &&
-           c.B * c.M * c.N >= kFp32TensorMinPairs;
+           c.B * c.M * c.N >= least;
 }
 
 // Plans the call; returns GS_OK and the workspace size, or an error.

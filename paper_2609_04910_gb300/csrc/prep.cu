@@ -1140,8 +1140,19 @@ __global__ void finalize_kernel(const float* __restrict__ part, int splits,
     const int c = static_cast<int>(idx - m * Cv);
     float acc = 0.f;
     const int ns = m < main_rows ? 1 : splits;
-    for (int s = 0; s < ns; ++s)
-        acc += part[(static_cast<int64_t>(s) * split_stride_rows + m) * part_ld + c];
+    const float* p = part + m * part_ld + c;
+    const int64_t step = split_stride_rows * part_ld;
+    int s = 0;
+    // Eight splits' loads in flight together where there are that many (the
+    // sum keeps the split order).
+    for (; s + 8 <= ns; s += 8, p += 8 * step) {
+        float x[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) x[i] = p[i * step];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) acc += x[i];
+    }
+    for (; s < ns; ++s, p += step) acc += *p;
     out[idx] = acc * (inv_scale ? inv_scale[c] : 1.f);
 }
 

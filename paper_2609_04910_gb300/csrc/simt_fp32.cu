@@ -1,13 +1,12 @@
-// fp32 SIMT Gauss-sum kernel (the single-precision regime of the paper's
+// fp32 SIMT Gauss-sum kernels (the single-precision regime of the paper's
 // appendix, where tensor-core attention is not available).
 //
-// Each thread owns one query row, held in registers and zero padded to
-// DMAX coordinates.  Keys stream through shared memory in tiles of KT keys
-// (zero padded to DMAX, so padded coordinates add (0 - 0)^2 = 0).  For each
-// pair the squared distance is formed in the direct-difference form
-// sum_d (q_d - k_d)^2 (no Gram identity, hence no cancellation), the kernel
-// value is 2^(-(c/2) d^2) with c = tau log2 e, and the values are
-// accumulated with fp32 FMAs:
+// Query rows live in registers, zero padded; keys stream through shared
+// memory in tiles (zero padded likewise, so padded coordinates add
+// (0 - 0)^2 = 0).  For each pair the squared distance is formed in the
+// direct-difference form sum_d (q_d - k_d)^2 (no Gram identity, hence no
+// cancellation), the kernel value is 2^(-(c/2) d^2) with c = tau log2 e, and
+// the values are accumulated with fp32 FMAs:
 //   forward (Eq. 1):     acc[j] += Phi v[n, c0 + j]       for CBLK channels
 //   gradient (Sec. 3):   acc[d] += Phi w_n (k_d - q_d),   acc[D] += Phi w_n
 //                        with w_n = v[n, c] for one weight channel c
@@ -15,7 +14,7 @@
 // are added in a fixed order by the finalise kernel.  Coordinates are
 // handled in pairs with the packed f32x2 subtract / FMA of sm_100+ (the
 // squared distance accumulates even and odd coordinates separately and
-// adds the two at the end).
+// adds the two at the end).  Bound: the fp32 lanes, 2 D operations per pair.
 #include <algorithm>
 
 #include "internal.h"
@@ -24,22 +23,199 @@
 namespace gs {
 namespace {
 
-constexpr int KT = 64;       // keys per shared-memory tile
-constexpr int THREADS = 128; // query rows per block
+constexpr int KT = 64;       // keys per shared-memory tile (gradient; forward: key_tile)
+constexpr int THREADS = 128; // threads per block
 
-template <int DMAX, int CBLK, bool GRAD>
+// ---------------------------------------------------------------- forward
+// Each thread holds ROWS = 4 query rows of up to 32 coordinates, so that one
+// broadcast load of four key coordinates serves 16 packed operations: with
+// one row per thread the 16-byte loads, not the packed subtracts and FMAs,
+// set the pace (in-register rate of the mix by rows per load: 1 row 66 % of
+// the fp32 lanes, 2 rows 74 %, 4 rows 80 %, 8 rows 84 %).  Wider points are
+// shared by L = 2 or 4 neighbouring lanes: lane l of a group holds the
+// coordinate quads l, l + L, .. of the group's four rows, and the lanes
+// exchange partial squared distances so that each ends up with 4 / L rows of
+// its own for the exponential and the values.  Key tiles are copied with
+// cp.async into two buffers, the next one under the arithmetic of the current
+// one.  Measured (one GB300, whole calls, C = 1, one row per thread in tiles
+// of 16, 32, 64 or 128 coordinates / this kernel): M = N = 16384, D = 4 435 /
+// 113 us, D = 16 435 / 296, D = 32 794 / 566, D = 48 1306 / 895, D = 64 1316
+// / 1144 (75 % of the lanes), D = 128 2919 / 2359; 4096^2, D = 16 39 / 31 us.
+constexpr int ROWS = 4;
+__host__ __device__ constexpr int lanes_per_group(int dmax) { return dmax <= 32 ? 1 : dmax <= 64 ? 2 : 4; }
+__host__ __device__ constexpr int key_tile(int dmax) { return dmax <= 64 ? 64 : 32; }
+// Blocks per SM that the registers are limited to (65536 / (128 x blocks)).
+__host__ __device__ constexpr int min_blocks(int dmax, int cblk) {
+    return dmax <= 16 ? 4 : dmax == 32 && cblk == 4 ? 2 : 3;
+}
+
+__device__ __forceinline__ void cp_async4(float* dst, const float* src, bool valid) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(smem_u32(dst)), "l"(src),
+                 "r"(valid ? 4 : 0)
+                 : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int PENDING>
+__device__ __forceinline__ void cp_async_wait() {
+    asm volatile("cp.async.wait_group %0;" ::"n"(PENDING) : "memory");
+}
+
+template <int DMAX, int CBLK>
+__global__ void __launch_bounds__(THREADS, min_blocks(DMAX, CBLK))
+simt_sum_kernel(const float* __restrict__ q, const float* __restrict__ k,
+                const float* __restrict__ v, int64_t M, int64_t N, int D, int Cv, float half_c,
+                int64_t keys_per_split, float* __restrict__ part) {
+    pdl_trigger();
+    pdl_wait();
+    constexpr int L = lanes_per_group(DMAX);
+    constexpr int DL = DMAX / L;          // coordinates per lane
+    constexpr int OWN = ROWS / L;         // rows whose sums a lane keeps
+    constexpr int GROUPS = THREADS / L;
+    constexpr int KTF = key_tile(DMAX);
+    static_assert(DL % 4 == 0 && DL <= 32, "coordinate quads of a lane");
+    __shared__ __align__(16) float ks[2][KTF][DMAX];
+    __shared__ __align__(16) float vs[2][KTF][CBLK];
+
+    const int sub = threadIdx.x % L;
+    const int64_t m0 = static_cast<int64_t>(blockIdx.x) * (GROUPS * ROWS) + threadIdx.x / L;
+    const int split = blockIdx.y;
+    const int c0 = blockIdx.z * CBLK;
+    const int64_t n_begin = static_cast<int64_t>(split) * keys_per_split;
+    const int64_t n_end = min(N, n_begin + keys_per_split);
+
+    // Tile of KTF keys from t0 into buffer b; rows past n_end and the
+    // coordinates and channels past D and Cv are filled with zeros (nothing
+    // is read for them; their source address is v, which is never null here,
+    // as k may be when D = 0).
+    auto load_tile = [&](int b, int64_t t0) {
+        const int cnt = static_cast<int>(min(static_cast<int64_t>(KTF), n_end - t0));
+        const float* kt = k + t0 * D;
+        for (int i = threadIdx.x; i < KTF * DMAX; i += THREADS) {
+            const int kk = i / DMAX, d = i - kk * DMAX;
+            const bool in = kk < cnt && d < D;
+            cp_async4(&ks[b][kk][d], in ? kt + kk * D + d : v, in);
+        }
+        const float* vt = v + t0 * Cv + c0;
+        for (int i = threadIdx.x; i < KTF * CBLK; i += THREADS) {
+            const int kk = i / CBLK, j = i - kk * CBLK;
+            const bool in = kk < cnt && c0 + j < Cv;
+            cp_async4(&vs[b][kk][j], in ? vt + static_cast<int64_t>(kk) * Cv + j : v, in);
+        }
+        cp_async_commit();
+    };
+    if (n_begin < n_end) load_tile(0, n_begin);
+
+    uint64_t qr[ROWS][DL / 2];   // coordinate pairs of the query rows
+    // Sums of the key tiles, added up tile by tile (two-level summation: the
+    // rounding error of a split's sum grows with the keys per tile plus the
+    // tiles, not with all its keys).
+    float acc[OWN][CBLK];
+#pragma unroll
+    for (int r = 0; r < ROWS; ++r) {
+        const int64_t m = m0 + r * GROUPS;
+#pragma unroll
+        for (int i = 0; i < DL; i += 2) {
+            const int d = (i & ~3) * L + 4 * sub + (i & 3);
+            qr[r][i / 2] = f32x2_pack((m < M && d < D) ? q[m * D + d] : 0.f,
+                                      (m < M && d + 1 < D) ? q[m * D + d + 1] : 0.f);
+        }
+    }
+#pragma unroll
+    for (int r = 0; r < OWN; ++r)
+#pragma unroll
+        for (int j = 0; j < CBLK; ++j) acc[r][j] = 0.f;
+
+    int b = 0;
+    for (int64_t t0 = n_begin; t0 < n_end; t0 += KTF, b ^= 1) {
+        const int cnt = static_cast<int>(min(static_cast<int64_t>(KTF), n_end - t0));
+        if (t0 + KTF < n_end) {
+            load_tile(b ^ 1, t0 + KTF);
+            cp_async_wait<1>();
+        } else {
+            cp_async_wait<0>();
+        }
+        __syncthreads();
+        float tile[OWN][CBLK];
+#pragma unroll
+        for (int r = 0; r < OWN; ++r)
+#pragma unroll
+            for (int j = 0; j < CBLK; ++j) tile[r][j] = 0.f;
+        for (int kk = 0; kk < cnt; ++kk) {
+            uint64_t d2p[ROWS];   // (even, odd) partial squared distances
+#pragma unroll
+            for (int r = 0; r < ROWS; ++r) d2p[r] = 0ull;
+#pragma unroll
+            for (int i = 0; i < DL; i += 4) {
+                const float4 kv = *reinterpret_cast<const float4*>(&ks[b][kk][i * L + 4 * sub]);
+                const uint64_t k01 = f32x2_pack(kv.x, kv.y), k23 = f32x2_pack(kv.z, kv.w);
+#pragma unroll
+                for (int r = 0; r < ROWS; ++r) {
+                    const uint64_t t01 = f32x2_sub(qr[r][i / 2], k01);
+                    const uint64_t t23 = f32x2_sub(qr[r][i / 2 + 1], k23);
+                    d2p[r] = f32x2_fma(t01, t01, d2p[r]);
+                    d2p[r] = f32x2_fma(t23, t23, d2p[r]);
+                }
+            }
+            float d2[ROWS];
+#pragma unroll
+            for (int r = 0; r < ROWS; ++r) {
+                float d2e, d2o;
+                f32x2_unpack(d2p[r], d2e, d2o);
+                d2[r] = d2e + d2o;
+            }
+            // Halve the rows with the neighbouring lanes: each keeps the
+            // half that own_row names and hands over the other.
+            if (L >= 2) {
+                const bool hi = (threadIdx.x & 1) != 0;
+#pragma unroll
+                for (int r = 0; r < 2; ++r) {
+                    const float give = hi ? d2[r] : d2[r + 2], keep = hi ? d2[r + 2] : d2[r];
+                    d2[r] = keep + __shfl_xor_sync(0xffffffffu, give, 1);
+                }
+            }
+            if (L >= 4) {
+                const bool hi = (threadIdx.x & 2) != 0;
+                const float give = hi ? d2[0] : d2[1], keep = hi ? d2[1] : d2[0];
+                d2[0] = keep + __shfl_xor_sync(0xffffffffu, give, 2);
+            }
+#pragma unroll
+            for (int r = 0; r < OWN; ++r) {
+                const float phi = ex2_approx(-half_c * d2[r]);
+#pragma unroll
+                for (int j = 0; j < CBLK; ++j) tile[r][j] = fmaf(phi, vs[b][kk][j], tile[r][j]);
+            }
+        }
+#pragma unroll
+        for (int r = 0; r < OWN; ++r)
+#pragma unroll
+            for (int j = 0; j < CBLK; ++j) acc[r][j] += tile[r][j];
+        __syncthreads();   // every thread is done with buffer b
+    }
+#pragma unroll
+    for (int r = 0; r < OWN; ++r) {
+        const int own_row = L == 1 ? r : L == 2 ? 2 * (sub & 1) + r : 2 * (sub & 1) + (sub >> 1);
+        const int64_t m = m0 + own_row * GROUPS;
+        if (m >= M) continue;
+        float* out = part + (static_cast<int64_t>(split) * M + m) * Cv + c0;
+#pragma unroll
+        for (int j = 0; j < CBLK; ++j)
+            if (c0 + j < Cv) out[j] = acc[r][j];
+    }
+}
+
+// ---------------------------------------------------------------- gradient
+template <int DMAX>
 __global__ void __launch_bounds__(THREADS)
-simt_gauss_kernel(const float* __restrict__ q, const float* __restrict__ k,
-                  const float* __restrict__ v, int64_t M, int64_t N, int D, int Cv,
-                  int wch, float half_c, int64_t keys_per_split, float* __restrict__ part) {
+simt_grad_kernel(const float* __restrict__ q, const float* __restrict__ k,
+                 const float* __restrict__ v, int64_t M, int64_t N, int D, int Cv,
+                 int wch, float half_c, int64_t keys_per_split, float* __restrict__ part) {
     pdl_trigger();
     pdl_wait();
     __shared__ __align__(16) float ks[KT][DMAX];
-    __shared__ float vs[KT][GRAD ? 1 : CBLK];
+    __shared__ float vs[KT];
 
     const int64_t m = static_cast<int64_t>(blockIdx.x) * THREADS + threadIdx.x;
     const int split = blockIdx.y;
-    const int c0 = GRAD ? 0 : blockIdx.z * CBLK;
     const int64_t n_begin = static_cast<int64_t>(split) * keys_per_split;
     const int64_t n_end = min(N, n_begin + keys_per_split);
 
@@ -48,12 +224,10 @@ simt_gauss_kernel(const float* __restrict__ q, const float* __restrict__ k,
     for (int d = 0; d < DMAX; d += 2)
         qr[d / 2] = f32x2_pack((m < M && d < D) ? q[m * D + d] : 0.f,
                                (m < M && d + 1 < D) ? q[m * D + d + 1] : 0.f);
-    float acc[GRAD ? 1 : CBLK];      // forward channels; gradient: sum of w
-    uint64_t acc2[GRAD ? DMAX / 2 : 1];   // gradient coordinates, in pairs
+    float acc = 0.f;              // sum of Phi w
+    uint64_t acc2[DMAX / 2];      // gradient coordinates, in pairs
 #pragma unroll
-    for (int j = 0; j < (GRAD ? 1 : CBLK); ++j) acc[j] = 0.f;
-#pragma unroll
-    for (int j = 0; j < (GRAD ? DMAX / 2 : 1); ++j) acc2[j] = 0ull;
+    for (int j = 0; j < DMAX / 2; ++j) acc2[j] = 0ull;
 
     for (int64_t t0 = n_begin; t0 < n_end; t0 += KT) {
         const int cnt = static_cast<int>(min(static_cast<int64_t>(KT), n_end - t0));
@@ -62,16 +236,9 @@ simt_gauss_kernel(const float* __restrict__ q, const float* __restrict__ k,
             const int kk = i / DMAX, d = i - kk * DMAX;
             ks[kk][d] = (kk < cnt && d < D) ? k[(t0 + kk) * D + d] : 0.f;
         }
-        if (GRAD) {
-            // v is N x Cv here; the weight is its channel wch.
-            for (int i = threadIdx.x; i < KT; i += THREADS)
-                vs[i][0] = i < cnt ? v[(t0 + i) * Cv + wch] : 0.f;
-        } else {
-            for (int i = threadIdx.x; i < KT * CBLK; i += THREADS) {
-                const int kk = i / CBLK, j = i - kk * CBLK;
-                vs[kk][j] = (kk < cnt && c0 + j < Cv) ? v[(t0 + kk) * Cv + c0 + j] : 0.f;
-            }
-        }
+        // v is N x Cv; the weight is its channel wch.
+        for (int i = threadIdx.x; i < KT; i += THREADS)
+            vs[i] = i < cnt ? v[(t0 + i) * Cv + wch] : 0.f;
         __syncthreads();
         for (int kk = 0; kk < cnt; ++kk) {
             uint64_t d2p = 0ull;   // (even, odd) partial squared distances
@@ -86,60 +253,59 @@ simt_gauss_kernel(const float* __restrict__ q, const float* __restrict__ k,
             float d2e, d2o;
             f32x2_unpack(d2p, d2e, d2o);
             const float phi = ex2_approx(-half_c * (d2e + d2o));
-            if (GRAD) {
-                const float w = phi * vs[kk][0];
-                const uint64_t w2 = f32x2_pack(w, w);
+            const float w = phi * vs[kk];
+            const uint64_t w2 = f32x2_pack(w, w);
 #pragma unroll
-                for (int d = 0; d < DMAX; d += 4) {
-                    const float4 kv = *reinterpret_cast<const float4*>(&ks[kk][d]);
-                    acc2[d / 2] = f32x2_fma(w2, f32x2_sub(f32x2_pack(kv.x, kv.y), qr[d / 2]), acc2[d / 2]);
-                    acc2[d / 2 + 1] =
-                        f32x2_fma(w2, f32x2_sub(f32x2_pack(kv.z, kv.w), qr[d / 2 + 1]), acc2[d / 2 + 1]);
-                }
-                acc[0] += w;
-            } else {
-#pragma unroll
-                for (int j = 0; j < CBLK; ++j) acc[j] = fmaf(phi, vs[kk][j], acc[j]);
+            for (int d = 0; d < DMAX; d += 4) {
+                const float4 kv = *reinterpret_cast<const float4*>(&ks[kk][d]);
+                acc2[d / 2] = f32x2_fma(w2, f32x2_sub(f32x2_pack(kv.x, kv.y), qr[d / 2]), acc2[d / 2]);
+                acc2[d / 2 + 1] =
+                    f32x2_fma(w2, f32x2_sub(f32x2_pack(kv.z, kv.w), qr[d / 2 + 1]), acc2[d / 2 + 1]);
             }
+            acc += w;
         }
     }
     if (m >= M) return;
-    if (GRAD) {
-        float* out = part + (static_cast<int64_t>(split) * M + m) * (D + 1);
+    float* out = part + (static_cast<int64_t>(split) * M + m) * (D + 1);
 #pragma unroll
-        for (int d = 0; d < DMAX; d += 2) {
-            float lo, hi;
-            f32x2_unpack(acc2[d / 2], lo, hi);
-            if (d < D) out[d] = lo;
-            if (d + 1 < D) out[d + 1] = hi;
-        }
-        out[D] = acc[0];
-    } else {
-        float* out = part + (static_cast<int64_t>(split) * M + m) * Cv + c0;
-#pragma unroll
-        for (int j = 0; j < CBLK; ++j)
-            if (c0 + j < Cv) out[j] = acc[j];
+    for (int d = 0; d < DMAX; d += 2) {
+        float lo, hi;
+        f32x2_unpack(acc2[d / 2], lo, hi);
+        if (d < D) out[d] = lo;
+        if (d + 1 < D) out[d + 1] = hi;
     }
+    out[D] = acc;
 }
 
-template <int DMAX, int CBLK, bool GRAD>
-cudaError_t launch_cblk(const SimtPlan& p, const float* q, const float* k, const float* v,
-                        int Cw, int wch, float half_c, float* part, cudaStream_t s) {
-    dim3 grid(static_cast<unsigned>((p.M + THREADS - 1) / THREADS), p.splits,
-              GRAD ? 1u : static_cast<unsigned>((p.Cv + CBLK - 1) / CBLK));
-    launch_kernel(simt_gauss_kernel<DMAX, CBLK, GRAD>, grid, THREADS, 0, s, 
-        q, k, v, p.M, p.N, static_cast<int>(p.D), GRAD ? Cw : static_cast<int>(p.Cv), wch,
-        half_c, p.keys_per_split, part);
+template <int DMAX>
+cudaError_t launch_grad(const SimtPlan& p, const float* q, const float* k, const float* v, int Cw,
+                        int wch, float half_c, float* part, cudaStream_t s) {
+    dim3 grid(static_cast<unsigned>((p.M + THREADS - 1) / THREADS), p.splits);
+    launch_kernel(simt_grad_kernel<DMAX>, grid, THREADS, 0, s, q, k, v, p.M, p.N,
+                  static_cast<int>(p.D), Cw, wch, half_c, p.keys_per_split, part);
     note_launches(1);
     return cudaGetLastError();
 }
 
-// Channel blocks of 4, or of 1 for a single channel (no idle FMAs).
-template <int DMAX, bool GRAD>
+template <int DMAX, int CBLK>
+cudaError_t launch_cblk(const SimtPlan& p, const float* q, const float* k, const float* v,
+                        float half_c, float* part, cudaStream_t s) {
+    constexpr int rows = THREADS / lanes_per_group(DMAX) * ROWS;
+    dim3 grid(static_cast<unsigned>((p.M + rows - 1) / rows), p.splits,
+              static_cast<unsigned>((p.Cv + CBLK - 1) / CBLK));
+    launch_kernel(simt_sum_kernel<DMAX, CBLK>, grid, THREADS, 0, s, q, k, v, p.M, p.N,
+                  static_cast<int>(p.D), static_cast<int>(p.Cv), half_c, p.keys_per_split, part);
+    note_launches(1);
+    return cudaGetLastError();
+}
+
+// Channel blocks of 4, or of 1 or 2 for as few channels (no idle FMAs).
+template <int DMAX>
 cudaError_t launch_dmax(const SimtPlan& p, const float* q, const float* k, const float* v,
-                        int Cw, int wch, float half_c, float* part, cudaStream_t s) {
-    if (!GRAD && p.Cv == 1) return launch_cblk<DMAX, 1, GRAD>(p, q, k, v, Cw, wch, half_c, part, s);
-    return launch_cblk<DMAX, 4, GRAD>(p, q, k, v, Cw, wch, half_c, part, s);
+                        float half_c, float* part, cudaStream_t s) {
+    if (p.cblk == 1) return launch_cblk<DMAX, 1>(p, q, k, v, half_c, part, s);
+    if (p.cblk == 2) return launch_cblk<DMAX, 2>(p, q, k, v, half_c, part, s);
+    return launch_cblk<DMAX, 4>(p, q, k, v, half_c, part, s);
 }
 
 }  // namespace
@@ -155,17 +321,45 @@ bool plan_simt(int64_t M, int64_t N, int64_t D, int64_t C, bool grad, int split_
         *why = grad ? "fp32 gradient supports D <= 64" : "fp32 path supports D <= 128";
         return false;
     }
-    p->dmax = D <= 16 ? 16 : D <= 32 ? 32 : D <= 64 ? 64 : 128;
-    p->cblk = 4;
-    const int64_t rowblocks = (M + THREADS - 1) / THREADS;
-    const int64_t chunks = grad ? 1 : (p->Cv + 3) / 4;
-    const int64_t key_tiles = (N + KT - 1) / KT;
-    int64_t splits = split_override > 0 ? split_override
-                                        : (4LL * sms + rowblocks * chunks - 1) / (rowblocks * chunks);
-    splits = std::max<int64_t>(1, std::min<int64_t>(splits, std::max<int64_t>(1, key_tiles)));
-    splits = std::min<int64_t>(splits, 65535);
-    const int64_t tiles_per_split = (key_tiles + splits - 1) / splits;
-    p->keys_per_split = std::max<int64_t>(KT, tiles_per_split * KT);
+    p->cblk = p->Cv >= 3 ? 4 : static_cast<int>(std::max<int64_t>(1, p->Cv));
+    int64_t rows, keys;   // query rows per block, keys per shared-memory tile
+    if (grad) {
+        p->dmax = D <= 16 ? 16 : D <= 32 ? 32 : 64;
+        rows = THREADS;
+        keys = KT;
+    } else {
+        // Register tiles of the query rows: the smallest that holds D.
+        p->dmax = D <= 4 ? 4 : D <= 8 ? 8 : D <= 16 ? 16 : D <= 24 ? 24 : D <= 32 ? 32
+                : D <= 48 ? 48 : D <= 64 ? 64 : 128;
+        rows = THREADS / lanes_per_group(p->dmax) * ROWS;
+        keys = key_tile(p->dmax);
+    }
+    const int64_t chunks = grad ? 1 : (p->Cv + p->cblk - 1) / p->cblk;
+    const int64_t blocks = (M + rows - 1) / rows * chunks;   // per key split
+    const int64_t key_tiles = std::max<int64_t>(1, (N + keys - 1) / keys);
+    if (grad || split_override > 0) {
+        int64_t splits = split_override > 0 ? split_override : (4LL * sms + blocks - 1) / blocks;
+        splits = std::max<int64_t>(1, std::min<int64_t>(splits, key_tiles));
+        splits = std::min<int64_t>(splits, 65535);
+        p->keys_per_split = grad ? (key_tiles + splits - 1) / splits * keys
+                                 : std::max<int64_t>(4, ((N + splits - 1) / splits + 3) / 4 * 4);
+    } else {
+        // The blocks of an SM share its fp32 lanes, so a call takes as long
+        // as the SM with the most keys: blocks per SM x (keys per block +
+        // about 48 keys' worth of start-up).  Tried: as many splits as give
+        // 1, 2, .. 16 blocks per SM, each of N / splits keys rounded up to 4,
+        // no fewer than 16; few splits win ties (fewer partial sums to add).
+        // Measured, 4096^2 pairs, D = 16: 1 and 2 blocks per SM (19 and 38
+        // splits) 30.5 us, 24, 32, 64 splits 39.7, 32.7, 36.9 us.
+        double best = 1e300;
+        for (int64_t per = 1; per <= 16; ++per) {
+            const int64_t want = std::min<int64_t>(256, std::max<int64_t>(1, per * sms / blocks));
+            const int64_t kps = std::max<int64_t>(16, ((N + want - 1) / want + 3) / 4 * 4);
+            const int64_t per_sm = (blocks * ((N + kps - 1) / kps) + sms - 1) / sms;
+            const double cost = static_cast<double>(per_sm) * (kps + 48.0);
+            if (cost < best * 0.99) { best = cost; p->keys_per_split = kps; }
+        }
+    }
     p->splits = static_cast<int>((N + p->keys_per_split - 1) / p->keys_per_split);
     if (p->splits < 1) p->splits = 1;
     p->off_part = 0;
@@ -179,16 +373,20 @@ cudaError_t launch_simt(const SimtPlan& p, bool grad, const float* q, const floa
                         cudaStream_t s) {
     if (grad) {
         switch (p.dmax) {
-            case 16: return launch_dmax<16, true>(p, q, k, v, Cw, wch, half_c, part, s);
-            case 32: return launch_dmax<32, true>(p, q, k, v, Cw, wch, half_c, part, s);
-            default: return launch_dmax<64, true>(p, q, k, v, Cw, wch, half_c, part, s);
+            case 16: return launch_grad<16>(p, q, k, v, Cw, wch, half_c, part, s);
+            case 32: return launch_grad<32>(p, q, k, v, Cw, wch, half_c, part, s);
+            default: return launch_grad<64>(p, q, k, v, Cw, wch, half_c, part, s);
         }
     }
     switch (p.dmax) {
-        case 16: return launch_dmax<16, false>(p, q, k, v, 0, 0, half_c, part, s);
-        case 32: return launch_dmax<32, false>(p, q, k, v, 0, 0, half_c, part, s);
-        case 64: return launch_dmax<64, false>(p, q, k, v, 0, 0, half_c, part, s);
-        default: return launch_dmax<128, false>(p, q, k, v, 0, 0, half_c, part, s);
+        case 4: return launch_dmax<4>(p, q, k, v, half_c, part, s);
+        case 8: return launch_dmax<8>(p, q, k, v, half_c, part, s);
+        case 16: return launch_dmax<16>(p, q, k, v, half_c, part, s);
+        case 24: return launch_dmax<24>(p, q, k, v, half_c, part, s);
+        case 32: return launch_dmax<32>(p, q, k, v, half_c, part, s);
+        case 48: return launch_dmax<48>(p, q, k, v, half_c, part, s);
+        case 64: return launch_dmax<64>(p, q, k, v, half_c, part, s);
+        default: return launch_dmax<128>(p, q, k, v, half_c, part, s);
     }
 }
 
