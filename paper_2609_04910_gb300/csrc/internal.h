@@ -241,9 +241,9 @@ cudaError_t launch_simt(const SimtPlan& p, bool grad, const float* q, const floa
                         const float* v, int Cw, int wch, float half_c, float* part,
                         cudaStream_t s);
 
-// Key records of the FMA kernel: per key pair (2t, 2t+1) the floats
-// B_2t, B_2t+1 (omitted when B is null), v_2t[0], v_2t+1[0], ...,
-// v_2t[C-1], v_2t+1[C-1].
+// Key records of the FMA kernel: without B per key pair (2t, 2t+1) the floats
+// v_2t[0], v_2t+1[0], ..., v_2t[C-1], v_2t+1[C-1]; with B per four keys their
+// four B and then, channel by channel, their values.
 cudaError_t launch_key_records(InType t, const void* v, const float* B, int64_t N, int64_t Npad,
                                int C, float* rec, cudaStream_t s, int batch = 1, bool signs = false);
 // 3xTF32 operands of fp32 inputs (see prep.cu): rows of 2 Dp floats

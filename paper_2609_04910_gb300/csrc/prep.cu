@@ -1050,8 +1050,10 @@ __global__ void value_prep_kernel(const W* __restrict__ w, const T* __restrict__
 }
 
 // ---------------------------------------------------------------- key records
-// One thread per key pair t: B_2t, B_2t+1 (only when B is given), then the
-// values of both keys channel by channel, in fp32 (zero for padded keys).
+// One thread per key pair t, values in fp32, zero for padded keys.  Without B
+// (augmented operands) the pair's values channel by channel; with B per four
+// keys their B and then, channel by channel, their values (see
+// tc_gauss_fma.cu).
 template <typename T>
 __global__ void key_record_kernel(const T* __restrict__ v, const float* __restrict__ B, int64_t N,
                                   int64_t pairs, int C, float* __restrict__ rec) {
@@ -1060,19 +1062,21 @@ __global__ void key_record_kernel(const T* __restrict__ v, const float* __restri
     const int64_t t = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
     if (t >= pairs) return;
     const int64_t n0 = 2 * t, n1 = 2 * t + 1;
-    const int head = B ? 2 : 0;
     // Problem blockIdx.y of a batch (2 pairs keys per problem).
     v += static_cast<int64_t>(blockIdx.y) * N * C;
     if (B) B += static_cast<int64_t>(blockIdx.y) * 2 * pairs;
-    rec += static_cast<int64_t>(blockIdx.y) * pairs * (head + 2 * C);
-    float* out = rec + t * (head + 2 * C);
+    rec += static_cast<int64_t>(blockIdx.y) * pairs * ((B ? 2 : 0) + 2 * C);
+    // The pair's first float, and the distance between its channels.
+    float* out = rec + (B ? (t >> 1) * (4 + 4 * C) + (t & 1) * 2 : t * (2 * C));
+    const int step = B ? 4 : 2;
     if (B) {
         out[0] = B[n0];
         out[1] = B[n1];
+        out += step;
     }
-    for (int c = 0; c < C; ++c) {
-        out[head + 2 * c] = n0 < N ? to_f(v[n0 * C + c]) : 0.f;
-        out[head + 1 + 2 * c] = n1 < N ? to_f(v[n1 * C + c]) : 0.f;
+    for (int c = 0; c < C; ++c, out += step) {
+        out[0] = n0 < N ? to_f(v[n0 * C + c]) : 0.f;
+        out[1] = n1 < N ? to_f(v[n1 * C + c]) : 0.f;
     }
 }
 

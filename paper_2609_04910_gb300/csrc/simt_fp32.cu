@@ -346,17 +346,19 @@ bool plan_simt(int64_t M, int64_t N, int64_t D, int64_t C, bool grad, int split_
     } else {
         // The blocks of an SM share its fp32 lanes, so a call takes as long
         // as the SM with the most keys: blocks per SM x (keys per block +
-        // about 48 keys' worth of start-up).  Tried: as many splits as give
-        // 1, 2, .. 16 blocks per SM, each of N / splits keys rounded up to 4,
-        // no fewer than 16; few splits win ties (fewer partial sums to add).
+        // about 48 keys' worth of start-up), with a single block per SM
+        // leaving its latencies exposed.  Tried: as many splits as give 1, 2,
+        // .. 16 blocks per SM, each of N / splits keys rounded up to 4, no
+        // fewer than 16; few splits win ties (fewer partial sums to add).
         // Measured, 4096^2 pairs, D = 16: 1 and 2 blocks per SM (19 and 38
-        // splits) 30.5 us, 24, 32, 64 splits 39.7, 32.7, 36.9 us.
+        // splits) 30.5 us, 24, 32, 64 splits 39.7, 32.7, 36.9 us; 5800^2
+        // pairs, D = 32: one block per SM 124 us, three 95 us.
         double best = 1e300;
         for (int64_t per = 1; per <= 16; ++per) {
             const int64_t want = std::min<int64_t>(256, std::max<int64_t>(1, per * sms / blocks));
             const int64_t kps = std::max<int64_t>(16, ((N + want - 1) / want + 3) / 4 * 4);
             const int64_t per_sm = (blocks * ((N + kps - 1) / kps) + sms - 1) / sms;
-            const double cost = static_cast<double>(per_sm) * (kps + 48.0);
+            const double cost = static_cast<double>(per_sm) * (kps + 48.0) * (per_sm < 2 ? 1.3 : 1.0);
             if (cost < best * 0.99) { best = cost; p->keys_per_split = kps; }
         }
     }

@@ -35,12 +35,18 @@
 //     the segment are complete and release each stage when they next load
 //     it, so the next segment's copies and MMAs run while the exponent
 //     warps finish the current one.
-//   * TMEM holds SL slots of two 128-column S buffers (one per query
-//     tile); key tile j uses slot j % SL, so the MMAs of key tile j only
-//     wait for the release of key tile j - SL.  With Dp <= 128 the query
-//     tiles q^ stay in shared memory (A operand read by the MMA from shared
-//     memory) and SL = 2; with larger Dp they would not fit next to the key
-//     stages, so q^ is copied into TMEM (A operand from TMEM) and SL = 1.
+//   * With Dp <= 128 the query tiles q^ stay in shared memory (A operand read
+//     by the MMA from shared memory) and TMEM holds two slots of two
+//     128-column S buffers (one per query tile); key tile j uses slot j % 2,
+//     so the MMAs of key tile j only wait for the release of key tile j - 2.
+//     With larger Dp the query tiles would not fit next to the key stages, so
+//     q^ is copied into TMEM (A operand from TMEM) beside one S buffer per
+//     query tile; each of the two is handed over and handed back by itself,
+//     so that the MMAs of one run while the other is read.  (One barrier for
+//     both left the tensor pipe idle from the last MMA of a key tile to the
+//     TMEM loads: 1M keys of D = 256 against 16384 queries, whole calls, C = 1
+//     6.11 -> 5.44 ms = 1617 TFLOP/s, C = 4, with its records in 16-byte
+//     loads, 6.62 -> 6.29 ms.)
 //   * The kernel is bound by instruction dispatch next to the MUFU pipe,
 //     and TMEM lane quarters tie every row to one SMSP, so each SMSP must
 //     carry the same extra work: the MMA issue and key loads are split over
@@ -56,8 +62,9 @@
 //                their k^ rows and key records (TMA) and issues and commits
 //                their MMAs.  Warp 16 also allocates TMEM and loads q^.
 // Key records: for each pair of keys (2t, 2t + 1) the floats
-//   [B_2t, B_2t+1,] v_2t[0], v_2t+1[0], ..., v_2t[C-1], v_2t+1[C-1]
-// (B only without augmented operands).  With folded values (VF: C = 1,
+//   v_2t[0], v_2t+1[0], ..., v_2t[C-1], v_2t+1[C-1]
+// with augmented operands, else for each four keys (4t .. 4t + 3) their B
+// and then, channel by channel, their values.  With folded values (VF: C = 1,
 // fp16 values, augmented operands whose query rows carry the exponent
 // scale c and whose key norm terms carry log2(|v_n| 2^-16), so that
 // 2^S = Phi |v_n| 2^-16 with no multiply), the records of a key tile are
@@ -94,7 +101,6 @@ constexpr int CTRL_WARP0 = 16;     // control warps 16..19, one per SMSP
 constexpr int NCTRL_MAX = 4;
 constexpr int THREADS = (NEXP + NCTRL_MAX) * 32;
 constexpr int NPART = 4;           // column groups (partial sums) per row
-constexpr int MAX_SL = 2;          // TMEM slots of two S buffers
 constexpr uint32_t TMEM_COLS = 512;
 constexpr int MAX_STAGES = NCTRL_MAX;   // one stage per control warp
 // Augmented operands keep q^ in shared memory (two TMEM slots of S).
@@ -140,8 +146,12 @@ struct FmaParams {
 struct __align__(8) FmaBarriers {
     uint64_t qa_ready;          // q^ available to the MMAs
     uint64_t q_free;            // OVL: every MMA of the segment has read q^ (one arrival per control warp)
-    uint64_t s_full[MAX_SL];    // slot phase: both S tiles of a key tile computed
-    uint64_t s_free[MAX_SL];    // slot phase: both S tiles of a key tile in registers
+    // q^ in shared memory: slot sl holds both S tiles of key tiles g = sl
+    // (mod 2); s_full[sl]: they are computed, s_free[sl]: they are in
+    // registers.  q^ in TMEM: s_full[h]: the S tile of query tile h is
+    // computed, s_free[2 h + g % 2]: that of key tile g is in registers.
+    uint64_t s_full[2];
+    uint64_t s_free[4];
     uint64_t kv_full[MAX_STAGES];
     uint64_t kv_empty[MAX_STAGES];
     uint64_t stall;             // test hook: a barrier nothing arrives on
@@ -328,10 +338,8 @@ tc_gauss_fma_kernel(const __grid_constant__ CUtensorMap tm_q,
         mbar_init(&bars->q_free, NCTRL_MAX);
         mbar_init(&bars->stall, 1);
         for (int k = 0; k < NCTRL_MAX; ++k) mbar_init(&bars->drain[k], 1);
-        for (int sl = 0; sl < SL; ++sl) {
-            mbar_init(&bars->s_full[sl], 1);
-            mbar_init(&bars->s_free[sl], NEXP);        // one arrival per exponent warp
-        }
+        for (int i = 0; i < 2; ++i) mbar_init(&bars->s_full[i], 1);
+        for (int i = 0; i < 4; ++i) mbar_init(&bars->s_free[i], NEXP);   // one arrival per exponent warp
         for (int s = 0; s < p.stages; ++s) {
             mbar_init(&bars->kv_full[s], 1);
             mbar_init(&bars->kv_empty[s], 1 + NEXP);  // MMA commit + exponent warps
@@ -464,9 +472,13 @@ tc_gauss_fma_kernel(const __grid_constant__ CUtensorMap tm_q,
                     // completes once per tile of the slot, and tile g reuses the
                     // slot that tile g - SL released.
                     const int g = g0 + j;
-                    const int sl = SL == 2 ? (g & 1) : 0;
-                    const uint32_t full_parity = static_cast<uint32_t>(SL == 2 ? (g >> 1) : g) & 1u;
-                    const uint32_t free_parity = full_parity ^ 1u;
+                    // q^ in TMEM: query tile 0's S tile of key tile g - 1 is in
+                    // registers once s_free[(g - 1) % 2] has completed for it
+                    // (query tile 1's: s_free[2 + ..], waited for below).
+                    const int sl = QSM ? (g & 1) : ((g - 1) & 1);
+                    const uint32_t free_parity =
+                        QSM ? (static_cast<uint32_t>(g >> 1) & 1u) ^ 1u
+                            : static_cast<uint32_t>((g - 1) >> 1) & 1u;
                     const bool ready = __all_sync(
                         0xffffffffu, g < SL ? mbar_test_wait(&bars->kv_full[k], ph)
                                             : mbar_test_wait2(&bars->s_free[sl], free_parity,
@@ -481,7 +493,7 @@ tc_gauss_fma_kernel(const __grid_constant__ CUtensorMap tm_q,
                     }
                     pending = false;
                     tc_fence_after();
-                    const uint32_t d0 = tmem + sl * (2 * BN), d1 = d0 + BN;
+                    const uint32_t d0 = tmem + (QSM ? sl * (2 * BN) : 0), d1 = d0 + BN;
                     if (leader && TF) {
                         // 3xTF32: per K step of 8 coordinates (32 bytes),
                         // hi.lo + lo.hi + hi.hi; the lo blocks follow the
@@ -502,25 +514,48 @@ tc_gauss_fma_kernel(const __grid_constant__ CUtensorMap tm_q,
                         mma_commit(&bars->s_full[sl]);
                         mma_commit(&bars->kv_empty[k]);
                         if (OVL && j + nctrl >= T) mma_commit(&bars->q_free);
-                    } else if (leader) {
-                        for (int h = 0; h < NQ; ++h) {
-                            for (int kk = 0; kk < ksteps; ++kk) {
-                                const uint32_t koff = static_cast<uint32_t>((kk >> 2) * (BN * 128 / 16) + (kk & 3) * 2);
-                                if (QSM) {
+                    } else if (QSM) {
+                        if (leader) {
+                            for (int h = 0; h < NQ; ++h) {
+                                for (int kk = 0; kk < ksteps; ++kk) {
+                                    const uint32_t koff = static_cast<uint32_t>((kk >> 2) * (BN * 128 / 16) + (kk & 3) * 2);
                                     const uint32_t qoff = h * qdesc_h + static_cast<uint32_t>((kk >> 2) * (BM * 128 / 16) + (kk & 3) * 2);
                                     mma_ss_f16(h ? d1 : d0, qdesc0 + qoff, kdesc + koff, p.idesc, kk > 0 ? 1u : 0u);
-                                } else {
+                                }
+                            }
+                            mma_commit(&bars->s_full[sl]);
+                            mma_commit(&bars->kv_empty[k]);
+                            // OVL, the warp's last tile of the segment: q_free
+                            // arrives once these MMAs, and so all of this warp's
+                            // MMAs that read the segment's q^, are complete.
+                            if (OVL && j + nctrl >= T) mma_commit(&bars->q_free);
+                        }
+                    } else {
+                        // One S tile per query tile, each handed over as soon
+                        // as it is done: the exponent warps take query tile
+                        // 0's S while query tile 1's MMAs run, so the MMAs of
+                        // key tile g + 1 follow those of key tile g without a
+                        // gap (one barrier for both S tiles left the tensor
+                        // pipe idle from the last MMA to the TMEM loads).
+                        for (int h = 0; h < NQ; ++h) {
+                            if (h == 1 && g >= 1) {
+                                ok = warp_wait(&bars->s_free[2 + sl], free_parity, abort_flag, p.status);
+                                if (!ok) break;
+                                tc_fence_after();
+                            }
+                            if (leader) {
+                                for (int kk = 0; kk < ksteps; ++kk) {
+                                    const uint32_t koff = static_cast<uint32_t>((kk >> 2) * (BN * 128 / 16) + (kk & 3) * 2);
                                     mma_ts_f16(h ? d1 : d0, (h ? a1 : a0) + kk * 8, kdesc + koff, p.idesc,
                                                kk > 0 ? 1u : 0u);
                                 }
+                                mma_commit(&bars->s_full[h]);
+                                if (h == 1) mma_commit(&bars->kv_empty[k]);
                             }
+                            __syncwarp();
+                            issued = true;
                         }
-                        mma_commit(&bars->s_full[sl]);
-                        mma_commit(&bars->kv_empty[k]);
-                        // OVL, the warp's last tile of the segment: q_free
-                        // arrives once these MMAs, and so all of this warp's
-                        // MMAs that read the segment's q^, are complete.
-                        if (OVL && j + nctrl >= T) mma_commit(&bars->q_free);
+                        if (!ok) break;
                     }
                     __syncwarp();
                     issued = true;
@@ -649,6 +684,7 @@ tc_gauss_fma_kernel(const __grid_constant__ CUtensorMap tm_q,
                 for (int j = 0; j < T; ++j, st.advance(p.stages), sl.advance(SL)) {
                     const int s = st.idx;
                     const uint32_t col0 = static_cast<uint32_t>(sl.idx * 2 * BN);
+                    // (q^ in TMEM: s_full[0], query tile 0's S tile, phase = tile parity.)
                     if (!__all_sync(0xffffffffu, ready || mbar_test_wait2(&bars->kv_full[s], st.phase,
                                                                           &bars->s_full[sl.idx], sl.phase))) {
                         ok = warp_wait(&bars->kv_full[s], st.phase, abort_flag, p.status);
@@ -658,27 +694,38 @@ tc_gauss_fma_kernel(const __grid_constant__ CUtensorMap tm_q,
                     tc_fence_after();
                     uint32_t r0[32], r1[32];
                     tmem_ld_32x32b_x32(tmem + lane_base + col0 + cg * 32, r0);
-                    tmem_ld_32x32b_x32(tmem + lane_base + col0 + BN + cg * 32, r1);
-                    // The wait names r0 and r1, so that no use of the loaded
-                    // values is scheduled above it (the loads land asynchronously).
-                    tmem_wait_ld_regs(r0, r1);
-                    // When and where the S slot is handed back: with two slots
-                    // (q^ in shared memory) only after the exponent work of this
-                    // tile (with the stage, below), because releasing it right
-                    // after the loads let the next MMAs into the slot corrupt S
-                    // values of this tile in some warps when the MMAs were long
-                    // (measured with 3xTF32 operands and three or more stages,
-                    // also with the loads' registers named in the wait; the early
-                    // release was no faster on the 65536^2, D = 64 sum either:
-                    // 0.6428 against 0.6418 ms).
-                    // With one slot (q^ in TMEM) a late release would serialise
-                    // the MMAs and the exponent work, so it is released here; no
-                    // corruption was seen there in repeated runs (regression
-                    // test: repeated calls agree bit for bit).
-                    if (!QSM) {
+                    if (QSM) {
+                        tmem_ld_32x32b_x32(tmem + lane_base + col0 + BN + cg * 32, r1);
+                        // The wait names r0 and r1, so that no use of the loaded
+                        // values is scheduled above it (the loads land asynchronously).
+                        // With two slots (q^ in shared memory) the S slot is handed
+                        // back only after the exponent work of this tile (with the
+                        // stage, below), because releasing it right after the loads
+                        // let the next MMAs into the slot corrupt S values of this
+                        // tile in some warps when the MMAs were long (measured with
+                        // 3xTF32 operands and three or more stages, also with the
+                        // loads' registers named in the wait; the early release was
+                        // no faster on the 65536^2, D = 64 sum either: 0.6428
+                        // against 0.6418 ms).
+                        tmem_wait_ld_regs(r0, r1);
+                    } else {
+                        // q^ in TMEM: one S tile per query tile, handed back as
+                        // soon as it is in registers, since the MMAs of the next
+                        // key tile need it (a late release would serialise MMAs
+                        // and exponent work; regression test: repeated calls
+                        // agree bit for bit).
+                        tmem_wait_ld_regs(r0);
                         tc_fence_before();
                         __syncwarp();
-                        mbar_arrive_if_zero(&bars->s_free[sl.idx], lane);
+                        mbar_arrive_if_zero(&bars->s_free[sl.phase], lane);
+                        ok = warp_wait(&bars->s_full[1], sl.phase, abort_flag, p.status);
+                        if (!ok) break;
+                        tc_fence_after();
+                        tmem_ld_32x32b_x32(tmem + lane_base + BN + cg * 32, r1);
+                        tmem_wait_ld_regs(r1);
+                        tc_fence_before();
+                        __syncwarp();
+                        mbar_arrive_if_zero(&bars->s_free[2 + sl.phase], lane);
                     }
                     // Query the barriers of key tile j + 1 now and read the answer
                     // after the exponent work of tile j: the query latency overlaps
@@ -757,40 +804,41 @@ tc_gauss_fma_kernel(const __grid_constant__ CUtensorMap tm_q,
                             }
                         }
                     } else {
+                        // Quad records: B and then each channel's values of
+                        // four keys, one 16-byte load each.  (In key pairs,
+                        // 8-byte loads, the records took half of the shared-
+                        // memory pipe's wavefronts on 1M keys of D = 256,
+                        // C = 4, next to the 29 % of the MMAs' operand reads.)
         #pragma unroll
-                    for (int t = 0; t < 16; ++t) {
-                        // Keys 32 cg + 2t and + 1, rows row0 (S0) and row1 (S1).
-                        const float* pr = rec + t * REC_PAIR;
-                        float2 bb, v0;
-                        if (C == 1) {
-                            const float4 bv = *reinterpret_cast<const float4*>(pr);
-                            bb = make_float2(bv.x, bv.y);
-                            v0 = make_float2(bv.z, bv.w);
-                        } else {
-                            bb = *reinterpret_cast<const float2*>(pr);
-                            v0 = *reinterpret_cast<const float2*>(pr + 2);
-                        }
-                        const uint64_t b2 = f32x2_pack(bb.x, bb.y);
-                        const uint64_t x01 = f32x2_fma(f32x2_pack(__uint_as_float(r0[2 * t]), __uint_as_float(r0[2 * t + 1])),
-                                                       c2, f32x2_add(b2, a2_0));
-                        const uint64_t y01 = f32x2_fma(f32x2_pack(__uint_as_float(r1[2 * t]), __uint_as_float(r1[2 * t + 1])),
-                                                       c2, f32x2_add(b2, a2_1));
-                        float x0, x1, y0, y1;
-                        f32x2_unpack(x01, x0, x1);
-                        f32x2_unpack(y01, y0, y1);
-                        const uint64_t px = f32x2_pack(ex2_nonpos(x0), ex2_nonpos(x1));
-                        const uint64_t py = f32x2_pack(ex2_nonpos(y0), ex2_nonpos(y1));
-                        const uint64_t vv0 = f32x2_pack(v0.x, v0.y);
-                        acc0[0] = f32x2_fma(px, vv0, acc0[0]);
-                        acc1[0] = f32x2_fma(py, vv0, acc1[0]);
+                        for (int t = 0; t < 8; ++t) {
+                            // Keys 32 cg + 4t .. + 3, rows row0 (S0) and row1 (S1).
+                            const float4* pr = reinterpret_cast<const float4*>(rec + t * (2 * REC_PAIR));
+                            const float4 bb = pr[0];
+                            uint64_t px[2], py[2];
         #pragma unroll
-                        for (int cc = 1; cc < C; ++cc) {
-                            const float2 vc = *reinterpret_cast<const float2*>(pr + 2 + 2 * cc);
-                            const uint64_t vv = f32x2_pack(vc.x, vc.y);
-                            acc0[cc] = f32x2_fma(px, vv, acc0[cc]);
-                            acc1[cc] = f32x2_fma(py, vv, acc1[cc]);
+                            for (int h = 0; h < 2; ++h) {
+                                const uint64_t b2 = h ? f32x2_pack(bb.z, bb.w) : f32x2_pack(bb.x, bb.y);
+                                const int i = 4 * t + 2 * h;
+                                float x0, x1, y0, y1;
+                                f32x2_unpack(f32x2_fma(f32x2_pack(__uint_as_float(r0[i]), __uint_as_float(r0[i + 1])),
+                                                       c2, f32x2_add(b2, a2_0)),
+                                             x0, x1);
+                                f32x2_unpack(f32x2_fma(f32x2_pack(__uint_as_float(r1[i]), __uint_as_float(r1[i + 1])),
+                                                       c2, f32x2_add(b2, a2_1)),
+                                             y0, y1);
+                                px[h] = f32x2_pack(ex2_nonpos(x0), ex2_nonpos(x1));
+                                py[h] = f32x2_pack(ex2_nonpos(y0), ex2_nonpos(y1));
+                            }
+        #pragma unroll
+                            for (int cc = 0; cc < C; ++cc) {
+                                const float4 vc = pr[1 + cc];
+                                const uint64_t v01 = f32x2_pack(vc.x, vc.y), v23 = f32x2_pack(vc.z, vc.w);
+                                acc0[cc] = f32x2_fma(px[0], v01, acc0[cc]);
+                                acc1[cc] = f32x2_fma(py[0], v01, acc1[cc]);
+                                acc0[cc] = f32x2_fma(px[1], v23, acc0[cc]);
+                                acc1[cc] = f32x2_fma(py[1], v23, acc1[cc]);
+                            }
                         }
-                    }
                     }
                     tc_fence_before();
                     __syncwarp();
@@ -846,8 +894,8 @@ tc_gauss_fma_kernel(const __grid_constant__ CUtensorMap tm_q,
 
 size_t align1k(size_t x) { return (x + 1023) & ~static_cast<size_t>(1023); }
 
-// Floats per key pair in the key records: (B_2t, B_2t+1 unless the norms
-// are folded into augmented operands) + both keys' values.
+// Floats per key pair in the key records: both keys' B (unless the norms
+// are folded into augmented operands) and values.
 int rec_pair_floats(int C, bool aug) { return (aug ? 0 : 2) + 2 * C; }
 
 // Key-record bytes of one key tile (VF: the signs and four group words).
@@ -984,14 +1032,16 @@ bool plan_fma_kernel(int Dp, int C, bool aug, bool tf, int* nq, int* stages, siz
     const size_t fixed = fixed_bytes_for(C, q_bytes_for(nkb, qsm));
     if (fixed >= budget) return false;
     // Control warp k owns stage k (stages = control warps) and checks the
-    // S-slot release of key tile j - SL before the MMAs of tile j.  An
+    // S release of an earlier key tile before the MMAs of tile j.  An
     // mbarrier parity test is only unambiguous while the barrier is at most
     // one phase behind the phase it asks about; the warp knows every key
-    // tile up to j - stages is done (its previous stage release), and the
-    // slot's previous phase is tile j - 2 SL, so stages <= 2 SL.
-    const int sl = qsm ? 2 : 1;
+    // tile up to j - stages is done (its previous stage release).  Two slots:
+    // it asks about tile j - 2, the slot's previous phase is tile j - 4, so
+    // stages <= 4.  One S tile per query tile (q^ in TMEM): it asks about
+    // tile j - 1 on the barrier of that tile's parity, whose previous phase
+    // is tile j - 3, so stages <= 3.
     const int st = static_cast<int>(
-        std::min<size_t>(std::min(MAX_STAGES, 2 * sl), (budget - fixed) / stage));
+        std::min<size_t>(qsm ? MAX_STAGES : 3, (budget - fixed) / stage));
     if (st < 2) return false;
     *nq = NQ;
     *stages = st;
