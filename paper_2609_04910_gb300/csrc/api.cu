@@ -218,10 +218,45 @@ bool fp32_on_tensor_cores(const Call& c) {
            c.B * c.M * c.N >= least;
 }
 
+// Wider rows (32 < D <= 64) of large single forward sums also go to the
+// tensor cores, guarded: both paths are launched, and the operand kernel's
+// look at the points decides on the device which one works (see
+// kGuardMaxBits).  From 2^24 pairs, where its extra launches are repaid.
+// Measured on a GB300, whole calls, SIMT / guarded: 16384^2, D = 64, C = 1
+// 1145 / 140 us (the tensor cores' share of the work at three tf32 MMAs per
+// product is 80 us), 8192^2, D = 50 305 / 66 us, 6000^2, D = 64 176 / 57 us.
+// Error against 64 bits (relative, 2-norm, N(0, I) points and values): 1.0 to
+// 6.6e-7, the SIMT kernel's 1.1 to 7.7e-7 on the same inputs.
+constexpr int64_t kFp32GuardedMinPairs = int64_t(1) << 24;
+
+bool fp32_guarded(const Call& c) {
+    return c.dtype == GS_FP32 && c.opt.path == GS_PATH_AUTO && !c.grad && c.B == 1 &&
+           c.C <= gs::kFmaMaxChannels && c.D > gs::kTf32MaxDp && c.D <= gs::kTf32WideMaxDp &&
+           c.M * c.N >= kFp32GuardedMinPairs;
+}
+
 // Plans the call; returns GS_OK and the workspace size, or an error.
 gs_status plan(const Call& c, int sms, bool* tensor, gs::TcPlan* tp, gs::SimtPlan* sp,
                size_t* bytes) {
     const char* why = "unsupported shape";
+    if (fp32_guarded(c) && c.opt.split_n == 0 && c.opt.exp2_fma == 0) {
+        // The guarded pair of paths, unless a caller's workspace holds only
+        // what the SIMT path needs.
+        const bool alias = c.q == c.k && c.M == c.N && c.q != nullptr;
+        if (gs::plan_tensor(gs::InType::F32, c.M, c.N, c.D, c.C, false, c.opt.center != 0, alias, 0,
+                            sms, tp, &why) &&
+            gs::plan_simt(c.M, c.N, c.D, c.C, false, 0, sms, sp, &why)) {
+            sp->off_part = tp->total;
+            *bytes = tp->total + sp->total;
+            if (!c.opt.workspace || c.opt.workspace_bytes >= *bytes) {
+                tp->exp2_fma = 0;
+                tp->cfold = tp->vfold = false;
+                *tensor = true;
+                return GS_OK;
+            }
+        }
+        *tp = gs::TcPlan{};
+    }
     *tensor = c.dtype != GS_FP32 || fp32_on_tensor_cores(c);
     if (*tensor) {
         const bool alias = c.q == c.k && c.M == c.N && c.q != nullptr;
@@ -347,6 +382,13 @@ gs_status run(Call c) {
     if (tensor) {
         const gs::InType t = in_type(c.dtype);
         float* mu = (tp.center && c.D > 0) ? reinterpret_cast<float*>(ws + tp.off_mu) : nullptr;
+        // Guarded sums: the word behind the key records (B and Cv values per key).
+        unsigned* guard = tp.guard ? reinterpret_cast<unsigned*>(ws + tp.off_rec) + tp.Npad * (1 + tp.Cv)
+                                   : nullptr;
+        if (guard && !mu) {
+            e = cudaMemsetAsync(guard, 0, sizeof(unsigned), c.stream);
+            where = "cudaMemsetAsync";
+        }
         // Key records of the FMA kernel with augmented operands depend on the
         // values only: the mean launch writes them where it can.
         bool records_done = false;
@@ -356,7 +398,7 @@ gs_status run(Call c) {
                                         reinterpret_cast<float*>(ws + tp.off_rec), tp.vfold};
             e = gs::launch_mean(t, c.q, c.k, c.M, c.N, static_cast<int>(c.D), tp.mean_blocks,
                                 reinterpret_cast<float*>(ws + tp.off_mean_part), mu, c.stream,
-                                batch, (tp.fma && tp.aug) ? &rec : nullptr, &records_done);
+                                batch, (tp.fma && tp.aug) ? &rec : nullptr, &records_done, guard);
             where = "mean kernel";
         }
         const float ninf = -INFINITY;
@@ -368,14 +410,14 @@ gs_status run(Call c) {
                                       static_cast<int>(c.D), tp.Dp, mu, half_c,
                                       reinterpret_cast<float*>(ws + tp.off_qh),
                                       reinterpret_cast<float*>(ws + tp.off_A), ninf, c.stream,
-                                      batch);
+                                      batch, guard);
             where = "tf32 split kernel (q)";
             if (e == cudaSuccess && !tp.alias) {
                 e = gs::launch_tf32_split(static_cast<const float*>(c.k), c.N, tp.Npad,
                                           static_cast<int>(c.D), tp.Dp, mu, half_c,
                                           reinterpret_cast<float*>(ws + tp.off_kh),
                                           reinterpret_cast<float*>(ws + tp.off_B), ninf,
-                                          c.stream, batch);
+                                          c.stream, batch, guard);
                 where = "tf32 split kernel (k)";
             }
         } else {
@@ -425,8 +467,21 @@ gs_status run(Call c) {
                                               c.M, static_cast<int>(tp.Cv), 128 * tp.nq,
                                               tp.Npad / tp.BN, tp.unit_len, c.out, c.stream,
                                               batch, tp.band_len > 0 ? tp.splits : 0,
-                                              tp.tri ? tp.Npad / tp.BN : 0);
+                                              tp.tri ? tp.Npad / tp.BN : 0, guard);
                 where = "finalise kernel";
+            }
+            if (e == cudaSuccess && guard) {
+                // The other side of the guard.
+                float* part = reinterpret_cast<float*>(ws + sp.off_part);
+                e = gs::launch_simt(sp, false, static_cast<const float*>(c.q),
+                                    static_cast<const float*>(c.k), static_cast<const float*>(c.v),
+                                    static_cast<int>(c.C), 0, half_c, part, c.stream, guard);
+                where = "fp32 kernel";
+                if (e == cudaSuccess) {
+                    e = gs::launch_finalize(part, sp.splits, c.M, c.M, static_cast<int>(sp.Cv),
+                                            static_cast<int>(sp.Cv), nullptr, c.out, c.stream, 0, guard);
+                    where = "finalise kernel";
+                }
             }
         } else if (e == cudaSuccess) {
             // Two-MMA kernel, once per chunk of value channels (one chunk for
@@ -599,11 +654,13 @@ namespace gs {
 
 gs_status forward_workspace_bytes(const void* q, const void* k, const void* v, double tau,
                                   int64_t M, int64_t N, int64_t D, int64_t C, gs_dtype dtype,
-                                  float* out, size_t* bytes) {
+                                  float* out, void* workspace, size_t limit, size_t* bytes) {
     Call c{q, k, v, tau, M, N, D, C, dtype, false, out, nullptr, nullptr, defaults()};
     *bytes = 0;
     gs_status st = validate(c);
     if (st != GS_OK) return st;
+    c.opt.workspace = workspace;
+    c.opt.workspace_bytes = limit;
     if (M == 0 || N == 0 || C == 0) return GS_OK;
     int dev = 0;
     unsigned* status = nullptr;

@@ -47,6 +47,16 @@ constexpr int kFmaMaxChannels = 4;
 // four channels when the augmented rows fit (plan_tensor, tc_gauss.cu).
 constexpr int64_t kTwoMmaMinPairs = int64_t(1) << 28;
 
+// Guard of fp32 sums of wide rows.  The tensor cores form the exponent as
+// c q^.k^ + A_m + B_n from the points' norms, the SIMT kernel from coordinate
+// differences; the first is as accurate only while the norm terms stay small
+// (its error is a few units in the last place of |A_m| + |B_n|, whatever the
+// distance).  The operand kernel writes the bits of the largest
+// (c/2)||x - mu||^2 of the call; up to 4.0 the tensor-core kernels work and
+// above it (or NaN, whose bits are larger still) the SIMT kernels do.  Points
+// ~ N(0, I_D) with tau = 1/D stay below 2.
+constexpr unsigned kGuardMaxBits = 0x40800000u;   // 4.0f
+
 // Workspace plan of the tensor-core path.  All offsets are bytes from the
 // workspace base and are 1024-byte aligned.
 struct TcPlan {
@@ -76,6 +86,11 @@ struct TcPlan {
                              // rounded to 16)
     bool tf;                 // fp32 inputs on the FMA kernel with 3xTF32 MMAs: q^ and k^
                              // rows are [hi | lo] of Dp (a multiple of 32) floats each
+    // 3xTF32 with a guard (rows of more than kTf32MaxDp coordinates): the
+    // kernels of the tensor-core path and of the SIMT path are both launched,
+    // and a word written with the operands (kGuardMaxBits) says which of
+    // them work; the others return at once.
+    bool guard;
     int nq;                  // query tiles of 128 rows per CTA (FMA kernel)
     bool early_s;            // two-MMA kernel: S buffers handed back as soon as they are
                              // in registers (exponent-bound shapes), else with P
@@ -159,12 +174,15 @@ struct RecordArgs {
     bool signs;          // sign records of folded value magnitudes (fp16 values, C = 1;
                          // per key tile of 128 keys: 128 signed 2^16 and 4 group words)
 };
+// With zero_word, the launch also clears that word (before any later kernel
+// of the call).
 // Common mean of q and k per problem.  With `rec`, the launch also writes
 // those key records where it can (the vectorised path); *rec_done says
 // whether it did.
 cudaError_t launch_mean(InType t, const void* q, const void* k, int64_t M, int64_t N, int D,
                         int blocks, float* partial, float* mu, cudaStream_t s, int batch = 1,
-                        const RecordArgs* rec = nullptr, bool* rec_done = nullptr);
+                        const RecordArgs* rec = nullptr, bool* rec_done = nullptr,
+                        unsigned* zero_word = nullptr);
 // (cf > 0 with vw: the exponent scale c folds into the query rows and the
 // magnitudes of the fp16 values vw into the key rows' norm terms;
 // vf_rec: sign records already written, whose per-problem flags the launch
@@ -206,7 +224,8 @@ cudaError_t launch_weight_prep(InType t, const void* rsrc, bool r_f32, int64_t R
 // in split order; rows below main_rows have one split.
 cudaError_t launch_finalize(const float* part, int splits, int64_t split_stride_rows,
                             int64_t M, int Cv, int part_ld, const float* inv_scale, float* out,
-                            cudaStream_t s, int64_t main_rows = 0);
+                            cudaStream_t s, int64_t main_rows = 0,
+                            const unsigned* guard = nullptr);
 // Gradient contraction of one launch's channels ch0 .. ch0 + Cc - 1 (see
 // prep.cu): out[m, d] (+)= tau sum_c u[m, c] (S_{c,d} - x^_{m,d} S_{c,D}),
 // s_out[m, c] = S_{c,D}.  direct: fp32 kernel partials (difference form).
@@ -232,14 +251,15 @@ cudaError_t launch_mmd2_reduce(InType t, const float* s, const void* v, int64_t 
 cudaError_t launch_finalize_slots(const float* part, int64_t Mpad, int64_t M, int C,
                                   int rows_per_unit, int64_t key_tiles, int64_t unit_len,
                                   float* out, cudaStream_t s, int batch = 1,
-                                  int fixed_slots = 0, int64_t tri_key_tiles = 0);
+                                  int fixed_slots = 0, int64_t tri_key_tiles = 0,
+                                  const unsigned* guard = nullptr);
 
 // simt_fp32.cu ---------------------------------------------------------
 // grad: keys weighted by channel wch of v (N x Cw); partials have D + 1
 // channels (sum Phi w (k - q), sum Phi w).
 cudaError_t launch_simt(const SimtPlan& p, bool grad, const float* q, const float* k,
                         const float* v, int Cw, int wch, float half_c, float* part,
-                        cudaStream_t s);
+                        cudaStream_t s, const unsigned* guard = nullptr);
 
 // Key records of the FMA kernel: without B per key pair (2t, 2t+1) the floats
 // v_2t[0], v_2t+1[0], ..., v_2t[C-1], v_2t+1[C-1]; with B per four keys their
@@ -250,7 +270,8 @@ cudaError_t launch_key_records(InType t, const void* v, const float* B, int64_t 
 // [hi | lo] into out, nrm = -(c/2)||x - mu||^2 (pad_value for padded rows).
 cudaError_t launch_tf32_split(const float* x, int64_t rows, int64_t rows_pad, int D, int Dp,
                               const float* mu, float half_c, float* out, float* nrm,
-                              float pad_value, cudaStream_t s, int batch = 1);
+                              float pad_value, cudaStream_t s, int batch = 1,
+                              unsigned* guard = nullptr);
 constexpr int aug_norm_terms(InType t) { return t == InType::BF16 ? 3 : 2; }
 
 // tc_gauss.cu ----------------------------------------------------------
@@ -261,9 +282,11 @@ cudaError_t launch_tc(const TcPlan& p, InType t, float c, char* ws, unsigned* st
 // Largest (augmented) Dp for which the FMA kernel keeps q^ in shared memory
 // and folds the norms into the MMA.
 constexpr int kAugMaxDp = 128;
-// Largest D of the 3xTF32 (fp32) variant: q^ hi and lo tiles of two query
-// tiles stay in shared memory next to the key stages.
+// Largest D of the 3xTF32 (fp32) variant whose q^ hi and lo tiles of two
+// query tiles stay in shared memory next to the key stages; and the largest
+// D of the one that keeps them in tensor memory.
 constexpr int kTf32MaxDp = 32;
+constexpr int kTf32WideMaxDp = 64;
 bool plan_fma_kernel(int Dp, int C, bool aug, bool tf, int* nq, int* stages, size_t* smem);
 // vf_pass (plans with vfold): 1 = the problems whose 32-key groups all have
 // values of one sign, 2 = the others (launched after pass 1); 0 otherwise.
@@ -279,12 +302,12 @@ cudaError_t launch_vf_flags(float* rec, int64_t Npad, int batch, cudaStream_t s)
 // (mix false), or the FMA kernel's exponent-loop instruction mix (true).
 cudaError_t run_ex2_probe(cudaStream_t s, double* rate, bool mix);
 
-// api.cu: workspace bytes that a forward call with exactly these arguments
-// and default options needs (through *bytes), or the status the call
-// would fail with; and recording a message for gauss_sum_last_error().
+// api.cu: workspace bytes that a forward call with exactly these arguments,
+// default options and a workspace of `limit` bytes needs (through *bytes), or
+// the status the call would fail with; and recording a message for gauss_sum_last_error().
 gs_status forward_workspace_bytes(const void* q, const void* k, const void* v, double tau,
                                   int64_t M, int64_t N, int64_t D, int64_t C, gs_dtype dtype,
-                                  float* out, size_t* bytes);
+                                  float* out, void* workspace, size_t limit, size_t* bytes);
 gs_status set_last_error(gs_status st, const char* msg);
 // Adds n to the count behind gauss_sum_kernel_launches(); called right
 // after each kernel launch of the library.

@@ -69,8 +69,11 @@ cudaError_t scratch_for_current_device(void** ptr) {
 extern "C" gs_status gauss_sum_noalloc(const void* q, const void* k, const void* v, double tau,
                                        int64_t M, int64_t N, int64_t D, int64_t C,
                                        gs_dtype dtype, float* out, void* stream) {
+    void* scratch = nullptr;
+    cudaError_t e = scratch_for_current_device(&scratch);
     size_t need = 0;
-    gs_status st = gs::forward_workspace_bytes(q, k, v, tau, M, N, D, C, dtype, out, &need);
+    gs_status st = gs::forward_workspace_bytes(q, k, v, tau, M, N, D, C, dtype, out, scratch,
+                                               GS_NOALLOC_SCRATCH_BYTES, &need);
     if (st != GS_OK) return st;
     if (need > static_cast<size_t>(GS_NOALLOC_SCRATCH_BYTES)) {
         char msg[200];
@@ -80,8 +83,6 @@ extern "C" gs_status gauss_sum_noalloc(const void* q, const void* k, const void*
                       need, static_cast<size_t>(GS_NOALLOC_SCRATCH_BYTES));
         return gs::set_last_error(GS_ERR_UNSUPPORTED, msg);
     }
-    void* scratch = nullptr;
-    cudaError_t e = scratch_for_current_device(&scratch);
     if (e != cudaSuccess) {
         char msg[200];
         std::snprintf(msg, sizeof(msg), "gauss_sum_noalloc: cudaGetSymbolAddress failed: %s",

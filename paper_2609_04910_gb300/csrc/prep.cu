@@ -288,9 +288,11 @@ constexpr int kMeanFinalThreadMax = 32;
 
 __global__ void __launch_bounds__(kMeanFinalThreads)
 mean_final_block_kernel(const float* __restrict__ partial, int G, int D, float total,
-                        int mant_bits, int min_exp, float* __restrict__ mu) {
+                        int mant_bits, int min_exp, float* __restrict__ mu,
+                        unsigned* __restrict__ zero_word) {
     pdl_trigger();
     pdl_wait();
+    if (zero_word && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *zero_word = 0u;
     constexpr int W = kMeanFinalThreads / 32;
     __shared__ float red_s[W];
     __shared__ float red_m[W];
@@ -328,9 +330,11 @@ mean_final_block_kernel(const float* __restrict__ partial, int G, int D, float t
 // per item = (problem b, coordinate d), folding the G partials in order.
 __global__ void __launch_bounds__(kMeanFinalThreads)
 mean_final_kernel(const float* __restrict__ partial, int G, int D, int64_t items, float total,
-                  int mant_bits, int min_exp, float* __restrict__ mu) {
+                  int mant_bits, int min_exp, float* __restrict__ mu,
+                  unsigned* __restrict__ zero_word) {
     pdl_trigger();
     pdl_wait();
+    if (zero_word && blockIdx.x == 0 && threadIdx.x == 0) *zero_word = 0u;
     const int64_t it = static_cast<int64_t>(blockIdx.x) * kMeanFinalThreads + threadIdx.x;
     if (it >= items) return;
     const int64_t b = it / D;
@@ -541,37 +545,59 @@ operand_kernel(const T* __restrict__ x, int64_t rows, int64_t rows_pad, int D, i
 __global__ void tf32_split_kernel(const float* __restrict__ x, int64_t rows, int64_t rows_pad,
                                   int64_t total_rows, int D, int Dp,
                                   const float* __restrict__ mu, float half_c, float pad_value,
-                                  float* __restrict__ out, float* __restrict__ nrm) {
+                                  float* __restrict__ out, float* __restrict__ nrm,
+                                  unsigned* __restrict__ guard) {
     pdl_trigger();
     pdl_wait();
+    // guard: the largest (c/2) ||x - mu||^2, as the bits of a non-negative
+    // float (or of a NaN, above them all), which order like the floats.
+    __shared__ unsigned big;
+    if (guard) {
+        if (threadIdx.x == 0) big = 0u;
+        __syncthreads();
+    }
     const int64_t w = (static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
-    if (w >= total_rows) return;
-    const int64_t b = w / rows_pad;
-    const int64_t r = w - b * rows_pad;
-    const bool valid = r < rows;
-    const float* xr = x + (b * rows + r) * D;
-    const float* mb = mu ? mu + b * D : nullptr;
-    float* o = out + w * 2 * Dp;
-    float acc = 0.f;
-    for (int d = lane; d < Dp; d += 32) {
-        const float xv = (valid && d < D) ? xr[d] - (mb ? mb[d] : 0.f) : 0.f;
-        const float hi = round_tf32(xv);
-        o[d] = hi;
-        o[Dp + d] = round_tf32(xv - hi);
-        acc = fmaf(xv, xv, acc);
-    }
+    if (w < total_rows) {
+        const int64_t b = w / rows_pad;
+        const int64_t r = w - b * rows_pad;
+        const bool valid = r < rows;
+        const float* xr = x + (b * rows + r) * D;
+        const float* mb = mu ? mu + b * D : nullptr;
+        float* o = out + w * 2 * Dp;
+        float acc = 0.f;
+        for (int d = lane; d < Dp; d += 32) {
+            const float xv = (valid && d < D) ? xr[d] - (mb ? mb[d] : 0.f) : 0.f;
+            const float hi = round_tf32(xv);
+            o[d] = hi;
+            o[Dp + d] = round_tf32(xv - hi);
+            acc = fmaf(xv, xv, acc);
+        }
 #pragma unroll
-    for (int s = 16; s > 0; s >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, s);
-    if (lane == 0) nrm[w] = valid ? -half_c * acc : pad_value;
+        for (int s = 16; s > 0; s >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, s);
+        if (lane == 0) {
+            nrm[w] = valid ? -half_c * acc : pad_value;
+            if (guard && valid) atomicMax(&big, __float_as_uint(half_c * acc) & 0x7fffffffu);
+        }
+    }
+    if (guard) {
+        __syncthreads();
+        if (threadIdx.x == 0) atomicMax(guard, big);
+    }
 }
+
+// Guarded sums (see kGuardMaxBits): whether the call's points exceed the
+// tensor-core path's range.  Read after pdl_wait only.
+__device__ __forceinline__ bool guard_above(const unsigned* guard) { return *guard > kGuardMaxBits; }
 
 __global__ void finalize_slots_kernel(const float* __restrict__ part, int64_t Mpad, int64_t M,
                                       int C, int rows_per_unit, int64_t key_tiles,
                                       int64_t unit_len, int64_t batch, int fixed_slots,
-                                      int64_t tri_kt, float* __restrict__ out) {
+                                      int64_t tri_kt, float* __restrict__ out,
+                                      const unsigned* __restrict__ guard) {
     pdl_trigger();
     pdl_wait();
+    if (guard && guard_above(guard)) return;   // the SIMT path's sums count
     // out: batch x M x C; partial rows are batch-stacked with Mpad rows per
     // problem and batch Mpad rows per slot.
     const int64_t idx = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
@@ -1135,9 +1161,10 @@ weight_prep_kernel(const TR* __restrict__ rsrc, int64_t R, int64_t Rpad,
 __global__ void finalize_kernel(const float* __restrict__ part, int splits,
                                 int64_t split_stride_rows, int64_t M, int Cv, int part_ld,
                                 const float* __restrict__ inv_scale, float* __restrict__ out,
-                                int64_t main_rows) {
+                                int64_t main_rows, const unsigned* __restrict__ guard) {
     pdl_trigger();
     pdl_wait();
+    if (guard && !guard_above(guard)) return;   // the tensor-core path's sums count
     const int64_t idx = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
     if (idx >= M * Cv) return;
     const int64_t m = div_nonneg(idx, Cv);
@@ -1265,7 +1292,7 @@ cudaError_t finalize_points_typed(const float* part, int splits, int64_t stride_
 
 cudaError_t launch_mean(InType t, const void* q, const void* k, int64_t M, int64_t N, int D,
                         int blocks, float* partial, float* mu, cudaStream_t s, int batch,
-                        const RecordArgs* rec, bool* rec_done) {
+                        const RecordArgs* rec, bool* rec_done, unsigned* zero_word) {
     if (rec_done) *rec_done = false;
     // q and k the same points: the mean of [q; q] is the mean of q.
     if (q == k && M == N) N = 0;
@@ -1330,13 +1357,13 @@ cudaError_t launch_mean(InType t, const void* q, const void* k, int64_t M, int64
     const int min_exp = t == InType::F16 ? -24 : t == InType::BF16 ? -133 : -149;
     if (G > kMeanFinalThreadMax) {
         launch_kernel(mean_final_block_kernel, dim3(D, batch), kMeanFinalThreads, 0, s, partial,
-                      G, D, static_cast<float>(total), mant_bits, min_exp, mu);
+                      G, D, static_cast<float>(total), mant_bits, min_exp, mu, zero_word);
     } else {
         const int64_t items = static_cast<int64_t>(batch) * D;
         launch_kernel(mean_final_kernel,
                       dim3(static_cast<unsigned>((items + kMeanFinalThreads - 1) / kMeanFinalThreads)),
                       kMeanFinalThreads, 0, s, partial, G, D, items, static_cast<float>(total),
-                      mant_bits, min_exp, mu);
+                      mant_bits, min_exp, mu, zero_word);
     }
     note_launches(1);
     return cudaGetLastError();
@@ -1422,13 +1449,13 @@ cudaError_t launch_mmd2_reduce(InType t, const float* s, const void* v, int64_t 
 cudaError_t launch_finalize_slots(const float* part, int64_t Mpad, int64_t M, int C,
                                   int rows_per_unit, int64_t key_tiles, int64_t unit_len,
                                   float* out, cudaStream_t s, int batch, int fixed_slots,
-                                  int64_t tri_key_tiles) {
+                                  int64_t tri_key_tiles, const unsigned* guard) {
     const int64_t total = static_cast<int64_t>(batch) * M * C;
     if (total == 0) return cudaSuccess;
     const int threads = 256;
     launch_kernel(finalize_slots_kernel, static_cast<unsigned>((total + threads - 1) / threads), threads, 0, s, 
         part, Mpad, M, C, rows_per_unit, key_tiles, unit_len, static_cast<int64_t>(batch),
-        fixed_slots, tri_key_tiles, out);
+        fixed_slots, tri_key_tiles, out, guard);
     note_launches(1);
     return cudaGetLastError();
 }
@@ -1469,13 +1496,13 @@ cudaError_t launch_operands(InType t, bool aug, const void* q, int64_t M, int64_
 
 cudaError_t launch_tf32_split(const float* x, int64_t rows, int64_t rows_pad, int D, int Dp,
                               const float* mu, float half_c, float* out, float* nrm,
-                              float pad_value, cudaStream_t s, int batch) {
+                              float pad_value, cudaStream_t s, int batch, unsigned* guard) {
     const int64_t total = rows_pad * batch;
     if (total == 0) return cudaSuccess;
     const int threads = 256;
     const int64_t blocks = (total * 32 + threads - 1) / threads;
     launch_kernel(tf32_split_kernel, static_cast<unsigned>(blocks), threads, 0, s, 
-        x, rows, rows_pad, total, D, Dp, mu, half_c, pad_value, out, nrm);
+        x, rows, rows_pad, total, D, Dp, mu, half_c, pad_value, out, nrm, guard);
     note_launches(1);
     return cudaGetLastError();
 }
@@ -1571,13 +1598,13 @@ cudaError_t launch_weight_prep(InType t, const void* rsrc, bool r_f32, int64_t R
 
 cudaError_t launch_finalize(const float* part, int splits, int64_t split_stride_rows,
                             int64_t M, int Cv, int part_ld, const float* inv_scale, float* out,
-                            cudaStream_t s, int64_t main_rows) {
+                            cudaStream_t s, int64_t main_rows, const unsigned* guard) {
     const int64_t total = M * Cv;
     if (total == 0) return cudaSuccess;
     const int threads = 256;
     const int64_t blocks = (total + threads - 1) / threads;
     launch_kernel(finalize_kernel, static_cast<unsigned>(blocks), threads, 0, s, 
-        part, splits, split_stride_rows, M, Cv, part_ld, inv_scale, out, main_rows);
+        part, splits, split_stride_rows, M, Cv, part_ld, inv_scale, out, main_rows, guard);
     note_launches(1);
     return cudaGetLastError();
 }

@@ -64,9 +64,11 @@ template <int DMAX, int CBLK>
 __global__ void __launch_bounds__(THREADS, min_blocks(DMAX, CBLK))
 simt_sum_kernel(const float* __restrict__ q, const float* __restrict__ k,
                 const float* __restrict__ v, int64_t M, int64_t N, int D, int Cv, float half_c,
-                int64_t keys_per_split, float* __restrict__ part) {
+                int64_t keys_per_split, float* __restrict__ part,
+                const unsigned* __restrict__ guard) {
     pdl_trigger();
     pdl_wait();
+    if (guard && *guard <= kGuardMaxBits) return;   // the tensor-core path does the call
     constexpr int L = lanes_per_group(DMAX);
     constexpr int DL = DMAX / L;          // coordinates per lane
     constexpr int OWN = ROWS / L;         // rows whose sums a lane keeps
@@ -289,12 +291,13 @@ cudaError_t launch_grad(const SimtPlan& p, const float* q, const float* k, const
 
 template <int DMAX, int CBLK>
 cudaError_t launch_cblk(const SimtPlan& p, const float* q, const float* k, const float* v,
-                        float half_c, float* part, cudaStream_t s) {
+                        float half_c, float* part, cudaStream_t s, const unsigned* guard) {
     constexpr int rows = THREADS / lanes_per_group(DMAX) * ROWS;
     dim3 grid(static_cast<unsigned>((p.M + rows - 1) / rows), p.splits,
               static_cast<unsigned>((p.Cv + CBLK - 1) / CBLK));
     launch_kernel(simt_sum_kernel<DMAX, CBLK>, grid, THREADS, 0, s, q, k, v, p.M, p.N,
-                  static_cast<int>(p.D), static_cast<int>(p.Cv), half_c, p.keys_per_split, part);
+                  static_cast<int>(p.D), static_cast<int>(p.Cv), half_c, p.keys_per_split, part,
+                  guard);
     note_launches(1);
     return cudaGetLastError();
 }
@@ -302,10 +305,10 @@ cudaError_t launch_cblk(const SimtPlan& p, const float* q, const float* k, const
 // Channel blocks of 4, or of 1 or 2 for as few channels (no idle FMAs).
 template <int DMAX>
 cudaError_t launch_dmax(const SimtPlan& p, const float* q, const float* k, const float* v,
-                        float half_c, float* part, cudaStream_t s) {
-    if (p.cblk == 1) return launch_cblk<DMAX, 1>(p, q, k, v, half_c, part, s);
-    if (p.cblk == 2) return launch_cblk<DMAX, 2>(p, q, k, v, half_c, part, s);
-    return launch_cblk<DMAX, 4>(p, q, k, v, half_c, part, s);
+                        float half_c, float* part, cudaStream_t s, const unsigned* guard) {
+    if (p.cblk == 1) return launch_cblk<DMAX, 1>(p, q, k, v, half_c, part, s, guard);
+    if (p.cblk == 2) return launch_cblk<DMAX, 2>(p, q, k, v, half_c, part, s, guard);
+    return launch_cblk<DMAX, 4>(p, q, k, v, half_c, part, s, guard);
 }
 
 }  // namespace
@@ -372,7 +375,7 @@ bool plan_simt(int64_t M, int64_t N, int64_t D, int64_t C, bool grad, int split_
 
 cudaError_t launch_simt(const SimtPlan& p, bool grad, const float* q, const float* k,
                         const float* v, int Cw, int wch, float half_c, float* part,
-                        cudaStream_t s) {
+                        cudaStream_t s, const unsigned* guard) {
     if (grad) {
         switch (p.dmax) {
             case 16: return launch_grad<16>(p, q, k, v, Cw, wch, half_c, part, s);
@@ -381,14 +384,14 @@ cudaError_t launch_simt(const SimtPlan& p, bool grad, const float* q, const floa
         }
     }
     switch (p.dmax) {
-        case 4: return launch_dmax<4>(p, q, k, v, half_c, part, s);
-        case 8: return launch_dmax<8>(p, q, k, v, half_c, part, s);
-        case 16: return launch_dmax<16>(p, q, k, v, half_c, part, s);
-        case 24: return launch_dmax<24>(p, q, k, v, half_c, part, s);
-        case 32: return launch_dmax<32>(p, q, k, v, half_c, part, s);
-        case 48: return launch_dmax<48>(p, q, k, v, half_c, part, s);
-        case 64: return launch_dmax<64>(p, q, k, v, half_c, part, s);
-        default: return launch_dmax<128>(p, q, k, v, half_c, part, s);
+        case 4: return launch_dmax<4>(p, q, k, v, half_c, part, s, guard);
+        case 8: return launch_dmax<8>(p, q, k, v, half_c, part, s, guard);
+        case 16: return launch_dmax<16>(p, q, k, v, half_c, part, s, guard);
+        case 24: return launch_dmax<24>(p, q, k, v, half_c, part, s, guard);
+        case 32: return launch_dmax<32>(p, q, k, v, half_c, part, s, guard);
+        case 48: return launch_dmax<48>(p, q, k, v, half_c, part, s, guard);
+        case 64: return launch_dmax<64>(p, q, k, v, half_c, part, s, guard);
+        default: return launch_dmax<128>(p, q, k, v, half_c, part, s, guard);
     }
 }
 

@@ -670,6 +670,7 @@ bool plan_tensor(InType t, int64_t M, int64_t N, int64_t D, int64_t C, bool grad
     p->alias = alias;
     p->center = center;
     p->tf = false;
+    p->guard = false;
     p->early_s = false;
     p->tri = false;
     p->tri_units = 0;
@@ -684,13 +685,15 @@ bool plan_tensor(InType t, int64_t M, int64_t N, int64_t D, int64_t C, bool grad
     if (t == InType::F32) {
         // fp32 inputs on the tensor cores: the FMA kernel with 3xTF32 MMAs
         // (forward sum, few channels, small D).
-        if (grad || p->Cv > kFmaMaxChannels || D > kTf32MaxDp) {
+        // (More than kTf32MaxDp coordinates: single problems, guarded.)
+        if (grad || p->Cv > kFmaMaxChannels || D > kTf32WideMaxDp || (D > kTf32MaxDp && batch > 1)) {
             *why = "the fp32 tensor-core path takes the forward sum with C <= 4 and D <= 32";
             return false;
         }
         p->tf = true;
         p->aug = false;
-        p->Dp = 32;
+        p->Dp = D <= kTf32MaxDp ? kTf32MaxDp : kTf32WideMaxDp;
+        p->guard = D > kTf32MaxDp;
         if (!plan_fma_kernel(p->Dp, static_cast<int>(p->Cv), false, true, &nq, &fma_stages,
                              &fma_smem)) {
             *why = "shared-memory budget exceeded";
@@ -936,7 +939,7 @@ bool plan_tensor(InType t, int64_t M, int64_t N, int64_t D, int64_t C, bool grad
         // when the value magnitudes are folded) 132 floats per key tile.
         size_t rec_floats = static_cast<size_t>(p->Npad / 2) * ((p->aug ? 0 : 2) + 2 * p->Cv);
         if (p->aug && p->Cv == 1) rec_floats = std::max<size_t>(rec_floats, (p->Npad / 128) * 132);
-        // (+ one word per problem: the folded-value pass flags.)
+        // (+ one word per problem: the folded-value pass flags, or the guard.)
         p->off_rec = take(static_cast<size_t>(B) * (rec_floats + 1) * 4);
         p->off_part = take(static_cast<size_t>(p->splits) * B * p->Mpad * p->Cv * 4);
     } else {

@@ -274,7 +274,9 @@ __global__ void __launch_bounds__(THREADS, 1)
 tc_gauss_fma_kernel(const __grid_constant__ CUtensorMap tm_q,
                     const __grid_constant__ CUtensorMap tm_k, const FmaParams p) {
     // TF (3xTF32): q^ in shared memory, norm terms from A and the records.
-    static_assert(!TF || (QSM && !AUG), "3xTF32 runs with q^ in shared memory");
+    // TF without QSM: q^ in TMEM, guarded (the call's points may be left to
+    // the SIMT path, see kGuardMaxBits).
+    static_assert(!TF || !AUG, "3xTF32 takes plain rows");
     static_assert(!OVL || QSM, "overlapped segments keep q^ in shared memory");
     static_assert(VF == 0 || (AUG && SOFT == 0 && !TF), "folded operands: augmented fp16 rows");
     static_assert(VF != 1 || C == 1, "folded values: one channel");
@@ -297,6 +299,12 @@ tc_gauss_fma_kernel(const __grid_constant__ CUtensorMap tm_q,
     volatile int* abort_flag = &bars->abort_flag;
 
     pdl_trigger();
+    if (TF && !QSM) {
+        // Guarded sums: the word follows the key records.
+        pdl_wait();
+        const int64_t rec_floats = static_cast<int64_t>(p.npad / 2) * REC_PAIR;
+        if (*reinterpret_cast<const unsigned*>(p.rec + rec_floats) > kGuardMaxBits) return;
+    }
     if (VF == 2) {
         // The second folded-value pass often has nothing to do (every problem
         // of the call went to the first): a CTA none of whose segments is of
@@ -321,6 +329,7 @@ tc_gauss_fma_kernel(const __grid_constant__ CUtensorMap tm_q,
     tc_fence_after();
     const uint32_t tmem = bars->tmem_base;
     const uint32_t qa_col = static_cast<uint32_t>(2 * SL * BN);   // TMEM q^ (not QSM)
+    const int q_cols = TF ? 2 * p.Dp : p.Dp / 2;                  // its columns per query tile
 
     auto kh_smem = [&](int s) { return stage0 + s * p.stage_bytes; };
     auto rec_smem = [&](int s) {
@@ -464,7 +473,7 @@ tc_gauss_fma_kernel(const __grid_constant__ CUtensorMap tm_q,
                 const uint64_t kdesc = smem_desc_kmajor_sw128(smem_u32(kh_smem(k)));
                 const uint64_t qdesc0 = smem_desc_kmajor_sw128(smem_u32(q_smem));
                 const uint32_t qdesc_h = static_cast<uint32_t>((p.nkb * BM * 128) >> 4);
-                const uint32_t a0 = tmem + qa_col, a1 = a0 + (p.Dp / 2);
+                const uint32_t a0 = tmem + qa_col, a1 = a0 + q_cols;
                 bool pending = ok;            // keys of tile j requested, not yet waited for
                 int j = j_first;
                 for (; ok && j < T; j += nctrl, ph ^= 1u) {
@@ -494,7 +503,7 @@ tc_gauss_fma_kernel(const __grid_constant__ CUtensorMap tm_q,
                     pending = false;
                     tc_fence_after();
                     const uint32_t d0 = tmem + (QSM ? sl * (2 * BN) : 0), d1 = d0 + BN;
-                    if (leader && TF) {
+                    if (leader && TF && QSM) {
                         // 3xTF32: per K step of 8 coordinates (32 bytes),
                         // hi.lo + lo.hi + hi.hi; the lo blocks follow the
                         // hi blocks (nkb / 2 of each).
@@ -543,7 +552,20 @@ tc_gauss_fma_kernel(const __grid_constant__ CUtensorMap tm_q,
                                 if (!ok) break;
                                 tc_fence_after();
                             }
-                            if (leader) {
+                            if (leader && TF) {
+                                // 3xTF32 as above, A = [hi | lo] from TMEM.
+                                const uint32_t klo = static_cast<uint32_t>((p.nkb / 2) * (BN * 128 / 16));
+                                const uint32_t d = h ? d1 : d0, a = h ? a1 : a0;
+                                for (int kk = 0; kk < ksteps; ++kk) {
+                                    const uint64_t kd = kdesc + (kk >> 2) * (BN * 128 / 16) +
+                                                        static_cast<uint32_t>((kk & 3) * 2);
+                                    mma_ts_tf32(d, a + kk * 8, kd + klo, p.idesc, kk > 0 ? 1u : 0u);
+                                    mma_ts_tf32(d, a + p.Dp + kk * 8, kd, p.idesc, 1u);
+                                    mma_ts_tf32(d, a + kk * 8, kd, p.idesc, 1u);
+                                }
+                                mma_commit(&bars->s_full[h]);
+                                if (h == 1) mma_commit(&bars->kv_empty[k]);
+                            } else if (leader) {
                                 for (int kk = 0; kk < ksteps; ++kk) {
                                     const uint32_t koff = static_cast<uint32_t>((kk >> 2) * (BN * 128 / 16) + (kk & 3) * 2);
                                     mma_ts_f16(h ? d1 : d0, (h ? a1 : a0) + kk * 8, kdesc + koff, p.idesc,
@@ -642,14 +664,14 @@ tc_gauss_fma_kernel(const __grid_constant__ CUtensorMap tm_q,
 
             if (!QSM) {
                 // q^ rows -> TMEM (A operand).  Column group cg copies query tile
-                // cg / 2, 8-column chunks ck = cg % 2 (mod 2) of its Dp / 2 columns.
+                // cg / 2, 8-column chunks ck = cg % 2 (mod 2) of its q_cols columns.
                 const int h = cg >> 1;
-                const uint32_t* src = p.qh + (row0 + h * BM) * (p.Dp / 2);
-                for (int ck = cg & 1; ck < p.Dp / 16; ck += 2) {
+                const uint32_t* src = p.qh + (row0 + h * BM) * q_cols;
+                for (int ck = cg & 1; ck < q_cols / 8; ck += 2) {
                     const uint4 lo = *reinterpret_cast<const uint4*>(src + ck * 8);
                     const uint4 hi = *reinterpret_cast<const uint4*>(src + ck * 8 + 4);
                     const uint32_t r[8] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z, hi.w};
-                    tmem_st_32x32b_x8(tmem + lane_base + qa_col + h * (p.Dp / 2) + ck * 8, r);
+                    tmem_st_32x32b_x8(tmem + lane_base + qa_col + h * q_cols + ck * 8, r);
                 }
                 tmem_wait_st();
                 tc_fence_before();
@@ -804,6 +826,18 @@ tc_gauss_fma_kernel(const __grid_constant__ CUtensorMap tm_q,
                             }
                         }
                     } else {
+                        // Guarded fp32 sums: the sums of the key tile by
+                        // themselves, added to acc at its end, so that rounding
+                        // grows with the keys of a tile plus the tiles, not
+                        // with all keys (with q^ in shared memory, where the
+                        // exponent warps set the pace, it cost 2 %).
+                        constexpr bool TILE_SUMS = TF && !QSM;
+                        uint64_t t0[C], t1[C];
+        #pragma unroll
+                        for (int cc = 0; cc < C; ++cc) {
+                            t0[cc] = TILE_SUMS ? 0ull : acc0[cc];
+                            t1[cc] = TILE_SUMS ? 0ull : acc1[cc];
+                        }
                         // Quad records: B and then each channel's values of
                         // four keys, one 16-byte load each.  (In key pairs,
                         // 8-byte loads, the records took half of the shared-
@@ -833,11 +867,16 @@ tc_gauss_fma_kernel(const __grid_constant__ CUtensorMap tm_q,
                             for (int cc = 0; cc < C; ++cc) {
                                 const float4 vc = pr[1 + cc];
                                 const uint64_t v01 = f32x2_pack(vc.x, vc.y), v23 = f32x2_pack(vc.z, vc.w);
-                                acc0[cc] = f32x2_fma(px[0], v01, acc0[cc]);
-                                acc1[cc] = f32x2_fma(py[0], v01, acc1[cc]);
-                                acc0[cc] = f32x2_fma(px[1], v23, acc0[cc]);
-                                acc1[cc] = f32x2_fma(py[1], v23, acc1[cc]);
+                                t0[cc] = f32x2_fma(px[0], v01, t0[cc]);
+                                t1[cc] = f32x2_fma(py[0], v01, t1[cc]);
+                                t0[cc] = f32x2_fma(px[1], v23, t0[cc]);
+                                t1[cc] = f32x2_fma(py[1], v23, t1[cc]);
                             }
+                        }
+        #pragma unroll
+                        for (int cc = 0; cc < C; ++cc) {
+                            acc0[cc] = TILE_SUMS ? f32x2_add(acc0[cc], t0[cc]) : t0[cc];
+                            acc1[cc] = TILE_SUMS ? f32x2_add(acc1[cc], t1[cc]) : t1[cc];
                         }
                     }
                     tc_fence_before();
@@ -980,7 +1019,9 @@ cudaError_t launch_typed(const TcPlan& pl, InType t, float c, char* ws, unsigned
 template <int C>
 cudaError_t launch_c(const TcPlan& pl, InType t, float c, char* ws, unsigned* status,
                      cudaStream_t s, const char** why, int vf_pass) {
-    if (pl.tf) return launch_typed<C, false, true, true>(pl, t, c, ws, status, s, why);
+    if (pl.tf)
+        return pl.guard ? launch_typed<C, false, false, true>(pl, t, c, ws, status, s, why)
+                        : launch_typed<C, false, true, true>(pl, t, c, ws, status, s, why);
     // Folded operands (template parameter VF): 1 / 2 = folded values, the
     // pass of the problems whose groups all share a sign / of the others;
     // 3 = only the exponent scale folded, value records as usual.
@@ -1022,10 +1063,10 @@ cudaError_t launch_c(const TcPlan& pl, InType t, float c, char* ws, unsigned* st
 bool plan_fma_kernel(int Dp, int C, bool aug, bool tf, int* nq, int* stages, size_t* smem) {
     if (C < 1 || C > kFmaMaxChannels || Dp > 256) return false;
     if (aug && Dp > kAugMaxDp) return false;
-    if (tf && (aug || Dp > kTf32MaxDp)) return false;
+    if (tf && (aug || Dp > kTf32WideMaxDp)) return false;
     // TMEM: q^ in TMEM needs Dp columns beside one slot of two S buffers.
-    const bool qsm = tf || (aug && kAugQsm);
-    if (!qsm && static_cast<int>(TMEM_COLS) - 2 * BN < Dp) return false;
+    const bool qsm = tf ? Dp <= kTf32MaxDp : (aug && kAugQsm);
+    if (!qsm && static_cast<int>(TMEM_COLS) - 2 * BN < (tf ? NQ * 2 * Dp : Dp)) return false;
     const int nkb = nkb_for(Dp, tf);
     const size_t budget = 232448;
     const size_t stage = stage_bytes_for(nkb, C, aug);
@@ -1051,7 +1092,7 @@ bool plan_fma_kernel(int Dp, int C, bool aug, bool tf, int* nq, int* stages, siz
 
 cudaError_t launch_tc_fma(const TcPlan& p, InType t, float c, char* ws, unsigned* status,
                           cudaStream_t s, const char** why, int vf_pass) {
-    const bool qsm = p.tf || (p.aug && kAugQsm);
+    const bool qsm = (p.tf && !p.guard) || (p.aug && kAugQsm);
     note_fma_variant((p.aug && kAugQsm && p.overlap && !p.tri && p.exp2_fma == 0 ? 1 : 0) |
                      (p.band_len > 0 ? 2 : 0) | (qsm ? 0 : 4) |
                      (p.vfold ? 8 : 0) | (p.cfold || p.vfold ? 16 : 0));
