@@ -255,6 +255,137 @@ mean_partial_vec_kernel(const T* __restrict__ q, const T* __restrict__ k, int64_
     }
 }
 
+// Any other width up to 256 (16-bit inputs): the partial sums and maxima of
+// mean_partial_kernel, in the same order of additions (bit for bit), read in
+// 16-byte vectors.  Eight rows are D vectors, and a block of
+// mean_partial_kernel adds up every eighth row, so thread t of the D threads
+// of a chunk (one block's rows there) owns vector t of each group of eight
+// rows: its eight elements are of fixed (row mod 8, coordinate) all along.
+// Chunks that do not start on 16 bytes take narrower loads; groups that
+// straddle q and k or end with the chunk are read element by element.  A block holds `chunks` chunks of D
+// threads; blocks from mblocks on write key records (see RecordJob).
+// Bound: load latency (ncu, with the records: 50021 points of D = 50 6.4 us,
+// where mean_partial_kernel took 7.2 us and the records and their flags two
+// more launches, 7.5 us).
+template <typename T, typename TV>
+__global__ void __launch_bounds__(kMeanVecThreads)
+mean_partial_rows_kernel(const T* __restrict__ q, const T* __restrict__ k, int64_t M, int64_t N,
+                         int D, int64_t rows_per_block, int G, int chunks, int mblocks,
+                         float* __restrict__ partial, const RecordJob<TV> rj) {
+    pdl_trigger();
+    pdl_wait();
+    if (static_cast<int>(blockIdx.x) >= mblocks) {
+        const int64_t t = static_cast<int64_t>(blockIdx.x - mblocks) * kMeanVecThreads + threadIdx.x;
+        if (rj.signs) {
+            if constexpr (std::is_same<TV, __half>::value) {
+                if (t < 2 * rj.pairs) write_sign_record(rj.v, rj.N, rj.rec, t, blockIdx.y, 2 * rj.pairs);
+            }
+        } else if (t < rj.pairs) {
+            write_key_record(rj, t, blockIdx.y);
+        }
+        return;
+    }
+    __shared__ float s_sum[kMeanVecThreads][9];
+    __shared__ float s_max[kMeanVecThreads][9];
+    // Problem blockIdx.y of a batch: its own points and partial rows.
+    q += static_cast<int64_t>(blockIdx.y) * M * D;
+    k += static_cast<int64_t>(blockIdx.y) * N * D;
+    partial += static_cast<int64_t>(blockIdx.y) * 2 * G * D;
+    const int local = static_cast<int>(threadIdx.x) / D;     // chunk of this block
+    const int t = static_cast<int>(threadIdx.x) - local * D;
+    const int chunk = static_cast<int>(blockIdx.x) * chunks + local;
+    float sum[8], mx[8];
+#pragma unroll
+    for (int e = 0; e < 8; ++e) sum[e] = mx[e] = 0.f;
+    if (local < chunks && chunk < G) {
+        const int64_t r0 = static_cast<int64_t>(chunk) * rows_per_block;
+        const int64_t r1 = min(r0 + rows_per_block, M + N);
+        auto add = [&](const uint4 u) {
+            const T* h = reinterpret_cast<const T*>(&u);
+#pragma unroll
+            for (int e = 0; e < 8; ++e) {
+                const float f = to_f(h[e]);
+                sum[e] += f;
+                mx[e] = fmaxf(mx[e], fabsf(f));
+            }
+        };
+        // Whole groups of eight rows from r on: in q up to M, in k after it; in
+        // the widest loads that the first row's address allows.
+        auto groups = [&](int64_t r, int64_t end) {
+            const T* x = (r < M ? q : k - M * D) + r * D + 8 * t;
+            const int64_t n = (end - r) / 8;
+            const int64_t step = 8 * static_cast<int64_t>(D);
+            auto walk = [&](auto tag) {
+                using L = decltype(tag);
+                constexpr int PER = 16 / static_cast<int>(sizeof(L));
+                auto load = [&](const T* p) {
+                    uint4 u;
+                    L* w = reinterpret_cast<L*>(&u);
+#pragma unroll
+                    for (int i = 0; i < PER; ++i) w[i] = reinterpret_cast<const L*>(p)[i];
+                    return u;
+                };
+                int64_t g = 0;
+                for (; g + 8 <= n; g += 8, x += 8 * step) {
+                    uint4 u[8];
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) u[i] = load(x + i * step);
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) add(u[i]);
+                }
+                for (; g < n; ++g, x += step) add(load(x));
+            };
+            const unsigned at = static_cast<unsigned>(reinterpret_cast<uintptr_t>(x)) & 15u;
+            if (at == 0) walk(uint4());
+            else if ((at & 7u) == 0) walk(uint2());
+            else if ((at & 3u) == 0) walk(unsigned());
+            else walk(static_cast<unsigned short>(0));
+            return r + 8 * n;
+        };
+        // One group (or what is left of it), element by element.
+        auto single = [&](int64_t r) {
+            for (int e = 0; e < 8; ++e) {
+                const int i = 8 * t + e;
+                const int64_t row = r + i / D;
+                if (row < r1) {
+                    const int d = i % D;
+                    const float f = to_f(row < M ? q[row * D + d] : k[(row - M) * D + d]);
+                    sum[e] += f;
+                    mx[e] = fmaxf(mx[e], fabsf(f));
+                }
+            }
+        };
+        int64_t r = r0;
+        while (r < r1) {
+            const int64_t end = r < M ? min(r1, M) : r1;
+            const int64_t next = groups(r, end);
+            if (next == r) {
+                single(r);
+                r += 8;
+            } else {
+                r = next;
+            }
+        }
+    }
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+        s_sum[threadIdx.x][e] = sum[e];
+        s_max[threadIdx.x][e] = mx[e];
+    }
+    __syncthreads();
+    if (local >= chunks || chunk >= G) return;
+    // Coordinate t of the chunk: rows 0 .. 7 (mod 8) in order.
+    float a = 0.f, m = 0.f;
+#pragma unroll
+    for (int y = 0; y < 8; ++y) {
+        const int i = y * D + t, u = local * D + (i >> 3), e = i & 7;
+        a += s_sum[u][e];
+        m = fmaxf(m, s_max[u][e]);
+    }
+    partial[static_cast<int64_t>(chunk) * D + t] = a;
+    partial[static_cast<int64_t>(G + chunk) * D + t] = m;
+}
+
 // mu_d = the mean of coordinate d rounded to a multiple of g_d, the spacing
 // of the input format at max |x_d| (2^(e - mant_bits) for max |x_d| in
 // [2^e, 2^(e+1)), at least the subnormal spacing 2^min_exp).  Every input
@@ -630,12 +761,10 @@ __global__ void finalize_slots_kernel(const float* __restrict__ part, int64_t Mp
     out[idx] = acc;
 }
 
-// Vectorised variant of operand_kernel for D a multiple of 8: G lanes
-// (G = the power of two >= D / 8) share a row, each converting one 16-byte
-// vector of 8 coordinates straight from global memory to global memory;
-// the squared norm is reduced over the G lanes and the group's first lane
-// writes the columns past D (norm terms or zeros).  Same outputs as
-// operand_kernel.
+// Vectorised variant of operand_kernel for D >= 1: G lanes share a row, each
+// converting up to kOperandVecs vectors of 8 coordinates; the squared norm is
+// reduced over the G lanes and the group's first lane writes the columns past
+// D (norm terms or zeros).  Same outputs as operand_kernel.
 constexpr int kOperandVecThreads = 256;
 
 template <typename T> __device__ __forceinline__ T bits_to(unsigned short b);
@@ -682,7 +811,7 @@ template <> struct Pair<__nv_bfloat16> {
 // layout: -(c/2)||x^||^2, or pad_value) in every lane.
 constexpr int kOperandVecs = 8;
 
-template <typename T, bool AUG, int G>
+template <typename T, bool AUG, int G, bool RAGGED>
 __device__ __forceinline__ float operand_row(const uint4 (&in)[kOperandVecs],
                                              const uint4* __restrict__ smean, int vi,
                                              bool in_pad, bool valid, int D, int Dp, int nt,
@@ -690,9 +819,19 @@ __device__ __forceinline__ float operand_row(const uint4 (&in)[kOperandVecs],
                                              T* __restrict__ out_q, T* __restrict__ out_k,
                                              float cf, const __half* vw) {
     using PT = Pair<T>;
-    const int V = D / 8;
+    const int V = RAGGED ? (D + 7) / 8 : D / 8;   // (coordinates past D are 0 - 0)
     const bool fold = AUG && cf > 0.f;
     float acc = 0.f, accu = 0.f;
+    // RAGGED: the squares are added in operand_kernel's order (coordinates of
+    // one residue mod 32 in sequence, then a tree over the residues), so that
+    // rows of any width keep their norms bit for bit: ps[8 j + e] is residue
+    // 8 (vi + G j) + e mod 32 of this lane.
+    constexpr int R8 = RAGGED ? 4 / G : 1;            // residue groups of 8 per lane
+    float ps[8 * R8], pu[8 * R8];
+    if (RAGGED) {
+#pragma unroll
+        for (int i = 0; i < 8 * R8; ++i) ps[i] = pu[i] = 0.f;
+    }
     if (in_pad) {
         uint64_t acc2 = 0ull, accu2 = 0ull;
 #pragma unroll
@@ -710,13 +849,24 @@ __device__ __forceinline__ float operand_row(const uint4 (&in)[kOperandVecs],
                     h[k] = PT::sub(x2[k], mm[k]);
                     const float2 f = PT::to_f2(h[k]);
                     const uint64_t f2 = f32x2_pack(f.x, f.y);
-                    acc2 = f32x2_fma(f2, f2, acc2);
+                    const int i = RAGGED ? 8 * (e % R8) + 2 * k : 0;
+                    if (RAGGED) {
+                        ps[i] = fmaf(f.x, f.x, ps[i]);
+                        ps[i + 1] = fmaf(f.y, f.y, ps[i + 1]);
+                    } else {
+                        acc2 = f32x2_fma(f2, f2, acc2);
+                    }
                     if (fold) {
                         // Folded scale: the query row holds rn(c x^).
                         hs[k] = PT::from_f2(cf * f.x, cf * f.y);
                         const float2 g = PT::to_f2(hs[k]);
                         const uint64_t g2 = f32x2_pack(g.x, g.y);
-                        accu2 = f32x2_fma(g2, g2, accu2);
+                        if (RAGGED) {
+                            pu[i] = fmaf(g.x, g.x, pu[i]);
+                            pu[i + 1] = fmaf(g.y, g.y, pu[i + 1]);
+                        } else {
+                            accu2 = f32x2_fma(g2, g2, accu2);
+                        }
                     }
                 }
                 u = *reinterpret_cast<const uint4*>(h);
@@ -725,21 +875,52 @@ __device__ __forceinline__ float operand_row(const uint4 (&in)[kOperandVecs],
             if (out_q) *reinterpret_cast<uint4*>(out_q + 8 * v) = fold ? us : u;
             if (out_k) *reinterpret_cast<uint4*>(out_k + 8 * v) = u;
         }
-        float lo, hi;
-        f32x2_unpack(acc2, lo, hi);
-        acc = lo + hi;
-        f32x2_unpack(accu2, lo, hi);
-        accu = lo + hi;
+        if (!RAGGED) {
+            float lo, hi;
+            f32x2_unpack(acc2, lo, hi);
+            acc = lo + hi;
+            f32x2_unpack(accu2, lo, hi);
+            accu = lo + hi;
+        }
     }
+    if (RAGGED) {
+        // The tree over residues: 16 apart, then 8, 4, 2, 1.  G = 1: all in this
+        // lane; G = 2: 16 apart in this lane (j, j + 1), 8 apart in the other;
+        // G = 4: 16 and 8 apart in other lanes.
+        auto tree = [&](float (&p)[8 * R8]) {
+            float t[8];
 #pragma unroll
-    for (int o = G / 2; o > 0; o >>= 1) {
-        acc += __shfl_xor_sync(0xffffffffu, acc, o, G);
-        if (fold) accu += __shfl_xor_sync(0xffffffffu, accu, o, G);
+            for (int i = 0; i < 8; ++i) {
+                if (G == 1) {
+                    t[i] = (p[i] + p[(16 + i) % (8 * R8)]) + (p[(8 + i) % (8 * R8)] + p[(24 + i) % (8 * R8)]);
+                } else if (G == 2) {
+                    t[i] = p[i] + p[(8 + i) % (8 * R8)];
+                    t[i] += __shfl_xor_sync(0xffffffffu, t[i], 1);
+                } else {
+                    t[i] = p[i] + __shfl_xor_sync(0xffffffffu, p[i], 2);
+                    t[i] += __shfl_xor_sync(0xffffffffu, t[i], 1);
+                }
+            }
+#pragma unroll
+            for (int i = 0; i < 4; ++i) t[i] += t[i + 4];
+            t[0] += t[2];
+            t[1] += t[3];
+            return t[0] + t[1];
+        };
+        acc = tree(ps);
+        if (fold) accu = tree(pu);
+    } else {
+#pragma unroll
+        for (int o = G / 2; o > 0; o >>= 1) {
+            acc += __shfl_xor_sync(0xffffffffu, acc, o, G);
+            if (fold) accu += __shfl_xor_sync(0xffffffffu, accu, o, G);
+        }
     }
     const float nrm = valid ? -half_c * acc : pad_value;
+    if (RAGGED) __syncwarp();   // the last vector's lane has written columns past D
     if (!in_pad || vi != 0) return nrm;
     if (!AUG) {
-        for (int c = D; c < Dp; c += 8)
+        for (int c = 8 * V; c < Dp; c += 8)
             *reinterpret_cast<uint4*>(out_q + c) = make_uint4(0u, 0u, 0u, 0u);
         return nrm;
     }
@@ -764,7 +945,11 @@ __device__ __forceinline__ float operand_row(const uint4 (&in)[kOperandVecs],
             // Folded: a = -||u||^2 / (2c) from the rounded scaled row, and
             // b = -c ||k^||^2 / 2 + log2(|v| 2^-16) (see log_weight).
             split(-0.5f * accu / cf, t0, t1, t2);
-            split(-0.5f * cf * acc + log_weight(vw), k0, k1, k2);
+            // (Explicitly one rounding for RAGGED rows, as in operand_kernel, and
+            // two for the others: a last bit of b moves signed sums of 65536
+            // keys by 2e-5 of their norm, so the choice is not the compiler's.)
+            const float lw = log_weight(vw);
+            split(RAGGED ? fmaf(-0.5f * cf, acc, lw) : __fadd_rn(__fmul_rn(-0.5f * cf, acc), lw), k0, k1, k2);
         } else {
             split(-0.5f * acc, t0, t1, t2);
             k0 = t0; k1 = t1; k2 = t2;
@@ -782,6 +967,19 @@ __device__ __forceinline__ float operand_row(const uint4 (&in)[kOperandVecs],
     auto tail_k = [&](int e) -> unsigned {
         return e < nt ? term(e) : e < 2 * nt ? partner(e - nt) : 0u;
     };
+    if (RAGGED) {
+        // The columns past D start anywhere: zeros to the end of the row, then
+        // the norm terms and their partners one by one.
+        for (int c = 8 * V; c < Dp; c += 8) {
+            if (out_q) *reinterpret_cast<uint4*>(out_q + c) = make_uint4(0u, 0u, 0u, 0u);
+            if (out_k) *reinterpret_cast<uint4*>(out_k + c) = make_uint4(0u, 0u, 0u, 0u);
+        }
+        for (int e = 0; e < 2 * nt; ++e) {
+            if (out_q) out_q[D + e] = bits_to<T>(static_cast<unsigned short>(tail_q(e)));
+            if (out_k) out_k[D + e] = bits_to<T>(static_cast<unsigned short>(tail_k(e)));
+        }
+        return nrm;
+    }
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
         const int c = D + 8 * h;
@@ -814,7 +1012,7 @@ struct OperandJob {
     const void* vw;      // fp16 values of the rows written to out_k (folded magnitudes), or null
 };
 
-// Vector path of the operand preparation (D a multiple of 8): G lanes per
+// Vector path of the operand preparation: G lanes per
 // row (G = 1 up to D = 64, 2 up to 128, 4 up to 256), each lane converting
 // up to eight 16-byte vectors of its row, all loaded before any is
 // converted; so every lane of a warp does its own row's work (no lanes idle
@@ -828,7 +1026,12 @@ struct OperandJob {
 // both arrays of every problem take one launch; a block never straddles
 // two problems.  The problem's mean is staged once per block in shared
 // memory as packed pairs of the input format.
-template <typename T, bool AUG, int G>
+// RAGGED (D not a multiple of 8, rows that start anywhere): the block's
+// input rows, one contiguous run, are copied to shared memory in 16-byte
+// vectors first and each lane gathers its row's vectors there.  (One warp per
+// row in operand_kernel before: 50021 points, D = 50, both layouts: 26.7 ->
+// 10.1 us, 19 MB moved.)
+template <typename T, bool AUG, int G, bool RAGGED>
 __global__ void __launch_bounds__(kOperandVecThreads)
 operand_vec_kernel(const OperandJob j0, const OperandJob j1, unsigned blocks0, int D, int Dp,
                    int nt, float F, const float* __restrict__ mu, float half_c, float pad_value,
@@ -851,35 +1054,74 @@ operand_vec_kernel(const OperandJob j0, const OperandJob j1, unsigned blocks0, i
     const int blk = static_cast<int>(second ? blockIdx.x - blocks0 : blockIdx.x);
     const int vi = threadIdx.x % G;                  // first vector of this lane
     const int slot = threadIdx.x / G;
-    const int V = D / 8;
+    const int V = RAGGED ? (D + 7) / 8 : D / 8;
     const int rows_pad = static_cast<int>(j.rows_pad);
     const int rows = static_cast<int>(j.rows);
     const int i = blk * SLOTS + slot;                // row of problem b
-    const T* xr = static_cast<const T*>(j.x) + (static_cast<int64_t>(b) * rows + i) * D;
+    const bool wq = AUG ? j.out_q != nullptr : true;
+    const bool wk = AUG && j.out_k != nullptr;
+    const int sv = (Dp / 8) | 1;                     // staged row stride (odd) in 16-byte vectors
     uint4 in[kOperandVecs];
+    if (RAGGED) {
+        // Behind the staged output rows (see operand_typed).
+        T* raw = reinterpret_cast<T*>(staged + ((wq ? 1 : 0) + (wk ? 1 : 0)) * SLOTS * sv);
+        const int i0 = blk * SLOTS;
+        const int n_el = max(0, min(SLOTS, rows - i0)) * D;
+        const T* src = static_cast<const T*>(j.x) + (static_cast<int64_t>(b) * rows + i0) * D;
+        // (A later problem of a batch may start anywhere.)
+        const int nvec = (reinterpret_cast<uintptr_t>(src) & 15u) == 0 ? n_el / 8 : 0;
+        for (int u = threadIdx.x; u < nvec; u += kOperandVecThreads)
+            reinterpret_cast<uint4*>(raw)[u] = reinterpret_cast<const uint4*>(src)[u];
+        for (int u = nvec * 8 + threadIdx.x; u < n_el; u += kOperandVecThreads) raw[u] = src[u];
+        __syncthreads();
+        const T* row = raw + slot * D;
 #pragma unroll
-    for (int e = 0; e < kOperandVecs; ++e) {
-        const int v = vi + G * e;
-        in[e] = (i < rows && v < V) ? *reinterpret_cast<const uint4*>(xr + 8 * v)
-                                    : make_uint4(0u, 0u, 0u, 0u);
+        for (int e = 0; e < kOperandVecs; ++e) {
+            const int c = 8 * (vi + G * e);
+            uint32_t w[4];
+#pragma unroll
+            for (int h = 0; h < 4; ++h) {
+                const int c2 = c + 2 * h;
+                unsigned lo = 0u, hi = 0u;
+                if (i < rows && c2 < D) {
+                    if (D & 1) {
+                        lo = to_bits(row[c2]);
+                        hi = c2 + 1 < D ? to_bits(row[c2 + 1]) : 0u;
+                        lo |= hi << 16;
+                    } else {
+                        lo = *reinterpret_cast<const uint32_t*>(row + c2);   // even row starts
+                    }
+                }
+                w[h] = lo;
+            }
+            in[e] = make_uint4(w[0], w[1], w[2], w[3]);
+        }
+    } else {
+        const T* xr = static_cast<const T*>(j.x) + (static_cast<int64_t>(b) * rows + i) * D;
+#pragma unroll
+        for (int e = 0; e < kOperandVecs; ++e) {
+            const int v = vi + G * e;
+            in[e] = (i < rows && v < V) ? *reinterpret_cast<const uint4*>(xr + 8 * v)
+                                        : make_uint4(0u, 0u, 0u, 0u);
+        }
     }
     const float* mb = mu ? mu + static_cast<int64_t>(b) * D : nullptr;
     typename PT::P* sm = reinterpret_cast<typename PT::P*>(smean);
-    for (int c = threadIdx.x; c < D / 2; c += kOperandVecThreads)
-        sm[c] = mb ? PT::from_f2(mb[2 * c], mb[2 * c + 1]) : PT::from_f2(0.f, 0.f);
+    for (int c = threadIdx.x; c < 4 * V; c += kOperandVecThreads) {
+        const float m0 = mb && 2 * c < D ? mb[2 * c] : 0.f;
+        const float m1 = mb && 2 * c + 1 < D ? mb[2 * c + 1] : 0.f;
+        sm[c] = PT::from_f2(m0, m1);
+    }
     __syncthreads();
-    const bool wq = AUG ? j.out_q != nullptr : true;
-    const bool wk = AUG && j.out_k != nullptr;
     const bool in_pad = i < rows_pad;
     const int64_t row = static_cast<int64_t>(b) * rows_pad + i;   // batch-stacked output row
     const __half* vw = (wk && j.vw && i < rows)
                            ? static_cast<const __half*>(j.vw) + static_cast<int64_t>(b) * rows + i
                            : nullptr;
     const int nv = Dp / 8;                           // 16-byte vectors per output row
-    const int sv = nv | 1;                           // staged row stride (odd)
     uint4* stage_q = staged;
     uint4* stage_k = staged + (wq ? SLOTS * sv : 0);
-    const float n = operand_row<T, AUG, G>(
+    const float n = operand_row<T, AUG, G, RAGGED>(
         in, smean, vi, in_pad, i < rows, D, Dp, nt, F, half_c, pad_value,
         wq ? reinterpret_cast<T*>(stage_q + slot * sv) : nullptr,
         wk ? reinterpret_cast<T*>(stage_k + slot * sv) : nullptr, cf, vw);
@@ -912,10 +1154,11 @@ cudaError_t operand_typed(const OperandJob& j0, const OperandJob* j1, int D, int
         return cudaErrorInvalidValue;
     // The vector path indexes rows with 32-bit integers.
     const int64_t most_rows = std::max(j0.rows_pad, j1 ? j1->rows_pad : int64_t(0)) * batch;
-    if (D % 8 == 0 && D >= 8 && (!AUG || Dp - D >= 2 * nt) && most_rows < (int64_t(1) << 30)) {
+    if (D >= 1 && (!AUG || Dp - D >= 2 * nt) && most_rows < (int64_t(1) << 30)) {
         // Vector path: G lanes per row (up to kOperandVecs vectors each),
         // both arrays in one launch.
-        const int V = D / 8;
+        const bool ragged = D % 8 != 0;
+        const int V = (D + 7) / 8;
         const int G = V <= kOperandVecs ? 1 : V <= 2 * kOperandVecs ? 2 : 4;
         const int64_t per_block = kOperandVecThreads / G;
         const int64_t b0 = (j0.rows_pad + per_block - 1) / per_block;
@@ -928,7 +1171,8 @@ cudaError_t operand_typed(const OperandJob& j0, const OperandJob* j1, int D, int
             return j ? (AUG ? (j->out_q ? 1 : 0) + (j->out_k ? 1 : 0) : 1) : 0;
         };
         const size_t smem = static_cast<size_t>(std::max(nout(&j0), nout(j1))) * per_block *
-                            ((Dp / 8) | 1) * 16;
+                                ((Dp / 8) | 1) * 16 +
+                            (ragged ? (static_cast<size_t>(per_block) * D * sizeof(T) + 15) / 16 * 16 : 0);
         auto go = [&](auto kern) {
             cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                  static_cast<int>(smem));
@@ -941,9 +1185,9 @@ cudaError_t operand_typed(const OperandJob& j0, const OperandJob* j1, int D, int
         if (flags_done) *flags_done = vf_rec != nullptr;
         cudaError_t e;
         switch (G) {
-            case 1: e = go(operand_vec_kernel<T, AUG, 1>); break;
-            case 2: e = go(operand_vec_kernel<T, AUG, 2>); break;
-            default: e = go(operand_vec_kernel<T, AUG, 4>); break;
+            case 1: e = ragged ? go(operand_vec_kernel<T, AUG, 1, true>) : go(operand_vec_kernel<T, AUG, 1, false>); break;
+            case 2: e = ragged ? go(operand_vec_kernel<T, AUG, 2, true>) : go(operand_vec_kernel<T, AUG, 2, false>); break;
+            default: e = ragged ? go(operand_vec_kernel<T, AUG, 4, true>) : go(operand_vec_kernel<T, AUG, 4, false>); break;
         }
         if (e != cudaSuccess) return e;
         note_launches(1);
@@ -1321,6 +1565,34 @@ cudaError_t launch_mean(InType t, const void* q, const void* k, int64_t M, int64
             launch_kernel(mean_partial_vec_kernel<T, TV>, dim3(G + rblocks, batch), kMeanVecThreads, 0,
                           s, static_cast<const T*>(q), static_cast<const T*>(k), M, N, D, rpb, Gq, G,
                           partial, rj);
+        };
+        const bool vf = rec && rec->v_f32;
+        if (t == InType::F16) {
+            if (vf) go(__half(), float()); else go(__half(), __half());
+        } else {
+            if (vf) go(__nv_bfloat16(), float()); else go(__nv_bfloat16(), __nv_bfloat16());
+        }
+        if (rec_done) *rec_done = rec != nullptr;
+        note_launches(1);
+    } else if (t != InType::F32 && D >= 1 && D <= kMeanVecThreads) {
+        const int64_t rpb = (total + blocks - 1) / blocks;
+        G = static_cast<int>((total + rpb - 1) / rpb);
+        // As many chunks per block as leave about 300 blocks.
+        const int chunks = static_cast<int>(
+            std::min<int64_t>(kMeanVecThreads / D, std::max<int64_t>(1, static_cast<int64_t>(G) * batch / 304)));
+        const int mblocks = (G + chunks - 1) / chunks;
+        const int64_t pairs = rec ? rec->Npad / 2 : 0;
+        const int64_t rthreads = rec && rec->signs ? 2 * pairs : pairs;
+        const int rblocks = static_cast<int>((rthreads + kMeanVecThreads - 1) / kMeanVecThreads);
+        auto go = [&](auto tag, auto vtag) {
+            using T = decltype(tag);
+            using TV = decltype(vtag);
+            const RecordJob<TV> rj = {rec ? static_cast<const TV*>(rec->v) : nullptr, rec ? rec->N : 0,
+                                      pairs, rec ? rec->C : 0, rec ? rec->out : nullptr,
+                                      rec && rec->signs};
+            launch_kernel(mean_partial_rows_kernel<T, TV>, dim3(mblocks + rblocks, batch), kMeanVecThreads,
+                          0, s, static_cast<const T*>(q), static_cast<const T*>(k), M, N, D, rpb, G,
+                          chunks, mblocks, partial, rj);
         };
         const bool vf = rec && rec->v_f32;
         if (t == InType::F16) {
