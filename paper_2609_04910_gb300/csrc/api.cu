@@ -394,11 +394,16 @@ gs_status run(Call c) {
         bool records_done = false;
         bool flags_done = false;   // folded values: per-problem flags written by the operand launch
         if (mu) {
+            // Words that later launches take maxima into: the guard, or the
+            // two-MMA kernel's channel and weight maxima.
+            gs::ZeroWords zero;
+            if (guard) zero = {guard, 1};
+            else if (!tp.fma) zero = {reinterpret_cast<unsigned*>(ws + tp.off_vmax), tp.Cp + 2 * tp.wt};
             const gs::RecordArgs rec = {c.v, c.w_f32, c.N, tp.Npad, static_cast<int>(tp.Cv),
                                         reinterpret_cast<float*>(ws + tp.off_rec), tp.vfold};
             e = gs::launch_mean(t, c.q, c.k, c.M, c.N, static_cast<int>(c.D), tp.mean_blocks,
                                 reinterpret_cast<float*>(ws + tp.off_mean_part), mu, c.stream,
-                                batch, (tp.fma && tp.aug) ? &rec : nullptr, &records_done, guard);
+                                batch, (tp.fma && tp.aug) ? &rec : nullptr, &records_done, zero);
             where = "mean kernel";
         }
         const float ninf = -INFINITY;
@@ -496,7 +501,7 @@ gs_status run(Call c) {
                                           static_cast<int>(c.D), static_cast<int>(c.C),
                                           static_cast<int>(ch0), cc, tp.Cp,
                                           reinterpret_cast<unsigned*>(ws + tp.off_vmax),
-                                          ws + tp.off_vt, inv, c.stream);
+                                          ws + tp.off_vt, inv, c.stream, mu && ch0 == 0);
                 where = "value kernel";
                 if (e == cudaSuccess && tp.wt > 0) {
                     e = gs::launch_weight_prep(t, c.rw, c.rw_f32, c.M, tp.Mpad, c.kw, c.kw_f32, c.N,
@@ -504,7 +509,7 @@ gs_status run(Call c) {
                                                reinterpret_cast<float*>(ws + tp.off_rowf),
                                                reinterpret_cast<float*>(ws + tp.off_colT),
                                                reinterpret_cast<unsigned*>(ws + tp.off_wmax),
-                                               c.stream);
+                                               c.stream, mu && ch0 == 0);
                     where = "pair-weight kernel";
                 }
                 if (e == cudaSuccess && ch0 == 0) e = record_event(c.opt.main_events[0], c.stream);

@@ -174,15 +174,19 @@ struct RecordArgs {
     bool signs;          // sign records of folded value magnitudes (fp16 values, C = 1;
                          // per key tile of 128 keys: 128 signed 2^16 and 4 group words)
 };
-// With zero_word, the launch also clears that word (before any later kernel
-// of the call).
+// The launches also clear the words of `zero` (before any later kernel of the
+// call).
+struct ZeroWords {
+    unsigned* p = nullptr;
+    int n = 0;
+};
 // Common mean of q and k per problem.  With `rec`, the launch also writes
 // those key records where it can (the vectorised path); *rec_done says
 // whether it did.
 cudaError_t launch_mean(InType t, const void* q, const void* k, int64_t M, int64_t N, int D,
                         int blocks, float* partial, float* mu, cudaStream_t s, int batch = 1,
                         const RecordArgs* rec = nullptr, bool* rec_done = nullptr,
-                        unsigned* zero_word = nullptr);
+                        ZeroWords zero = {});
 // (cf > 0 with vw: the exponent scale c folds into the query rows and the
 // magnitudes of the fp16 values vw into the key rows' norm terms;
 // vf_rec: sign records already written, whose per-problem flags the launch
@@ -205,11 +209,12 @@ cudaError_t launch_operands(InType t, bool aug, const void* q, int64_t M, int64_
 // power-of-two scales.  Forward: channel ch of key n is w[n, ch] (w has the
 // input dtype, Cw = channels).  grad: channel c (D + 1) + d is
 // w[n, c] (x[n, d] - mu_d) for d < D and w[n, c] for d = D (w is N x Cw,
-// float32 when w_f32, else the input dtype; x is N x D).
+// float32 when w_f32, else the input dtype; x is N x D).  zeroed: an earlier
+// launch of the call has cleared the Cp words of vmax_bits (wmax below).
 cudaError_t launch_value_prep(InType t, bool grad, bool w_f32, const void* w, const void* x,
                               const float* mu, int64_t N, int64_t Npad, int D, int Cw, int ch0,
                               int Cc, int Cp, unsigned* vmax_bits, void* vt, float* inv_scale,
-                              cudaStream_t s);
+                              cudaStream_t s, bool zeroed = false);
 // Factors of the pair weights w_mn = sum_c r[m, c] k[n, c] of the weighted
 // vector-Jacobian pass (see prep.cu): row factors rsrc (R x C) into rowf
 // (Rpad x WT float32), column factors csrc (Ncol x C) into colT (per key
@@ -219,7 +224,7 @@ cudaError_t launch_value_prep(InType t, bool grad, bool w_f32, const void* w, co
 cudaError_t launch_weight_prep(InType t, const void* rsrc, bool r_f32, int64_t R, int64_t Rpad,
                                const void* csrc, bool c_f32, int64_t Ncol, int64_t Npad, int C,
                                int WT, int BN, float* rowf, float* colT, unsigned* wmax,
-                               cudaStream_t s);
+                               cudaStream_t s, bool zeroed = false);
 // Forward: out (M x Cv) = inv_scale (when given) x the split partials summed
 // in split order; rows below main_rows have one split.
 cudaError_t launch_finalize(const float* part, int splits, int64_t split_stride_rows,

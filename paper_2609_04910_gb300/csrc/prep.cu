@@ -420,10 +420,11 @@ constexpr int kMeanFinalThreadMax = 32;
 __global__ void __launch_bounds__(kMeanFinalThreads)
 mean_final_block_kernel(const float* __restrict__ partial, int G, int D, float total,
                         int mant_bits, int min_exp, float* __restrict__ mu,
-                        unsigned* __restrict__ zero_word) {
+                        const ZeroWords zero) {
     pdl_trigger();
     pdl_wait();
-    if (zero_word && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *zero_word = 0u;
+    if (blockIdx.x == 0 && blockIdx.y == 0)
+        for (int i = threadIdx.x; i < zero.n; i += kMeanFinalThreads) zero.p[i] = 0u;
     constexpr int W = kMeanFinalThreads / 32;
     __shared__ float red_s[W];
     __shared__ float red_m[W];
@@ -462,10 +463,11 @@ mean_final_block_kernel(const float* __restrict__ partial, int G, int D, float t
 __global__ void __launch_bounds__(kMeanFinalThreads)
 mean_final_kernel(const float* __restrict__ partial, int G, int D, int64_t items, float total,
                   int mant_bits, int min_exp, float* __restrict__ mu,
-                  unsigned* __restrict__ zero_word) {
+                  const ZeroWords zero) {
     pdl_trigger();
     pdl_wait();
-    if (zero_word && blockIdx.x == 0 && threadIdx.x == 0) *zero_word = 0u;
+    if (blockIdx.x == 0)
+        for (int i = threadIdx.x; i < zero.n; i += kMeanFinalThreads) zero.p[i] = 0u;
     const int64_t it = static_cast<int64_t>(blockIdx.x) * kMeanFinalThreads + threadIdx.x;
     if (it >= items) return;
     const int64_t b = it / D;
@@ -1431,6 +1433,46 @@ __global__ void finalize_kernel(const float* __restrict__ part, int splits,
     out[idx] = acc * (inv_scale ? inv_scale[c] : 1.f);
 }
 
+// The same for Cv a multiple of 4 (part_ld is a multiple of 16): one thread
+// per quad of channels.  (Bound: HBM and load latency; 65536 rows of 64
+// channels, ncu: one thread per channel 26.0 us, quads 10.9.)
+constexpr int kFinalizeThreads = 256;
+
+// The sum over ns splits of one quad, added in split order.
+__device__ __forceinline__ float4 sum_splits4(const float* __restrict__ p, int64_t step, int ns) {
+    float4 a = *reinterpret_cast<const float4*>(p);
+#pragma unroll 4
+    for (int s = 1; s < ns; ++s) {
+        const float4 x = *reinterpret_cast<const float4*>(p + s * step);
+        a.x += x.x;
+        a.y += x.y;
+        a.z += x.z;
+        a.w += x.w;
+    }
+    return a;
+}
+
+__global__ void __launch_bounds__(kFinalizeThreads)
+finalize_quads_kernel(const float* __restrict__ part, int splits, int64_t split_stride_rows,
+                      int64_t M, int Cv, int part_ld, const float* __restrict__ inv_scale,
+                      float* __restrict__ out, int64_t main_rows) {
+    pdl_trigger();
+    pdl_wait();
+    const int Q = Cv / 4;
+    const int64_t idx = static_cast<int64_t>(blockIdx.x) * kFinalizeThreads + threadIdx.x;
+    if (idx >= M * Q) return;
+    const int64_t m = div_nonneg(idx, Q);
+    const int c = 4 * static_cast<int>(idx - m * Q);
+    const float4 sc = inv_scale ? *reinterpret_cast<const float4*>(inv_scale + c)
+                                : make_float4(1.f, 1.f, 1.f, 1.f);
+    float4 a = sum_splits4(part + m * part_ld + c, split_stride_rows * part_ld, m < main_rows ? 1 : splits);
+    a.x *= sc.x;
+    a.y *= sc.y;
+    a.z *= sc.z;
+    a.w *= sc.w;
+    reinterpret_cast<float4*>(out)[idx] = a;
+}
+
 // Gradient contraction for the channels ch0 .. ch0 + Cc - 1 of one launch
 // (channel ch = c (D + 1) + d, as in value_at).  With S_j the sum over
 // splits of partial channel j (times inv_scale[j] when given):
@@ -1489,13 +1531,200 @@ __global__ void finalize_points_kernel(const float* __restrict__ part, int split
     if (out && d < D) out[m * D + d] = (accumulate ? out[m * D + d] : 0.f) + tau * acc;
 }
 
+// finalize_points_kernel for one weight channel whose D + 1 channels are one
+// launch's (the q-gradient and the weighted vector-Jacobian passes): one
+// thread per quad of coordinates, all its loads issued before any is used.
+// The same operations per output, in the same order.  (Bound: HBM and load
+// latency, about 4 (D + 16) bytes read and 4 D written per row; 131072 rows,
+// D = 32, ncu: one thread per output 56.5 us, quads 14.3.)
+template <typename T, typename U>
+__global__ void __launch_bounds__(kFinalizeThreads, 5)
+finalize_point_quads_kernel(const float* __restrict__ part, int splits, int64_t split_stride_rows,
+                            int64_t M, int part_ld, const float* __restrict__ inv_scale,
+                            const T* __restrict__ x, const float* __restrict__ mu, float tau, int D,
+                            const U* __restrict__ u, float* __restrict__ out,
+                            float* __restrict__ s_out, int64_t main_rows) {
+    pdl_trigger();
+    pdl_wait();
+    const int Q = (D + 3) / 4;
+    const int64_t idx = static_cast<int64_t>(blockIdx.x) * kFinalizeThreads + threadIdx.x;
+    if (idx >= M * Q) return;
+    const int64_t m = div_nonneg(idx, Q);
+    const int d = 4 * static_cast<int>(idx - m * Q);
+    const int ns = m < main_rows ? 1 : splits;
+    const int64_t step = split_stride_rows * part_ld;
+    const float* p = part + m * part_ld;
+    const bool whole = (D & 3) == 0;    // quads of x and out are aligned
+    float xf[4];
+    if (whole) {
+        T h[4];
+        *reinterpret_cast<uint2*>(h) = *reinterpret_cast<const uint2*>(x + m * D + d);
+#pragma unroll
+        for (int e = 0; e < 4; ++e) xf[e] = to_f(h[e]);
+    } else {
+#pragma unroll
+        for (int e = 0; e < 4; ++e) xf[e] = d + e < D ? to_f(x[m * D + d + e]) : 0.f;
+    }
+    const float w = u ? to_f(u[m]) : 1.f;
+    // (Channels up to d + 3 < part_ld exist; mu has D values.)
+    const float4 is = *reinterpret_cast<const float4*>(inv_scale + d);
+    const float isd = inv_scale[D];
+    float mf[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) mf[e] = mu && d + e < D ? mu[d + e] : 0.f;
+    float4 a = *reinterpret_cast<const float4*>(p + d);
+    float ss = p[D];
+    // (Two at a time: more in flight cost registers, and most rows have one.)
+#pragma unroll 2
+    for (int s = 1; s < ns; ++s) {
+        const float4 b = *reinterpret_cast<const float4*>(p + s * step + d);
+        ss += p[s * step + D];
+        a.x += b.x;
+        a.y += b.y;
+        a.z += b.z;
+        a.w += b.w;
+    }
+    const float sd = ss * isd;
+    if (d == 0 && s_out) s_out[m] = sd;
+    if (!out) return;
+    const float v[4] = {a.x * is.x, a.y * is.y, a.z * is.z, a.w * is.w};
+    float o[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) o[e] = tau * (w * fmaf(-(xf[e] - mf[e]), sd, v[e]));
+    float* dst = out + m * D + d;
+    if (whole) {
+        *reinterpret_cast<float4*>(dst) = make_float4(o[0], o[1], o[2], o[3]);
+    } else {
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+            if (d + e < D) dst[e] = o[e];
+    }
+}
+
+// ---------------------------------------------------------------- values of one weight channel
+// value_max_kernel and value_prep_kernel for the D + 1 channels of one weight
+// channel (channels w (x - mu) and w).  A block stages kValueRows rows of x,
+// one contiguous run, in shared memory with 16-byte loads (any D), then takes
+// per-channel maxima, or writes 16 keys of a channel per thread (two 16-byte
+// stores, whole sectors).  The element-wise kernels read 2 bytes at a time and
+// stored 4: 131072 keys, D = 32, ncu: 19.6 + 24.1 us, these 9.3 + 11.8.
+constexpr int kValueRows = 128;
+constexpr int kValueThreads = 128;
+
+// Rows [n0, n0 + kValueRows) of x into raw (zeros past N); weights into sw (1
+// without weights, 0 past N).
+template <typename T, typename W>
+__device__ __forceinline__ void stage_value_rows(const W* __restrict__ w, const T* __restrict__ x,
+                                                 int64_t N, int D, int64_t n0, T* raw, float* sw) {
+    const int rows = static_cast<int>(max(int64_t(0), min(static_cast<int64_t>(kValueRows), N - n0)));
+    const T* src = x + n0 * D;          // n0 is a multiple of 128: 16-byte aligned
+    const int n_el = rows * D, nvec = n_el / 8;
+    for (int i = threadIdx.x; i < nvec; i += kValueThreads)
+        reinterpret_cast<uint4*>(raw)[i] = reinterpret_cast<const uint4*>(src)[i];
+    for (int i = nvec * 8 + threadIdx.x; i < n_el; i += kValueThreads) raw[i] = src[i];
+    for (int i = n_el + threadIdx.x; i < kValueRows * D; i += kValueThreads) raw[i] = from_f<T>(0.f);
+    for (int i = threadIdx.x; i < kValueRows; i += kValueThreads)
+        sw[i] = i < rows ? (w ? to_f(w[n0 + i]) : 1.f) : 0.f;
+    __syncthreads();
+}
+
+template <typename T, typename W>
+__global__ void __launch_bounds__(kValueThreads)
+point_value_max_kernel(const W* __restrict__ w, const T* __restrict__ x,
+                       const float* __restrict__ mu, int64_t N, int D,
+                       unsigned* __restrict__ vmax_bits) {
+    pdl_trigger();
+    pdl_wait();
+    extern __shared__ __align__(16) uint8_t value_smem[];
+    T* raw = reinterpret_cast<T*>(value_smem);
+    __shared__ float sw[kValueRows];
+    __shared__ unsigned big[257];
+    for (int i = threadIdx.x; i <= D; i += kValueThreads) big[i] = 0u;
+    const int64_t n0 = static_cast<int64_t>(blockIdx.x) * kValueRows;
+    stage_value_rows(w, x, N, D, n0, raw, sw);
+    const int rows = static_cast<int>(min(static_cast<int64_t>(kValueRows), N - n0));
+    // Lanes take coordinates, warps rows.
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int d = lane; d <= D; d += 32) {
+        const float m = d < D && mu ? mu[d] : 0.f;
+        float mx = 0.f;
+        for (int r = warp; r < rows; r += kValueThreads / 32)
+            mx = fmaxf(mx, fabsf(d < D ? sw[r] * (to_f(raw[r * D + d]) - m) : sw[r]));
+        // Non-negative floats order like their bit patterns.
+        atomicMax(&big[d], __float_as_uint(mx));
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i <= D; i += kValueThreads)
+        if (big[i] != 0u) atomicMax(&vmax_bits[i], big[i]);
+}
+
+template <typename T, typename W>
+__global__ void __launch_bounds__(kValueThreads)
+point_value_prep_kernel(const W* __restrict__ w, const T* __restrict__ x,
+                        const float* __restrict__ mu, int64_t N, int64_t Npad, int D, int Cp,
+                        const unsigned* __restrict__ vmax_bits, __half* __restrict__ vt,
+                        float* __restrict__ inv_scale) {
+    pdl_trigger();
+    pdl_wait();
+    extern __shared__ __align__(16) uint8_t value_smem[];
+    T* raw = reinterpret_cast<T*>(value_smem);
+    __shared__ float sw[kValueRows];
+    const int64_t n0 = static_cast<int64_t>(blockIdx.x) * kValueRows;
+    stage_value_rows(w, x, N, D, n0, raw, sw);
+    // (Npad is a multiple of 128, so the block's keys are all inside.)  Item
+    // i: channel i mod Cp, keys 16 (i / Cp) .. + 15 of the block.
+    for (int i = threadIdx.x; i < Cp * (kValueRows / 16); i += kValueThreads) {
+        const int g = i / Cp, c = i - g * Cp;
+        const float sc = c <= D ? pow2f(channel_exponent(vmax_bits[c])) : 0.f;
+        const float m = c < D && mu ? mu[c] : 0.f;
+        __half2 h[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            float v[2];
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                const int r = 16 * g + 2 * k + e;
+                v[e] = c < D ? sw[r] * (to_f(raw[r * D + c]) - m) : c == D ? sw[r] : 0.f;
+            }
+            h[k] = __floats2half2_rn(v[0] * sc, v[1] * sc);
+        }
+        uint4* dst = reinterpret_cast<uint4*>(vt + static_cast<int64_t>(c) * Npad + n0 + 16 * g);
+        dst[0] = reinterpret_cast<const uint4*>(h)[0];
+        dst[1] = reinterpret_cast<const uint4*>(h)[1];
+    }
+    if (blockIdx.x == 0)
+        for (int c = threadIdx.x; c < Cp; c += kValueThreads)
+            inv_scale[c] = c <= D ? pow2f(-channel_exponent(vmax_bits[c])) : 0.f;
+}
+
 template <typename T, typename W, bool GRAD>
 cudaError_t value_prep_typed(const void* w, const void* x, const float* mu, int64_t N,
                              int64_t Npad, int D, int Cw, int ch0, int Cc, int Cp,
-                             unsigned* vmax_bits, void* vt, float* inv_scale, cudaStream_t s) {
-    cudaError_t e = cudaMemsetAsync(vmax_bits, 0, sizeof(unsigned) * Cp, s);
-    if (e != cudaSuccess) return e;
-    pdl_reset();   // the next kernel follows a memset
+                             unsigned* vmax_bits, void* vt, float* inv_scale, cudaStream_t s,
+                             bool zeroed) {
+    cudaError_t e = cudaSuccess;
+    if (!zeroed) {
+        e = cudaMemsetAsync(vmax_bits, 0, sizeof(unsigned) * Cp, s);
+        if (e != cudaSuccess) return e;
+        pdl_reset();   // the next kernel follows a memset
+    }
+    if (GRAD && Cw == 1 && ch0 == 0 && Cc == D + 1 && D >= 1 && N > 0) {
+        const size_t smem = static_cast<size_t>(kValueRows) * D * sizeof(T);
+        auto go = [&](auto kern, unsigned blocks, auto... args) {
+            cudaError_t r = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                 static_cast<int>(smem));
+            if (r != cudaSuccess) return r;
+            launch_kernel(kern, blocks, kValueThreads, smem, s, args...);
+            note_launches(1);
+            return cudaGetLastError();
+        };
+        e = go(point_value_max_kernel<T, W>, static_cast<unsigned>((N + kValueRows - 1) / kValueRows),
+               static_cast<const W*>(w), static_cast<const T*>(x), mu, N, D, vmax_bits);
+        if (e != cudaSuccess) return e;
+        return go(point_value_prep_kernel<T, W>, static_cast<unsigned>(Npad / kValueRows),
+                  static_cast<const W*>(w), static_cast<const T*>(x), mu, N, Npad, D, Cp,
+                  static_cast<const unsigned*>(vmax_bits), static_cast<__half*>(vt), inv_scale);
+    }
     // 64 rows per block: several blocks per SM even for N of a few 10^4.
     const int64_t rows_per_block = 64;
     const int64_t blocks = N > 0 ? (N + rows_per_block - 1) / rows_per_block : 0;
@@ -1523,6 +1752,17 @@ cudaError_t finalize_points_typed(const float* part, int splits, int64_t stride_
                                   cudaStream_t s, int64_t main_rows) {
     const int64_t total = M * (D > 0 ? D : 1);
     if (total == 0) return cudaSuccess;
+    if constexpr (!DIRECT) {
+        if (D >= 1 && Cw == 1 && ch0 == 0 && Cc == D + 1 && !accumulate && inv_scale && part_ld % 4 == 0) {
+            launch_kernel(finalize_point_quads_kernel<T, U>,
+                          static_cast<unsigned>((M * ((D + 3) / 4) + kFinalizeThreads - 1) / kFinalizeThreads),
+                          kFinalizeThreads, 0, s, part, splits, stride_rows, M, part_ld, inv_scale,
+                          static_cast<const T*>(x), mu, tau, D, static_cast<const U*>(u), out, s_out,
+                          main_rows);
+            note_launches(1);
+            return cudaGetLastError();
+        }
+    }
     const int threads = 256;
     const int64_t blocks = (total + threads - 1) / threads;
     launch_kernel(finalize_points_kernel<DIRECT, T, U>, static_cast<unsigned>(blocks), threads, 0, s, 
@@ -1536,7 +1776,7 @@ cudaError_t finalize_points_typed(const float* part, int splits, int64_t stride_
 
 cudaError_t launch_mean(InType t, const void* q, const void* k, int64_t M, int64_t N, int D,
                         int blocks, float* partial, float* mu, cudaStream_t s, int batch,
-                        const RecordArgs* rec, bool* rec_done, unsigned* zero_word) {
+                        const RecordArgs* rec, bool* rec_done, ZeroWords zero) {
     if (rec_done) *rec_done = false;
     // q and k the same points: the mean of [q; q] is the mean of q.
     if (q == k && M == N) N = 0;
@@ -1629,13 +1869,13 @@ cudaError_t launch_mean(InType t, const void* q, const void* k, int64_t M, int64
     const int min_exp = t == InType::F16 ? -24 : t == InType::BF16 ? -133 : -149;
     if (G > kMeanFinalThreadMax) {
         launch_kernel(mean_final_block_kernel, dim3(D, batch), kMeanFinalThreads, 0, s, partial,
-                      G, D, static_cast<float>(total), mant_bits, min_exp, mu, zero_word);
+                      G, D, static_cast<float>(total), mant_bits, min_exp, mu, zero);
     } else {
         const int64_t items = static_cast<int64_t>(batch) * D;
         launch_kernel(mean_final_kernel,
                       dim3(static_cast<unsigned>((items + kMeanFinalThreads - 1) / kMeanFinalThreads)),
                       kMeanFinalThreads, 0, s, partial, G, D, items, static_cast<float>(total),
-                      mant_bits, min_exp, mu, zero_word);
+                      mant_bits, min_exp, mu, zero);
     }
     note_launches(1);
     return cudaGetLastError();
@@ -1782,9 +2022,9 @@ cudaError_t launch_tf32_split(const float* x, int64_t rows, int64_t rows_pad, in
 cudaError_t launch_value_prep(InType t, bool grad, bool w_f32, const void* w, const void* x,
                               const float* mu, int64_t N, int64_t Npad, int D, int Cw, int ch0,
                               int Cc, int Cp, unsigned* vmax_bits, void* vt, float* inv_scale,
-                              cudaStream_t s) {
+                              cudaStream_t s, bool zeroed) {
 #define GS_VALUE_PREP(T, W, G) \
-    value_prep_typed<T, W, G>(w, x, mu, N, Npad, D, Cw, ch0, Cc, Cp, vmax_bits, vt, inv_scale, s)
+    value_prep_typed<T, W, G>(w, x, mu, N, Npad, D, Cw, ch0, Cc, Cp, vmax_bits, vt, inv_scale, s, zeroed)
     if (t == InType::BF16) {
         if (!grad)
             return w_f32 ? GS_VALUE_PREP(__nv_bfloat16, float, false)
@@ -1837,11 +2077,13 @@ cudaError_t launch_vf_flags(float* rec, int64_t Npad, int batch, cudaStream_t s)
 cudaError_t launch_weight_prep(InType t, const void* rsrc, bool r_f32, int64_t R, int64_t Rpad,
                                const void* csrc, bool c_f32, int64_t Ncol, int64_t Npad, int C,
                                int WT, int BN, float* rowf, float* colT, unsigned* wmax,
-                               cudaStream_t s) {
+                               cudaStream_t s, bool zeroed) {
     if (WT <= 0 || kWeightThreads % WT != 0 || C > WT) return cudaErrorInvalidValue;
-    cudaError_t e = cudaMemsetAsync(wmax, 0, sizeof(unsigned) * 2 * WT, s);
-    if (e != cudaSuccess) return e;
-    pdl_reset();   // the next kernel follows a memset
+    if (!zeroed) {
+        const cudaError_t e = cudaMemsetAsync(wmax, 0, sizeof(unsigned) * 2 * WT, s);
+        if (e != cudaSuccess) return e;
+        pdl_reset();   // the next kernel follows a memset
+    }
     const int64_t rb = (Rpad * WT + kWeightThreads - 1) / kWeightThreads;
     const int64_t cb = (Npad * WT + kWeightThreads - 1) / kWeightThreads;
     if (rb + cb == 0) return cudaSuccess;
@@ -1873,6 +2115,13 @@ cudaError_t launch_finalize(const float* part, int splits, int64_t split_stride_
                             cudaStream_t s, int64_t main_rows, const unsigned* guard) {
     const int64_t total = M * Cv;
     if (total == 0) return cudaSuccess;
+    if (Cv % 4 == 0 && part_ld % 4 == 0 && !guard) {
+        launch_kernel(finalize_quads_kernel,
+                      static_cast<unsigned>((total / 4 + kFinalizeThreads - 1) / kFinalizeThreads),
+                      kFinalizeThreads, 0, s, part, splits, split_stride_rows, M, Cv, part_ld, inv_scale, out, main_rows);
+        note_launches(1);
+        return cudaGetLastError();
+    }
     const int threads = 256;
     const int64_t blocks = (total + threads - 1) / threads;
     launch_kernel(finalize_kernel, static_cast<unsigned>(blocks), threads, 0, s, 

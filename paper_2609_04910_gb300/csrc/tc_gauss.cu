@@ -945,7 +945,9 @@ bool plan_tensor(InType t, int64_t M, int64_t N, int64_t D, int64_t C, bool grad
     } else {
         p->off_rec = 0;
         p->off_vt = take(static_cast<size_t>(p->Cp) * p->Npad * 2);
-        p->off_vmax = take(static_cast<size_t>(p->Cp) * 4);
+        // (The weighted passes' maxima wmax follow the channels' vmax, so that
+        // one launch clears both.)
+        p->off_vmax = take((static_cast<size_t>(p->Cp) + 2 * wt) * 4);
         p->off_inv = take(static_cast<size_t>(p->Cp) * 4);
         p->off_part = take(static_cast<size_t>(p->splits) * p->Mpad * p->Cp * 4);
     }
@@ -953,7 +955,7 @@ bool plan_tensor(InType t, int64_t M, int64_t N, int64_t D, int64_t C, bool grad
     if (wt > 0) {
         p->off_rowf = take(static_cast<size_t>(p->Mpad) * wt * 4);
         p->off_colT = take(static_cast<size_t>(p->Npad) * wt * 4);
-        p->off_wmax = take(static_cast<size_t>(2) * wt * 4);
+        p->off_wmax = p->off_vmax + static_cast<size_t>(p->Cp) * 4;
     }
     p->total = off;
     return true;
