@@ -393,6 +393,8 @@ gs_status run(Call c) {
         // values only: the mean launch writes them where it can.
         bool records_done = false;
         bool flags_done = false;   // folded values: per-problem flags written by the operand launch
+        const float ninf = -INFINITY;
+        bool prepared = false;     // mean and operands written
         if (mu) {
             // Words that later launches take maxima into: the guard, or the
             // two-MMA kernel's channel and weight maxima.
@@ -401,14 +403,30 @@ gs_status run(Call c) {
             else if (!tp.fma) zero = {reinterpret_cast<unsigned*>(ws + tp.off_vmax), tp.Cp + 2 * tp.wt};
             const gs::RecordArgs rec = {c.v, c.w_f32, c.N, tp.Npad, static_cast<int>(tp.Cv),
                                         reinterpret_cast<float*>(ws + tp.off_rec), tp.vfold};
-            e = gs::launch_mean(t, c.q, c.k, c.M, c.N, static_cast<int>(c.D), tp.mean_blocks,
-                                reinterpret_cast<float*>(ws + tp.off_mean_part), mu, c.stream,
-                                batch, (tp.fma && tp.aug) ? &rec : nullptr, &records_done, zero);
-            where = "mean kernel";
+            if (tp.fma && !tp.tf && gs::prep_cluster_fits(t, c.q, c.k, c.M, c.N, static_cast<int>(c.D), tp.Dp,
+                                                tp.mean_blocks, tp.aug, batch)) {
+                records_done = tp.fma && tp.aug;
+                flags_done = records_done && tp.vfold;
+                prepared = true;
+                e = gs::launch_prep_cluster(
+                    t, tp.aug, c.q, c.M, tp.Mpad, ws + tp.off_qh,
+                    (tp.aug && tp.alias) ? ws + tp.off_kh : nullptr,
+                    tp.aug ? nullptr : reinterpret_cast<float*>(ws + tp.off_A), !tp.alias, c.k, c.N,
+                    tp.Npad, ws + tp.off_kh, tp.aug ? nullptr : reinterpret_cast<float*>(ws + tp.off_B),
+                    static_cast<int>(c.D), tp.Dp, tp.mean_blocks, mu, half_c, ninf, c.stream, batch,
+                    tp.vfold ? c.v : nullptr, (tp.vfold || tp.cfold) ? cexp : 0.f,
+                    records_done ? &rec : nullptr,
+                    flags_done ? reinterpret_cast<float*>(ws + tp.off_rec) : nullptr, zero);
+                where = "preparation kernel";
+            } else {
+                e = gs::launch_mean(t, c.q, c.k, c.M, c.N, static_cast<int>(c.D), tp.mean_blocks,
+                                    reinterpret_cast<float*>(ws + tp.off_mean_part), mu, c.stream,
+                                    batch, (tp.fma && tp.aug) ? &rec : nullptr, &records_done, zero);
+                where = "mean kernel";
+            }
         }
-        const float ninf = -INFINITY;
-        if (e != cudaSuccess) {
-            // an error: nothing more is launched
+        if (e != cudaSuccess || prepared) {
+            // an error: nothing more is launched; or nothing left to prepare
         } else if (tp.tf) {
             // 3xTF32 operands: hi / lo tf32 halves and the norm terms.
             e = gs::launch_tf32_split(static_cast<const float*>(c.q), c.M, tp.Mpad,

@@ -204,6 +204,19 @@ cudaError_t launch_operands(InType t, bool aug, const void* q, int64_t M, int64_
                             const float* mu, float half_c, float pad_value, cudaStream_t s,
                             int batch = 1, const void* vw = nullptr, float cf = 0.f,
                             float* vf_rec = nullptr, bool* flags_done = nullptr);
+// Small 16-bit problems: the mean, operands, records and flags of the two
+// launches above in one, with the same results; see prep_cluster_kernel.
+// prep_cluster_fits says whether a call is one.
+constexpr int64_t kPrepMaxRows = 2048;       // M + N (M for q = k) per problem
+constexpr int64_t kPrepMaxElements = int64_t(1) << 17;   // (M + N) D
+constexpr int64_t kPrepMaxBlocks = 152;      // clusters' blocks, at most one wave
+bool prep_cluster_fits(InType t, const void* q, const void* k, int64_t M, int64_t N, int D, int Dp, int blocks,
+                       bool aug, int batch);
+cudaError_t launch_prep_cluster(InType t, bool aug, const void* q, int64_t M, int64_t Mpad, void* qh,
+                                void* qh_as_key, float* nrm_q, bool with_k, const void* k, int64_t N,
+                                int64_t Npad, void* kh, float* nrm_k, int D, int Dp, int blocks, float* mu,
+                                float half_c, float pad_value, cudaStream_t s, int batch, const void* vw,
+                                float cf, const RecordArgs* rec, float* vf_rec, ZeroWords zero);
 // Transposed fp16 value operand of the two-MMA kernel for the channels
 // ch0 .. ch0 + Cc - 1 (Cp >= Cc rows of Npad keys), with per-channel
 // power-of-two scales.  Forward: channel ch of key n is w[n, ch] (w has the

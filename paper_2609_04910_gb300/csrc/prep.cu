@@ -17,6 +17,7 @@
 #include <algorithm>
 #include <type_traits>
 
+#include <cooperative_groups.h>
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 #include <math_constants.h>
@@ -106,6 +107,13 @@ __global__ void mean_partial_kernel(const T* __restrict__ q, const T* __restrict
 // a launch of their own later in the chain.
 constexpr int kMeanVecThreads = 256;
 
+// How the rows of [q; k] are split into partial sums (see mean_split).
+struct MeanSplit {
+    bool vec;            // mean_partial_vec_kernel's split, else mean_partial_rows_kernel's
+    int64_t rpb;         // rows per partial
+    int Gq, G;           // partials of q (vec), of both
+};
+
 template <typename TV>
 struct RecordJob {
     const TV* v;         // N x C values per problem (batch-stacked)
@@ -179,33 +187,22 @@ __device__ __forceinline__ void write_key_record(const RecordJob<TV>& j, int64_t
     }
 }
 
-template <typename T, typename TV>
-__global__ void __launch_bounds__(kMeanVecThreads)
-mean_partial_vec_kernel(const T* __restrict__ q, const T* __restrict__ k, int64_t M, int64_t N,
-                        int D, int64_t rows_per_block, int Gq, int G, float* __restrict__ partial,
-                        const RecordJob<TV> rj) {
-    pdl_trigger();
-    pdl_wait();
-    if (static_cast<int>(blockIdx.x) >= G) {
-        const int64_t t = static_cast<int64_t>(blockIdx.x - G) * kMeanVecThreads + threadIdx.x;
-        if (rj.signs) {
-            if constexpr (std::is_same<TV, __half>::value) {
-                if (t < 2 * rj.pairs) write_sign_record(rj.v, rj.N, rj.rec, t, blockIdx.y, 2 * rj.pairs);
-            }
-        } else if (t < rj.pairs) {
-            write_key_record(rj, t, blockIdx.y);
-        }
-        return;
-    }
-    __shared__ float s_sum[kMeanVecThreads][9];
-    __shared__ float s_max[kMeanVecThreads][9];
+struct MeanShared {
+    float sum[kMeanVecThreads][9];
+    float max[kMeanVecThreads][9];
+};
+
+// Partial sums and maxima of block `block` of the split, by the whole thread
+// block, into D values each.
+template <typename T>
+__device__ __forceinline__ void mean_vec_block(const T* __restrict__ q, const T* __restrict__ k, int64_t M,
+                                               int64_t N, int D, int64_t rows_per_block, int Gq, int block,
+                                               MeanShared& sh, float* out_sum, float* out_max) {
+    auto& s_sum = sh.sum;
+    auto& s_max = sh.max;
     const int t = threadIdx.x;
-    // Problem blockIdx.y of a batch: its own points and partial rows.
-    q += static_cast<int64_t>(blockIdx.y) * M * D;
-    k += static_cast<int64_t>(blockIdx.y) * N * D;
-    partial += static_cast<int64_t>(blockIdx.y) * 2 * G * D;
-    const bool on_q = static_cast<int>(blockIdx.x) < Gq;
-    const int64_t b = on_q ? blockIdx.x : blockIdx.x - Gq;
+    const bool on_q = block < Gq;
+    const int64_t b = on_q ? block : block - Gq;
     const int64_t rows = on_q ? M : N;
     const T* x = on_q ? q : k;
     const int64_t r0 = b * rows_per_block;
@@ -250,9 +247,36 @@ mean_partial_vec_kernel(const T* __restrict__ q, const T* __restrict__ k, int64_
             a += s_sum[u][e];
             m = fmaxf(m, s_max[u][e]);
         }
-        partial[static_cast<int64_t>(blockIdx.x) * D + d] = a;
-        partial[static_cast<int64_t>(G + blockIdx.x) * D + d] = m;
+        out_sum[d] = a;
+        out_max[d] = m;
     }
+}
+
+template <typename T, typename TV>
+__global__ void __launch_bounds__(kMeanVecThreads)
+mean_partial_vec_kernel(const T* __restrict__ q, const T* __restrict__ k, int64_t M, int64_t N,
+                        int D, int64_t rows_per_block, int Gq, int G, float* __restrict__ partial,
+                        const RecordJob<TV> rj) {
+    pdl_trigger();
+    pdl_wait();
+    if (static_cast<int>(blockIdx.x) >= G) {
+        const int64_t t = static_cast<int64_t>(blockIdx.x - G) * kMeanVecThreads + threadIdx.x;
+        if (rj.signs) {
+            if constexpr (std::is_same<TV, __half>::value) {
+                if (t < 2 * rj.pairs) write_sign_record(rj.v, rj.N, rj.rec, t, blockIdx.y, 2 * rj.pairs);
+            }
+        } else if (t < rj.pairs) {
+            write_key_record(rj, t, blockIdx.y);
+        }
+        return;
+    }
+    // Problem blockIdx.y of a batch: its own points and partial rows.
+    __shared__ MeanShared sh;
+    partial += static_cast<int64_t>(blockIdx.y) * 2 * G * D;
+    mean_vec_block(q + static_cast<int64_t>(blockIdx.y) * M * D, k + static_cast<int64_t>(blockIdx.y) * N * D,
+                   M, N, D, rows_per_block, Gq, static_cast<int>(blockIdx.x), sh,
+                   partial + static_cast<int64_t>(blockIdx.x) * D,
+                   partial + static_cast<int64_t>(G + blockIdx.x) * D);
 }
 
 // Any other width up to 256 (16-bit inputs): the partial sums and maxima of
@@ -267,33 +291,17 @@ mean_partial_vec_kernel(const T* __restrict__ q, const T* __restrict__ k, int64_
 // Bound: load latency (ncu, with the records: 50021 points of D = 50 6.4 us,
 // where mean_partial_kernel took 7.2 us and the records and their flags two
 // more launches, 7.5 us).
-template <typename T, typename TV>
-__global__ void __launch_bounds__(kMeanVecThreads)
-mean_partial_rows_kernel(const T* __restrict__ q, const T* __restrict__ k, int64_t M, int64_t N,
-                         int D, int64_t rows_per_block, int G, int chunks, int mblocks,
-                         float* __restrict__ partial, const RecordJob<TV> rj) {
-    pdl_trigger();
-    pdl_wait();
-    if (static_cast<int>(blockIdx.x) >= mblocks) {
-        const int64_t t = static_cast<int64_t>(blockIdx.x - mblocks) * kMeanVecThreads + threadIdx.x;
-        if (rj.signs) {
-            if constexpr (std::is_same<TV, __half>::value) {
-                if (t < 2 * rj.pairs) write_sign_record(rj.v, rj.N, rj.rec, t, blockIdx.y, 2 * rj.pairs);
-            }
-        } else if (t < rj.pairs) {
-            write_key_record(rj, t, blockIdx.y);
-        }
-        return;
-    }
-    __shared__ float s_sum[kMeanVecThreads][9];
-    __shared__ float s_max[kMeanVecThreads][9];
-    // Problem blockIdx.y of a batch: its own points and partial rows.
-    q += static_cast<int64_t>(blockIdx.y) * M * D;
-    k += static_cast<int64_t>(blockIdx.y) * N * D;
-    partial += static_cast<int64_t>(blockIdx.y) * 2 * G * D;
+// Chunks [chunk0, chunk0 + chunks) of the split into G, by the whole thread
+// block; put(chunk, d, sum, max) takes the results.
+template <typename T, typename Put>
+__device__ __forceinline__ void mean_rows_block(const T* __restrict__ q, const T* __restrict__ k, int64_t M,
+                                                int64_t N, int D, int64_t rows_per_block, int G, int chunks,
+                                                int chunk0, MeanShared& sh, Put put) {
+    auto& s_sum = sh.sum;
+    auto& s_max = sh.max;
     const int local = static_cast<int>(threadIdx.x) / D;     // chunk of this block
     const int t = static_cast<int>(threadIdx.x) - local * D;
-    const int chunk = static_cast<int>(blockIdx.x) * chunks + local;
+    const int chunk = chunk0 + local;
     float sum[8], mx[8];
 #pragma unroll
     for (int e = 0; e < 8; ++e) sum[e] = mx[e] = 0.f;
@@ -382,8 +390,36 @@ mean_partial_rows_kernel(const T* __restrict__ q, const T* __restrict__ k, int64
         a += s_sum[u][e];
         m = fmaxf(m, s_max[u][e]);
     }
-    partial[static_cast<int64_t>(chunk) * D + t] = a;
-    partial[static_cast<int64_t>(G + chunk) * D + t] = m;
+    put(chunk, t, a, m);
+}
+
+template <typename T, typename TV>
+__global__ void __launch_bounds__(kMeanVecThreads)
+mean_partial_rows_kernel(const T* __restrict__ q, const T* __restrict__ k, int64_t M, int64_t N,
+                         int D, int64_t rows_per_block, int G, int chunks, int mblocks,
+                         float* __restrict__ partial, const RecordJob<TV> rj) {
+    pdl_trigger();
+    pdl_wait();
+    if (static_cast<int>(blockIdx.x) >= mblocks) {
+        const int64_t t = static_cast<int64_t>(blockIdx.x - mblocks) * kMeanVecThreads + threadIdx.x;
+        if (rj.signs) {
+            if constexpr (std::is_same<TV, __half>::value) {
+                if (t < 2 * rj.pairs) write_sign_record(rj.v, rj.N, rj.rec, t, blockIdx.y, 2 * rj.pairs);
+            }
+        } else if (t < rj.pairs) {
+            write_key_record(rj, t, blockIdx.y);
+        }
+        return;
+    }
+    // Problem blockIdx.y of a batch: its own points and partial rows.
+    __shared__ MeanShared sh;
+    partial += static_cast<int64_t>(blockIdx.y) * 2 * G * D;
+    mean_rows_block(q + static_cast<int64_t>(blockIdx.y) * M * D, k + static_cast<int64_t>(blockIdx.y) * N * D,
+                    M, N, D, rows_per_block, G, chunks, static_cast<int>(blockIdx.x) * chunks, sh,
+                    [&](int chunk, int d, float sum, float mx) {
+                        partial[static_cast<int64_t>(chunk) * D + d] = sum;
+                        partial[static_cast<int64_t>(G + chunk) * D + d] = mx;
+                    });
 }
 
 // mu_d = the mean of coordinate d rounded to a multiple of g_d, the spacing
@@ -1033,27 +1069,15 @@ struct OperandJob {
 // vectors first and each lane gathers its row's vectors there.  (One warp per
 // row in operand_kernel before: 50021 points, D = 50, both layouts: 26.7 ->
 // 10.1 us, 19 MB moved.)
-template <typename T, bool AUG, int G, bool RAGGED>
-__global__ void __launch_bounds__(kOperandVecThreads)
-operand_vec_kernel(const OperandJob j0, const OperandJob j1, unsigned blocks0, int D, int Dp,
-                   int nt, float F, const float* __restrict__ mu, float half_c, float pad_value,
-                   float cf, unsigned op_blocks, float* __restrict__ vf_rec, int64_t vf_tiles) {
-    using PT = Pair<T>;
-    pdl_trigger();
-    pdl_wait();
-    if (blockIdx.x >= op_blocks) {
-        // Folded values: the per-problem flag of the sign records (written
-        // by an earlier launch of the call), one extra block per problem.
-        write_vf_flag(vf_rec, vf_tiles, static_cast<int>(gridDim.y), blockIdx.y);
-        return;
-    }
-    constexpr int SLOTS = kOperandVecThreads / G;   // rows of a block
-    __shared__ uint4 smean[kOperandMaxCols / 8];
-    extern __shared__ uint4 staged[];                // SLOTS rows of each output
-    const int b = blockIdx.y;                        // problem of the batch
-    const bool second = blockIdx.x >= blocks0;
-    const OperandJob j = second ? j1 : j0;
-    const int blk = static_cast<int>(second ? blockIdx.x - blocks0 : blockIdx.x);
+// Rows [blk SLOTS, (blk + 1) SLOTS) of job j, problem b, by the whole block:
+// stage_mean() stages the problem's mean in smean (it runs between the row
+// loads and their use), staged holds the output rows (and, RAGGED, behind
+// them the input rows).
+template <typename T, bool AUG, int G, bool RAGGED, typename StageMean>
+__device__ __forceinline__ void operand_block(const OperandJob& j, int b, int blk, int D, int Dp, int nt,
+                                              float F, float half_c, float pad_value, float cf,
+                                              const uint4* smean, uint4* staged, StageMean stage_mean) {
+    constexpr int SLOTS = kOperandVecThreads / G;    // rows of a block
     const int vi = threadIdx.x % G;                  // first vector of this lane
     const int slot = threadIdx.x / G;
     const int V = RAGGED ? (D + 7) / 8 : D / 8;
@@ -1107,13 +1131,7 @@ operand_vec_kernel(const OperandJob j0, const OperandJob j1, unsigned blocks0, i
                                         : make_uint4(0u, 0u, 0u, 0u);
         }
     }
-    const float* mb = mu ? mu + static_cast<int64_t>(b) * D : nullptr;
-    typename PT::P* sm = reinterpret_cast<typename PT::P*>(smean);
-    for (int c = threadIdx.x; c < 4 * V; c += kOperandVecThreads) {
-        const float m0 = mb && 2 * c < D ? mb[2 * c] : 0.f;
-        const float m1 = mb && 2 * c + 1 < D ? mb[2 * c + 1] : 0.f;
-        sm[c] = PT::from_f2(m0, m1);
-    }
+    stage_mean();
     __syncthreads();
     const bool in_pad = i < rows_pad;
     const int64_t row = static_cast<int64_t>(b) * rows_pad + i;   // batch-stacked output row
@@ -1142,6 +1160,38 @@ operand_vec_kernel(const OperandJob j0, const OperandJob j1, unsigned blocks0, i
         if (wq) gq[u] = stage_q[s];
         if (wk) gk[u] = stage_k[s];
     }
+}
+
+template <typename T, bool AUG, int G, bool RAGGED>
+__global__ void __launch_bounds__(kOperandVecThreads)
+operand_vec_kernel(const OperandJob j0, const OperandJob j1, unsigned blocks0, int D, int Dp,
+                   int nt, float F, const float* __restrict__ mu, float half_c, float pad_value,
+                   float cf, unsigned op_blocks, float* __restrict__ vf_rec, int64_t vf_tiles) {
+    using PT = Pair<T>;
+    pdl_trigger();
+    pdl_wait();
+    if (blockIdx.x >= op_blocks) {
+        // Folded values: the per-problem flag of the sign records (written
+        // by an earlier launch of the call), one extra block per problem.
+        write_vf_flag(vf_rec, vf_tiles, static_cast<int>(gridDim.y), blockIdx.y);
+        return;
+    }
+    __shared__ uint4 smean[kOperandMaxCols / 8];
+    extern __shared__ uint4 staged[];                // the block's rows of each output
+    const int b = blockIdx.y;                        // problem of the batch
+    const bool second = blockIdx.x >= blocks0;
+    const OperandJob j = second ? j1 : j0;
+    const int blk = static_cast<int>(second ? blockIdx.x - blocks0 : blockIdx.x);
+    const int V = RAGGED ? (D + 7) / 8 : D / 8;
+    operand_block<T, AUG, G, RAGGED>(j, b, blk, D, Dp, nt, F, half_c, pad_value, cf, smean, staged, [&] {
+        const float* mb = mu ? mu + static_cast<int64_t>(b) * D : nullptr;
+        typename PT::P* sm = reinterpret_cast<typename PT::P*>(smean);
+        for (int c = threadIdx.x; c < 4 * V; c += kOperandVecThreads) {
+            const float m0 = mb && 2 * c < D ? mb[2 * c] : 0.f;
+            const float m1 = mb && 2 * c + 1 < D ? mb[2 * c + 1] : 0.f;
+            sm[c] = PT::from_f2(m0, m1);
+        }
+    });
 }
 
 template <typename T, bool AUG>
@@ -1612,68 +1662,47 @@ constexpr int kValueRows = 128;
 constexpr int kValueThreads = 128;
 
 // Rows [n0, n0 + kValueRows) of x into raw (zeros past N); weights into sw (1
-// without weights, 0 past N).
+// without weights, 0 past N).  By the whole block.
 template <typename T, typename W>
 __device__ __forceinline__ void stage_value_rows(const W* __restrict__ w, const T* __restrict__ x,
                                                  int64_t N, int D, int64_t n0, T* raw, float* sw) {
     const int rows = static_cast<int>(max(int64_t(0), min(static_cast<int64_t>(kValueRows), N - n0)));
+    const int nt = blockDim.x;
     const T* src = x + n0 * D;          // n0 is a multiple of 128: 16-byte aligned
     const int n_el = rows * D, nvec = n_el / 8;
-    for (int i = threadIdx.x; i < nvec; i += kValueThreads)
+    for (int i = threadIdx.x; i < nvec; i += nt)
         reinterpret_cast<uint4*>(raw)[i] = reinterpret_cast<const uint4*>(src)[i];
-    for (int i = nvec * 8 + threadIdx.x; i < n_el; i += kValueThreads) raw[i] = src[i];
-    for (int i = n_el + threadIdx.x; i < kValueRows * D; i += kValueThreads) raw[i] = from_f<T>(0.f);
-    for (int i = threadIdx.x; i < kValueRows; i += kValueThreads)
+    for (int i = nvec * 8 + threadIdx.x; i < n_el; i += nt) raw[i] = src[i];
+    for (int i = n_el + threadIdx.x; i < kValueRows * D; i += nt) raw[i] = from_f<T>(0.f);
+    for (int i = threadIdx.x; i < kValueRows; i += nt)
         sw[i] = i < rows ? (w ? to_f(w[n0 + i]) : 1.f) : 0.f;
     __syncthreads();
 }
 
-template <typename T, typename W>
-__global__ void __launch_bounds__(kValueThreads)
-point_value_max_kernel(const W* __restrict__ w, const T* __restrict__ x,
-                       const float* __restrict__ mu, int64_t N, int D,
-                       unsigned* __restrict__ vmax_bits) {
-    pdl_trigger();
-    pdl_wait();
-    extern __shared__ __align__(16) uint8_t value_smem[];
-    T* raw = reinterpret_cast<T*>(value_smem);
-    __shared__ float sw[kValueRows];
-    __shared__ unsigned big[257];
-    for (int i = threadIdx.x; i <= D; i += kValueThreads) big[i] = 0u;
-    const int64_t n0 = static_cast<int64_t>(blockIdx.x) * kValueRows;
-    stage_value_rows(w, x, N, D, n0, raw, sw);
-    const int rows = static_cast<int>(min(static_cast<int64_t>(kValueRows), N - n0));
-    // Lanes take coordinates, warps rows.
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+// Largest |value| per channel of the staged rows, into big (float bits; lanes
+// take coordinates, warps rows).
+template <typename T>
+__device__ __forceinline__ void value_rows_max(const T* raw, const float* sw, const float* mu, int rows,
+                                               int D, unsigned* big) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
     for (int d = lane; d <= D; d += 32) {
         const float m = d < D && mu ? mu[d] : 0.f;
         float mx = 0.f;
-        for (int r = warp; r < rows; r += kValueThreads / 32)
+        for (int r = warp; r < rows; r += warps)
             mx = fmaxf(mx, fabsf(d < D ? sw[r] * (to_f(raw[r * D + d]) - m) : sw[r]));
         // Non-negative floats order like their bit patterns.
         atomicMax(&big[d], __float_as_uint(mx));
     }
-    __syncthreads();
-    for (int i = threadIdx.x; i <= D; i += kValueThreads)
-        if (big[i] != 0u) atomicMax(&vmax_bits[i], big[i]);
 }
 
-template <typename T, typename W>
-__global__ void __launch_bounds__(kValueThreads)
-point_value_prep_kernel(const W* __restrict__ w, const T* __restrict__ x,
-                        const float* __restrict__ mu, int64_t N, int64_t Npad, int D, int Cp,
-                        const unsigned* __restrict__ vmax_bits, __half* __restrict__ vt,
-                        float* __restrict__ inv_scale) {
-    pdl_trigger();
-    pdl_wait();
-    extern __shared__ __align__(16) uint8_t value_smem[];
-    T* raw = reinterpret_cast<T*>(value_smem);
-    __shared__ float sw[kValueRows];
-    const int64_t n0 = static_cast<int64_t>(blockIdx.x) * kValueRows;
-    stage_value_rows(w, x, N, D, n0, raw, sw);
-    // (Npad is a multiple of 128, so the block's keys are all inside.)  Item
-    // i: channel i mod Cp, keys 16 (i / Cp) .. + 15 of the block.
-    for (int i = threadIdx.x; i < Cp * (kValueRows / 16); i += kValueThreads) {
+// The staged rows' scaled values into vt: item i is channel i mod Cp, keys
+// 16 (i / Cp) .. + 15 of the block.  (Npad is a multiple of 128, so the
+// block's keys are all inside.)
+template <typename T>
+__device__ __forceinline__ void value_rows_write(const T* raw, const float* sw, const float* mu, int D, int Cp,
+                                                 const unsigned* vmax_bits, int64_t Npad, int64_t n0,
+                                                 __half* __restrict__ vt) {
+    for (int i = threadIdx.x; i < Cp * (kValueRows / 16); i += blockDim.x) {
         const int g = i / Cp, c = i - g * Cp;
         const float sc = c <= D ? pow2f(channel_exponent(vmax_bits[c])) : 0.f;
         const float m = c < D && mu ? mu[c] : 0.f;
@@ -1692,9 +1721,186 @@ point_value_prep_kernel(const W* __restrict__ w, const T* __restrict__ x,
         dst[0] = reinterpret_cast<const uint4*>(h)[0];
         dst[1] = reinterpret_cast<const uint4*>(h)[1];
     }
+}
+
+template <typename T, typename W>
+__global__ void __launch_bounds__(kValueThreads)
+point_value_max_kernel(const W* __restrict__ w, const T* __restrict__ x,
+                       const float* __restrict__ mu, int64_t N, int D,
+                       unsigned* __restrict__ vmax_bits) {
+    pdl_trigger();
+    pdl_wait();
+    extern __shared__ __align__(16) uint8_t value_smem[];
+    T* raw = reinterpret_cast<T*>(value_smem);
+    __shared__ float sw[kValueRows];
+    __shared__ unsigned big[kOperandMaxCols + 1];
+    for (int i = threadIdx.x; i <= D; i += kValueThreads) big[i] = 0u;
+    const int64_t n0 = static_cast<int64_t>(blockIdx.x) * kValueRows;
+    stage_value_rows(w, x, N, D, n0, raw, sw);
+    value_rows_max(raw, sw, mu, static_cast<int>(min(static_cast<int64_t>(kValueRows), N - n0)), D, big);
+    __syncthreads();
+    for (int i = threadIdx.x; i <= D; i += kValueThreads)
+        if (big[i] != 0u) atomicMax(&vmax_bits[i], big[i]);
+}
+
+template <typename T, typename W>
+__global__ void __launch_bounds__(kValueThreads)
+point_value_prep_kernel(const W* __restrict__ w, const T* __restrict__ x,
+                        const float* __restrict__ mu, int64_t N, int64_t Npad, int D, int Cp,
+                        const unsigned* __restrict__ vmax_bits, __half* __restrict__ vt,
+                        float* __restrict__ inv_scale) {
+    pdl_trigger();
+    pdl_wait();
+    extern __shared__ __align__(16) uint8_t value_smem[];
+    T* raw = reinterpret_cast<T*>(value_smem);
+    __shared__ float sw[kValueRows];
+    const int64_t n0 = static_cast<int64_t>(blockIdx.x) * kValueRows;
+    stage_value_rows(w, x, N, D, n0, raw, sw);
+    value_rows_write(raw, sw, mu, D, Cp, vmax_bits, Npad, n0, vt);
     if (blockIdx.x == 0)
         for (int c = threadIdx.x; c < Cp; c += kValueThreads)
             inv_scale[c] = c <= D ? pow2f(-channel_exponent(vmax_bits[c])) : 0.f;
+}
+
+// ---------------------------------------------------------------- small problems in one launch
+// The whole preparation of a small problem by one cluster of kPrepCluster
+// blocks: the partial sums of the mean (the blocks' shares of the split that
+// the separate kernels would use, so that the mean has the same bits), their
+// fold through distributed shared memory, the operand rows, and what rides
+// along: key or sign records, folded-value flags and cleared words.  The
+// smallest calls wait for the host, about 2 us per launch; this takes two
+// launches out.  Its own chain (loads, reduction, two cluster barriers, rows)
+// is longer than that of the three kernels it replaces once a block has more
+// than one chunk of the mean and one block of rows, hence kPrepMaxRows.
+// Measured (whole calls, one GB300, three launches / this one): 1024^2, D = 64
+// 25.3 / 21.0 us, 16 problems of 512^2 25.0 / 22.8, of 600 points (MMD^2)
+// 29.9 / 26.7; beyond the limit 1500 x 2500, D = 64 24.8 / 27.9, 4000 points,
+// D = 50 30.4 / 34.5 us.
+constexpr int kPrepCluster = 8;
+constexpr int kPrepMaxChunks = 8;            // mean chunks per block of the cluster
+constexpr int kPrepMaxParts = 32;            // mean partials folded in sequence (kMeanFinalThreadMax)
+
+template <typename T>
+struct PrepArgs {
+    const T* q;
+    const T* k;
+    int64_t M, N;                            // N = 0 for q = k
+    MeanSplit split;
+    int chunks;                              // chunks per block and step (rows form; 1 otherwise)
+    float total;
+    int mant_bits, min_exp;
+    float* mu;
+    ZeroWords zero;
+    // Records (out null: none) and folded-value flags (vf_rec null: none).
+    RecordArgs rec;
+    float* vf_rec;
+    int64_t vf_tiles;
+    // Operands: blocks [0, nb0) of j0, then of j1.
+    OperandJob j0, j1;
+    int nb0, nb;
+    int D, Dp, nt;
+    float F, half_c, pad_value, cf;
+};
+
+template <typename T, bool AUG, int G, bool RAGGED>
+__global__ void __cluster_dims__(kPrepCluster, 1, 1) __launch_bounds__(kOperandVecThreads)
+prep_cluster_kernel(const PrepArgs<T> a) {
+    namespace cg = cooperative_groups;
+    using PT = Pair<T>;
+    static_assert(kOperandVecThreads == kMeanVecThreads, "one block does both");
+    pdl_trigger();
+    pdl_wait();
+    extern __shared__ uint4 staged[];
+    __shared__ float part[2][kPrepMaxChunks][kOperandMaxCols];
+    __shared__ float mean[kOperandMaxCols];
+    __shared__ uint4 smean[kOperandMaxCols / 8];
+    cg::cluster_group cluster = cg::this_cluster();
+    const int rank = static_cast<int>(cluster.block_rank());
+    const int b = blockIdx.y;                // problem of the batch
+    const int tid = threadIdx.x;
+    const int D = a.D;
+
+    // What depends on the values alone.
+    if (a.rec.out) {
+        const int64_t pairs = a.rec.Npad / 2;
+        const int64_t n = a.rec.signs ? 2 * pairs : pairs;     // signs: whole warps (n % 32 == 0)
+        for (int64_t t = rank * kOperandVecThreads + tid; t < n; t += kPrepCluster * kOperandVecThreads) {
+            if (a.rec.signs) {
+                if constexpr (std::is_same<T, __half>::value)
+                    write_sign_record(static_cast<const __half*>(a.rec.v), a.rec.N, a.rec.out, t, b, a.rec.Npad);
+            } else if (a.rec.v_f32) {
+                write_key_record(RecordJob<float>{static_cast<const float*>(a.rec.v), a.rec.N, pairs, a.rec.C,
+                                                  a.rec.out, false}, t, b);
+            } else {
+                write_key_record(RecordJob<T>{static_cast<const T*>(a.rec.v), a.rec.N, pairs, a.rec.C,
+                                              a.rec.out, false}, t, b);
+            }
+        }
+    }
+    if (rank == 0 && b == 0)
+        for (int i = tid; i < a.zero.n; i += kOperandVecThreads) a.zero.p[i] = 0u;
+
+    // Mean: this block's chunks of the split, then the fold over all of them.
+    const T* q = a.q + static_cast<int64_t>(b) * a.M * D;
+    const T* k = a.k + static_cast<int64_t>(b) * a.N * D;
+    const int W = a.chunks, parts = a.split.G;
+    MeanShared& sh = *reinterpret_cast<MeanShared*>(staged);
+    for (int it = 0;; ++it) {
+        const int chunk0 = (it * kPrepCluster + rank) * W;
+        if (chunk0 >= parts) break;
+        float* ps = part[0][it * W];
+        float* pm = part[1][it * W];
+        if (a.split.vec)
+            mean_vec_block(q, k, a.M, a.N, D, a.split.rpb, a.split.Gq, chunk0, sh, ps, pm);
+        else
+            mean_rows_block(q, k, a.M, a.N, D, a.split.rpb, parts, W, chunk0, sh,
+                            [&](int chunk, int d, float sum, float mx) {
+                                ps[(chunk - chunk0) * kOperandMaxCols + d] = sum;
+                                pm[(chunk - chunk0) * kOperandMaxCols + d] = mx;
+                            });
+        __syncthreads();
+    }
+    cluster.sync();
+    // All partials into this block's own shared memory, then the fold in order
+    // (one thread per coordinate reading the other blocks' memory partial by
+    // partial would wait for each in turn).
+    float* all_sum = reinterpret_cast<float*>(staged);
+    float* all_max = all_sum + kPrepMaxParts * D;
+    for (int g = tid >> 5; g < parts; g += kOperandVecThreads / 32) {
+        const int step = g / W, slot = (step / kPrepCluster) * W + (g - step * W);
+        const float* rp = cluster.map_shared_rank(&part[0][0][0], step % kPrepCluster) + slot * kOperandMaxCols;
+        for (int d = tid & 31; d < D; d += 32) {
+            all_sum[g * D + d] = rp[d];
+            all_max[g * D + d] = rp[kPrepMaxChunks * kOperandMaxCols + d];
+        }
+    }
+    __syncthreads();
+    for (int d = tid; d < D; d += kOperandVecThreads) {
+        float s = 0.f, mx = 0.f;
+#pragma unroll 8
+        for (int g = 0; g < parts; ++g) {
+            s += all_sum[g * D + d];
+            mx = fmaxf(mx, all_max[g * D + d]);
+        }
+        const float m = rounded_mean(s, mx, a.total, a.mant_bits, a.min_exp);
+        mean[d] = m;
+        if (rank == 0) a.mu[static_cast<int64_t>(b) * D + d] = m;
+    }
+    __syncthreads();
+    {
+        typename PT::P* sm = reinterpret_cast<typename PT::P*>(smean);
+        for (int c = tid; c < 4 * ((D + 7) / 8); c += kOperandVecThreads)
+            sm[c] = PT::from_f2(2 * c < D ? mean[2 * c] : 0.f, 2 * c + 1 < D ? mean[2 * c + 1] : 0.f);
+    }
+    if (a.vf_rec && rank == kPrepCluster - 1)   // (the records are visible since the cluster barrier)
+        write_vf_flag(a.vf_rec, a.vf_tiles, static_cast<int>(gridDim.y), b);
+    for (int blk = rank; blk < a.nb; blk += kPrepCluster) {
+        __syncthreads();                        // staged: the previous use is over
+        const bool second = blk >= a.nb0;
+        operand_block<T, AUG, G, RAGGED>(second ? a.j1 : a.j0, b, second ? blk - a.nb0 : blk, D, a.Dp, a.nt,
+                                         a.F, a.half_c, a.pad_value, a.cf, smean, staged, [] {});
+    }
+    cluster.sync();     // other blocks may still read this block's shared memory
 }
 
 template <typename T, typename W, bool GRAD>
@@ -1774,6 +1980,34 @@ cudaError_t finalize_points_typed(const float* part, int splits, int64_t stride_
 
 }  // namespace
 
+namespace {
+
+// How the rows of [q; k] (N = 0 for q = k) are split into at most `blocks`
+// partial sums.
+MeanSplit mean_split(InType t, int64_t M, int64_t N, int D, int blocks) {
+    MeanSplit r;
+    const int64_t total = M + N;
+    r.vec = t != InType::F32 && D >= 8 && D <= 2048 && (D & (D - 1)) == 0 && 2048 % D == 0 && blocks >= 4;
+    if (r.vec) {
+        // At most `blocks` blocks over both arrays (the partial buffer holds
+        // `blocks` rows of 2 D floats).
+        r.rpb = std::max<int64_t>(1, (total + blocks - 3) / (blocks - 2));
+        r.Gq = static_cast<int>((M + r.rpb - 1) / r.rpb);
+        r.G = r.Gq + static_cast<int>((N + r.rpb - 1) / r.rpb);
+    } else {
+        r.rpb = (total + blocks - 1) / blocks;
+        r.Gq = 0;
+        r.G = static_cast<int>((total + r.rpb - 1) / r.rpb);
+    }
+    return r;
+}
+
+// Spacing of the input format that the mean is rounded to.
+int mean_mant_bits(InType t) { return t == InType::F16 ? 10 : t == InType::BF16 ? 7 : 23; }
+int mean_min_exp(InType t) { return t == InType::F16 ? -24 : t == InType::BF16 ? -133 : -149; }
+
+}  // namespace
+
 cudaError_t launch_mean(InType t, const void* q, const void* k, int64_t M, int64_t N, int D,
                         int blocks, float* partial, float* mu, cudaStream_t s, int batch,
                         const RecordArgs* rec, bool* rec_done, ZeroWords zero) {
@@ -1781,16 +2015,10 @@ cudaError_t launch_mean(InType t, const void* q, const void* k, int64_t M, int64
     // q and k the same points: the mean of [q; q] is the mean of q.
     if (q == k && M == N) N = 0;
     const int64_t total = M + N;
-    int G = 0;
-    const bool vec = t != InType::F32 && D >= 8 && D <= 2048 && (D & (D - 1)) == 0 &&
-                     2048 % D == 0 && blocks >= 4;
-    if (vec) {
-        // At most `blocks` blocks over both arrays (the partial buffer holds
-        // `blocks` rows of 2 D floats).
-        const int64_t rpb = std::max<int64_t>(1, (total + blocks - 3) / (blocks - 2));
-        const int Gq = static_cast<int>((M + rpb - 1) / rpb);
-        const int Gk = static_cast<int>((N + rpb - 1) / rpb);
-        G = Gq + Gk;
+    const MeanSplit sp = mean_split(t, M, N, D, blocks);
+    const int G = sp.G, Gq = sp.Gq;
+    const int64_t rpb = sp.rpb;
+    if (sp.vec) {
         // Key records (see RecordJob) in blocks G .. G + rblocks - 1.
         const int64_t pairs = rec ? rec->Npad / 2 : 0;
         // One thread per key pair, or per key for sign records.
@@ -1815,8 +2043,6 @@ cudaError_t launch_mean(InType t, const void* q, const void* k, int64_t M, int64
         if (rec_done) *rec_done = rec != nullptr;
         note_launches(1);
     } else if (t != InType::F32 && D >= 1 && D <= kMeanVecThreads) {
-        const int64_t rpb = (total + blocks - 1) / blocks;
-        G = static_cast<int>((total + rpb - 1) / rpb);
         // As many chunks per block as leave about 300 blocks.
         const int chunks = static_cast<int>(
             std::min<int64_t>(kMeanVecThreads / D, std::max<int64_t>(1, static_cast<int64_t>(G) * batch / 304)));
@@ -1843,8 +2069,6 @@ cudaError_t launch_mean(InType t, const void* q, const void* k, int64_t M, int64
         if (rec_done) *rec_done = rec != nullptr;
         note_launches(1);
     } else {
-        const int64_t rpb = (total + blocks - 1) / blocks;
-        G = static_cast<int>((total + rpb - 1) / rpb);
         switch (t) {
             case InType::F16:
                 launch_kernel(mean_partial_kernel<__half>, dim3(G, batch), dim3(32, 8), 0, s, 
@@ -1865,8 +2089,7 @@ cudaError_t launch_mean(InType t, const void* q, const void* k, int64_t M, int64
     }
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    const int mant_bits = t == InType::F16 ? 10 : t == InType::BF16 ? 7 : 23;
-    const int min_exp = t == InType::F16 ? -24 : t == InType::BF16 ? -133 : -149;
+    const int mant_bits = mean_mant_bits(t), min_exp = mean_min_exp(t);
     if (G > kMeanFinalThreadMax) {
         launch_kernel(mean_final_block_kernel, dim3(D, batch), kMeanFinalThreads, 0, s, partial,
                       G, D, static_cast<float>(total), mant_bits, min_exp, mu, zero);
@@ -2004,6 +2227,95 @@ cudaError_t launch_operands(InType t, bool aug, const void* q, int64_t M, int64_
                                              cf, vf_rec, vf_tiles, flags_done)
                : operand_typed<__half, false>(jq, j1, D, Dp, 0, 1.f, mu, half_c, pad_value, s,
                                               batch, cf, vf_rec, vf_tiles, flags_done);
+}
+
+namespace {
+
+template <typename T, bool AUG>
+cudaError_t prep_cluster_typed(PrepArgs<T> a, int batch, cudaStream_t s) {
+    const bool ragged = a.D % 8 != 0;
+    const int V = (a.D + 7) / 8;
+    const int G = V <= kOperandVecs ? 1 : V <= 2 * kOperandVecs ? 2 : 4;
+    const int64_t slots = kOperandVecThreads / G;
+    a.nb0 = static_cast<int>((a.j0.rows_pad + slots - 1) / slots);
+    a.nb = a.nb0 + static_cast<int>(a.j1.x ? (a.j1.rows_pad + slots - 1) / slots : 0);
+    auto nout = [](const OperandJob& j) { return AUG ? (j.out_q ? 1 : 0) + (j.out_k ? 1 : 0) : 1; };
+    size_t smem = static_cast<size_t>(std::max(nout(a.j0), nout(a.j1))) * slots * ((a.Dp / 8) | 1) * 16 +
+                  (ragged ? (static_cast<size_t>(slots) * a.D * sizeof(T) + 15) / 16 * 16 : 0);
+    smem = std::max(smem, std::max(sizeof(MeanShared), sizeof(float) * 2 * kPrepMaxParts * a.D));
+    auto go = [&](auto kern) {
+        const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                   static_cast<int>(smem));
+        if (e != cudaSuccess) return e;
+        launch_kernel(kern, dim3(kPrepCluster, static_cast<unsigned>(batch)), kOperandVecThreads, smem, s, a);
+        note_launches(1);
+        return cudaGetLastError();
+    };
+    switch (G) {
+        case 1: return ragged ? go(prep_cluster_kernel<T, AUG, 1, true>) : go(prep_cluster_kernel<T, AUG, 1, false>);
+        case 2: return ragged ? go(prep_cluster_kernel<T, AUG, 2, true>) : go(prep_cluster_kernel<T, AUG, 2, false>);
+        default: return ragged ? go(prep_cluster_kernel<T, AUG, 4, true>) : go(prep_cluster_kernel<T, AUG, 4, false>);
+    }
+}
+
+}  // namespace
+
+bool prep_cluster_fits(InType t, const void* q, const void* k, int64_t M, int64_t N, int D, int Dp, int blocks,
+                       bool aug, int batch) {
+    if (t == InType::F32 || D < 1 || D > kOperandMaxCols || batch > 65535) return false;
+    if (aug && (Dp - D < 2 * aug_norm_terms(t) || 2 * Dp > kOperandMaxCols)) return false;
+    if (q == k && M == N) N = 0;
+    if (M + N > kPrepMaxRows || (M + N) * D > kPrepMaxElements || static_cast<int64_t>(batch) * kPrepCluster > kPrepMaxBlocks) return false;
+    return mean_split(t, M, N, D, blocks).G <= kPrepMaxParts;
+}
+
+cudaError_t launch_prep_cluster(InType t, bool aug, const void* q, int64_t M, int64_t Mpad, void* qh,
+                                void* qh_as_key, float* nrm_q, bool with_k, const void* k, int64_t N,
+                                int64_t Npad, void* kh, float* nrm_k, int D, int Dp, int blocks, float* mu,
+                                float half_c, float pad_value, cudaStream_t s, int batch, const void* vw,
+                                float cf, const RecordArgs* rec, float* vf_rec, ZeroWords zero) {
+    auto fill = [&](auto tag) {
+        using T = decltype(tag);
+        PrepArgs<T> a = {};
+        const int64_t kN = q == k && M == N ? 0 : N;
+        a.q = static_cast<const T*>(q);
+        a.k = static_cast<const T*>(k);
+        a.M = M;
+        a.N = kN;
+        a.split = mean_split(t, M, kN, D, blocks);
+        // (Rows form: as many chunks of D threads per step as the cluster has
+        // use for; at most kPrepMaxChunks slots per block either way.)
+        a.chunks = a.split.vec ? 1 : std::max(1, std::min(kMeanVecThreads / D,
+                                                          (a.split.G + kPrepCluster - 1) / kPrepCluster));
+        a.total = static_cast<float>(M + kN);
+        a.mant_bits = mean_mant_bits(t);
+        a.min_exp = mean_min_exp(t);
+        a.mu = mu;
+        a.zero = zero;
+        if (rec) a.rec = *rec;
+        a.vf_rec = vf_rec;
+        a.vf_tiles = Npad / kRecTile;
+        a.D = D;
+        a.Dp = Dp;
+        a.nt = aug ? aug_norm_terms(t) : 0;
+        a.F = aug && t == InType::F16 ? 1024.f : 1.f;
+        a.half_c = aug ? 0.f : half_c;
+        a.pad_value = aug ? 0.f : pad_value;
+        a.cf = aug ? cf : 0.f;
+        if (aug) {
+            a.j0 = {q, M, Mpad, qh, qh_as_key, nullptr, qh_as_key ? vw : nullptr};
+            if (with_k) a.j1 = {k, N, Npad, nullptr, kh, nullptr, vw};
+        } else {
+            a.j0 = {q, M, Mpad, qh, nullptr, nrm_q, nullptr};
+            if (with_k) a.j1 = {k, N, Npad, kh, nullptr, nrm_k, nullptr};
+        }
+        return a;
+    };
+    if (t == InType::BF16)
+        return aug ? prep_cluster_typed<__nv_bfloat16, true>(fill(__nv_bfloat16()), batch, s)
+                   : prep_cluster_typed<__nv_bfloat16, false>(fill(__nv_bfloat16()), batch, s);
+    return aug ? prep_cluster_typed<__half, true>(fill(__half()), batch, s)
+               : prep_cluster_typed<__half, false>(fill(__half()), batch, s);
 }
 
 cudaError_t launch_tf32_split(const float* x, int64_t rows, int64_t rows_pad, int D, int Dp,
