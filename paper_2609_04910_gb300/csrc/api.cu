@@ -135,6 +135,12 @@ struct Call {
     // upper triangle of tile pairs, and out then holds row sums s' with
     // sum_m v_m s'_m = v^T K v instead of K v.
     bool tri = false;
+    // ... and its value per problem is wanted in mmd_out (float64 partial sums
+    // in mmd_part), taken from the FMA kernel's partial sums directly where it
+    // runs (*mmd_done says so; out is then not written).
+    float* mmd_out = nullptr;
+    double* mmd_part = nullptr;
+    bool* mmd_done = nullptr;
     // Weighted vector-Jacobian pass (gradient mode with C = 1 and v null):
     // the kernel values are multiplied by the pair weights
     // w_mn = sum_c r[m, c] k[n, c] of wc channels, r = rw (M x wc, float32
@@ -281,7 +287,7 @@ gs_status plan(const Call& c, int sms, bool* tensor, gs::TcPlan* tp, gs::SimtPla
         const double cx = c.tau * 1.4426950408889634;
         tp->cfold = tp->fma && tp->aug && !tp->tf && c.dtype == GS_FP16 && tp->exp2_fma == 0 &&
                     cx <= 0.5 && cx >= 1.0 / 16384.0;
-        tp->vfold = tp->cfold && tp->Cv == 1 && !c.w_f32 && c.C == 1 && !tp->overlap;
+        tp->vfold = tp->cfold && tp->Cv == 1 && !c.w_f32 && c.C == 1 && (!tp->overlap || tp->tri);
         *bytes = tp->total;
     } else {
         if (c.opt.exp2_fma > 0)
@@ -349,6 +355,7 @@ gs_status run(Call c) {
         for (int64_t b = 0; b < c.B; ++b) {
             Call cb = c;
             cb.B = 1;
+            cb.mmd_out = nullptr;
             cb.q = static_cast<const char*>(c.q) + b * c.M * c.D * es;
             cb.k = static_cast<const char*>(c.k) + b * c.N * c.D * es;
             cb.v = static_cast<const char*>(c.v) + b * c.N * c.C * ws_;
@@ -486,11 +493,19 @@ gs_status run(Call c) {
             }
             if (e == cudaSuccess) e = record_event(c.opt.main_events[1], c.stream);
             if (e == cudaSuccess) {
-                e = gs::launch_finalize_slots(reinterpret_cast<float*>(ws + tp.off_part), tp.Mpad,
-                                              c.M, static_cast<int>(tp.Cv), 128 * tp.nq,
-                                              tp.Npad / tp.BN, tp.unit_len, c.out, c.stream,
-                                              batch, tp.band_len > 0 ? tp.splits : 0,
-                                              tp.tri ? tp.Npad / tp.BN : 0, guard);
+                const int fixed = tp.band_len > 0 ? tp.splits : 0;
+                const int64_t kt = tp.Npad / tp.BN;
+                const float* part = reinterpret_cast<float*>(ws + tp.off_part);
+                if (c.mmd_out && !guard && t != gs::InType::F32) {
+                    e = gs::launch_mmd2_slots(t, part, tp.Mpad, c.M, 128 * tp.nq, kt, tp.unit_len, c.v,
+                                              c.mmd_part, c.mmd_out, c.stream, batch, fixed,
+                                              tp.tri ? kt : 0);
+                    *c.mmd_done = true;
+                } else {
+                    e = gs::launch_finalize_slots(part, tp.Mpad, c.M, static_cast<int>(tp.Cv), 128 * tp.nq,
+                                                  kt, tp.unit_len, c.out, c.stream, batch, fixed,
+                                                  tp.tri ? kt : 0, guard);
+                }
                 where = "finalise kernel";
             }
             if (e == cudaSuccess && guard) {
@@ -798,11 +813,14 @@ gs_status gauss_sum_mmd2(const void* x, const void* v, double tau, int64_t B, in
                                     s_bytes + gs::mmd2_partial_bytes(B, N), st);
     if (e != cudaSuccess) return cuda_fail(e, "workspace allocation");
     c.out = s_buf;
+    bool done = false;
+    c.mmd_out = mmd2;
+    c.mmd_part = reinterpret_cast<double*>(reinterpret_cast<char*>(s_buf) + s_bytes);
+    c.mmd_done = &done;
     status = run(c);
-    if (status == GS_OK) {
+    if (status == GS_OK && !done) {
         e = gs::launch_mmd2_reduce(in_type(dtype), s_buf, v, B, N,
-                                   reinterpret_cast<double*>(reinterpret_cast<char*>(s_buf) + s_bytes),
-                                   mmd2, st);
+                                   c.mmd_part, mmd2, st);
         if (e != cudaSuccess) status = cuda_fail(e, "MMD reduction kernel");
     }
     cudaError_t ef = cudaFreeAsync(s_buf, st);

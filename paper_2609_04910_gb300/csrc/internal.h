@@ -259,6 +259,12 @@ cudaError_t launch_finalize_points(bool direct, InType t, bool u_f32, const floa
 size_t mmd2_partial_bytes(int64_t B, int64_t N);
 cudaError_t launch_mmd2_reduce(InType t, const float* s, const void* v, int64_t B, int64_t N,
                                double* partial, float* out, cudaStream_t st);
+// The same from the FMA kernel's partial sums (one channel; arguments as
+// launch_finalize_slots): s is not written.
+cudaError_t launch_mmd2_slots(InType t, const float* part, int64_t Mpad, int64_t M, int rows_per_unit,
+                              int64_t key_tiles, int64_t unit_len, const void* v, double* partial,
+                              float* out, cudaStream_t s, int batch, int fixed_slots,
+                              int64_t tri_key_tiles);
 // Forward sum of the FMA kernel's contributor slots, added in slot order:
 // every row has slots 0 .. fixed_slots - 1 when fixed_slots > 0 (banded
 // order); otherwise rows of the pair of query tiles r = m / rows_per_unit

@@ -759,6 +759,24 @@ __global__ void tf32_split_kernel(const float* __restrict__ x, int64_t rows, int
 // tensor-core path's range.  Read after pdl_wait only.
 __device__ __forceinline__ bool guard_above(const unsigned* guard) { return *guard > kGuardMaxBits; }
 
+// Contributor slots of pair of query tiles r of the FMA kernel (see
+// launch_finalize_slots in internal.h).
+__device__ __forceinline__ int64_t contributor_slots(int64_t r, int fixed_slots, int64_t key_tiles,
+                                                     int64_t unit_len, int64_t tri_kt) {
+    if (fixed_slots > 0) return fixed_slots;
+    if (tri_kt > 0) {
+        // Upper-triangle order (folded rows of tri_kt + 2 units: pair s,
+        // then pair ppb - 1 - s): pair P of problem b holds tri_kt - 2P units.
+        const int64_t ppb = tri_kt / 2;
+        const int64_t bb = r / ppb, P = r - bb * ppb;
+        const int64_t U = ppb * tri_kt - ppb * (ppb - 1);
+        const int64_t s = 2 * P <= ppb - 1 ? P : ppb - 1 - P;
+        const int64_t start = bb * U + s * (tri_kt + 2) + (s == P ? 0 : tri_kt - 2 * s);
+        return (start + tri_kt - 2 * P - 1) / unit_len - start / unit_len + 1;
+    }
+    return ((r + 1) * key_tiles - 1) / unit_len - r * key_tiles / unit_len + 1;
+}
+
 __global__ void finalize_slots_kernel(const float* __restrict__ part, int64_t Mpad, int64_t M,
                                       int C, int rows_per_unit, int64_t key_tiles,
                                       int64_t unit_len, int64_t batch, int fixed_slots,
@@ -775,25 +793,8 @@ __global__ void finalize_slots_kernel(const float* __restrict__ part, int64_t Mp
     const int c = static_cast<int>(idx - bm * C);
     const int64_t b = M <= 0x7fffffff ? div_nonneg(bm, static_cast<int>(M)) : bm / M;
     const int64_t m = (bm - b * M) + b * Mpad;
-    int64_t nslots = fixed_slots;
-    if (nslots == 0 && tri_kt > 0) {
-        // Upper-triangle order (folded rows of tri_kt + 2 units: pair s,
-        // then pair ppb - 1 - s): pair P of problem b holds tri_kt - 2P units.
-        const int64_t r = m / rows_per_unit;
-        const int64_t ppb = tri_kt / 2;
-        const int64_t bb = r / ppb, P = r - bb * ppb;
-        const int64_t U = ppb * tri_kt - ppb * (ppb - 1);
-        const int64_t s = 2 * P <= ppb - 1 ? P : ppb - 1 - P;
-        const int64_t start = bb * U + s * (tri_kt + 2) + (s == P ? 0 : tri_kt - 2 * s);
-        const int64_t first = start / unit_len;
-        const int64_t last = (start + tri_kt - 2 * P - 1) / unit_len;
-        nslots = last - first + 1;
-    } else if (nslots == 0) {
-        const int64_t r = m / rows_per_unit;
-        const int64_t first = r * key_tiles / unit_len;
-        const int64_t last = ((r + 1) * key_tiles - 1) / unit_len;
-        nslots = last - first + 1;
-    }
+    const int64_t nslots =
+        contributor_slots(m / rows_per_unit, fixed_slots, key_tiles, unit_len, tri_kt);
     float acc = 0.f;
     for (int64_t sl = 0; sl < nslots; ++sl) acc += part[(sl * batch * Mpad + m) * C + c];
     out[idx] = acc;
@@ -1005,7 +1006,7 @@ __device__ __forceinline__ float operand_row(const uint4 (&in)[kOperandVecs],
     auto tail_k = [&](int e) -> unsigned {
         return e < nt ? term(e) : e < 2 * nt ? partner(e - nt) : 0u;
     };
-    if (RAGGED) {
+    if constexpr (RAGGED) {
         // The columns past D start anywhere: zeros to the end of the row, then
         // the norm terms and their partners one by one.
         for (int c = 8 * V; c < Dp; c += 8) {
@@ -1016,24 +1017,24 @@ __device__ __forceinline__ float operand_row(const uint4 (&in)[kOperandVecs],
             if (out_q) out_q[D + e] = bits_to<T>(static_cast<unsigned short>(tail_q(e)));
             if (out_k) out_k[D + e] = bits_to<T>(static_cast<unsigned short>(tail_k(e)));
         }
-        return nrm;
-    }
+    } else {
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
-        const int c = D + 8 * h;
-        if (c >= Dp) break;
-        uint32_t wq[4], wk[4];
+        for (int h = 0; h < 2; ++h) {
+            const int c = D + 8 * h;
+            if (c >= Dp) break;
+            uint32_t wq[4], wk[4];
 #pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            wq[e] = tail_q(8 * h + 2 * e) | (tail_q(8 * h + 2 * e + 1) << 16);
-            wk[e] = tail_k(8 * h + 2 * e) | (tail_k(8 * h + 2 * e + 1) << 16);
+            for (int e = 0; e < 4; ++e) {
+                wq[e] = tail_q(8 * h + 2 * e) | (tail_q(8 * h + 2 * e + 1) << 16);
+                wk[e] = tail_k(8 * h + 2 * e) | (tail_k(8 * h + 2 * e + 1) << 16);
+            }
+            if (out_q) *reinterpret_cast<uint4*>(out_q + c) = make_uint4(wq[0], wq[1], wq[2], wq[3]);
+            if (out_k) *reinterpret_cast<uint4*>(out_k + c) = make_uint4(wk[0], wk[1], wk[2], wk[3]);
         }
-        if (out_q) *reinterpret_cast<uint4*>(out_q + c) = make_uint4(wq[0], wq[1], wq[2], wq[3]);
-        if (out_k) *reinterpret_cast<uint4*>(out_k + c) = make_uint4(wk[0], wk[1], wk[2], wk[3]);
-    }
-    for (int c = D + 16; c < Dp; c += 8) {
-        if (out_q) *reinterpret_cast<uint4*>(out_q + c) = make_uint4(0u, 0u, 0u, 0u);
-        if (out_k) *reinterpret_cast<uint4*>(out_k + c) = make_uint4(0u, 0u, 0u, 0u);
+        for (int c = D + 16; c < Dp; c += 8) {
+            if (out_q) *reinterpret_cast<uint4*>(out_q + c) = make_uint4(0u, 0u, 0u, 0u);
+            if (out_k) *reinterpret_cast<uint4*>(out_k + c) = make_uint4(0u, 0u, 0u, 0u);
+        }
     }
     return nrm;
 }
@@ -2136,6 +2137,78 @@ mmd2_reduce_kernel(const float* __restrict__ s, const T* __restrict__ v, int64_t
     if (t == 0) partial[b * gridDim.x + blockIdx.x] = red[0];
 }
 
+// The same with s_n added up here from the FMA kernel's contributor slots (in
+// slot order, as finalize_slots_kernel does), which saves writing and reading
+// s and a launch; with one chunk per problem the result is written at once.
+// kMmdChunk points are 16 pairs of 128-row query tiles, whose slot counts are
+// worked out once per block; the sums s_n of the chunk are formed by all
+// threads, four points each with their loads in flight together (with two
+// passes of few blocks the loads' latency is what this costs: one point at a
+// time by 256 threads took 10 to 20 us more), and folded in
+// mmd2_reduce_kernel's order.  Whole calls, with the overlapped segments
+// before and after: 64 problems of 2000 points 70.0 -> 62.5 us, 16 of 4096
+// 82 -> 56, 8 of 8000 79.3 -> 73.5, one of 30000 105.3 -> 105.3 us.
+constexpr int kMmdThreads = 1024;
+
+template <typename T>
+__global__ void __launch_bounds__(kMmdThreads)
+mmd2_slots_kernel(const float* __restrict__ part, int64_t Mpad, int64_t N, int rows_per_unit,
+                  int64_t key_tiles, int64_t unit_len, int fixed_slots, int64_t tri_kt,
+                  const T* __restrict__ v, double* __restrict__ partial, float* __restrict__ out) {
+    pdl_trigger();
+    pdl_wait();
+    constexpr int PER = static_cast<int>(kMmdChunk) / kMmdThreads;
+    __shared__ double red[256];
+    __shared__ float sums[kMmdChunk];
+    __shared__ int slots[kMmdChunk / 256];
+    const int t = threadIdx.x;
+    const int64_t b = blockIdx.y, batch = gridDim.y;
+    const int64_t n0 = static_cast<int64_t>(blockIdx.x) * kMmdChunk;
+    const int64_t n1 = min(N, n0 + kMmdChunk);
+    if (t < kMmdChunk / 256)
+        slots[t] = n0 + 256 * t < n1
+                       ? static_cast<int>(contributor_slots((b * Mpad + n0 + 256 * t) / rows_per_unit,
+                                                            fixed_slots, key_tiles, unit_len, tri_kt))
+                       : 0;
+    __syncthreads();
+    const int64_t step = batch * Mpad;
+    const float* p = part + b * Mpad + n0 + t;     // (rows up to Mpad exist; those past N are not used)
+    int ns[PER], most = 0;
+    float s[PER];
+#pragma unroll
+    for (int i = 0; i < PER; ++i) {
+        ns[i] = n0 + t + i * kMmdThreads < n1 ? slots[(t + i * kMmdThreads) / 256] : 0;
+        most = max(most, ns[i]);
+        s[i] = 0.f;
+    }
+#pragma unroll 2
+    for (int sl = 0; sl < most; ++sl) {
+        float x[PER];
+#pragma unroll
+        for (int i = 0; i < PER; ++i) x[i] = sl < ns[i] ? p[sl * step + i * kMmdThreads] : 0.f;
+#pragma unroll
+        for (int i = 0; i < PER; ++i)
+            if (sl < ns[i]) s[i] += x[i];
+    }
+#pragma unroll
+    for (int i = 0; i < PER; ++i) sums[t + i * kMmdThreads] = s[i];
+    __syncthreads();
+    if (t < 256) {
+        double acc = 0.0;
+        for (int64_t n = n0 + t; n < n1; n += 256)
+            acc += static_cast<double>(to_f(v[b * N + n])) * static_cast<double>(sums[n - n0]);
+        red[t] = acc;
+    }
+    __syncthreads();
+    for (int w = 128; w > 0; w >>= 1) {
+        if (t < w) red[t] += red[t + w];
+        __syncthreads();
+    }
+    if (t != 0) return;
+    if (gridDim.x == 1) out[b] = static_cast<float>(red[0]);
+    else partial[b * gridDim.x + blockIdx.x] = red[0];
+}
+
 __global__ void mmd2_final_kernel(const double* __restrict__ partial, int chunks, int64_t B,
                                   float* __restrict__ out) {
     pdl_trigger();
@@ -2177,6 +2250,29 @@ cudaError_t launch_mmd2_reduce(InType t, const float* s, const void* v, int64_t 
     if (e != cudaSuccess) return e;
     launch_kernel(mmd2_final_kernel, static_cast<unsigned>((B + 127) / 128), 128, 0, st, 
         partial, static_cast<int>(chunks), B, out);
+    note_launches(1);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_mmd2_slots(InType t, const float* part, int64_t Mpad, int64_t M, int rows_per_unit,
+                              int64_t key_tiles, int64_t unit_len, const void* v, double* partial,
+                              float* out, cudaStream_t st, int batch, int fixed_slots,
+                              int64_t tri_key_tiles) {
+    if (rows_per_unit != 256) return cudaErrorInvalidValue;   // (slot counts per 256 rows)
+    const int64_t chunks = std::max<int64_t>(1, (M + kMmdChunk - 1) / kMmdChunk);
+    const dim3 grid(static_cast<unsigned>(chunks), static_cast<unsigned>(batch));
+    if (t == InType::BF16)
+        launch_kernel(mmd2_slots_kernel<__nv_bfloat16>, grid, kMmdThreads, 0, st, part, Mpad, M, rows_per_unit,
+                      key_tiles, unit_len, fixed_slots, tri_key_tiles,
+                      static_cast<const __nv_bfloat16*>(v), partial, out);
+    else
+        launch_kernel(mmd2_slots_kernel<__half>, grid, kMmdThreads, 0, st, part, Mpad, M, rows_per_unit, key_tiles,
+                      unit_len, fixed_slots, tri_key_tiles, static_cast<const __half*>(v), partial, out);
+    note_launches(1);
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess || chunks == 1) return e;
+    launch_kernel(mmd2_final_kernel, static_cast<unsigned>((batch + 127) / 128), 128, 0, st, partial,
+                  static_cast<int>(chunks), static_cast<int64_t>(batch), out);
     note_launches(1);
     return cudaGetLastError();
 }

@@ -906,10 +906,11 @@ bool plan_tensor(InType t, int64_t M, int64_t N, int64_t D, int64_t C, bool grad
     // the FMA kernel overlaps the restart with the previous segment's tail
     // (forward sums with augmented operands; measured on one GB300: B = 256
     // problems of 1024 points 0.205 -> 0.137 ms per call, B = 64 x 16384
-    // 3.06 -> 2.96 ms).  Long segments keep the barrier, whose code measured
-    // faster there.
+    // 3.06 -> 2.96 ms; upper triangle, whole MMD^2 calls: 64 problems of 2000
+    // points 74.9 -> 72.1 us, 200 of 1000 90.5 -> 84.3).  Long segments keep
+    // the barrier, whose code measured faster there.
     p->overlap = false;
-    if (p->fma && p->aug && !p->tf && !p->tri) {
+    if (p->fma && p->aug && !p->tf) {
         const int64_t seg = p->band_len > 0 ? p->band_len : std::min<int64_t>(key_tiles, p->unit_len);
         p->overlap = seg <= kOverlapMaxTiles;
     }

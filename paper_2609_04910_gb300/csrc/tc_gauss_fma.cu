@@ -1027,6 +1027,14 @@ cudaError_t launch_c(const TcPlan& pl, InType t, float c, char* ws, unsigned* st
     // 3 = only the exponent scale folded, value records as usual.
     const int vf = pl.vfold ? vf_pass : pl.cfold ? 3 : 0;
     if constexpr (C == 1 && kAugQsm) {
+        if (pl.tri && pl.aug && pl.overlap) {
+            switch (vf) {
+                case 1: return launch_typed<1, true, true, false, true, 0, true, 1>(pl, t, c, ws, status, s, why);
+                case 2: return launch_typed<1, true, true, false, true, 0, true, 2>(pl, t, c, ws, status, s, why);
+                case 3: return launch_typed<1, true, true, false, true, 0, true, 3>(pl, t, c, ws, status, s, why);
+                default: return launch_typed<1, true, true, false, true, 0, true>(pl, t, c, ws, status, s, why);
+            }
+        }
         if (pl.tri && pl.aug) {
             switch (vf) {
                 case 1: return launch_typed<1, true, true, false, true, 0, false, 1>(pl, t, c, ws, status, s, why);
@@ -1093,7 +1101,7 @@ bool plan_fma_kernel(int Dp, int C, bool aug, bool tf, int* nq, int* stages, siz
 cudaError_t launch_tc_fma(const TcPlan& p, InType t, float c, char* ws, unsigned* status,
                           cudaStream_t s, const char** why, int vf_pass) {
     const bool qsm = (p.tf && !p.guard) || (p.aug && kAugQsm);
-    note_fma_variant((p.aug && kAugQsm && p.overlap && !p.tri && p.exp2_fma == 0 ? 1 : 0) |
+    note_fma_variant((p.aug && kAugQsm && p.overlap && p.exp2_fma == 0 ? 1 : 0) |
                      (p.band_len > 0 ? 2 : 0) | (qsm ? 0 : 4) |
                      (p.vfold ? 8 : 0) | (p.cfold || p.vfold ? 16 : 0));
     switch (p.Cv) {
