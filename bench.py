@@ -287,9 +287,11 @@ def kernel_source_hash():
 def main_kernel_name(w):
     """Fused kernel the library picks for this workload (plan in csrc)."""
     if w.dtype == "fp32":
-        # fp32 forward sums with C <= 4, D <= 32 from 2^25 pairs: 3xTF32 variant.
-        tf32 = not w.grad and w.C <= 4 and w.D <= 32 and w.M * w.N >= 2 ** 25
-        return "tc_gauss_fma_kernel" if tf32 else "simt_gauss_kernel"
+        # fp32 forward sums with C <= 4 and D <= 64 from a size that depends on
+        # D: 3xTF32 variant (above D = 32 guarded by the points' norms).
+        least = 2 ** 26 if w.D <= 4 else 2 ** 25 if w.D <= 32 else 2 ** 24
+        tf32 = not w.grad and w.C <= 4 and w.D <= 64 and w.M * w.N >= least
+        return "tc_gauss_fma_kernel" if tf32 else "simt_grad_kernel" if w.grad else "simt_sum_kernel"
     if w.grad or w.C > 4:
         return "tc_gauss_kernel"
     # Three or four channels on augmented rows (D + 4 <= 128 for fp16, + 6

@@ -38,8 +38,14 @@
  *    C) or, for forward sums with C <= 4 and D <= 32, on the tensor cores
  *    with three tf32 MMAs per product (q^ k^T ~ hi.hi + hi.lo + lo.hi of the
  *    tf32 splits x = hi + lo, fp32-level accuracy): chosen automatically
- *    from 2^25 pairs (per call, summed over a batch), or forced with
- *    GS_PATH_TENSOR / GS_PATH_SIMT.
+ *    from 2^25 pairs (per call, summed over a batch; single problems with
+ *    D <= 4 from 2^26), or forced with GS_PATH_TENSOR / GS_PATH_SIMT.  Single forward sums with C <= 4 and
+ *    32 < D <= 64 from 2^24 pairs launch both: a device-side look at the
+ *    points' norms lets the tensor cores work only where they are as accurate
+ *    as the SIMT kernel's coordinate differences (largest
+ *    (tau/2) log2(e) ||x - mean||^2 at most 4), else the SIMT kernel does.
+ *    Their workspace holds both; where a caller's workspace, or the scratch of
+ *    gauss_sum_noalloc, is too small for both, the SIMT kernel runs alone.
  *  - On a non-OK return gauss_sum_last_error() describes the failure.
  */
 #ifndef GAUSS_SUM_H
@@ -84,9 +90,10 @@ typedef enum { GS_PATH_AUTO = 0, GS_PATH_TENSOR = 1, GS_PATH_SIMT = 2 } gs_path;
  *                  required size is gauss_sum_workspace_size().
  *  path            GS_PATH_AUTO picks the tensor-core kernels for fp16/bf16
  *                  and, for fp32, the 3xTF32 tensor-core variant for large
- *                  forward sums with C <= 4 and D <= 32, else the SIMT
- *                  kernel; GS_PATH_TENSOR takes fp32 only within that
- *                  range (GS_ERR_UNSUPPORTED otherwise); GS_PATH_SIMT
+ *                  forward sums with C <= 4 and D <= 32 (with the SIMT kernel
+ *                  behind it up to D = 64, see above), else the SIMT
+ *                  kernel; GS_PATH_TENSOR takes fp32 only with D <= 32
+ *                  (GS_ERR_UNSUPPORTED otherwise); GS_PATH_SIMT
  *                  rejects fp16/bf16.
  *  main_events     measurement hook: two cudaEvent_t handles (or NULL) that
  *                  the call records on `stream` immediately before and after

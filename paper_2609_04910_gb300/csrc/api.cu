@@ -204,12 +204,12 @@ gs::InType in_type(gs_dtype d) {
 // fp32 inputs go to the tensor cores (3xTF32) when the path is chosen
 // explicitly, or automatically for forward sums that the variant covers
 // and that are large enough to repay its extra operand kernels: from 2^25
-// pairs, and single problems of few coordinates, whose squared distances
-// are cheap on the SIMT kernel (it works in register tiles of 4, 8, 16, ..
-// coordinates), from 3 x 2^25 pairs (D <= 4) or 3 x 2^24 (D <= 8).  Measured
-// on a GB300, C = 1, whole calls, SIMT / tensor cores: 5800^2 pairs D = 4
-// 24 / 40 us, D = 16 50 / 43 us; 16384^2 pairs D = 4 113 / 71 us, D = 8 172 /
-// 71 us, D = 16 296 / 76 us.
+// pairs, and single problems of at most four coordinates, whose squared
+// distances are cheap on the SIMT kernel (it works in register tiles of 4, 8,
+// 16, .. coordinates), from 2^26.  Measured on a GB300, C = 1, whole calls,
+// SIMT / tensor cores: 5800^2 pairs D = 4 24 / 35 us, 18684 x 2500, D = 7 37 /
+// 35 us, 5800^2, D = 16 50 / 37 us; 16384^2 pairs D = 4 113 / 70 us, D = 8
+// 172 / 70 us, D = 16 296 / 74 us.
 // Batches keep 2^25 for every D: the tensor-core path runs them in one
 // launch of each kernel, the SIMT kernel problem by problem.
 constexpr int64_t kFp32TensorMinPairs = int64_t(1) << 25;
@@ -217,9 +217,7 @@ constexpr int64_t kFp32TensorMinPairs = int64_t(1) << 25;
 bool fp32_on_tensor_cores(const Call& c) {
     if (c.opt.path == GS_PATH_TENSOR) return true;
     if (c.opt.path != GS_PATH_AUTO) return false;
-    const int64_t least = c.B > 1 || c.D > 8 ? kFp32TensorMinPairs
-                          : c.D > 4          ? kFp32TensorMinPairs / 2 * 3
-                                             : kFp32TensorMinPairs * 3;
+    const int64_t least = c.B > 1 || c.D > 4 ? kFp32TensorMinPairs : 2 * kFp32TensorMinPairs;
     return !c.grad && c.C <= gs::kFmaMaxChannels && c.D <= gs::kTf32MaxDp &&
            c.B * c.M * c.N >= least;
 }
@@ -436,20 +434,15 @@ gs_status run(Call c) {
             // an error: nothing more is launched; or nothing left to prepare
         } else if (tp.tf) {
             // 3xTF32 operands: hi / lo tf32 halves and the norm terms.
-            e = gs::launch_tf32_split(static_cast<const float*>(c.q), c.M, tp.Mpad,
-                                      static_cast<int>(c.D), tp.Dp, mu, half_c,
-                                      reinterpret_cast<float*>(ws + tp.off_qh),
-                                      reinterpret_cast<float*>(ws + tp.off_A), ninf, c.stream,
-                                      batch, guard);
-            where = "tf32 split kernel (q)";
-            if (e == cudaSuccess && !tp.alias) {
-                e = gs::launch_tf32_split(static_cast<const float*>(c.k), c.N, tp.Npad,
-                                          static_cast<int>(c.D), tp.Dp, mu, half_c,
-                                          reinterpret_cast<float*>(ws + tp.off_kh),
-                                          reinterpret_cast<float*>(ws + tp.off_B), ninf,
-                                          c.stream, batch, guard);
-                where = "tf32 split kernel (k)";
-            }
+            const gs::Tf32Job jq = {static_cast<const float*>(c.q), c.M, tp.Mpad,
+                                    reinterpret_cast<float*>(ws + tp.off_qh),
+                                    reinterpret_cast<float*>(ws + tp.off_A)};
+            const gs::Tf32Job jk = {static_cast<const float*>(c.k), c.N, tp.Npad,
+                                    reinterpret_cast<float*>(ws + tp.off_kh),
+                                    reinterpret_cast<float*>(ws + tp.off_B)};
+            e = gs::launch_tf32_split(jq, tp.alias ? nullptr : &jk, static_cast<int>(c.D), tp.Dp, mu,
+                                      half_c, ninf, c.stream, batch, guard);
+            where = "tf32 split kernel";
         } else {
             // Centred, rounded operands of q and (unless q is k) k in one
             // launch: augmented rows (norms folded into the MMA), or plain
@@ -491,6 +484,14 @@ gs_status run(Call c) {
                     e = gs::launch_tc_fma(tp, t, cexp, ws, status, c.stream, &why, 2);
                 where = "fused tensor-core kernel";
             }
+            if (e == cudaSuccess && guard) {
+                // The other side of the guard.
+                e = gs::launch_simt(sp, false, static_cast<const float*>(c.q),
+                                    static_cast<const float*>(c.k), static_cast<const float*>(c.v),
+                                    static_cast<int>(c.C), 0, half_c,
+                                    reinterpret_cast<float*>(ws + sp.off_part), c.stream, guard);
+                where = "fp32 kernel";
+            }
             if (e == cudaSuccess) e = record_event(c.opt.main_events[1], c.stream);
             if (e == cudaSuccess) {
                 const int fixed = tp.band_len > 0 ? tp.splits : 0;
@@ -509,17 +510,10 @@ gs_status run(Call c) {
                 where = "finalise kernel";
             }
             if (e == cudaSuccess && guard) {
-                // The other side of the guard.
-                float* part = reinterpret_cast<float*>(ws + sp.off_part);
-                e = gs::launch_simt(sp, false, static_cast<const float*>(c.q),
-                                    static_cast<const float*>(c.k), static_cast<const float*>(c.v),
-                                    static_cast<int>(c.C), 0, half_c, part, c.stream, guard);
-                where = "fp32 kernel";
-                if (e == cudaSuccess) {
-                    e = gs::launch_finalize(part, sp.splits, c.M, c.M, static_cast<int>(sp.Cv),
-                                            static_cast<int>(sp.Cv), nullptr, c.out, c.stream, 0, guard);
-                    where = "finalise kernel";
-                }
+                e = gs::launch_finalize(reinterpret_cast<float*>(ws + sp.off_part), sp.splits, c.M, c.M,
+                                        static_cast<int>(sp.Cv), static_cast<int>(sp.Cv), nullptr, c.out,
+                                        c.stream, 0, guard);
+                where = "finalise kernel";
             }
         } else if (e == cudaSuccess) {
             // Two-MMA kernel, once per chunk of value channels (one chunk for

@@ -148,6 +148,7 @@ struct SimtPlan {
     int64_t M, N, D, Cv;
     int dmax;          // register tile of the query row (16, 32, 64 or 128)
     int cblk;          // channels per launch slice
+    int threads;       // threads per block of the forward kernel
     int splits;
     int64_t keys_per_split;
     size_t off_part, total;
@@ -291,11 +292,17 @@ cudaError_t launch_simt(const SimtPlan& p, bool grad, const float* q, const floa
 cudaError_t launch_key_records(InType t, const void* v, const float* B, int64_t N, int64_t Npad,
                                int C, float* rec, cudaStream_t s, int batch = 1, bool signs = false);
 // 3xTF32 operands of fp32 inputs (see prep.cu): rows of 2 Dp floats
-// [hi | lo] into out, nrm = -(c/2)||x - mu||^2 (pad_value for padded rows).
-cudaError_t launch_tf32_split(const float* x, int64_t rows, int64_t rows_pad, int D, int Dp,
-                              const float* mu, float half_c, float* out, float* nrm,
-                              float pad_value, cudaStream_t s, int batch = 1,
-                              unsigned* guard = nullptr);
+// [hi | lo] into out, nrm = -(c/2)||x - mu||^2 (pad_value for padded rows), of
+// q and, unless q is k, of k; guard takes the bits of the largest -nrm.
+struct Tf32Job {
+    const float* x;          // batch x rows x D
+    int64_t rows, rows_pad;
+    float* out;
+    float* nrm;
+};
+cudaError_t launch_tf32_split(const Tf32Job& q, const Tf32Job* k, int D, int Dp, const float* mu,
+                              float half_c, float pad_value, cudaStream_t s, int batch,
+                              unsigned* guard);
 constexpr int aug_norm_terms(InType t) { return t == InType::BF16 ? 3 : 2; }
 
 // tc_gauss.cu ----------------------------------------------------------

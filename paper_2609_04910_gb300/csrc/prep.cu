@@ -711,11 +711,10 @@ operand_kernel(const T* __restrict__ x, int64_t rows, int64_t rows_pad, int D, i
 // lo.lo term (2^-22 relative).  nrm = -(c/2) ||x^||^2 from the fp32 x^;
 // rows in [rows, rows_pad) are zero with norm pad_value.  One warp per row,
 // over all problems of a batch.
-__global__ void tf32_split_kernel(const float* __restrict__ x, int64_t rows, int64_t rows_pad,
-                                  int64_t total_rows, int D, int Dp,
-                                  const float* __restrict__ mu, float half_c, float pad_value,
-                                  float* __restrict__ out, float* __restrict__ nrm,
-                                  unsigned* __restrict__ guard) {
+// Rows of job j0 (all problems), then of j1, in one launch.
+__global__ void tf32_split_kernel(const Tf32Job j0, const Tf32Job j1, int64_t total0, int64_t total_rows,
+                                  int D, int Dp, const float* __restrict__ mu, float half_c,
+                                  float pad_value, unsigned* __restrict__ guard) {
     pdl_trigger();
     pdl_wait();
     // guard: the largest (c/2) ||x - mu||^2, as the bits of a non-negative
@@ -728,12 +727,15 @@ __global__ void tf32_split_kernel(const float* __restrict__ x, int64_t rows, int
     const int64_t w = (static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
     if (w < total_rows) {
-        const int64_t b = w / rows_pad;
-        const int64_t r = w - b * rows_pad;
-        const bool valid = r < rows;
-        const float* xr = x + (b * rows + r) * D;
+        const bool second = w >= total0;
+        const Tf32Job j = second ? j1 : j0;
+        const int64_t i = second ? w - total0 : w;         // batch-stacked output row
+        const int64_t b = i / j.rows_pad;
+        const int64_t r = i - b * j.rows_pad;
+        const bool valid = r < j.rows;
+        const float* xr = j.x + (b * j.rows + r) * D;
         const float* mb = mu ? mu + b * D : nullptr;
-        float* o = out + w * 2 * Dp;
+        float* o = j.out + i * 2 * Dp;
         float acc = 0.f;
         for (int d = lane; d < Dp; d += 32) {
             const float xv = (valid && d < D) ? xr[d] - (mb ? mb[d] : 0.f) : 0.f;
@@ -745,7 +747,7 @@ __global__ void tf32_split_kernel(const float* __restrict__ x, int64_t rows, int
 #pragma unroll
         for (int s = 16; s > 0; s >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, s);
         if (lane == 0) {
-            nrm[w] = valid ? -half_c * acc : pad_value;
+            j.nrm[i] = valid ? -half_c * acc : pad_value;
             if (guard && valid) atomicMax(&big, __float_as_uint(half_c * acc) & 0x7fffffffu);
         }
     }
@@ -2070,22 +2072,9 @@ cudaError_t launch_mean(InType t, const void* q, const void* k, int64_t M, int64
         if (rec_done) *rec_done = rec != nullptr;
         note_launches(1);
     } else {
-        switch (t) {
-            case InType::F16:
-                launch_kernel(mean_partial_kernel<__half>, dim3(G, batch), dim3(32, 8), 0, s, 
-                    static_cast<const __half*>(q), static_cast<const __half*>(k), M, N, D, rpb,
-                    partial);
-                break;
-            case InType::BF16:
-                launch_kernel(mean_partial_kernel<__nv_bfloat16>, dim3(G, batch), dim3(32, 8), 0, s, 
-                    static_cast<const __nv_bfloat16*>(q), static_cast<const __nv_bfloat16*>(k), M, N,
-                    D, rpb, partial);
-                break;
-            default:
-                launch_kernel(mean_partial_kernel<float>, dim3(G, batch), dim3(32, 8), 0, s, 
-                    static_cast<const float*>(q), static_cast<const float*>(k), M, N, D, rpb,
-                    partial);
-        }
+        // fp32 inputs (16-bit ones have D <= 256).
+        launch_kernel(mean_partial_kernel<float>, dim3(G, batch), dim3(32, 8), 0, s,
+                      static_cast<const float*>(q), static_cast<const float*>(k), M, N, D, rpb, partial);
         note_launches(1);
     }
     cudaError_t e = cudaGetLastError();
@@ -2414,15 +2403,16 @@ cudaError_t launch_prep_cluster(InType t, bool aug, const void* q, int64_t M, in
                : prep_cluster_typed<__half, false>(fill(__half()), batch, s);
 }
 
-cudaError_t launch_tf32_split(const float* x, int64_t rows, int64_t rows_pad, int D, int Dp,
-                              const float* mu, float half_c, float* out, float* nrm,
-                              float pad_value, cudaStream_t s, int batch, unsigned* guard) {
-    const int64_t total = rows_pad * batch;
+cudaError_t launch_tf32_split(const Tf32Job& q, const Tf32Job* k, int D, int Dp, const float* mu,
+                              float half_c, float pad_value, cudaStream_t s, int batch,
+                              unsigned* guard) {
+    const int64_t total0 = q.rows_pad * batch;
+    const int64_t total = total0 + (k ? k->rows_pad * batch : 0);
     if (total == 0) return cudaSuccess;
     const int threads = 256;
     const int64_t blocks = (total * 32 + threads - 1) / threads;
-    launch_kernel(tf32_split_kernel, static_cast<unsigned>(blocks), threads, 0, s, 
-        x, rows, rows_pad, total, D, Dp, mu, half_c, pad_value, out, nrm, guard);
+    launch_kernel(tf32_split_kernel, static_cast<unsigned>(blocks), threads, 0, s, q, k ? *k : Tf32Job{},
+                  total0, total, D, Dp, mu, half_c, pad_value, guard);
     note_launches(1);
     return cudaGetLastError();
 }

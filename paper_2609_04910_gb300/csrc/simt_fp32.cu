@@ -24,7 +24,7 @@ namespace gs {
 namespace {
 
 constexpr int KT = 64;       // keys per shared-memory tile (gradient; forward: key_tile)
-constexpr int THREADS = 128; // threads per block
+constexpr int THREADS = 128; // threads per block (forward: or half of that, see plan_simt)
 
 // ---------------------------------------------------------------- forward
 // Each thread holds ROWS = 4 query rows of up to 32 coordinates, so that one
@@ -72,12 +72,12 @@ simt_sum_kernel(const float* __restrict__ q, const float* __restrict__ k,
     constexpr int L = lanes_per_group(DMAX);
     constexpr int DL = DMAX / L;          // coordinates per lane
     constexpr int OWN = ROWS / L;         // rows whose sums a lane keeps
-    constexpr int GROUPS = THREADS / L;
     constexpr int KTF = key_tile(DMAX);
     static_assert(DL % 4 == 0 && DL <= 32, "coordinate quads of a lane");
     __shared__ __align__(16) float ks[2][KTF][DMAX];
     __shared__ __align__(16) float vs[2][KTF][CBLK];
 
+    const int nthreads = blockDim.x, GROUPS = nthreads / L;
     const int sub = threadIdx.x % L;
     const int64_t m0 = static_cast<int64_t>(blockIdx.x) * (GROUPS * ROWS) + threadIdx.x / L;
     const int split = blockIdx.y;
@@ -92,13 +92,13 @@ simt_sum_kernel(const float* __restrict__ q, const float* __restrict__ k,
     auto load_tile = [&](int b, int64_t t0) {
         const int cnt = static_cast<int>(min(static_cast<int64_t>(KTF), n_end - t0));
         const float* kt = k + t0 * D;
-        for (int i = threadIdx.x; i < KTF * DMAX; i += THREADS) {
+        for (int i = threadIdx.x; i < KTF * DMAX; i += nthreads) {
             const int kk = i / DMAX, d = i - kk * DMAX;
             const bool in = kk < cnt && d < D;
             cp_async4(&ks[b][kk][d], in ? kt + kk * D + d : v, in);
         }
         const float* vt = v + t0 * Cv + c0;
-        for (int i = threadIdx.x; i < KTF * CBLK; i += THREADS) {
+        for (int i = threadIdx.x; i < KTF * CBLK; i += nthreads) {
             const int kk = i / CBLK, j = i - kk * CBLK;
             const bool in = kk < cnt && c0 + j < Cv;
             cp_async4(&vs[b][kk][j], in ? vt + static_cast<int64_t>(kk) * Cv + j : v, in);
@@ -292,10 +292,10 @@ cudaError_t launch_grad(const SimtPlan& p, const float* q, const float* k, const
 template <int DMAX, int CBLK>
 cudaError_t launch_cblk(const SimtPlan& p, const float* q, const float* k, const float* v,
                         float half_c, float* part, cudaStream_t s, const unsigned* guard) {
-    constexpr int rows = THREADS / lanes_per_group(DMAX) * ROWS;
+    const int rows = p.threads / lanes_per_group(DMAX) * ROWS;
     dim3 grid(static_cast<unsigned>((p.M + rows - 1) / rows), p.splits,
               static_cast<unsigned>((p.Cv + CBLK - 1) / CBLK));
-    launch_kernel(simt_sum_kernel<DMAX, CBLK>, grid, THREADS, 0, s, q, k, v, p.M, p.N,
+    launch_kernel(simt_sum_kernel<DMAX, CBLK>, grid, p.threads, 0, s, q, k, v, p.M, p.N,
                   static_cast<int>(p.D), static_cast<int>(p.Cv), half_c, p.keys_per_split, part,
                   guard);
     note_launches(1);
@@ -338,7 +338,8 @@ bool plan_simt(int64_t M, int64_t N, int64_t D, int64_t C, bool grad, int split_
         keys = key_tile(p->dmax);
     }
     const int64_t chunks = grad ? 1 : (p->Cv + p->cblk - 1) / p->cblk;
-    const int64_t blocks = (M + rows - 1) / rows * chunks;   // per key split
+    int64_t blocks = (M + rows - 1) / rows * chunks;   // per key split
+    p->threads = THREADS;
     const int64_t key_tiles = std::max<int64_t>(1, (N + keys - 1) / keys);
     if (grad || split_override > 0) {
         int64_t splits = split_override > 0 ? split_override : (4LL * sms + blocks - 1) / blocks;
@@ -356,13 +357,24 @@ bool plan_simt(int64_t M, int64_t N, int64_t D, int64_t C, bool grad, int split_
         // Measured, 4096^2 pairs, D = 16: 1 and 2 blocks per SM (19 and 38
         // splits) 30.5 us, 24, 32, 64 splits 39.7, 32.7, 36.9 us; 5800^2
         // pairs, D = 32: one block per SM 124 us, three 95 us.
+        // And blocks of half the threads, where the rows of the last full-sized
+        // block would be mostly padding (1100 rows in blocks of 512).
         double best = 1e300;
-        for (int64_t per = 1; per <= 16; ++per) {
-            const int64_t want = std::min<int64_t>(256, std::max<int64_t>(1, per * sms / blocks));
-            const int64_t kps = std::max<int64_t>(16, ((N + want - 1) / want + 3) / 4 * 4);
-            const int64_t per_sm = (blocks * ((N + kps - 1) / kps) + sms - 1) / sms;
-            const double cost = static_cast<double>(per_sm) * (kps + 48.0) * (per_sm < 2 ? 1.3 : 1.0);
-            if (cost < best * 0.99) { best = cost; p->keys_per_split = kps; }
+        for (int threads = THREADS; threads >= THREADS / 2; threads /= 2) {
+            const int64_t r = rows * threads / THREADS;
+            const double size = static_cast<double>(threads) / THREADS;
+            blocks = (M + r - 1) / r * chunks;
+            for (int64_t per = 1; per <= 16 * THREADS / threads; ++per) {
+                const int64_t want = std::min<int64_t>(256, std::max<int64_t>(1, per * sms / blocks));
+                const int64_t kps = std::max<int64_t>(16, ((N + want - 1) / want + 3) / 4 * 4);
+                const int64_t per_sm = (blocks * ((N + kps - 1) / kps) + sms - 1) / sms;
+                const double cost = static_cast<double>(per_sm) * size * (kps + 48.0) * (per_sm * size < 2 ? 1.3 : 1.0);
+                if (cost < best * 0.99) {
+                    best = cost;
+                    p->keys_per_split = kps;
+                    p->threads = threads;
+                }
+            }
         }
     }
     p->splits = static_cast<int>((N + p->keys_per_split - 1) / p->keys_per_split);

@@ -817,12 +817,25 @@ tc_gauss_fma_kernel(const __grid_constant__ CUtensorMap tm_q,
                                 py = f32x2_pack(TRI ? ex2_approx(y0) : ex2_nonpos(y0),
                                                 TRI ? ex2_approx(y1) : ex2_nonpos(y1));
                             }
+                            // (Two channels per 16-byte load where the records allow it:
+                            // the loads share the MUFU's issue path.)
+                            constexpr int PER = C % 2 == 0 ? 2 : 1;
         #pragma unroll
-                            for (int cc = 0; cc < C; ++cc) {
-                                const float2 vc = *reinterpret_cast<const float2*>(pr + 2 * cc);
-                                const uint64_t vv = f32x2_pack(vc.x, vc.y);
-                                acc0[cc] = f32x2_fma(px, vv, acc0[cc]);
-                                acc1[cc] = f32x2_fma(py, vv, acc1[cc]);
+                            for (int cc = 0; cc < C; cc += PER) {
+                                uint64_t vv[2];
+                                if (PER == 2) {
+                                    const float4 vc = *reinterpret_cast<const float4*>(pr + 2 * cc);
+                                    vv[0] = f32x2_pack(vc.x, vc.y);
+                                    vv[1] = f32x2_pack(vc.z, vc.w);
+                                } else {
+                                    const float2 vc = *reinterpret_cast<const float2*>(pr + 2 * cc);
+                                    vv[0] = f32x2_pack(vc.x, vc.y);
+                                }
+        #pragma unroll
+                                for (int e = 0; e < PER; ++e) {
+                                    acc0[cc + e] = f32x2_fma(px, vv[e], acc0[cc + e]);
+                                    acc1[cc + e] = f32x2_fma(py, vv[e], acc1[cc + e]);
+                                }
                             }
                         }
                     } else {
