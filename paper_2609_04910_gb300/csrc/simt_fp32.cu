@@ -112,14 +112,31 @@ simt_sum_kernel(const float* __restrict__ q, const float* __restrict__ k,
     // rounding error of a split's sum grows with the keys per tile plus the
     // tiles, not with all its keys).
     float acc[OWN][CBLK];
+    // (In the widest loads that every row's alignment allows: each load touches
+    // 32 rows, and 4-byte loads of four 32-coordinate rows kept the load path
+    // busy for about 8 us per block.)
 #pragma unroll
     for (int r = 0; r < ROWS; ++r) {
         const int64_t m = m0 + r * GROUPS;
+        const float* qm = q + m * D;
 #pragma unroll
-        for (int i = 0; i < DL; i += 2) {
-            const int d = (i & ~3) * L + 4 * sub + (i & 3);
-            qr[r][i / 2] = f32x2_pack((m < M && d < D) ? q[m * D + d] : 0.f,
-                                      (m < M && d + 1 < D) ? q[m * D + d + 1] : 0.f);
+        for (int i = 0; i < DL; i += 4) {
+            const int d = i * L + 4 * sub;
+            float x[4] = {0.f, 0.f, 0.f, 0.f};
+            if (m < M && d < D) {
+                if ((D & 3) == 0) {
+                    *reinterpret_cast<float4*>(x) = *reinterpret_cast<const float4*>(qm + d);
+                } else if ((D & 1) == 0) {
+                    *reinterpret_cast<float2*>(x) = *reinterpret_cast<const float2*>(qm + d);
+                    if (d + 2 < D) *reinterpret_cast<float2*>(x + 2) = *reinterpret_cast<const float2*>(qm + d + 2);
+                } else {
+#pragma unroll
+                    for (int e = 0; e < 4; ++e)
+                        if (d + e < D) x[e] = qm[d + e];
+                }
+            }
+            qr[r][i / 2] = f32x2_pack(x[0], x[1]);
+            qr[r][i / 2 + 1] = f32x2_pack(x[2], x[3]);
         }
     }
 #pragma unroll
@@ -368,7 +385,9 @@ bool plan_simt(int64_t M, int64_t N, int64_t D, int64_t C, bool grad, int split_
                 const int64_t want = std::min<int64_t>(256, std::max<int64_t>(1, per * sms / blocks));
                 const int64_t kps = std::max<int64_t>(16, ((N + want - 1) / want + 3) / 4 * 4);
                 const int64_t per_sm = (blocks * ((N + kps - 1) / kps) + sms - 1) / sms;
-                const double cost = static_cast<double>(per_sm) * size * (kps + 48.0) * (per_sm * size < 2 ? 1.3 : 1.0);
+                // (A warp per SMSP and less take as long as a full block.)
+                const double share = std::max(1.0, per_sm * size);
+                const double cost = share * (kps + 48.0) * (share < 2 ? 1.3 : 1.0);
                 if (cost < best * 0.99) {
                     best = cost;
                     p->keys_per_split = kps;
