@@ -267,7 +267,8 @@ def gauss_sum_vjp(q, k, v, g, tau, want=("q", "k", "v"), grad_q=None, grad_k=Non
     lib = _lib or load_library()
     for t, n in ((q, "q"), (k, "k"), (v, "v"), (g, "g")):
         _check_tensor(t, n)
-    if _dtype_code(g) != GS_FP32:
+    import torch
+    if g.dtype != torch.float32:
         raise ValueError("g must be float32")
     M, D = q.shape
     N = k.shape[0]
