@@ -91,3 +91,16 @@ def test_scratch_limits_keep_the_simt_path():
     full = torch.empty(need, dtype=torch.uint8, device="cuda")
     assert torch.equal(gs.gauss_sum(q, k, v, 1.0 / 64, workspace=full),
                        gs.gauss_sum(q, k, v, 1.0 / 64))
+
+
+@pytest.mark.parametrize("M,N,D,C", [(16384, 16384, 64, 1), (16384, 16384, 33, 4),
+                                     (5000, 30001, 48, 2)])
+def test_many_key_tiles_repeat_bitwise(M, N, D, C):
+    """Long sequences of tf32 MMAs with the S tiles handed back as soon as they
+    are in registers: repeated calls agree bit for bit."""
+    import paper_2609_04910_gb300 as gs
+    q, k, v = device_inputs(generate(case(M, N, D, C, "fp32"), seed=6))
+    first = gs.gauss_sum(q, k, v, 1.0 / D)
+    again = [gs.gauss_sum(q, k, v, 1.0 / D) for _ in range(20)]
+    gs.gauss_sum_device_status()
+    assert all(torch.equal(first, a) for a in again)
