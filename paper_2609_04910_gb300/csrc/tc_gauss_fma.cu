@@ -52,6 +52,10 @@
 //     carry the same extra work: the MMA issue and key loads are split over
 //     one control warp per SMSP (round robin over key tiles) rather than
 //     given to one MMA warp, whose SMSP would otherwise pace all others.
+//     With q^ in TMEM the MMAs set the pace, and one control warp issues all
+//     of them: an S tile then goes back to a warp whose own earlier MMAs are
+//     the only ones that may still run (the same time as with one issuing warp
+//     per stage: 16384 x 1048576, D = 256, C = 4 6.31 ms).
 //
 // Warp roles (20 warps):
 //   warps 0-15   exponent warps.  Warp w reads TMEM lanes 32 (w % 4) .. +31
@@ -60,7 +64,9 @@
 //   warps 16-19  control warps, one per SMSP.  Control warp k owns shared-
 //                memory stage k and key tiles j = k (mod stages): it loads
 //                their k^ rows and key records (TMA) and issues and commits
-//                their MMAs.  Warp 16 also allocates TMEM and loads q^.
+//                their MMAs (q^ in TMEM: at most three stages, and warp 19
+//                issues and commits the MMAs of all key tiles).  Warp 16 also
+//                allocates TMEM and loads q^.
 // Key records: for each pair of keys (2t, 2t + 1) the floats
 //   v_2t[0], v_2t+1[0], ..., v_2t[C-1], v_2t+1[C-1]
 // with augmented operands, else for each four keys (4t .. 4t + 3) their B
@@ -147,11 +153,11 @@ struct __align__(8) FmaBarriers {
     uint64_t qa_ready;          // q^ available to the MMAs
     uint64_t q_free;            // OVL: every MMA of the segment has read q^ (one arrival per control warp)
     // q^ in shared memory: slot sl holds both S tiles of key tiles g = sl
-    // (mod 2); s_full[sl]: they are computed, s_free[sl]: they are in
-    // registers.  q^ in TMEM: s_full[h]: the S tile of query tile h is
-    // computed, s_free[2 h + g % 2]: that of key tile g is in registers.
+    // (mod 2); s_full[sl]: they are computed, s_free[sl]: the exponent warps
+    // are done with them.  q^ in TMEM: the same for the S tile of query tile h,
+    // s_full[h] and s_free[h].
     uint64_t s_full[2];
-    uint64_t s_free[4];
+    uint64_t s_free[2];
     uint64_t kv_full[MAX_STAGES];
     uint64_t kv_empty[MAX_STAGES];
     uint64_t stall;             // test hook: a barrier nothing arrives on
@@ -275,7 +281,10 @@ tc_gauss_fma_kernel(const __grid_constant__ CUtensorMap tm_q,
                     const __grid_constant__ CUtensorMap tm_k, const FmaParams p) {
     // TF (3xTF32): q^ in shared memory, norm terms from A and the records.
     // TF without QSM: q^ in TMEM, guarded (the call's points may be left to
-    // the SIMT path, see kGuardMaxBits).
+    // the SIMT path, see kGuardMaxBits), and HALVES: query tile 0's exponentials
+    // are summed before its S tile goes back, then query tile 1's.  The three
+    // MMAs per K step take longer than the exponentials, so the later handback
+    // costs little (16384^2, D = 64 140 -> 148 us).
     static_assert(!TF || !AUG, "3xTF32 takes plain rows");
     static_assert(!OVL || QSM, "overlapped segments keep q^ in shared memory");
     static_assert(VF == 0 || (AUG && SOFT == 0 && !TF), "folded operands: augmented fp16 rows");
@@ -285,6 +294,7 @@ tc_gauss_fma_kernel(const __grid_constant__ CUtensorMap tm_q,
     constexpr int kSoftMask = soft_mask(SOFT);
     constexpr int REC_PAIR = (AUG ? 0 : 2) + 2 * C;   // floats per key pair
     constexpr int SL = QSM ? 2 : 1;
+    constexpr bool HALVES = TF && !QSM;
     extern __shared__ uint8_t smem_raw[];
     const uint32_t raw_addr = smem_u32(smem_raw);
     uint8_t* smem = smem_raw + (((raw_addr + 1023u) & ~1023u) - raw_addr);
@@ -347,8 +357,10 @@ tc_gauss_fma_kernel(const __grid_constant__ CUtensorMap tm_q,
         mbar_init(&bars->q_free, NCTRL_MAX);
         mbar_init(&bars->stall, 1);
         for (int k = 0; k < NCTRL_MAX; ++k) mbar_init(&bars->drain[k], 1);
-        for (int i = 0; i < 2; ++i) mbar_init(&bars->s_full[i], 1);
-        for (int i = 0; i < 4; ++i) mbar_init(&bars->s_free[i], NEXP);   // one arrival per exponent warp
+        for (int i = 0; i < 2; ++i) {
+            mbar_init(&bars->s_full[i], 1);
+            mbar_init(&bars->s_free[i], NEXP);         // one arrival per exponent warp
+        }
         for (int s = 0; s < p.stages; ++s) {
             mbar_init(&bars->kv_full[s], 1);
             mbar_init(&bars->kv_empty[s], 1 + NEXP);  // MMA commit + exponent warps
@@ -433,18 +445,91 @@ tc_gauss_fma_kernel(const __grid_constant__ CUtensorMap tm_q,
                                     kb * p.kb_elems, (tile_m * NQ + h) * BM);
             }
             __syncwarp();
-            if (has_tiles && ok) {
-                auto load_keys = [&](int j) {
-                    mbar_arrive_expect_tx(&bars->kv_full[k], p.kh_bytes + p.rec_bytes);
-                    const int n0 = kbase + (kt0 + j) * BN;
-                    for (int kb = 0; kb < p.nkb; ++kb)
-                        tma_load_2d(kh_smem(k) + kb * (BN * 128), &tm_k, &bars->kv_full[k],
-                                    kb * p.kb_elems, n0);
-                    bulk_load(const_cast<float*>(rec_smem(k)),
-                              p.rec + ((VF == 1 || VF == 2) ? static_cast<int64_t>(n0 / BN) * (BN + BN / 32)
-                                          : static_cast<int64_t>(n0 / 2) * REC_PAIR),
-                              p.rec_bytes, &bars->kv_full[k]);
-                };
+            auto load_keys = [&](int j) {
+                mbar_arrive_expect_tx(&bars->kv_full[k], p.kh_bytes + p.rec_bytes);
+                const int n0 = kbase + (kt0 + j) * BN;
+                for (int kb = 0; kb < p.nkb; ++kb)
+                    tma_load_2d(kh_smem(k) + kb * (BN * 128), &tm_k, &bars->kv_full[k],
+                                kb * p.kb_elems, n0);
+                bulk_load(const_cast<float*>(rec_smem(k)),
+                          p.rec + ((VF == 1 || VF == 2) ? static_cast<int64_t>(n0 / BN) * (BN + BN / 32)
+                                      : static_cast<int64_t>(n0 / 2) * REC_PAIR),
+                          p.rec_bytes, &bars->kv_full[k]);
+            };
+            if (!QSM && k == NCTRL_MAX - 1) {
+                // q^ in TMEM: this warp issues every MMA of the CTA, in the
+                // order of the key tiles, one S tile per query tile.  Each is
+                // handed over as soon as it is done: the exponent warps take
+                // query tile 0's S while query tile 1's MMAs run, so the MMAs
+                // of key tile g + 1 follow those of key tile g without a gap
+                // (one barrier for both S tiles left the tensor pipe idle from
+                // the last MMA to the TMEM loads).  Tile g waits for the
+                // release of tile g - 1, whose own predecessor it has waited
+                // for before: no barrier is ever more than one phase behind.
+                ok = warp_wait(&bars->qa_ready, seg_parity, abort_flag, p.status);
+                // Test hook, as below.
+                if (ok && blockIdx.x == 0 && g0 == 0 &&
+                    *reinterpret_cast<volatile unsigned*>(p.status + kDevStallRequest) != 0u)
+                    ok = warp_wait(&bars->stall, 0, abort_flag, p.status);
+                const uint32_t kstep = BN * 128 / 16;                   // of the start-address field
+                const uint32_t klo = static_cast<uint32_t>(p.nkb / 2) * kstep;   // TF: the lo blocks
+                RingPos st;
+                st.idx = g0 % p.stages;
+                st.phase = static_cast<uint32_t>(g0 / p.stages) & 1u;
+                for (int j = 0; ok && j < T; ++j, st.advance(p.stages)) {
+                    const int g = g0 + j;
+                    ok = warp_wait(&bars->kv_full[st.idx], st.phase, abort_flag, p.status);
+                    const uint64_t kdesc = smem_desc_kmajor_sw128(smem_u32(kh_smem(st.idx)));
+                    for (int h = 0; h < NQ; ++h) {
+                        if (ok && g >= 1)
+                            ok = warp_wait(&bars->s_free[h], static_cast<uint32_t>(g - 1) & 1u, abort_flag,
+                                           p.status);
+                        if (!ok) break;
+                        tc_fence_after();
+                        if (leader) {
+                            const uint32_t d = tmem + h * BN, a = tmem + qa_col + h * q_cols;
+                            for (int kk = 0; kk < p.ksteps; ++kk) {
+                                const uint64_t kd = kdesc + (kk >> 2) * kstep + static_cast<uint32_t>((kk & 3) * 2);
+                                if (TF) {
+                                    // 3xTF32 as below, A = [hi | lo] from TMEM.
+                                    mma_ts_tf32(d, a + kk * 8, kd + klo, p.idesc, kk > 0 ? 1u : 0u);
+                                    mma_ts_tf32(d, a + p.Dp + kk * 8, kd, p.idesc, 1u);
+                                    mma_ts_tf32(d, a + kk * 8, kd, p.idesc, 1u);
+                                } else {
+                                    mma_ts_f16(d, a + kk * 8, kd, p.idesc, kk > 0 ? 1u : 0u);
+                                }
+                            }
+                            mma_commit(&bars->s_full[h]);
+                            if (h == NQ - 1) mma_commit(&bars->kv_empty[st.idx]);
+                        }
+                        __syncwarp();
+                        issued = true;
+                    }
+                }
+            } else if (!QSM && has_tiles) {
+                // Keys and records of this warp's stage; the stage is free
+                // again once the MMAs and the exponent warps are done with it.
+                uint32_t ph = static_cast<uint32_t>((g0 + j_first) / nctrl) & 1u;
+                bool pending = true;
+                if (leader) {
+                    tma_prefetch_desc(&tm_k);
+                    load_keys(j_first);
+                }
+                __syncwarp();
+                for (int j = j_first;; j += nctrl) {
+                    ok = warp_wait(&bars->kv_empty[k], ph, abort_flag, p.status);
+                    if (!ok) break;
+                    pending = false;
+                    if (j + nctrl >= T) break;
+                    ph ^= 1u;
+                    if (leader) load_keys(j + nctrl);
+                    __syncwarp();
+                    pending = true;
+                }
+                // (After an abort the copy may still be in flight.)
+                if (pending) mbar_wait_bounded(&bars->kv_full[k], ph, nullptr, p.status);
+                __syncwarp();
+            } else if (QSM && has_tiles && ok) {
                 // Parity of stage k's barriers for tile j: stage k completes once
                 // per tile g = k (mod nctrl).
                 uint32_t ph = static_cast<uint32_t>((g0 + j_first) / nctrl) & 1u;
@@ -473,7 +558,6 @@ tc_gauss_fma_kernel(const __grid_constant__ CUtensorMap tm_q,
                 const uint64_t kdesc = smem_desc_kmajor_sw128(smem_u32(kh_smem(k)));
                 const uint64_t qdesc0 = smem_desc_kmajor_sw128(smem_u32(q_smem));
                 const uint32_t qdesc_h = static_cast<uint32_t>((p.nkb * BM * 128) >> 4);
-                const uint32_t a0 = tmem + qa_col, a1 = a0 + q_cols;
                 bool pending = ok;            // keys of tile j requested, not yet waited for
                 int j = j_first;
                 for (; ok && j < T; j += nctrl, ph ^= 1u) {
@@ -481,13 +565,8 @@ tc_gauss_fma_kernel(const __grid_constant__ CUtensorMap tm_q,
                     // completes once per tile of the slot, and tile g reuses the
                     // slot that tile g - SL released.
                     const int g = g0 + j;
-                    // q^ in TMEM: query tile 0's S tile of key tile g - 1 is in
-                    // registers once s_free[(g - 1) % 2] has completed for it
-                    // (query tile 1's: s_free[2 + ..], waited for below).
-                    const int sl = QSM ? (g & 1) : ((g - 1) & 1);
-                    const uint32_t free_parity =
-                        QSM ? (static_cast<uint32_t>(g >> 1) & 1u) ^ 1u
-                            : static_cast<uint32_t>((g - 1) >> 1) & 1u;
+                    const int sl = g & 1;
+                    const uint32_t free_parity = (static_cast<uint32_t>(g >> 1) & 1u) ^ 1u;
                     const bool ready = __all_sync(
                         0xffffffffu, g < SL ? mbar_test_wait(&bars->kv_full[k], ph)
                                             : mbar_test_wait2(&bars->s_free[sl], free_parity,
@@ -502,8 +581,8 @@ tc_gauss_fma_kernel(const __grid_constant__ CUtensorMap tm_q,
                     }
                     pending = false;
                     tc_fence_after();
-                    const uint32_t d0 = tmem + (QSM ? sl * (2 * BN) : 0), d1 = d0 + BN;
-                    if (leader && TF && QSM) {
+                    const uint32_t d0 = tmem + sl * (2 * BN), d1 = d0 + BN;
+                    if (leader && TF) {
                         // 3xTF32: per K step of 8 coordinates (32 bytes),
                         // hi.lo + lo.hi + hi.hi; the lo blocks follow the
                         // hi blocks (nkb / 2 of each).
@@ -523,61 +602,20 @@ tc_gauss_fma_kernel(const __grid_constant__ CUtensorMap tm_q,
                         mma_commit(&bars->s_full[sl]);
                         mma_commit(&bars->kv_empty[k]);
                         if (OVL && j + nctrl >= T) mma_commit(&bars->q_free);
-                    } else if (QSM) {
-                        if (leader) {
-                            for (int h = 0; h < NQ; ++h) {
-                                for (int kk = 0; kk < ksteps; ++kk) {
-                                    const uint32_t koff = static_cast<uint32_t>((kk >> 2) * (BN * 128 / 16) + (kk & 3) * 2);
-                                    const uint32_t qoff = h * qdesc_h + static_cast<uint32_t>((kk >> 2) * (BM * 128 / 16) + (kk & 3) * 2);
-                                    mma_ss_f16(h ? d1 : d0, qdesc0 + qoff, kdesc + koff, p.idesc, kk > 0 ? 1u : 0u);
-                                }
-                            }
-                            mma_commit(&bars->s_full[sl]);
-                            mma_commit(&bars->kv_empty[k]);
-                            // OVL, the warp's last tile of the segment: q_free
-                            // arrives once these MMAs, and so all of this warp's
-                            // MMAs that read the segment's q^, are complete.
-                            if (OVL && j + nctrl >= T) mma_commit(&bars->q_free);
-                        }
-                    } else {
-                        // One S tile per query tile, each handed over as soon
-                        // as it is done: the exponent warps take query tile
-                        // 0's S while query tile 1's MMAs run, so the MMAs of
-                        // key tile g + 1 follow those of key tile g without a
-                        // gap (one barrier for both S tiles left the tensor
-                        // pipe idle from the last MMA to the TMEM loads).
+                    } else if (leader) {
                         for (int h = 0; h < NQ; ++h) {
-                            if (h == 1 && g >= 1) {
-                                ok = warp_wait(&bars->s_free[2 + sl], free_parity, abort_flag, p.status);
-                                if (!ok) break;
-                                tc_fence_after();
+                            for (int kk = 0; kk < ksteps; ++kk) {
+                                const uint32_t koff = static_cast<uint32_t>((kk >> 2) * (BN * 128 / 16) + (kk & 3) * 2);
+                                const uint32_t qoff = h * qdesc_h + static_cast<uint32_t>((kk >> 2) * (BM * 128 / 16) + (kk & 3) * 2);
+                                mma_ss_f16(h ? d1 : d0, qdesc0 + qoff, kdesc + koff, p.idesc, kk > 0 ? 1u : 0u);
                             }
-                            if (leader && TF) {
-                                // 3xTF32 as above, A = [hi | lo] from TMEM.
-                                const uint32_t klo = static_cast<uint32_t>((p.nkb / 2) * (BN * 128 / 16));
-                                const uint32_t d = h ? d1 : d0, a = h ? a1 : a0;
-                                for (int kk = 0; kk < ksteps; ++kk) {
-                                    const uint64_t kd = kdesc + (kk >> 2) * (BN * 128 / 16) +
-                                                        static_cast<uint32_t>((kk & 3) * 2);
-                                    mma_ts_tf32(d, a + kk * 8, kd + klo, p.idesc, kk > 0 ? 1u : 0u);
-                                    mma_ts_tf32(d, a + p.Dp + kk * 8, kd, p.idesc, 1u);
-                                    mma_ts_tf32(d, a + kk * 8, kd, p.idesc, 1u);
-                                }
-                                mma_commit(&bars->s_full[h]);
-                                if (h == 1) mma_commit(&bars->kv_empty[k]);
-                            } else if (leader) {
-                                for (int kk = 0; kk < ksteps; ++kk) {
-                                    const uint32_t koff = static_cast<uint32_t>((kk >> 2) * (BN * 128 / 16) + (kk & 3) * 2);
-                                    mma_ts_f16(h ? d1 : d0, (h ? a1 : a0) + kk * 8, kdesc + koff, p.idesc,
-                                               kk > 0 ? 1u : 0u);
-                                }
-                                mma_commit(&bars->s_full[h]);
-                                if (h == 1) mma_commit(&bars->kv_empty[k]);
-                            }
-                            __syncwarp();
-                            issued = true;
                         }
-                        if (!ok) break;
+                        mma_commit(&bars->s_full[sl]);
+                        mma_commit(&bars->kv_empty[k]);
+                        // OVL, the warp's last tile of the segment: q_free
+                        // arrives once these MMAs, and so all of this warp's
+                        // MMAs that read the segment's q^, are complete.
+                        if (OVL && j + nctrl >= T) mma_commit(&bars->q_free);
                     }
                     __syncwarp();
                     issued = true;
@@ -730,16 +768,17 @@ tc_gauss_fma_kernel(const __grid_constant__ CUtensorMap tm_q,
                         // no faster on the 65536^2, D = 64 sum either: 0.6428
                         // against 0.6418 ms).
                         tmem_wait_ld_regs(r0, r1);
-                    } else {
+                    } else if (!HALVES) {
                         // q^ in TMEM: one S tile per query tile, handed back as
                         // soon as it is in registers, since the MMAs of the next
-                        // key tile need it (a late release would serialise MMAs
-                        // and exponent work; regression test: repeated calls
-                        // agree bit for bit).
+                        // key tile need it: the exponentials take about as long
+                        // as the MMAs.  (Unlike with two slots, all MMAs come
+                        // from one warp here, which issues the next ones behind
+                        // its own earlier ones.)
                         tmem_wait_ld_regs(r0);
                         tc_fence_before();
                         __syncwarp();
-                        mbar_arrive_if_zero(&bars->s_free[sl.phase], lane);
+                        mbar_arrive_if_zero(&bars->s_free[0], lane);
                         ok = warp_wait(&bars->s_full[1], sl.phase, abort_flag, p.status);
                         if (!ok) break;
                         tc_fence_after();
@@ -747,7 +786,9 @@ tc_gauss_fma_kernel(const __grid_constant__ CUtensorMap tm_q,
                         tmem_wait_ld_regs(r1);
                         tc_fence_before();
                         __syncwarp();
-                        mbar_arrive_if_zero(&bars->s_free[2 + sl.phase], lane);
+                        mbar_arrive_if_zero(&bars->s_free[1], lane);
+                    } else {
+                        tmem_wait_ld_regs(r0);
                     }
                     // Query the barriers of key tile j + 1 now and read the answer
                     // after the exponent work of tile j: the query latency overlaps
@@ -838,19 +879,53 @@ tc_gauss_fma_kernel(const __grid_constant__ CUtensorMap tm_q,
                                 }
                             }
                         }
-                    } else {
-                        // Guarded fp32 sums: the sums of the key tile by
+                    } else if constexpr (HALVES) {
+                        // Query tile 0's rows, then query tile 1's: each S tile is
+                        // handed back once its exponentials are summed, while the
+                        // MMAs of the other one run.  The sums of the key tile by
                         // themselves, added to acc at its end, so that rounding
-                        // grows with the keys of a tile plus the tiles, not
-                        // with all keys (with q^ in shared memory, where the
-                        // exponent warps set the pace, it cost 2 %).
-                        constexpr bool TILE_SUMS = TF && !QSM;
-                        uint64_t t0[C], t1[C];
+                        // grows with the keys of a tile plus the tiles, not with
+                        // all keys.
+                        auto half = [&](const uint32_t (&r)[32], uint64_t a2, uint64_t (&acc)[C]) {
+                            uint64_t sum[C];
         #pragma unroll
-                        for (int cc = 0; cc < C; ++cc) {
-                            t0[cc] = TILE_SUMS ? 0ull : acc0[cc];
-                            t1[cc] = TILE_SUMS ? 0ull : acc1[cc];
-                        }
+                            for (int cc = 0; cc < C; ++cc) sum[cc] = 0ull;
+        #pragma unroll
+                            for (int t = 0; t < 8; ++t) {
+                                const float4* pr = reinterpret_cast<const float4*>(rec + t * (2 * REC_PAIR));
+                                const float4 bb = pr[0];
+                                uint64_t px[2];
+        #pragma unroll
+                                for (int e = 0; e < 2; ++e) {
+                                    const uint64_t b2 = e ? f32x2_pack(bb.z, bb.w) : f32x2_pack(bb.x, bb.y);
+                                    const int i = 4 * t + 2 * e;
+                                    float x0, x1;
+                                    f32x2_unpack(f32x2_fma(f32x2_pack(__uint_as_float(r[i]), __uint_as_float(r[i + 1])),
+                                                           c2, f32x2_add(b2, a2)),
+                                                 x0, x1);
+                                    px[e] = f32x2_pack(ex2_nonpos(x0), ex2_nonpos(x1));
+                                }
+        #pragma unroll
+                                for (int cc = 0; cc < C; ++cc) {
+                                    const float4 vc = pr[1 + cc];
+                                    sum[cc] = f32x2_fma(px[0], f32x2_pack(vc.x, vc.y), sum[cc]);
+                                    sum[cc] = f32x2_fma(px[1], f32x2_pack(vc.z, vc.w), sum[cc]);
+                                }
+                            }
+        #pragma unroll
+                            for (int cc = 0; cc < C; ++cc) acc[cc] = f32x2_add(acc[cc], sum[cc]);
+                        };
+                        half(r0, a2_0, acc0);
+                        tc_fence_before();
+                        __syncwarp();
+                        mbar_arrive_if_zero(&bars->s_free[0], lane);
+                        ok = warp_wait(&bars->s_full[1], sl.phase, abort_flag, p.status);
+                        if (!ok) break;
+                        tc_fence_after();
+                        tmem_ld_32x32b_x32(tmem + lane_base + BN + cg * 32, r1);
+                        tmem_wait_ld_regs(r1);
+                        half(r1, a2_1, acc1);
+                    } else {
                         // Quad records: B and then each channel's values of
                         // four keys, one 16-byte load each.  (In key pairs,
                         // 8-byte loads, the records took half of the shared-
@@ -880,16 +955,11 @@ tc_gauss_fma_kernel(const __grid_constant__ CUtensorMap tm_q,
                             for (int cc = 0; cc < C; ++cc) {
                                 const float4 vc = pr[1 + cc];
                                 const uint64_t v01 = f32x2_pack(vc.x, vc.y), v23 = f32x2_pack(vc.z, vc.w);
-                                t0[cc] = f32x2_fma(px[0], v01, t0[cc]);
-                                t1[cc] = f32x2_fma(py[0], v01, t1[cc]);
-                                t0[cc] = f32x2_fma(px[1], v23, t0[cc]);
-                                t1[cc] = f32x2_fma(py[1], v23, t1[cc]);
+                                acc0[cc] = f32x2_fma(px[0], v01, acc0[cc]);
+                                acc1[cc] = f32x2_fma(py[0], v01, acc1[cc]);
+                                acc0[cc] = f32x2_fma(px[1], v23, acc0[cc]);
+                                acc1[cc] = f32x2_fma(py[1], v23, acc1[cc]);
                             }
-                        }
-        #pragma unroll
-                        for (int cc = 0; cc < C; ++cc) {
-                            acc0[cc] = TILE_SUMS ? f32x2_add(acc0[cc], t0[cc]) : t0[cc];
-                            acc1[cc] = TILE_SUMS ? f32x2_add(acc1[cc], t1[cc]) : t1[cc];
                         }
                     }
                     tc_fence_before();
@@ -898,6 +968,7 @@ tc_gauss_fma_kernel(const __grid_constant__ CUtensorMap tm_q,
                     // predicated rather than branched: a divergent branch here
                     // cost 0.7 % of the kernel time.
                     if (QSM) mbar_arrive2_if_zero(&bars->s_free[sl.idx], &bars->kv_empty[s], lane);
+                    else if (HALVES) mbar_arrive2_if_zero(&bars->s_free[1], &bars->kv_empty[s], lane);
                     else mbar_arrive_if_zero(&bars->kv_empty[s], lane);
                 }
             };
@@ -1093,17 +1164,15 @@ bool plan_fma_kernel(int Dp, int C, bool aug, bool tf, int* nq, int* stages, siz
     const size_t stage = stage_bytes_for(nkb, C, aug);
     const size_t fixed = fixed_bytes_for(C, q_bytes_for(nkb, qsm));
     if (fixed >= budget) return false;
-    // Control warp k owns stage k (stages = control warps) and checks the
-    // S release of an earlier key tile before the MMAs of tile j.  An
-    // mbarrier parity test is only unambiguous while the barrier is at most
-    // one phase behind the phase it asks about; the warp knows every key
-    // tile up to j - stages is done (its previous stage release).  Two slots:
-    // it asks about tile j - 2, the slot's previous phase is tile j - 4, so
-    // stages <= 4.  One S tile per query tile (q^ in TMEM): it asks about
-    // tile j - 1 on the barrier of that tile's parity, whose previous phase
-    // is tile j - 3, so stages <= 3.
+    // q^ in shared memory: control warp k owns stage k (stages = control
+    // warps) and checks the slot release of key tile j - 2 before the MMAs of
+    // tile j.  An mbarrier parity test is only unambiguous while the barrier
+    // is at most one phase behind the phase it asks about; the warp knows
+    // every key tile up to j - stages is done (its previous stage release) and
+    // the slot's previous phase is tile j - 4, so stages <= 4.  q^ in TMEM:
+    // one control warp issues the MMAs, the others load a stage each.
     const int st = static_cast<int>(
-        std::min<size_t>(qsm ? MAX_STAGES : 3, (budget - fixed) / stage));
+        std::min<size_t>(qsm ? MAX_STAGES : NCTRL_MAX - 1, (budget - fixed) / stage));
     if (st < 2) return false;
     *nq = NQ;
     *stages = st;
