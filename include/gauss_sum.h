@@ -39,11 +39,16 @@
  *    with three tf32 MMAs per product (q^ k^T ~ hi.hi + hi.lo + lo.hi of the
  *    tf32 splits x = hi + lo, fp32-level accuracy): chosen automatically
  *    from 2^25 pairs (per call, summed over a batch; single problems with
- *    D <= 4 from 2^26), or forced with GS_PATH_TENSOR / GS_PATH_SIMT.  Single forward sums with C <= 4 and
- *    32 < D <= 64 from 2^24 pairs launch both: a device-side look at the
- *    points' norms lets the tensor cores work only where they are as accurate
- *    as the SIMT kernel's coordinate differences (largest
- *    (tau/2) log2(e) ||x - mean||^2 at most 4), else the SIMT kernel does.
+ *    D <= 4 from 2^26), or forced with GS_PATH_TENSOR / GS_PATH_SIMT.  Single
+ *    forward sums with C <= 4 and 32 < D <= 64 from 2^24 pairs launch both: a
+ *    look at the points on the device lets the tensor cores' sums count only
+ *    where every (tau/2) log2(e) ||x - mean||^2 is at most 2 and at most one
+ *    pair in 256 is close compared with its norms (tau log2(e)
+ *    (q - mean).(k - mean) > 1), else the SIMT kernel's do.  The norms' form
+ *    of the exponent is off by a few 2^-24 of the norm terms, the SIMT
+ *    kernel's differences by a few 2^-24 of the exponent; within these limits
+ *    both errors stay below 5e-7 of sum |v| Phi, which single-precision sums
+ *    have anyway.  GS_PATH_SIMT takes the differences whatever the points.
  *    Their workspace holds both; where a caller's workspace, or the scratch of
  *    gauss_sum_noalloc, is too small for both, the SIMT kernel runs alone.
  *  - On a non-OK return gauss_sum_last_error() describes the failure.

@@ -223,14 +223,16 @@ bool fp32_on_tensor_cores(const Call& c) {
 }
 
 // Wider rows (32 < D <= 64) of large single forward sums also go to the
-// tensor cores, guarded: both paths are launched, and the operand kernel's
-// look at the points decides on the device which one works (see
-// kGuardMaxBits).  From 2^24 pairs, where its extra launches are repaid.
+// tensor cores, guarded: both paths are launched, and a look at the points on
+// the device decides whose sums count (see Guard in internal.h).  From 2^24
+// pairs, where its extra launches are repaid.
 // Measured on a GB300, whole calls, SIMT / guarded: 16384^2, D = 64, C = 1
 // 1145 / 140 us (the tensor cores' share of the work at three tf32 MMAs per
 // product is 80 us), 8192^2, D = 50 305 / 66 us, 6000^2, D = 64 176 / 57 us.
-// Error against 64 bits (relative, 2-norm, N(0, I) points and values): 1.0 to
-// 6.6e-7, the SIMT kernel's 1.1 to 7.7e-7 on the same inputs.
+// Error against 64 bits at 8192^2, D = 33 to 64 (guarded / SIMT kernel): N(0, I)
+// points and values, relative 2-norm 1.0e-7 to 2.5e-7 / 1.3e-7 to 3.7e-7; two
+// clusters with norm terms of 0.4 to 2, largest error relative to the sum of
+// |v| Phi 4.3e-7 / 4.3e-7 (most of them summed by the SIMT kernel).
 constexpr int64_t kFp32GuardedMinPairs = int64_t(1) << 24;
 
 bool fp32_guarded(const Call& c) {
@@ -387,11 +389,14 @@ gs_status run(Call c) {
     if (tensor) {
         const gs::InType t = in_type(c.dtype);
         float* mu = (tp.center && c.D > 0) ? reinterpret_cast<float*>(ws + tp.off_mu) : nullptr;
-        // Guarded sums: the word behind the key records (B and Cv values per key).
-        unsigned* guard = tp.guard ? reinterpret_cast<unsigned*>(ws + tp.off_rec) + tp.Npad * (1 + tp.Cv)
-                                   : nullptr;
-        if (guard && !mu) {
-            e = cudaMemsetAsync(guard, 0, sizeof(unsigned), c.stream);
+        // Guarded sums: the words behind the key records (B and Cv values per key).
+        gs::Guard guard;
+        if (tp.guard) {
+            guard.words = reinterpret_cast<unsigned*>(ws + tp.off_rec) + tp.Npad * (1 + tp.Cv);
+            guard.most_close = static_cast<unsigned long long>(c.M) * c.N / (8 * 256);
+        }
+        if (guard.words && !mu) {
+            e = cudaMemsetAsync(guard.words, 0, gs::kGuardWords * sizeof(unsigned), c.stream);
             where = "cudaMemsetAsync";
         }
         // Key records of the FMA kernel with augmented operands depend on the
@@ -404,7 +409,7 @@ gs_status run(Call c) {
             // Words that later launches take maxima into: the guard, or the
             // two-MMA kernel's channel and weight maxima.
             gs::ZeroWords zero;
-            if (guard) zero = {guard, 1};
+            if (guard.words) zero = {guard.words, gs::kGuardWords};
             else if (!tp.fma) zero = {reinterpret_cast<unsigned*>(ws + tp.off_vmax), tp.Cp + 2 * tp.wt};
             const gs::RecordArgs rec = {c.v, c.w_f32, c.N, tp.Npad, static_cast<int>(tp.Cv),
                                         reinterpret_cast<float*>(ws + tp.off_rec), tp.vfold};
@@ -441,7 +446,7 @@ gs_status run(Call c) {
                                     reinterpret_cast<float*>(ws + tp.off_kh),
                                     reinterpret_cast<float*>(ws + tp.off_B)};
             e = gs::launch_tf32_split(jq, tp.alias ? nullptr : &jk, static_cast<int>(c.D), tp.Dp, mu,
-                                      half_c, ninf, c.stream, batch, guard);
+                                      half_c, ninf, c.stream, batch, guard.words);
             where = "tf32 split kernel";
         } else {
             // Centred, rounded operands of q and (unless q is k) k in one
@@ -484,7 +489,7 @@ gs_status run(Call c) {
                     e = gs::launch_tc_fma(tp, t, cexp, ws, status, c.stream, &why, 2);
                 where = "fused tensor-core kernel";
             }
-            if (e == cudaSuccess && guard) {
+            if (e == cudaSuccess && guard.words) {
                 // The other side of the guard.
                 e = gs::launch_simt(sp, false, static_cast<const float*>(c.q),
                                     static_cast<const float*>(c.k), static_cast<const float*>(c.v),
@@ -497,7 +502,7 @@ gs_status run(Call c) {
                 const int fixed = tp.band_len > 0 ? tp.splits : 0;
                 const int64_t kt = tp.Npad / tp.BN;
                 const float* part = reinterpret_cast<float*>(ws + tp.off_part);
-                if (c.mmd_out && !guard && t != gs::InType::F32) {
+                if (c.mmd_out && t != gs::InType::F32) {
                     e = gs::launch_mmd2_slots(t, part, tp.Mpad, c.M, 128 * tp.nq, kt, tp.unit_len, c.v,
                                               c.mmd_part, c.mmd_out, c.stream, batch, fixed,
                                               tp.tri ? kt : 0);
@@ -509,7 +514,7 @@ gs_status run(Call c) {
                 }
                 where = "finalise kernel";
             }
-            if (e == cudaSuccess && guard) {
+            if (e == cudaSuccess && guard.words) {
                 e = gs::launch_finalize(reinterpret_cast<float*>(ws + sp.off_part), sp.splits, c.M, c.M,
                                         static_cast<int>(sp.Cv), static_cast<int>(sp.Cv), nullptr, c.out,
                                         c.stream, 0, guard);

@@ -49,13 +49,34 @@ constexpr int64_t kTwoMmaMinPairs = int64_t(1) << 28;
 
 // Guard of fp32 sums of wide rows.  The tensor cores form the exponent as
 // c q^.k^ + A_m + B_n from the points' norms, the SIMT kernel from coordinate
-// differences; the first is as accurate only while the norm terms stay small
-// (its error is a few units in the last place of |A_m| + |B_n|, whatever the
-// distance).  The operand kernel writes the bits of the largest
-// (c/2)||x - mu||^2 of the call; up to 4.0 the tensor-core kernels work and
-// above it (or NaN, whose bits are larger still) the SIMT kernels do.  Points
-// ~ N(0, I_D) with tau = 1/D stay below 2.
-constexpr unsigned kGuardMaxBits = 0x40800000u;   // 4.0f
+// differences.  The first is off by a few units in the last place of
+// |A_m| + |B_n| and, because the MMAs round every partial sum of q^.k^ towards
+// zero, by up to as many of c q^.k^ as there are K steps, whatever the
+// distance; the second by a few of the exponent itself.  So the tensor cores'
+// sums only count where
+//  * the largest (c/2)||x - mu||^2 of the call is at most 2, and
+//  * at most one pair in 256 (of a sample of one key in eight) has
+//    c q^.k^ > 1, i.e. points that are close to one another compared with
+//    their distance from the mean.
+// Relative to the sum of |v| Phi, the largest error of clusters of points was
+// measured at 4.2e-6 (norm terms 3.9) and 2.5e-6 (1.95) without the second
+// condition, where the SIMT kernel has 2e-7 to 6e-7.  Points ~ N(0, I_D) with
+// tau = 1/D have norm terms below 2 and at D = 33 one pair in 10^4 above 1.
+// The words, behind the key records: [0] the bits of the largest norm term,
+// written with the operands (a NaN's are larger still); [2..3] the count of
+// sampled pairs above kGuardClose, added up by the tensor-core kernel.
+constexpr unsigned kGuardMaxBits = 0x40000000u;   // 2.0f
+constexpr float kGuardClose = 1.0f;
+constexpr int kGuardWords = 4;
+struct Guard {
+    unsigned* words = nullptr;
+    unsigned long long most_close = 0;   // sampled pairs: M N / 8 / 256
+};
+// Whether the SIMT path's sums count.  Read after pdl_wait only.
+__device__ __forceinline__ bool guard_simt(const Guard& g) {
+    return g.words[0] > kGuardMaxBits ||
+           *reinterpret_cast<const unsigned long long*>(g.words + 2) > g.most_close;
+}
 
 // Workspace plan of the tensor-core path.  All offsets are bytes from the
 // workspace base and are 1024-byte aligned.
@@ -88,8 +109,8 @@ struct TcPlan {
                              // rows are [hi | lo] of Dp (a multiple of 32) floats each
     // 3xTF32 with a guard (rows of more than kTf32MaxDp coordinates): the
     // kernels of the tensor-core path and of the SIMT path are both launched,
-    // and a word written with the operands (kGuardMaxBits) says which of
-    // them work; the others return at once.
+    // and the guard's words say whose sums count (see Guard); the SIMT kernels
+    // return at once where the tensor cores' do.
     bool guard;
     int nq;                  // query tiles of 128 rows per CTA (FMA kernel)
     bool early_s;            // two-MMA kernel: S buffers handed back as soon as they are
@@ -244,7 +265,7 @@ cudaError_t launch_weight_prep(InType t, const void* rsrc, bool r_f32, int64_t R
 cudaError_t launch_finalize(const float* part, int splits, int64_t split_stride_rows,
                             int64_t M, int Cv, int part_ld, const float* inv_scale, float* out,
                             cudaStream_t s, int64_t main_rows = 0,
-                            const unsigned* guard = nullptr);
+                            const Guard& guard = {});
 // Gradient contraction of one launch's channels ch0 .. ch0 + Cc - 1 (see
 // prep.cu): out[m, d] (+)= tau sum_c u[m, c] (S_{c,d} - x^_{m,d} S_{c,D}),
 // s_out[m, c] = S_{c,D}.  direct: fp32 kernel partials (difference form).
@@ -277,14 +298,14 @@ cudaError_t launch_finalize_slots(const float* part, int64_t Mpad, int64_t M, in
                                   int rows_per_unit, int64_t key_tiles, int64_t unit_len,
                                   float* out, cudaStream_t s, int batch = 1,
                                   int fixed_slots = 0, int64_t tri_key_tiles = 0,
-                                  const unsigned* guard = nullptr);
+                                  const Guard& guard = {});
 
 // simt_fp32.cu ---------------------------------------------------------
 // grad: keys weighted by channel wch of v (N x Cw); partials have D + 1
 // channels (sum Phi w (k - q), sum Phi w).
 cudaError_t launch_simt(const SimtPlan& p, bool grad, const float* q, const float* k,
                         const float* v, int Cw, int wch, float half_c, float* part,
-                        cudaStream_t s, const unsigned* guard = nullptr);
+                        cudaStream_t s, const Guard& guard = {});
 
 // Key records of the FMA kernel: without B per key pair (2t, 2t+1) the floats
 // v_2t[0], v_2t+1[0], ..., v_2t[C-1], v_2t+1[C-1]; with B per four keys their

@@ -779,10 +779,6 @@ __global__ void tf32_split_kernel(const Tf32Job j0, const Tf32Job j1, int64_t to
     }
 }
 
-// Guarded sums (see kGuardMaxBits): whether the call's points exceed the
-// tensor-core path's range.  Read after pdl_wait only.
-__device__ __forceinline__ bool guard_above(const unsigned* guard) { return *guard > kGuardMaxBits; }
-
 // Contributor slots of pair of query tiles r of the FMA kernel (see
 // launch_finalize_slots in internal.h).
 __device__ __forceinline__ int64_t contributor_slots(int64_t r, int fixed_slots, int64_t key_tiles,
@@ -805,10 +801,10 @@ __global__ void finalize_slots_kernel(const float* __restrict__ part, int64_t Mp
                                       int C, int rows_per_unit, int64_t key_tiles,
                                       int64_t unit_len, int64_t batch, int fixed_slots,
                                       int64_t tri_kt, float* __restrict__ out,
-                                      const unsigned* __restrict__ guard) {
+                                      const Guard guard) {
     pdl_trigger();
     pdl_wait();
-    if (guard && guard_above(guard)) return;   // the SIMT path's sums count
+    if (guard.words && guard_simt(guard)) return;
     // out: batch x M x C; partial rows are batch-stacked with Mpad rows per
     // problem and batch Mpad rows per slot.
     const int64_t idx = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
@@ -1482,10 +1478,10 @@ weight_prep_kernel(const TR* __restrict__ rsrc, int64_t R, int64_t Rpad,
 __global__ void finalize_kernel(const float* __restrict__ part, int splits,
                                 int64_t split_stride_rows, int64_t M, int Cv, int part_ld,
                                 const float* __restrict__ inv_scale, float* __restrict__ out,
-                                int64_t main_rows, const unsigned* __restrict__ guard) {
+                                int64_t main_rows, const Guard guard) {
     pdl_trigger();
     pdl_wait();
-    if (guard && !guard_above(guard)) return;   // the tensor-core path's sums count
+    if (guard.words && !guard_simt(guard)) return;
     const int64_t idx = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
     if (idx >= M * Cv) return;
     const int64_t m = div_nonneg(idx, Cv);
@@ -2291,7 +2287,7 @@ cudaError_t launch_mmd2_slots(InType t, const float* part, int64_t Mpad, int64_t
 cudaError_t launch_finalize_slots(const float* part, int64_t Mpad, int64_t M, int C,
                                   int rows_per_unit, int64_t key_tiles, int64_t unit_len,
                                   float* out, cudaStream_t s, int batch, int fixed_slots,
-                                  int64_t tri_key_tiles, const unsigned* guard) {
+                                  int64_t tri_key_tiles, const Guard& guard) {
     const int64_t total = static_cast<int64_t>(batch) * M * C;
     if (total == 0) return cudaSuccess;
     const int threads = 256;
@@ -2532,10 +2528,10 @@ cudaError_t launch_weight_prep(InType t, const void* rsrc, bool r_f32, int64_t R
 
 cudaError_t launch_finalize(const float* part, int splits, int64_t split_stride_rows,
                             int64_t M, int Cv, int part_ld, const float* inv_scale, float* out,
-                            cudaStream_t s, int64_t main_rows, const unsigned* guard) {
+                            cudaStream_t s, int64_t main_rows, const Guard& guard) {
     const int64_t total = M * Cv;
     if (total == 0) return cudaSuccess;
-    if (Cv % 4 == 0 && part_ld % 4 == 0 && !guard) {
+    if (Cv % 4 == 0 && part_ld % 4 == 0 && !guard.words) {
         launch_kernel(finalize_quads_kernel,
                       static_cast<unsigned>((total / 4 + kFinalizeThreads - 1) / kFinalizeThreads),
                       kFinalizeThreads, 0, s, part, splits, split_stride_rows, M, Cv, part_ld, inv_scale, out, main_rows);

@@ -65,10 +65,10 @@ __global__ void __launch_bounds__(THREADS, min_blocks(DMAX, CBLK))
 simt_sum_kernel(const float* __restrict__ q, const float* __restrict__ k,
                 const float* __restrict__ v, int64_t M, int64_t N, int D, int Cv, float half_c,
                 int64_t keys_per_split, float* __restrict__ part,
-                const unsigned* __restrict__ guard) {
+                const Guard guard) {
     pdl_trigger();
     pdl_wait();
-    if (guard && *guard <= kGuardMaxBits) return;   // the tensor-core path does the call
+    if (guard.words && !guard_simt(guard)) return;   // the tensor-core path does the call
     constexpr int L = lanes_per_group(DMAX);
     constexpr int DL = DMAX / L;          // coordinates per lane
     constexpr int OWN = ROWS / L;         // rows whose sums a lane keeps
@@ -308,7 +308,7 @@ cudaError_t launch_grad(const SimtPlan& p, const float* q, const float* k, const
 
 template <int DMAX, int CBLK>
 cudaError_t launch_cblk(const SimtPlan& p, const float* q, const float* k, const float* v,
-                        float half_c, float* part, cudaStream_t s, const unsigned* guard) {
+                        float half_c, float* part, cudaStream_t s, const Guard& guard) {
     const int rows = p.threads / lanes_per_group(DMAX) * ROWS;
     dim3 grid(static_cast<unsigned>((p.M + rows - 1) / rows), p.splits,
               static_cast<unsigned>((p.Cv + CBLK - 1) / CBLK));
@@ -322,7 +322,7 @@ cudaError_t launch_cblk(const SimtPlan& p, const float* q, const float* k, const
 // Channel blocks of 4, or of 1 or 2 for as few channels (no idle FMAs).
 template <int DMAX>
 cudaError_t launch_dmax(const SimtPlan& p, const float* q, const float* k, const float* v,
-                        float half_c, float* part, cudaStream_t s, const unsigned* guard) {
+                        float half_c, float* part, cudaStream_t s, const Guard& guard) {
     if (p.cblk == 1) return launch_cblk<DMAX, 1>(p, q, k, v, half_c, part, s, guard);
     if (p.cblk == 2) return launch_cblk<DMAX, 2>(p, q, k, v, half_c, part, s, guard);
     return launch_cblk<DMAX, 4>(p, q, k, v, half_c, part, s, guard);
@@ -406,7 +406,7 @@ bool plan_simt(int64_t M, int64_t N, int64_t D, int64_t C, bool grad, int split_
 
 cudaError_t launch_simt(const SimtPlan& p, bool grad, const float* q, const float* k,
                         const float* v, int Cw, int wch, float half_c, float* part,
-                        cudaStream_t s, const unsigned* guard) {
+                        cudaStream_t s, const Guard& guard) {
     if (grad) {
         switch (p.dmax) {
             case 16: return launch_grad<16>(p, q, k, v, Cw, wch, half_c, part, s);

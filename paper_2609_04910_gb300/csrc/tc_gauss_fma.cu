@@ -123,6 +123,7 @@ struct FmaParams {
     const float* rec;    // key records, Npad / 2 pairs
     float* part;         // contributor slots x Mpad x C partial sums
     unsigned* status;
+    unsigned* guard;     // guarded sums: the words behind the key records (see Guard)
     int64_t Mpad;
     int units;           // work units: (pair of query tiles, key tile), row major
     int unit_len;        // units per CTA (CTA i: units [i unit_len, (i + 1) unit_len))
@@ -310,10 +311,8 @@ tc_gauss_fma_kernel(const __grid_constant__ CUtensorMap tm_q,
 
     pdl_trigger();
     if (TF && !QSM) {
-        // Guarded sums: the word follows the key records.
         pdl_wait();
-        const int64_t rec_floats = static_cast<int64_t>(p.npad / 2) * REC_PAIR;
-        if (*reinterpret_cast<const unsigned*>(p.rec + rec_floats) > kGuardMaxBits) return;
+        if (*p.guard > kGuardMaxBits) return;
     }
     if (VF == 2) {
         // The second folded-value pass often has nothing to do (every problem
@@ -491,14 +490,19 @@ tc_gauss_fma_kernel(const __grid_constant__ CUtensorMap tm_q,
                             for (int kk = 0; kk < p.ksteps; ++kk) {
                                 const uint64_t kd = kdesc + (kk >> 2) * kstep + static_cast<uint32_t>((kk & 3) * 2);
                                 if (TF) {
-                                    // 3xTF32 as below, A = [hi | lo] from TMEM.
+                                    // 3xTF32, A = [hi | lo] from TMEM: the small
+                                    // products first, so that only the hi.hi steps
+                                    // round (towards zero) at the sum's magnitude.
                                     mma_ts_tf32(d, a + kk * 8, kd + klo, p.idesc, kk > 0 ? 1u : 0u);
                                     mma_ts_tf32(d, a + p.Dp + kk * 8, kd, p.idesc, 1u);
-                                    mma_ts_tf32(d, a + kk * 8, kd, p.idesc, 1u);
                                 } else {
                                     mma_ts_f16(d, a + kk * 8, kd, p.idesc, kk > 0 ? 1u : 0u);
                                 }
                             }
+                            for (int kk = 0; TF && kk < p.ksteps; ++kk)
+                                mma_ts_tf32(d, a + kk * 8,
+                                            kdesc + (kk >> 2) * kstep + static_cast<uint32_t>((kk & 3) * 2),
+                                            p.idesc, 1u);
                             mma_commit(&bars->s_full[h]);
                             if (h == NQ - 1) mma_commit(&bars->kv_empty[st.idx]);
                         }
@@ -724,6 +728,8 @@ tc_gauss_fma_kernel(const __grid_constant__ CUtensorMap tm_q,
             const uint64_t a2_1 = f32x2_pack(am1, am1);
             const uint64_t c2 = f32x2_pack(p.c, p.c);
             const float s_min = -127.0f / p.c;   // exp2_fma_x2 range limit
+            const float s_close = kGuardClose / p.c;
+            unsigned close = 0;                  // sampled pairs of close points (see Guard)
             uint64_t acc0[C], acc1[C];
     #pragma unroll
             for (int cc = 0; cc < C; ++cc) acc0[cc] = acc1[cc] = 0ull;
@@ -886,6 +892,7 @@ tc_gauss_fma_kernel(const __grid_constant__ CUtensorMap tm_q,
                         // themselves, added to acc at its end, so that rounding
                         // grows with the keys of a tile plus the tiles, not with
                         // all keys.
+                        const int probe = (sg.kt0 + j) & 7;   // the sampled quad of keys
                         auto half = [&](const uint32_t (&r)[32], uint64_t a2, uint64_t (&acc)[C]) {
                             uint64_t sum[C];
         #pragma unroll
@@ -894,6 +901,11 @@ tc_gauss_fma_kernel(const __grid_constant__ CUtensorMap tm_q,
                             for (int t = 0; t < 8; ++t) {
                                 const float4* pr = reinterpret_cast<const float4*>(rec + t * (2 * REC_PAIR));
                                 const float4 bb = pr[0];
+                                if (t == probe) {
+        #pragma unroll
+                                    for (int e = 0; e < 4; ++e)
+                                        close += __uint_as_float(r[4 * t + e]) > s_close ? 1u : 0u;
+                                }
                                 uint64_t px[2];
         #pragma unroll
                                 for (int e = 0; e < 2; ++e) {
@@ -973,6 +985,12 @@ tc_gauss_fma_kernel(const __grid_constant__ CUtensorMap tm_q,
                 }
             };
             tile_loop(std::integral_constant<bool, VF == 1>{});
+            if (HALVES) {
+                close = __reduce_add_sync(0xffffffffu, close);
+                if (lane == 0 && close != 0u)
+                    atomicAdd(reinterpret_cast<unsigned long long*>(p.guard + 2),
+                              static_cast<unsigned long long>(close));
+            }
             // Fixed-order reduction of the NPART column-group partial sums.
             // (The reduction area of the previous segment has been read by
             // every warp: they met at its end.)
@@ -1068,6 +1086,7 @@ cudaError_t launch_typed(const TcPlan& pl, InType t, float c, char* ws, unsigned
     p.rec = reinterpret_cast<const float*>(ws + pl.off_rec);
     p.part = reinterpret_cast<float*>(ws + pl.off_part);
     p.status = status;
+    p.guard = pl.guard ? reinterpret_cast<unsigned*>(ws + pl.off_rec) + pl.Npad * (1 + pl.Cv) : nullptr;
     p.Mpad = pl.Mpad * pl.batch;   // partial-sum rows per contributor slot
     p.key_tiles = static_cast<int>(pl.Npad / BN);
     p.pairs_per_batch = static_cast<int>(pl.Mpad / (NQ * BM));
