@@ -49,8 +49,9 @@
  *    kernel's differences by a few 2^-24 of the exponent; within these limits
  *    both errors stay below 5e-7 of sum |v| Phi, which single-precision sums
  *    have anyway.  GS_PATH_SIMT takes the differences whatever the points.
- *    Their workspace holds both; where a caller's workspace, or the scratch of
- *    gauss_sum_noalloc, is too small for both, the SIMT kernel runs alone.
+ *    Their workspace holds both; where a caller's workspace, the scratch of
+ *    gauss_sum_noalloc, or the memory left on the device is too small for
+ *    both, the SIMT kernel runs alone.
  *  - On a non-OK return gauss_sum_last_error() describes the failure.
  */
 #ifndef GAUSS_SUM_H

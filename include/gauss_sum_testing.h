@@ -24,6 +24,11 @@ extern "C" {
 void gauss_sum_testing_fail_allocations(int on);
 
 /*
+ * The same for the next `count` workspace allocations only (0: none).
+ */
+void gauss_sum_testing_fail_next_allocations(int count);
+
+/*
  * Makes one bounded device-side wait of every launch of the fused FMA
  * kernel (C <= 4 forward) on the current device run out until the request
  * is cleared: control warp 0 of block 0 waits on a barrier that nothing

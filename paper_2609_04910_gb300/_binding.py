@@ -29,8 +29,8 @@ EXPORTS = (
     "gauss_sum_vjp", "gauss_sum_probe_ex2_mix_rate",
 )
 # Test hooks declared in include/gauss_sum_testing.h.
-TESTING_EXPORTS = ("gauss_sum_testing_fail_allocations", "gauss_sum_testing_request_stall",
-                   "gauss_sum_testing_last_fma_variant")
+TESTING_EXPORTS = ("gauss_sum_testing_fail_allocations", "gauss_sum_testing_fail_next_allocations",
+                   "gauss_sum_testing_request_stall", "gauss_sum_testing_last_fma_variant")
 
 # Bytes of the static scratch array behind gauss_sum_noalloc
 # (GS_NOALLOC_SCRATCH_BYTES in include/gauss_sum.h).
@@ -116,6 +116,8 @@ def _declare(lib):
     lib.gauss_sum_vjp.restype = f
     lib.gauss_sum_testing_fail_allocations.argtypes = [f]
     lib.gauss_sum_testing_fail_allocations.restype = None
+    lib.gauss_sum_testing_fail_next_allocations.argtypes = [f]
+    lib.gauss_sum_testing_fail_next_allocations.restype = None
     lib.gauss_sum_testing_request_stall.argtypes = [vp]
     lib.gauss_sum_testing_request_stall.restype = f
     lib.gauss_sum_testing_last_fma_variant.argtypes = []
@@ -373,6 +375,11 @@ def gauss_sum_kernel_launches() -> int:
 def testing_fail_allocations(on: bool) -> None:
     """Test hook: make the library's workspace allocations fail (or not)."""
     load_library().gauss_sum_testing_fail_allocations(1 if on else 0)
+
+
+def testing_fail_next_allocations(count: int) -> None:
+    """Test hook: make the library's next ``count`` workspace allocations fail."""
+    load_library().gauss_sum_testing_fail_next_allocations(int(count))
 
 
 def testing_last_fma_variant() -> int:

@@ -310,9 +310,15 @@ cudaError_t record_event(void* ev, cudaStream_t s) {
 
 // Test hook (gauss_sum_testing_fail_allocations): workspace allocations
 // fail.  A relaxed atomic load per allocating call; nothing else reads it.
+// Another hook (gauss_sum_testing_fail_next_allocations) lets the next few fail.
 std::atomic<int> g_fail_allocations{0};
+std::atomic<int> g_fail_next{0};
 
-bool forced_alloc_failure() { return g_fail_allocations.load(std::memory_order_relaxed) != 0; }
+bool forced_alloc_failure() {
+    if (g_fail_allocations.load(std::memory_order_relaxed) != 0) return true;
+    return g_fail_next.load(std::memory_order_relaxed) > 0 &&
+           g_fail_next.fetch_sub(1, std::memory_order_relaxed) > 0;
+}
 
 gs_status run(Call c) {
     // The first kernel of a call follows whatever the caller queued before.
@@ -375,8 +381,16 @@ gs_status run(Call c) {
         if (c.opt.workspace_bytes < bytes)
             return fail(GS_ERR_OUT_OF_MEMORY, "caller workspace is smaller than gauss_sum_workspace_size()");
     } else if (bytes > 0) {
-        if (forced_alloc_failure()) return fail(GS_ERR_OUT_OF_MEMORY, "workspace allocation failed (test hook)");
-        e = pool_alloc(reinterpret_cast<void**>(&ws), bytes, c.stream);
+        const bool forced = forced_alloc_failure();
+        e = forced ? cudaErrorMemoryAllocation : pool_alloc(reinterpret_cast<void**>(&ws), bytes, c.stream);
+        if (e == cudaErrorMemoryAllocation && tensor && tp.guard) {
+            // No room for both paths of a guarded sum: the SIMT kernel alone,
+            // as in a caller's workspace too small for both.
+            if (!forced) cudaGetLastError();
+            c.opt.path = GS_PATH_SIMT;
+            return run(c);
+        }
+        if (forced) return fail(GS_ERR_OUT_OF_MEMORY, "workspace allocation failed (test hook)");
         if (e != cudaSuccess) return cuda_fail(e, "workspace allocation");
         owned = true;
     }
@@ -963,6 +977,10 @@ int gauss_sum_testing_last_fma_variant(void) { return g_last_fma_variant.load(st
 
 void gauss_sum_testing_fail_allocations(int on) {
     g_fail_allocations.store(on ? 1 : 0, std::memory_order_relaxed);
+}
+
+void gauss_sum_testing_fail_next_allocations(int count) {
+    g_fail_next.store(count, std::memory_order_relaxed);
 }
 
 gs_status gauss_sum_testing_request_stall(void* stream) {
