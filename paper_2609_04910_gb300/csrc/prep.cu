@@ -1504,6 +1504,44 @@ __global__ void finalize_kernel(const float* __restrict__ part, int splits,
     out[idx] = acc * (inv_scale ? inv_scale[c] : 1.f);
 }
 
+// The same for many splits of few rows (the fp32 SIMT path: inv_scale null, one
+// contiguous M x Cv block of partials per split): one thread per output walked
+// up to 256 splits with most of the chip idle (513 x 8192, D = 16, C = 4: 17 us
+// of a 43 us call).  Here kFinalizeLanes threads share an output: thread y adds
+// splits y, y + kFinalizeLanes, ... in order, and thread 0 the sums in order.
+constexpr int kFinalizeLanes = 8;
+constexpr int kFinalizeManySplits = 16;
+
+__global__ void __launch_bounds__(32 * kFinalizeLanes)
+finalize_many_kernel(const float* __restrict__ part, int splits, int64_t total, float* __restrict__ out,
+                     const Guard guard) {
+    pdl_trigger();
+    pdl_wait();
+    if (guard.words && !guard_simt(guard)) return;
+    __shared__ float sums[kFinalizeLanes][32];
+    const int64_t idx = static_cast<int64_t>(blockIdx.x) * 32 + threadIdx.x;
+    float acc = 0.f;
+    if (idx < total) {
+        const float* p = part + threadIdx.y * total + idx;
+        const int64_t step = kFinalizeLanes * total;
+        int s = threadIdx.y;
+        for (; s + 7 * kFinalizeLanes < splits; s += 8 * kFinalizeLanes, p += 8 * step) {
+            float x[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) x[i] = p[i * step];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) acc += x[i];
+        }
+        for (; s < splits; s += kFinalizeLanes, p += step) acc += *p;
+    }
+    sums[threadIdx.y][threadIdx.x] = acc;
+    __syncthreads();
+    if (threadIdx.y != 0 || idx >= total) return;
+#pragma unroll
+    for (int y = 1; y < kFinalizeLanes; ++y) acc += sums[y][threadIdx.x];
+    out[idx] = acc;
+}
+
 // The same for Cv a multiple of 4 (part_ld is a multiple of 16): one thread
 // per quad of channels.  (Bound: HBM and load latency; 65536 rows of 64
 // channels, ncu: one thread per channel 26.0 us, quads 10.9.)
@@ -2531,6 +2569,13 @@ cudaError_t launch_finalize(const float* part, int splits, int64_t split_stride_
                             cudaStream_t s, int64_t main_rows, const Guard& guard) {
     const int64_t total = M * Cv;
     if (total == 0) return cudaSuccess;
+    if (splits >= kFinalizeManySplits && !inv_scale && main_rows == 0 && part_ld == Cv &&
+        split_stride_rows == M) {
+        launch_kernel(finalize_many_kernel, static_cast<unsigned>((total + 31) / 32), dim3(32, kFinalizeLanes), 0,
+                      s, part, splits, total, out, guard);
+        note_launches(1);
+        return cudaGetLastError();
+    }
     if (Cv % 4 == 0 && part_ld % 4 == 0 && !guard.words) {
         launch_kernel(finalize_quads_kernel,
                       static_cast<unsigned>((total / 4 + kFinalizeThreads - 1) / kFinalizeThreads),

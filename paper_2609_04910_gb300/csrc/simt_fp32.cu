@@ -24,7 +24,10 @@ namespace gs {
 namespace {
 
 constexpr int KT = 64;       // keys per shared-memory tile (gradient; forward: key_tile)
-constexpr int THREADS = 128; // threads per block (forward: or half of that, see plan_simt)
+constexpr int THREADS = 128; // threads per block (forward: or fewer, see plan_simt)
+// Partial sums of more than one split (16 MiB): the scratch of gauss_sum_noalloc
+// holds every call that it would hold unsplit.
+constexpr int64_t kMaxSplitFloats = int64_t(1) << 22;
 
 // ---------------------------------------------------------------- forward
 // Each thread holds ROWS = 4 query rows of up to 32 coordinates, so that one
@@ -40,7 +43,7 @@ constexpr int THREADS = 128; // threads per block (forward: or half of that, see
 // one.  Measured (one GB300, whole calls, C = 1, one row per thread in tiles
 // of 16, 32, 64 or 128 coordinates / this kernel): M = N = 16384, D = 4 435 /
 // 113 us, D = 16 435 / 296, D = 32 794 / 566, D = 48 1306 / 895, D = 64 1316
-// / 1144 (75 % of the lanes), D = 128 2919 / 2359; 4096^2, D = 16 39 / 31 us.
+// / 1144 (75 % of the lanes), D = 128 2919 / 2359; 4096^2, D = 16 39 / 27 us.
 constexpr int ROWS = 4;
 __host__ __device__ constexpr int lanes_per_group(int dmax) { return dmax <= 32 ? 1 : dmax <= 64 ? 2 : 4; }
 __host__ __device__ constexpr int key_tile(int dmax) { return dmax <= 64 ? 64 : 32; }
@@ -354,7 +357,7 @@ bool plan_simt(int64_t M, int64_t N, int64_t D, int64_t C, bool grad, int split_
         rows = THREADS / lanes_per_group(p->dmax) * ROWS;
         keys = key_tile(p->dmax);
     }
-    const int64_t chunks = grad ? 1 : (p->Cv + p->cblk - 1) / p->cblk;
+    const int64_t chunks = grad ? 1 : std::max<int64_t>(1, (p->Cv + p->cblk - 1) / p->cblk);
     int64_t blocks = (M + rows - 1) / rows * chunks;   // per key split
     p->threads = THREADS;
     const int64_t key_tiles = std::max<int64_t>(1, (N + keys - 1) / keys);
@@ -365,30 +368,41 @@ bool plan_simt(int64_t M, int64_t N, int64_t D, int64_t C, bool grad, int split_
         p->keys_per_split = grad ? (key_tiles + splits - 1) / splits * keys
                                  : std::max<int64_t>(4, ((N + splits - 1) / splits + 3) / 4 * 4);
     } else {
-        // The blocks of an SM share its fp32 lanes, so a call takes as long
-        // as the SM with the most keys: blocks per SM x (keys per block +
-        // about 48 keys' worth of start-up), with a single block per SM
-        // leaving its latencies exposed.  Tried: as many splits as give 1, 2,
-        // .. 16 blocks per SM, each of N / splits keys rounded up to 4, no
-        // fewer than 16; few splits win ties (fewer partial sums to add).
-        // Measured, 4096^2 pairs, D = 16: 1 and 2 blocks per SM (19 and 38
-        // splits) 30.5 us, 24, 32, 64 splits 39.7, 32.7, 36.9 us; 5800^2
-        // pairs, D = 32: one block per SM 124 us, three 95 us.
-        // And blocks of half the threads, where the rows of the last full-sized
-        // block would be mostly padding (1100 rows in blocks of 512).
+        // Threads per block and key splits by an estimate of the busiest SM's
+        // cycles, fitted to whole calls (one GB300, 216 shapes of 1 to 262144
+        // rows, 32 to 262144 keys, 4 to 100 coordinates, 1 and 4 channels,
+        // each with 33 choices; the estimate's choice is 2.8 % slower than the
+        // best one on average, at most 14 %).  A warp takes `key` issue cycles
+        // per key of its rows: coordinates, exponentials, values and its share
+        // of copying the key tile, which few threads per block make dear; an
+        // SMSP with fewer than two warps waits for latencies instead.  Each
+        // block costs a start, each split a partial sum to add.  Blocks of 128
+        // threads share the copies best; 64 and 32 (128 query rows up to 32
+        // coordinates) are for few rows, which full blocks would pad: 32 x
+        // 65536, D = 64, 256 splits of 64-thread blocks 67 us, 608 of 32
+        // threads 40.
+        const int L = lanes_per_group(p->dmax);
+        const double issue = 2.8 * (p->dmax / L) + 10.0 + 1.6 * 4 * p->cblk / L + (L > 1 ? 6.0 : 0.0);
+        const int64_t smem = 2 * keys * (p->dmax + p->cblk) * 4 + 1024;
         double best = 1e300;
-        for (int threads = THREADS; threads >= THREADS / 2; threads /= 2) {
+        for (int threads = THREADS; threads >= 32; threads /= 2) {
             const int64_t r = rows * threads / THREADS;
-            const double size = static_cast<double>(threads) / THREADS;
+            const double key = issue + 18.0 * (p->dmax + p->cblk) / threads;
+            const double warps = threads / 128.0;              // per SMSP and block
+            const int64_t fit = std::min<int64_t>(228 * 1024 / smem, min_blocks(p->dmax, p->cblk) * THREADS / threads);
             blocks = (M + r - 1) / r * chunks;
-            for (int64_t per = 1; per <= 16 * THREADS / threads; ++per) {
-                const int64_t want = std::min<int64_t>(256, std::max<int64_t>(1, per * sms / blocks));
+            for (int64_t per : {1, 2, 3, 4, 6, 8, 12, 16, 32}) {
+                const int64_t want = std::max<int64_t>(1, per * sms / blocks);
                 const int64_t kps = std::max<int64_t>(16, ((N + want - 1) / want + 3) / 4 * 4);
-                const int64_t per_sm = (blocks * ((N + kps - 1) / kps) + sms - 1) / sms;
-                // (A warp per SMSP and less take as long as a full block.)
-                const double share = std::max(1.0, per_sm * size);
-                const double cost = share * (kps + 48.0) * (share < 2 ? 1.3 : 1.0);
-                if (cost < best * 0.99) {
+                const int64_t n = (N + kps - 1) / kps;
+                if (n > 1 && n * M * p->Cv > kMaxSplitFloats) break;
+                const int64_t per_sm = (blocks * n + sms - 1) / sms;
+                const int64_t conc = std::min(per_sm, fit), rounds = per_sm / conc, rem = per_sm % conc;
+                auto cycles = [&](int64_t nb) {
+                    return nb == 0 ? 0.0 : std::max(nb * warps, 2.0) * key * kps + 620.0 * (1.0 + 0.22 * nb * warps);
+                };
+                const double cost = rounds * cycles(conc) + cycles(rem) + 6.3 * n;
+                if (cost < best * 0.995) {
                     best = cost;
                     p->keys_per_split = kps;
                     p->threads = threads;
