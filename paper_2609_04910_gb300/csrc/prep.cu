@@ -731,14 +731,22 @@ operand_kernel(const T* __restrict__ x, int64_t rows, int64_t rows_pad, int D, i
 // x^ = x - mu (fp32), hi = x^ rounded to tf32 and lo = (x^ - hi) rounded to
 // tf32, zero padded; q^.k^ is then hi.hi + hi.lo + lo.hi up to the dropped
 // lo.lo term (2^-22 relative).  nrm = -(c/2) ||x^||^2 from the fp32 x^;
-// rows in [rows, rows_pad) are zero with norm pad_value.  One warp per row,
-// over all problems of a batch.
-// Rows of job j0 (all problems), then of j1, in one launch.
-__global__ void tf32_split_kernel(const Tf32Job j0, const Tf32Job j1, int64_t total0, int64_t total_rows,
-                                  int D, int Dp, const float* __restrict__ mu, float half_c,
-                                  float pad_value, unsigned* __restrict__ guard) {
+// rows in [rows, rows_pad) are zero with norm pad_value.  Rows of job j0 (all
+// problems), then of j1, in one launch; rows_pad is a multiple of 128, so the
+// kSplitRows rows of a warp are of one problem and job.  Bound: HBM, but for
+// the loads' latency: one row per warp took 303 us for 2^20 rows of D = 32
+// (1.3 TB/s), with the job and problem worked out again for each.
+constexpr int kSplitRows = 8;
+constexpr int kSplitThreads = 256;
+
+template <int P>   // Dp = 32 P
+__global__ void __launch_bounds__(kSplitThreads)
+tf32_split_kernel(const Tf32Job j0, const Tf32Job j1, int64_t total0, int64_t total_rows, int D,
+                  const float* __restrict__ mu, float half_c, float pad_value,
+                  unsigned* __restrict__ guard) {
     pdl_trigger();
     pdl_wait();
+    constexpr int Dp = 32 * P;
     // guard: the largest (c/2) ||x - mu||^2, as the bits of a non-negative
     // float (or of a NaN, above them all), which order like the floats.
     __shared__ unsigned big;
@@ -746,32 +754,50 @@ __global__ void tf32_split_kernel(const Tf32Job j0, const Tf32Job j1, int64_t to
         if (threadIdx.x == 0) big = 0u;
         __syncthreads();
     }
-    const int64_t w = (static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
+    const int64_t w = ((static_cast<int64_t>(blockIdx.x) * kSplitThreads + threadIdx.x) >> 5) * kSplitRows;
     const int lane = threadIdx.x & 31;
     if (w < total_rows) {
         const bool second = w >= total0;
-        const Tf32Job j = second ? j1 : j0;
-        const int64_t i = second ? w - total0 : w;         // batch-stacked output row
-        const int64_t b = i / j.rows_pad;
-        const int64_t r = i - b * j.rows_pad;
-        const bool valid = r < j.rows;
-        const float* xr = j.x + (b * j.rows + r) * D;
-        const float* mb = mu ? mu + b * D : nullptr;
-        float* o = j.out + i * 2 * Dp;
-        float acc = 0.f;
-        for (int d = lane; d < Dp; d += 32) {
-            const float xv = (valid && d < D) ? xr[d] - (mb ? mb[d] : 0.f) : 0.f;
-            const float hi = round_tf32(xv);
-            o[d] = hi;
-            o[Dp + d] = round_tf32(xv - hi);
-            acc = fmaf(xv, xv, acc);
+        const float* x = second ? j1.x : j0.x;
+        float* out = second ? j1.out : j0.out;
+        float* nrm = second ? j1.nrm : j0.nrm;
+        const int64_t rows = second ? j1.rows : j0.rows, pad = second ? j1.rows_pad : j0.rows_pad;
+        const int64_t i0 = second ? w - total0 : w;        // first batch-stacked output row
+        const int64_t b = pad <= 0x7fffffff ? div_nonneg(i0, static_cast<int>(pad)) : i0 / pad;
+        const int64_t r0 = i0 - b * pad;
+        x += (b * rows + r0) * D + lane;
+        out += i0 * 2 * Dp + lane;
+        const int left = static_cast<int>(min(static_cast<int64_t>(kSplitRows), rows - r0));
+        float m[P], v[kSplitRows][P], acc[kSplitRows];
+#pragma unroll
+        for (int p = 0; p < P; ++p) m[p] = mu && lane + 32 * p < D ? mu[b * D + lane + 32 * p] : 0.f;
+#pragma unroll
+        for (int r = 0; r < kSplitRows; ++r)
+#pragma unroll
+            for (int p = 0; p < P; ++p)
+                v[r][p] = r < left && lane + 32 * p < D ? x[r * D + 32 * p] - m[p] : 0.f;
+#pragma unroll
+        for (int r = 0; r < kSplitRows; ++r) {
+            acc[r] = 0.f;
+#pragma unroll
+            for (int p = 0; p < P; ++p) {
+                const float hi = round_tf32(v[r][p]);
+                out[r * 2 * Dp + 32 * p] = hi;
+                out[r * 2 * Dp + Dp + 32 * p] = round_tf32(v[r][p] - hi);
+                acc[r] = fmaf(v[r][p], v[r][p], acc[r]);
+            }
         }
 #pragma unroll
-        for (int s = 16; s > 0; s >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, s);
-        if (lane == 0) {
-            j.nrm[i] = valid ? -half_c * acc : pad_value;
-            if (guard && valid) atomicMax(&big, __float_as_uint(half_c * acc) & 0x7fffffffu);
+        for (int s = 16; s > 0; s >>= 1)
+#pragma unroll
+            for (int r = 0; r < kSplitRows; ++r) acc[r] += __shfl_xor_sync(0xffffffffu, acc[r], s);
+        unsigned most = 0u;
+#pragma unroll
+        for (int r = 0; r < kSplitRows; ++r) {
+            if (lane == r) nrm[i0 + r] = r < left ? -half_c * acc[r] : pad_value;
+            if (r < left) most = max(most, __float_as_uint(half_c * acc[r]) & 0x7fffffffu);
         }
+        if (guard && lane == 0) atomicMax(&big, most);
     }
     if (guard) {
         __syncthreads();
@@ -2465,10 +2491,17 @@ cudaError_t launch_tf32_split(const Tf32Job& q, const Tf32Job* k, int D, int Dp,
     const int64_t total0 = q.rows_pad * batch;
     const int64_t total = total0 + (k ? k->rows_pad * batch : 0);
     if (total == 0) return cudaSuccess;
-    const int threads = 256;
-    const int64_t blocks = (total * 32 + threads - 1) / threads;
-    launch_kernel(tf32_split_kernel, static_cast<unsigned>(blocks), threads, 0, s, q, k ? *k : Tf32Job{},
-                  total0, total, D, Dp, mu, half_c, pad_value, guard);
+    if ((Dp != 32 && Dp != 64) || q.rows_pad % kSplitRows != 0 || (k && k->rows_pad % kSplitRows != 0))
+        return cudaErrorInvalidValue;
+    const int64_t warps = total / kSplitRows;
+    const unsigned blocks = static_cast<unsigned>((warps * 32 + kSplitThreads - 1) / kSplitThreads);
+    const Tf32Job jk = k ? *k : Tf32Job{};
+    if (Dp == 32)
+        launch_kernel(tf32_split_kernel<1>, blocks, kSplitThreads, 0, s, q, jk, total0, total, D, mu, half_c,
+                      pad_value, guard);
+    else
+        launch_kernel(tf32_split_kernel<2>, blocks, kSplitThreads, 0, s, q, jk, total0, total, D, mu, half_c,
+                      pad_value, guard);
     note_launches(1);
     return cudaGetLastError();
 }
