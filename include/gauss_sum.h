@@ -39,8 +39,9 @@
  *    with three tf32 MMAs per product (q^ k^T ~ hi.hi + hi.lo + lo.hi of the
  *    tf32 splits x = hi + lo, fp32-level accuracy): chosen automatically
  *    from 2^25 pairs (per call, summed over a batch; single problems with
- *    D <= 4 from 2^26), or forced with GS_PATH_TENSOR / GS_PATH_SIMT.  Single
- *    forward sums with C <= 4 and 32 < D <= 64 from 2^24 pairs launch both: a
+ *    D <= 4 from 2^26, q = k from 3 2^24), or forced with GS_PATH_TENSOR /
+ *    GS_PATH_SIMT.  Single forward sums with C <= 4 and 32 < D <= 64 from 2^24
+ *    pairs, unless they have few queries or few keys, launch both: a
  *    look at the points on the device lets the tensor cores' sums count only
  *    where every (tau/2) log2(e) ||x - mean||^2 is at most 2 and at most one
  *    pair in 256 is close compared with its norms (tau log2(e)

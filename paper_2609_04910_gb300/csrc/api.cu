@@ -208,8 +208,10 @@ gs::InType in_type(gs_dtype d) {
 // distances are cheap on the SIMT kernel (it works in register tiles of 4, 8,
 // 16, .. coordinates), from 2^26.  Measured on a GB300, C = 1, whole calls,
 // SIMT / tensor cores: 5800^2 pairs D = 4 24 / 35 us, 18684 x 2500, D = 7 37 /
-// 35 us, 5800^2, D = 16 50 / 37 us; 16384^2 pairs D = 4 113 / 70 us, D = 8
-// 172 / 70 us, D = 16 296 / 74 us.
+// 31 us, 5800^2, D = 16 50 / 37 us; 16384^2 pairs D = 4 113 / 70 us, D = 8
+// 172 / 70 us, D = 16 296 / 74 us.  One cloud against itself (q is k), whose
+// operands are written once, from 3 x 2^24 pairs for D <= 4: MMD^2 of 8000
+// points, D = 3 41.5 / 39.2 us.
 // Batches keep 2^25 for every D: the tensor-core path runs them in one
 // launch of each kernel, the SIMT kernel problem by problem.
 constexpr int64_t kFp32TensorMinPairs = int64_t(1) << 25;
@@ -217,7 +219,10 @@ constexpr int64_t kFp32TensorMinPairs = int64_t(1) << 25;
 bool fp32_on_tensor_cores(const Call& c) {
     if (c.opt.path == GS_PATH_TENSOR) return true;
     if (c.opt.path != GS_PATH_AUTO) return false;
-    const int64_t least = c.B > 1 || c.D > 4 ? kFp32TensorMinPairs : 2 * kFp32TensorMinPairs;
+    const bool alias = c.q == c.k && c.M == c.N;
+    const int64_t least = c.B > 1 || c.D > 4 ? kFp32TensorMinPairs
+                          : alias            ? kFp32TensorMinPairs * 3 / 2
+                                             : kFp32TensorMinPairs * 2;
     return !c.grad && c.C <= gs::kFmaMaxChannels && c.D <= gs::kTf32MaxDp &&
            c.B * c.M * c.N >= least;
 }
@@ -227,8 +232,8 @@ bool fp32_on_tensor_cores(const Call& c) {
 // the device decides whose sums count (see Guard in internal.h).  From 2^24
 // pairs, where its extra launches are repaid.
 // Measured on a GB300, whole calls, SIMT / guarded: 16384^2, D = 64, C = 1
-// 1145 / 140 us (the tensor cores' share of the work at three tf32 MMAs per
-// product is 80 us), 8192^2, D = 50 305 / 66 us, 6000^2, D = 64 176 / 57 us.
+// 1145 / 150 us (the tensor cores' share of the work at three tf32 MMAs per
+// product is 80 us), 8192^2, D = 50 289 / 64 us, 5800^2, D = 64 154 / 53 us.
 // Error against 64 bits at 8192^2, D = 33 to 64 (guarded / SIMT kernel): N(0, I)
 // points and values, relative 2-norm 1.0e-7 to 2.5e-7 / 1.3e-7 to 3.7e-7; two
 // clusters with norm terms of 0.4 to 2, largest error relative to the sum of
@@ -236,22 +241,36 @@ bool fp32_on_tensor_cores(const Call& c) {
 constexpr int64_t kFp32GuardedMinPairs = int64_t(1) << 24;
 
 bool fp32_guarded(const Call& c) {
-    return c.dtype == GS_FP32 && c.opt.path == GS_PATH_AUTO && !c.grad && c.B == 1 &&
-           c.C <= gs::kFmaMaxChannels && c.D > gs::kTf32MaxDp && c.D <= gs::kTf32WideMaxDp &&
-           c.M * c.N >= kFp32GuardedMinPairs;
+    return c.dtype == GS_FP32 && c.opt.path == GS_PATH_AUTO && c.opt.split_n == 0 && c.opt.exp2_fma == 0 &&
+           !c.grad && c.B == 1 && c.C <= gs::kFmaMaxChannels && c.D > gs::kTf32MaxDp &&
+           c.D <= gs::kTf32WideMaxDp && c.M * c.N >= kFp32GuardedMinPairs;
+}
+
+// Whether a call that may be guarded is: the SIMT kernel's estimated time has to
+// be several times what the guard's launches cost a call that it then does
+// after all, about 15 us and 0.17 us per 1000 points (2^20 x 32 points 170 us).
+// With these factors such calls take about as long as on the SIMT kernel of one
+// row per thread whose place the pair of paths took (its width tile of 64
+// coordinates gained least, so the factors depend on D): left to the SIMT kernel
+// by the guard, 4096^2, D = 64 98 us (107 before), 4100 x 4500 113 (108), 5800^2,
+// D = 50 173 (158), 8192^2, D = 64 300 (347).  Few keys or few queries stay with
+// the SIMT kernel: 2^20 x 32, D = 48 118 us alone, 518 guarded.
+bool guard_pays(const Call& c, double simt_micros) {
+    const double launches = 15.0 + 0.17e-3 * static_cast<double>(c.M + c.N);
+    return simt_micros >= (c.D <= 48 ? 3.0 : c.D <= 56 ? 8.0 : 4.2) * launches;
 }
 
 // Plans the call; returns GS_OK and the workspace size, or an error.
 gs_status plan(const Call& c, int sms, bool* tensor, gs::TcPlan* tp, gs::SimtPlan* sp,
                size_t* bytes) {
     const char* why = "unsupported shape";
-    if (fp32_guarded(c) && c.opt.split_n == 0 && c.opt.exp2_fma == 0) {
+    if (fp32_guarded(c)) {
         // The guarded pair of paths, unless a caller's workspace holds only
         // what the SIMT path needs.
         const bool alias = c.q == c.k && c.M == c.N && c.q != nullptr;
-        if (gs::plan_tensor(gs::InType::F32, c.M, c.N, c.D, c.C, false, c.opt.center != 0, alias, 0,
-                            sms, tp, &why) &&
-            gs::plan_simt(c.M, c.N, c.D, c.C, false, 0, sms, sp, &why)) {
+        if (gs::plan_simt(c.M, c.N, c.D, c.C, false, 0, sms, sp, &why) && guard_pays(c, sp->micros) &&
+            gs::plan_tensor(gs::InType::F32, c.M, c.N, c.D, c.C, false, c.opt.center != 0, alias, 0,
+                            sms, tp, &why)) {
             sp->off_part = tp->total;
             *bytes = tp->total + sp->total;
             if (!c.opt.workspace || c.opt.workspace_bytes >= *bytes) {
@@ -459,8 +478,11 @@ gs_status run(Call c) {
             const gs::Tf32Job jk = {static_cast<const float*>(c.k), c.N, tp.Npad,
                                     reinterpret_cast<float*>(ws + tp.off_kh),
                                     reinterpret_cast<float*>(ws + tp.off_B)};
+            const gs::RecordArgs rec = {c.v, true, c.N, tp.Npad, static_cast<int>(tp.Cv),
+                                        reinterpret_cast<float*>(ws + tp.off_rec), false};
             e = gs::launch_tf32_split(jq, tp.alias ? nullptr : &jk, static_cast<int>(c.D), tp.Dp, mu,
-                                      half_c, ninf, c.stream, batch, guard.words);
+                                      half_c, ninf, c.stream, batch, guard.words, rec);
+            records_done = true;
             where = "tf32 split kernel";
         } else {
             // Centred, rounded operands of q and (unless q is k) k in one
@@ -504,7 +526,11 @@ gs_status run(Call c) {
                 where = "fused tensor-core kernel";
             }
             if (e == cudaSuccess && guard.words) {
-                // The other side of the guard.
+                // The other side of the guard.  Launched once the fused kernel
+                // has ended: blocks that start as its blocks leave pile up on
+                // the first free SMs (8192^2, D = 64, left to the SIMT kernel:
+                // 486 us).
+                gs::pdl_reset();
                 e = gs::launch_simt(sp, false, static_cast<const float*>(c.q),
                                     static_cast<const float*>(c.k), static_cast<const float*>(c.v),
                                     static_cast<int>(c.C), 0, half_c,
@@ -521,17 +547,16 @@ gs_status run(Call c) {
                                               c.mmd_part, c.mmd_out, c.stream, batch, fixed,
                                               tp.tri ? kt : 0);
                     *c.mmd_done = true;
+                } else if (guard.words) {
+                    e = gs::launch_finalize_guarded(part, tp.Mpad, c.M, static_cast<int>(tp.Cv), 128 * tp.nq, kt,
+                                                    tp.unit_len, fixed,
+                                                    reinterpret_cast<float*>(ws + sp.off_part), sp.splits,
+                                                    c.out, c.stream, guard);
                 } else {
                     e = gs::launch_finalize_slots(part, tp.Mpad, c.M, static_cast<int>(tp.Cv), 128 * tp.nq,
                                                   kt, tp.unit_len, c.out, c.stream, batch, fixed,
-                                                  tp.tri ? kt : 0, guard);
+                                                  tp.tri ? kt : 0);
                 }
-                where = "finalise kernel";
-            }
-            if (e == cudaSuccess && guard.words) {
-                e = gs::launch_finalize(reinterpret_cast<float*>(ws + sp.off_part), sp.splits, c.M, c.M,
-                                        static_cast<int>(sp.Cv), static_cast<int>(sp.Cv), nullptr, c.out,
-                                        c.stream, 0, guard);
                 where = "finalise kernel";
             }
         } else if (e == cudaSuccess) {

@@ -167,11 +167,13 @@ struct TcPlan {
 
 struct SimtPlan {
     int64_t M, N, D, Cv;
-    int dmax;          // register tile of the query row (16, 32, 64 or 128)
+    int dmax;          // register tile of the query row (forward: 4, 8, 16, 24, 32, 48, 64 or
+                       // 128 coordinates; gradient: 16, 32 or 64)
     int cblk;          // channels per launch slice
     int threads;       // threads per block of the forward kernel
     int splits;
     int64_t keys_per_split;
+    double micros;     // estimated time of a forward call in microseconds
     size_t off_part, total;
 };
 
@@ -264,8 +266,12 @@ cudaError_t launch_weight_prep(InType t, const void* rsrc, bool r_f32, int64_t R
 // in split order; rows below main_rows have one split.
 cudaError_t launch_finalize(const float* part, int splits, int64_t split_stride_rows,
                             int64_t M, int Cv, int part_ld, const float* inv_scale, float* out,
-                            cudaStream_t s, int64_t main_rows = 0,
-                            const Guard& guard = {});
+                            cudaStream_t s, int64_t main_rows = 0);
+// Guarded sums: the splits of the SIMT path or the slots of the FMA kernel,
+// arguments as launch_finalize and launch_finalize_slots.
+cudaError_t launch_finalize_guarded(const float* part, int64_t Mpad, int64_t M, int C, int rows_per_unit,
+                                    int64_t key_tiles, int64_t unit_len, int fixed_slots, const float* simt,
+                                    int simt_splits, float* out, cudaStream_t s, const Guard& guard);
 // Gradient contraction of one launch's channels ch0 .. ch0 + Cc - 1 (see
 // prep.cu): out[m, d] (+)= tau sum_c u[m, c] (S_{c,d} - x^_{m,d} S_{c,D}),
 // s_out[m, c] = S_{c,D}.  direct: fp32 kernel partials (difference form).
@@ -297,8 +303,7 @@ cudaError_t launch_mmd2_slots(InType t, const float* part, int64_t Mpad, int64_t
 cudaError_t launch_finalize_slots(const float* part, int64_t Mpad, int64_t M, int C,
                                   int rows_per_unit, int64_t key_tiles, int64_t unit_len,
                                   float* out, cudaStream_t s, int batch = 1,
-                                  int fixed_slots = 0, int64_t tri_key_tiles = 0,
-                                  const Guard& guard = {});
+                                  int fixed_slots = 0, int64_t tri_key_tiles = 0);
 
 // simt_fp32.cu ---------------------------------------------------------
 // grad: keys weighted by channel wch of v (N x Cw); partials have D + 1
@@ -314,7 +319,8 @@ cudaError_t launch_key_records(InType t, const void* v, const float* B, int64_t 
                                int C, float* rec, cudaStream_t s, int batch = 1, bool signs = false);
 // 3xTF32 operands of fp32 inputs (see prep.cu): rows of 2 Dp floats
 // [hi | lo] into out, nrm = -(c/2)||x - mu||^2 (pad_value for padded rows), of
-// q and, unless q is k, of k; guard takes the bits of the largest -nrm.
+// q and, unless q is k, of k; guard takes the bits of the largest -nrm; rec:
+// the key records with B, in the same launch.
 struct Tf32Job {
     const float* x;          // batch x rows x D
     int64_t rows, rows_pad;
@@ -323,7 +329,7 @@ struct Tf32Job {
 };
 cudaError_t launch_tf32_split(const Tf32Job& q, const Tf32Job* k, int D, int Dp, const float* mu,
                               float half_c, float pad_value, cudaStream_t s, int batch,
-                              unsigned* guard);
+                              unsigned* guard, const RecordArgs& rec);
 constexpr int aug_norm_terms(InType t) { return t == InType::BF16 ? 3 : 2; }
 
 // tc_gauss.cu ----------------------------------------------------------

@@ -735,7 +735,8 @@ operand_kernel(const T* __restrict__ x, int64_t rows, int64_t rows_pad, int D, i
 // problems), then of j1, in one launch; rows_pad is a multiple of 128, so the
 // kSplitRows rows of a warp are of one problem and job.  Bound: HBM, but for
 // the loads' latency: one row per warp took 303 us for 2^20 rows of D = 32
-// (1.3 TB/s), with the job and problem worked out again for each.
+// (1.3 TB/s), with the job and problem worked out again for each; whole call
+// (32 keys) 448 -> 263 us.  The key records ride along.
 constexpr int kSplitRows = 8;
 constexpr int kSplitThreads = 256;
 
@@ -743,7 +744,7 @@ template <int P>   // Dp = 32 P
 __global__ void __launch_bounds__(kSplitThreads)
 tf32_split_kernel(const Tf32Job j0, const Tf32Job j1, int64_t total0, int64_t total_rows, int D,
                   const float* __restrict__ mu, float half_c, float pad_value,
-                  unsigned* __restrict__ guard) {
+                  unsigned* __restrict__ guard, const RecordJob<float> rec) {
     pdl_trigger();
     pdl_wait();
     constexpr int Dp = 32 * P;
@@ -792,12 +793,27 @@ tf32_split_kernel(const Tf32Job j0, const Tf32Job j1, int64_t total0, int64_t to
 #pragma unroll
             for (int r = 0; r < kSplitRows; ++r) acc[r] += __shfl_xor_sync(0xffffffffu, acc[r], s);
         unsigned most = 0u;
+        float norm = 0.f;                                  // of row i0 + lane
 #pragma unroll
         for (int r = 0; r < kSplitRows; ++r) {
-            if (lane == r) nrm[i0 + r] = r < left ? -half_c * acc[r] : pad_value;
+            if (lane == r) norm = r < left ? -half_c * acc[r] : pad_value;
             if (r < left) most = max(most, __float_as_uint(half_c * acc[r]) & 0x7fffffffu);
         }
+        if (lane < kSplitRows) nrm[i0 + lane] = norm;
         if (guard && lane == 0) atomicMax(&big, most);
+        if (second || j1.x == nullptr) {
+            // Keys: their records (quads, see key_record_kernel), of which B are
+            // the norm terms; kSplitRows / 4 quads of 1 + C groups of four floats.
+            float* q = rec.rec + (i0 >> 2) * (4 + 4 * rec.C);
+            const int items = (1 + rec.C) * kSplitRows;
+            for (int t0 = 0; t0 < items; t0 += 32) {
+                const int t = t0 + lane;
+                const int quad = t / (4 + 4 * rec.C), e = t - quad * (4 + 4 * rec.C);
+                const int r = 4 * quad + (e & 3), c = (e >> 2) - 1;
+                const float B = __shfl_sync(0xffffffffu, norm, r);
+                if (t < items) q[t] = c < 0 ? B : r < left ? rec.v[(b * rows + r0 + r) * rec.C + c] : 0.f;
+            }
+        }
     }
     if (guard) {
         __syncthreads();
@@ -826,11 +842,9 @@ __device__ __forceinline__ int64_t contributor_slots(int64_t r, int fixed_slots,
 __global__ void finalize_slots_kernel(const float* __restrict__ part, int64_t Mpad, int64_t M,
                                       int C, int rows_per_unit, int64_t key_tiles,
                                       int64_t unit_len, int64_t batch, int fixed_slots,
-                                      int64_t tri_kt, float* __restrict__ out,
-                                      const Guard guard) {
+                                      int64_t tri_kt, float* __restrict__ out) {
     pdl_trigger();
     pdl_wait();
-    if (guard.words && guard_simt(guard)) return;
     // out: batch x M x C; partial rows are batch-stacked with Mpad rows per
     // problem and batch Mpad rows per slot.
     const int64_t idx = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
@@ -1504,10 +1518,9 @@ weight_prep_kernel(const TR* __restrict__ rsrc, int64_t R, int64_t Rpad,
 __global__ void finalize_kernel(const float* __restrict__ part, int splits,
                                 int64_t split_stride_rows, int64_t M, int Cv, int part_ld,
                                 const float* __restrict__ inv_scale, float* __restrict__ out,
-                                int64_t main_rows, const Guard guard) {
+                                int64_t main_rows) {
     pdl_trigger();
     pdl_wait();
-    if (guard.words && !guard_simt(guard)) return;
     const int64_t idx = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
     if (idx >= M * Cv) return;
     const int64_t m = div_nonneg(idx, Cv);
@@ -1538,34 +1551,72 @@ __global__ void finalize_kernel(const float* __restrict__ part, int splits,
 constexpr int kFinalizeLanes = 8;
 constexpr int kFinalizeManySplits = 16;
 
-__global__ void __launch_bounds__(32 * kFinalizeLanes)
-finalize_many_kernel(const float* __restrict__ part, int splits, int64_t total, float* __restrict__ out,
-                     const Guard guard) {
-    pdl_trigger();
-    pdl_wait();
-    if (guard.words && !guard_simt(guard)) return;
+// p[0], p[stride], .. (n of them) added up by the block's column of threads
+// threadIdx.x, into the return value of thread y = 0; fewer than
+// kFinalizeManySplits in order by that thread, as finalize_kernel adds them.
+// Every thread of the block calls this (n <= 0: none).
+__device__ __forceinline__ float sum_lanes(const float* __restrict__ p, int64_t stride, int n) {
     __shared__ float sums[kFinalizeLanes][32];
-    const int64_t idx = static_cast<int64_t>(blockIdx.x) * 32 + threadIdx.x;
+    const int lanes = n < kFinalizeManySplits ? 1 : kFinalizeLanes;
     float acc = 0.f;
-    if (idx < total) {
-        const float* p = part + threadIdx.y * total + idx;
-        const int64_t step = kFinalizeLanes * total;
-        int s = threadIdx.y;
-        for (; s + 7 * kFinalizeLanes < splits; s += 8 * kFinalizeLanes, p += 8 * step) {
+    int s = static_cast<int>(threadIdx.y);
+    if (s < lanes) {
+        p += s * stride;
+        const int64_t step = lanes * stride;
+        for (; s + 7 * lanes < n; s += 8 * lanes, p += 8 * step) {
             float x[8];
 #pragma unroll
             for (int i = 0; i < 8; ++i) x[i] = p[i * step];
 #pragma unroll
             for (int i = 0; i < 8; ++i) acc += x[i];
         }
-        for (; s < splits; s += kFinalizeLanes, p += step) acc += *p;
+        for (; s < n; s += lanes, p += step) acc += *p;
     }
     sums[threadIdx.y][threadIdx.x] = acc;
     __syncthreads();
-    if (threadIdx.y != 0 || idx >= total) return;
+    if (threadIdx.y == 0 && lanes > 1) {
 #pragma unroll
-    for (int y = 1; y < kFinalizeLanes; ++y) acc += sums[y][threadIdx.x];
-    out[idx] = acc;
+        for (int y = 1; y < kFinalizeLanes; ++y) acc += sums[y][threadIdx.x];
+    }
+    return acc;
+}
+
+__global__ void __launch_bounds__(32 * kFinalizeLanes)
+finalize_many_kernel(const float* __restrict__ part, int splits, int64_t total, float* __restrict__ out) {
+    pdl_trigger();
+    pdl_wait();
+    const int64_t idx = static_cast<int64_t>(blockIdx.x) * 32 + threadIdx.x;
+    const float sum = sum_lanes(part + idx, total, idx < total ? splits : 0);
+    if (threadIdx.y == 0 && idx < total) out[idx] = sum;
+}
+
+// Guarded sums of one problem (see Guard): the SIMT path's splits (simt,
+// simt_splits), or the FMA kernel's contributor slots as in
+// finalize_slots_kernel.
+__global__ void __launch_bounds__(32 * kFinalizeLanes)
+finalize_guarded_kernel(const float* __restrict__ part, int64_t Mpad, int64_t M, int C, int rows_per_unit,
+                        int64_t key_tiles, int64_t unit_len, int fixed_slots,
+                        const float* __restrict__ simt, int simt_splits, float* __restrict__ out,
+                        const Guard guard) {
+    pdl_trigger();
+    pdl_wait();
+    const int64_t total = M * C;
+    const int64_t idx = static_cast<int64_t>(blockIdx.x) * 32 + threadIdx.x;
+    const float* p = simt + idx;
+    int64_t stride = total;
+    int n = 0;
+    if (idx < total) {
+        if (guard_simt(guard)) {
+            n = simt_splits;
+        } else {
+            n = static_cast<int>(contributor_slots(div_nonneg(idx, C) / rows_per_unit, fixed_slots, key_tiles,
+                                                   unit_len, 0));
+            p = part + idx;
+            stride = Mpad * C;
+        }
+    }
+    const float sum = sum_lanes(p, stride, n);
+    if (threadIdx.y == 0 && idx < total) out[idx] = sum;
 }
 
 // The same for Cv a multiple of 4 (part_ld is a multiple of 16): one thread
@@ -2351,13 +2402,13 @@ cudaError_t launch_mmd2_slots(InType t, const float* part, int64_t Mpad, int64_t
 cudaError_t launch_finalize_slots(const float* part, int64_t Mpad, int64_t M, int C,
                                   int rows_per_unit, int64_t key_tiles, int64_t unit_len,
                                   float* out, cudaStream_t s, int batch, int fixed_slots,
-                                  int64_t tri_key_tiles, const Guard& guard) {
+                                  int64_t tri_key_tiles) {
     const int64_t total = static_cast<int64_t>(batch) * M * C;
     if (total == 0) return cudaSuccess;
     const int threads = 256;
     launch_kernel(finalize_slots_kernel, static_cast<unsigned>((total + threads - 1) / threads), threads, 0, s, 
         part, Mpad, M, C, rows_per_unit, key_tiles, unit_len, static_cast<int64_t>(batch),
-        fixed_slots, tri_key_tiles, out, guard);
+        fixed_slots, tri_key_tiles, out);
     note_launches(1);
     return cudaGetLastError();
 }
@@ -2487,7 +2538,8 @@ cudaError_t launch_prep_cluster(InType t, bool aug, const void* q, int64_t M, in
 
 cudaError_t launch_tf32_split(const Tf32Job& q, const Tf32Job* k, int D, int Dp, const float* mu,
                               float half_c, float pad_value, cudaStream_t s, int batch,
-                              unsigned* guard) {
+                              unsigned* guard, const RecordArgs& rec) {
+    const RecordJob<float> rj = {static_cast<const float*>(rec.v), rec.N, rec.Npad / 2, rec.C, rec.out, false};
     const int64_t total0 = q.rows_pad * batch;
     const int64_t total = total0 + (k ? k->rows_pad * batch : 0);
     if (total == 0) return cudaSuccess;
@@ -2498,10 +2550,10 @@ cudaError_t launch_tf32_split(const Tf32Job& q, const Tf32Job* k, int D, int Dp,
     const Tf32Job jk = k ? *k : Tf32Job{};
     if (Dp == 32)
         launch_kernel(tf32_split_kernel<1>, blocks, kSplitThreads, 0, s, q, jk, total0, total, D, mu, half_c,
-                      pad_value, guard);
+                      pad_value, guard, rj);
     else
         launch_kernel(tf32_split_kernel<2>, blocks, kSplitThreads, 0, s, q, jk, total0, total, D, mu, half_c,
-                      pad_value, guard);
+                      pad_value, guard, rj);
     note_launches(1);
     return cudaGetLastError();
 }
@@ -2599,17 +2651,17 @@ cudaError_t launch_weight_prep(InType t, const void* rsrc, bool r_f32, int64_t R
 
 cudaError_t launch_finalize(const float* part, int splits, int64_t split_stride_rows,
                             int64_t M, int Cv, int part_ld, const float* inv_scale, float* out,
-                            cudaStream_t s, int64_t main_rows, const Guard& guard) {
+                            cudaStream_t s, int64_t main_rows) {
     const int64_t total = M * Cv;
     if (total == 0) return cudaSuccess;
     if (splits >= kFinalizeManySplits && !inv_scale && main_rows == 0 && part_ld == Cv &&
         split_stride_rows == M) {
         launch_kernel(finalize_many_kernel, static_cast<unsigned>((total + 31) / 32), dim3(32, kFinalizeLanes), 0,
-                      s, part, splits, total, out, guard);
+                      s, part, splits, total, out);
         note_launches(1);
         return cudaGetLastError();
     }
-    if (Cv % 4 == 0 && part_ld % 4 == 0 && !guard.words) {
+    if (Cv % 4 == 0 && part_ld % 4 == 0) {
         launch_kernel(finalize_quads_kernel,
                       static_cast<unsigned>((total / 4 + kFinalizeThreads - 1) / kFinalizeThreads),
                       kFinalizeThreads, 0, s, part, splits, split_stride_rows, M, Cv, part_ld, inv_scale, out, main_rows);
@@ -2619,7 +2671,18 @@ cudaError_t launch_finalize(const float* part, int splits, int64_t split_stride_
     const int threads = 256;
     const int64_t blocks = (total + threads - 1) / threads;
     launch_kernel(finalize_kernel, static_cast<unsigned>(blocks), threads, 0, s, 
-        part, splits, split_stride_rows, M, Cv, part_ld, inv_scale, out, main_rows, guard);
+        part, splits, split_stride_rows, M, Cv, part_ld, inv_scale, out, main_rows);
+    note_launches(1);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_finalize_guarded(const float* part, int64_t Mpad, int64_t M, int C, int rows_per_unit,
+                                    int64_t key_tiles, int64_t unit_len, int fixed_slots, const float* simt,
+                                    int simt_splits, float* out, cudaStream_t s, const Guard& guard) {
+    const int64_t total = M * C;
+    if (total == 0) return cudaSuccess;
+    launch_kernel(finalize_guarded_kernel, static_cast<unsigned>((total + 31) / 32), dim3(32, kFinalizeLanes), 0, s,
+                  part, Mpad, M, C, rows_per_unit, key_tiles, unit_len, fixed_slots, simt, simt_splits, out, guard);
     note_launches(1);
     return cudaGetLastError();
 }

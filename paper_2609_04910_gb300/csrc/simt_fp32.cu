@@ -344,6 +344,7 @@ bool plan_simt(int64_t M, int64_t N, int64_t D, int64_t C, bool grad, int split_
         *why = grad ? "fp32 gradient supports D <= 64" : "fp32 path supports D <= 128";
         return false;
     }
+    p->micros = 0.0;
     p->cblk = p->Cv >= 3 ? 4 : static_cast<int>(std::max<int64_t>(1, p->Cv));
     int64_t rows, keys;   // query rows per block, keys per shared-memory tile
     if (grad) {
@@ -409,6 +410,8 @@ bool plan_simt(int64_t M, int64_t N, int64_t D, int64_t C, bool grad, int split_
                 }
             }
         }
+        // (Measured, D = 48 and 64: 630 to 830 of these cycles in a microsecond.)
+        p->micros = best / 720.0 + 5.0;
     }
     p->splits = static_cast<int>((N + p->keys_per_split - 1) / p->keys_per_split);
     if (p->splits < 1) p->splits = 1;
