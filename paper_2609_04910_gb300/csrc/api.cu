@@ -956,6 +956,15 @@ size_t gauss_sum_workspace_size(int64_t M, int64_t N, int64_t D, int64_t C, gs_d
     gs::SimtPlan sp{};
     size_t bytes = 0;
     if (plan(c, sms, &tensor, &tp, &sp, &bytes) != GS_OK) return static_cast<size_t>(-1);
+    if (M == N) {
+        // One cloud with itself needs less on the same path, but may take the
+        // tensor cores where two clouds do not (fp32_on_tensor_cores).
+        size_t alias = 0;
+        c.k = c.q;
+        tp = gs::TcPlan{};
+        if (plan(c, sms, &tensor, &tp, &sp, &alias) != GS_OK) return static_cast<size_t>(-1);
+        bytes = std::max(bytes, alias);
+    }
     return bytes;
 }
 

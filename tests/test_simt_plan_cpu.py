@@ -23,3 +23,10 @@ def test_no_channels(D):
 def test_split_sums_stay_small(M, N, D, C):
     need = gs.gauss_sum_workspace_size(M, N, D, C, gs.GS_FP32, path=gs.GS_PATH_SIMT)
     assert 0 < need <= max(16 << 20, 4 * M * C + 1023)
+
+
+@pytest.mark.parametrize("N,more", [(7093, False), (7095, True), (8191, True)])
+def test_one_cloud_may_need_the_tensor_cores_workspace(N, more):
+    need = gs.gauss_sum_workspace_size(N, N, 3, 1, gs.GS_FP32)
+    simt = gs.gauss_sum_workspace_size(N, N, 3, 1, gs.GS_FP32, path=gs.GS_PATH_SIMT)
+    assert (need > simt) == more

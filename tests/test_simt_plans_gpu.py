@@ -46,3 +46,17 @@ def test_shapes(M, N, D, C):
 @pytest.mark.parametrize("M,C", [(1, 1), (31, 3), (257, 4)])
 def test_splits(splits, M, C):
     _check(M, 6400, 20, C, split_n=splits)
+
+
+@pytest.mark.parametrize("N", [7093, 7094, 8191, 8192])
+@pytest.mark.parametrize("D", [2, 4])
+def test_workspace_serves_one_cloud_and_two(N, D):
+    """Sums of one cloud with itself change paths at another size than sums of
+    two clouds; the workspace asked for holds either."""
+    import paper_2609_04910_gb300 as gs
+    inp = generate(case(N, N, D, 1, "fp32"), seed=32)
+    q, k, v = device_inputs(inp)
+    ws = torch.empty(gs.gauss_sum_workspace_size(N, N, D, 1, gs.GS_FP32), dtype=torch.uint8, device="cuda")
+    for a in (k, q):
+        assert torch.equal(gs.gauss_sum(a, k, v, 1.0 / D, workspace=ws), gs.gauss_sum(a, k, v, 1.0 / D))
+        gs.gauss_sum_noalloc(a, k, v, 1.0 / D)
