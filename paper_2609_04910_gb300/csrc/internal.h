@@ -345,7 +345,9 @@ constexpr int kAugMaxDp = 128;
 // D of the one that keeps them in tensor memory.
 constexpr int kTf32MaxDp = 32;
 constexpr int kTf32WideMaxDp = 64;
-bool plan_fma_kernel(int Dp, int C, bool aug, bool tf, int* nq, int* stages, size_t* smem);
+// few_stages: q^ in TMEM, short runs of key tiles.
+bool plan_fma_kernel(int Dp, int C, bool aug, bool tf, bool few_stages, int* nq, int* stages,
+                     size_t* smem);
 // vf_pass (plans with vfold): 1 = the problems whose 32-key groups all have
 // values of one sign, 2 = the others (launched after pass 1); 0 otherwise.
 cudaError_t launch_tc_fma(const TcPlan& p, InType t, float c, char* ws, unsigned* status,

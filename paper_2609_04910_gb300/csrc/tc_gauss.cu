@@ -694,7 +694,7 @@ bool plan_tensor(InType t, int64_t M, int64_t N, int64_t D, int64_t C, bool grad
         p->aug = false;
         p->Dp = D <= kTf32MaxDp ? kTf32MaxDp : kTf32WideMaxDp;
         p->guard = D > kTf32MaxDp;
-        if (!plan_fma_kernel(p->Dp, static_cast<int>(p->Cv), false, true, &nq, &fma_stages,
+        if (!plan_fma_kernel(p->Dp, static_cast<int>(p->Cv), false, true, false, &nq, &fma_stages,
                              &fma_smem)) {
             *why = "shared-memory budget exceeded";
             return false;
@@ -721,7 +721,7 @@ bool plan_tensor(InType t, int64_t M, int64_t N, int64_t D, int64_t C, bool grad
         p->aug = !grad && p->Cv <= kFmaMaxChannels && dp_aug <= kAugMaxDp;
         const int dp_fma = p->aug ? dp_aug : p->Dp;
         p->fma = !grad && p->Cv <= kFmaMaxChannels && !channels_on_mma &&
-                 plan_fma_kernel(dp_fma, static_cast<int>(p->Cv), p->aug, false, &nq, &fma_stages,
+                 plan_fma_kernel(dp_fma, static_cast<int>(p->Cv), p->aug, false, false, &nq, &fma_stages,
                                  &fma_smem);
         if (!p->fma) p->aug = false;
     }
@@ -913,6 +913,17 @@ bool plan_tensor(InType t, int64_t M, int64_t N, int64_t D, int64_t C, bool grad
     if (p->fma && p->aug && !p->tf) {
         const int64_t seg = p->band_len > 0 ? p->band_len : std::min<int64_t>(key_tiles, p->unit_len);
         p->overlap = seg <= kOverlapMaxTiles;
+    }
+    // q^ in TMEM (16-bit rows too wide for the augmented layout): short runs of
+    // key tiles take two stages instead of three, whose loads would delay the
+    // first MMAs and q^ (three / two stages, whole calls, one GB300: 16384 x
+    // 1000, D = 256 37.0 / 34.6 us, D = 208, C = 4 41 / 35; runs of 14 tiles, 1000 x
+    // 65536, D = 240 70 / 63, D = 256, C = 4 77.7 / 75.3, D = 144 48 / 49; runs of 54
+    // tiles, 16384^2, D = 160 84 / 93).
+    if (p->fma && !p->aug && !p->tf) {
+        const int64_t seg = p->band_len > 0 ? p->band_len : std::min<int64_t>(key_tiles, p->unit_len);
+        if (seg <= 8 || (seg <= 16 && p->Dp > 192))
+            plan_fma_kernel(p->Dp, static_cast<int>(p->Cv), false, false, true, &nq, &p->stages, &p->smem_bytes);
     }
     // ~256 rows per block of the mean kernel, so that every SM has work.
     p->mean_blocks = static_cast<int>(std::max<int64_t>(1, std::min<int64_t>(4096, (M + N + 255) / 256)));

@@ -123,7 +123,6 @@ struct FmaParams {
     const float* rec;    // key records, Npad / 2 pairs
     float* part;         // contributor slots x Mpad x C partial sums
     unsigned* status;
-    unsigned* guard;     // guarded sums: the words behind the key records (see Guard)
     int64_t Mpad;
     int units;           // work units: (pair of query tiles, key tile), row major
     int unit_len;        // units per CTA (CTA i: units [i unit_len, (i + 1) unit_len))
@@ -252,6 +251,13 @@ __device__ __forceinline__ bool vf_takes(const FmaParams& p, int tile_m) {
     return (flags[problem] != 0u) == (VF == 1);
 }
 
+// Guarded sums: the guard's words behind the key records of one problem.  (Not a
+// kernel parameter: eight bytes more of them made the compiler spill in the
+// variant with q^ in shared memory.)
+__device__ __forceinline__ unsigned* guard_words(const float* rec, int npad, int rec_pair) {
+    return reinterpret_cast<unsigned*>(const_cast<float*>(rec + static_cast<int64_t>(npad / 2) * rec_pair));
+}
+
 __device__ __forceinline__ void exp_warps_sync() {
     asm volatile("bar.sync 1, %0;" ::"r"(NEXP * 32) : "memory");
 }
@@ -285,7 +291,7 @@ tc_gauss_fma_kernel(const __grid_constant__ CUtensorMap tm_q,
     // the SIMT path, see kGuardMaxBits), and HALVES: query tile 0's exponentials
     // are summed before its S tile goes back, then query tile 1's.  The three
     // MMAs per K step take longer than the exponentials, so the later handback
-    // costs little (16384^2, D = 64 140 -> 148 us).
+    // costs little (16384^2, D = 64 140 -> 150 us).
     static_assert(!TF || !AUG, "3xTF32 takes plain rows");
     static_assert(!OVL || QSM, "overlapped segments keep q^ in shared memory");
     static_assert(VF == 0 || (AUG && SOFT == 0 && !TF), "folded operands: augmented fp16 rows");
@@ -312,7 +318,7 @@ tc_gauss_fma_kernel(const __grid_constant__ CUtensorMap tm_q,
     pdl_trigger();
     if (TF && !QSM) {
         pdl_wait();
-        if (*p.guard > kGuardMaxBits) return;
+        if (*guard_words(p.rec, p.npad, REC_PAIR) > kGuardMaxBits) return;
     }
     if (VF == 2) {
         // The second folded-value pass often has nothing to do (every problem
@@ -444,16 +450,18 @@ tc_gauss_fma_kernel(const __grid_constant__ CUtensorMap tm_q,
                                     kb * p.kb_elems, (tile_m * NQ + h) * BM);
             }
             __syncwarp();
-            auto load_keys = [&](int j) {
-                mbar_arrive_expect_tx(&bars->kv_full[k], p.kh_bytes + p.rec_bytes);
+            // Key tile j into stage `stage` (the warp's own with q^ in shared memory).
+            auto load_keys = [&](int stage, int j) {
+                const int s = QSM ? k : stage;
+                mbar_arrive_expect_tx(&bars->kv_full[s], p.kh_bytes + p.rec_bytes);
                 const int n0 = kbase + (kt0 + j) * BN;
                 for (int kb = 0; kb < p.nkb; ++kb)
-                    tma_load_2d(kh_smem(k) + kb * (BN * 128), &tm_k, &bars->kv_full[k],
+                    tma_load_2d(kh_smem(s) + kb * (BN * 128), &tm_k, &bars->kv_full[s],
                                 kb * p.kb_elems, n0);
-                bulk_load(const_cast<float*>(rec_smem(k)),
+                bulk_load(const_cast<float*>(rec_smem(s)),
                           p.rec + ((VF == 1 || VF == 2) ? static_cast<int64_t>(n0 / BN) * (BN + BN / 32)
                                       : static_cast<int64_t>(n0 / 2) * REC_PAIR),
-                          p.rec_bytes, &bars->kv_full[k]);
+                          p.rec_bytes, &bars->kv_full[s]);
             };
             if (!QSM && k == NCTRL_MAX - 1) {
                 // q^ in TMEM: this warp issues every MMA of the CTA, in the
@@ -513,20 +521,25 @@ tc_gauss_fma_kernel(const __grid_constant__ CUtensorMap tm_q,
             } else if (!QSM && has_tiles) {
                 // Keys and records of this warp's stage; the stage is free
                 // again once the MMAs and the exponent warps are done with it.
+                // A segment's third tile is asked for once q^ is there, which
+                // its load would delay, and a block's first two by one warp,
+                // one after the other.
                 uint32_t ph = static_cast<uint32_t>((g0 + j_first) / nctrl) & 1u;
-                bool pending = true;
-                if (leader) {
+                if (j_first >= 2) ok = warp_wait(&bars->qa_ready, seg_parity, abort_flag, p.status);
+                bool pending = ok;
+                if (leader && ok && (g0 > 0 || k != 1)) {
                     tma_prefetch_desc(&tm_k);
-                    load_keys(j_first);
+                    load_keys(k, j_first);
+                    if (g0 == 0 && k == 0 && T > 1) load_keys(1, 1);
                 }
                 __syncwarp();
-                for (int j = j_first;; j += nctrl) {
+                for (int j = j_first; ok; j += nctrl) {
                     ok = warp_wait(&bars->kv_empty[k], ph, abort_flag, p.status);
                     if (!ok) break;
                     pending = false;
                     if (j + nctrl >= T) break;
                     ph ^= 1u;
-                    if (leader) load_keys(j + nctrl);
+                    if (leader) load_keys(k, j + nctrl);
                     __syncwarp();
                     pending = true;
                 }
@@ -545,7 +558,7 @@ tc_gauss_fma_kernel(const __grid_constant__ CUtensorMap tm_q,
                     ok = warp_wait(&bars->kv_empty[k], ph ^ 1u, abort_flag, p.status);
                 if (leader && ok) {
                     tma_prefetch_desc(&tm_k);
-                    load_keys(j_first);
+                    load_keys(k, j_first);
                 }
                 __syncwarp();
                 if (ok) ok = warp_wait(&bars->qa_ready, seg_parity, abort_flag, p.status);
@@ -633,7 +646,7 @@ tc_gauss_fma_kernel(const __grid_constant__ CUtensorMap tm_q,
                         if (!ok) break;
                     }
                     if (j + nctrl < T) {
-                        if (leader) load_keys(j + nctrl);
+                        if (leader) load_keys(k, j + nctrl);
                         __syncwarp();
                         pending = true;
                     }
@@ -728,8 +741,9 @@ tc_gauss_fma_kernel(const __grid_constant__ CUtensorMap tm_q,
             const uint64_t a2_1 = f32x2_pack(am1, am1);
             const uint64_t c2 = f32x2_pack(p.c, p.c);
             const float s_min = -127.0f / p.c;   // exp2_fma_x2 range limit
-            const float s_close = kGuardClose / p.c;
-            unsigned close = 0;                  // sampled pairs of close points (see Guard)
+            // HALVES: q^.k^ of close points, and the sampled pairs above it (see Guard).
+            const float s_close = HALVES ? kGuardClose / p.c : 0.f;
+            unsigned close = 0;
             uint64_t acc0[C], acc1[C];
     #pragma unroll
             for (int cc = 0; cc < C; ++cc) acc0[cc] = acc1[cc] = 0ull;
@@ -760,6 +774,11 @@ tc_gauss_fma_kernel(const __grid_constant__ CUtensorMap tm_q,
                     tc_fence_after();
                     uint32_t r0[32], r1[32];
                     tmem_ld_32x32b_x32(tmem + lane_base + col0 + cg * 32, r0);
+                    bool both = false;    // q^ in TMEM: query tile 1's S tile is done as well
+                    if (!QSM && !HALVES) {
+                        both = __all_sync(0xffffffffu, mbar_test_wait(&bars->s_full[1], sl.phase));
+                        if (both) tc_fence_after();
+                    }
                     if (QSM) {
                         tmem_ld_32x32b_x32(tmem + lane_base + col0 + BN + cg * 32, r1);
                         // The wait names r0 and r1, so that no use of the loaded
@@ -781,18 +800,28 @@ tc_gauss_fma_kernel(const __grid_constant__ CUtensorMap tm_q,
                         // as the MMAs.  (Unlike with two slots, all MMAs come
                         // from one warp here, which issues the next ones behind
                         // its own earlier ones.)
-                        tmem_wait_ld_regs(r0);
-                        tc_fence_before();
-                        __syncwarp();
-                        mbar_arrive_if_zero(&bars->s_free[0], lane);
-                        ok = warp_wait(&bars->s_full[1], sl.phase, abort_flag, p.status);
-                        if (!ok) break;
-                        tc_fence_after();
-                        tmem_ld_32x32b_x32(tmem + lane_base + BN + cg * 32, r1);
-                        tmem_wait_ld_regs(r1);
-                        tc_fence_before();
-                        __syncwarp();
-                        mbar_arrive_if_zero(&bars->s_free[1], lane);
+                        // (Both done, as in short key ranges and where the
+                        // exponentials set the pace: one round trip for both.)
+                        if (both) {
+                            tmem_ld_32x32b_x32(tmem + lane_base + BN + cg * 32, r1);
+                            tmem_wait_ld_regs(r0, r1);
+                            tc_fence_before();
+                            __syncwarp();
+                            mbar_arrive2_if_zero(&bars->s_free[0], &bars->s_free[1], lane);
+                        } else {
+                            tmem_wait_ld_regs(r0);
+                            tc_fence_before();
+                            __syncwarp();
+                            mbar_arrive_if_zero(&bars->s_free[0], lane);
+                            ok = warp_wait(&bars->s_full[1], sl.phase, abort_flag, p.status);
+                            if (!ok) break;
+                            tc_fence_after();
+                            tmem_ld_32x32b_x32(tmem + lane_base + BN + cg * 32, r1);
+                            tmem_wait_ld_regs(r1);
+                            tc_fence_before();
+                            __syncwarp();
+                            mbar_arrive_if_zero(&bars->s_free[1], lane);
+                        }
                     } else {
                         tmem_wait_ld_regs(r0);
                     }
@@ -988,7 +1017,7 @@ tc_gauss_fma_kernel(const __grid_constant__ CUtensorMap tm_q,
             if (HALVES) {
                 close = __reduce_add_sync(0xffffffffu, close);
                 if (lane == 0 && close != 0u)
-                    atomicAdd(reinterpret_cast<unsigned long long*>(p.guard + 2),
+                    atomicAdd(reinterpret_cast<unsigned long long*>(guard_words(p.rec, p.npad, REC_PAIR) + 2),
                               static_cast<unsigned long long>(close));
             }
             // Fixed-order reduction of the NPART column-group partial sums.
@@ -1086,7 +1115,6 @@ cudaError_t launch_typed(const TcPlan& pl, InType t, float c, char* ws, unsigned
     p.rec = reinterpret_cast<const float*>(ws + pl.off_rec);
     p.part = reinterpret_cast<float*>(ws + pl.off_part);
     p.status = status;
-    p.guard = pl.guard ? reinterpret_cast<unsigned*>(ws + pl.off_rec) + pl.Npad * (1 + pl.Cv) : nullptr;
     p.Mpad = pl.Mpad * pl.batch;   // partial-sum rows per contributor slot
     p.key_tiles = static_cast<int>(pl.Npad / BN);
     p.pairs_per_batch = static_cast<int>(pl.Mpad / (NQ * BM));
@@ -1171,7 +1199,8 @@ cudaError_t launch_c(const TcPlan& pl, InType t, float c, char* ws, unsigned* st
 
 }  // namespace
 
-bool plan_fma_kernel(int Dp, int C, bool aug, bool tf, int* nq, int* stages, size_t* smem) {
+bool plan_fma_kernel(int Dp, int C, bool aug, bool tf, bool few_stages, int* nq, int* stages,
+                     size_t* smem) {
     if (C < 1 || C > kFmaMaxChannels || Dp > 256) return false;
     if (aug && Dp > kAugMaxDp) return false;
     if (tf && (aug || Dp > kTf32WideMaxDp)) return false;
@@ -1189,9 +1218,12 @@ bool plan_fma_kernel(int Dp, int C, bool aug, bool tf, int* nq, int* stages, siz
     // is at most one phase behind the phase it asks about; the warp knows
     // every key tile up to j - stages is done (its previous stage release) and
     // the slot's previous phase is tile j - 4, so stages <= 4.  q^ in TMEM:
-    // one control warp issues the MMAs, the others load a stage each.
-    const int st = static_cast<int>(
-        std::min<size_t>(qsm ? MAX_STAGES : NCTRL_MAX - 1, (budget - fixed) / stage));
+    // one control warp issues the MMAs, the others load a stage each: three,
+    // or two with few_stages (see plan_tensor) and for 3xTF32, whose S tiles
+    // go back late (16384^2, C = 1, three / two stages: D = 33 130 / 120 us,
+    // D = 64 155 / 150).
+    const int st = static_cast<int>(std::min<size_t>(
+        qsm ? MAX_STAGES : tf || few_stages ? 2 : NCTRL_MAX - 1, (budget - fixed) / stage));
     if (st < 2) return false;
     *nq = NQ;
     *stages = st;
