@@ -1793,24 +1793,31 @@ finalize_point_quads_kernel(const float* __restrict__ part, int splits, int64_t 
 // one contiguous run, in shared memory with 16-byte loads (any D), then takes
 // per-channel maxima, or writes 16 keys of a channel per thread (two 16-byte
 // stores, whole sectors).  The element-wise kernels read 2 bytes at a time and
-// stored 4: 131072 keys, D = 32, ncu: 19.6 + 24.1 us, these 9.3 + 11.8.
+// stored 4: 131072 keys, D = 32, ncu: 19.6 + 24.1 us, these 9.3 + 11.8.  Blocks
+// of 128 rows and 128 threads, or of 32 rows and 256 threads where the first
+// would leave SMs idle and each thread's chain of rows is what a call waits for
+// (whole calls, with blocks of 128 rows / of 32: gradient of 3000 points, D = 128
+// 57 / 39 us; vector-Jacobian product of 300 points, D = 64 78 / 56).
 constexpr int kValueRows = 128;
 constexpr int kValueThreads = 128;
+constexpr int kFewValueRows = 32;
+constexpr int kFewValueThreads = 256;
+constexpr int64_t kFewValueBlocks = 304;     // (two per SM)
 
-// Rows [n0, n0 + kValueRows) of x into raw (zeros past N); weights into sw (1
+// Rows [n0, n0 + ROWS) of x into raw (zeros past N); weights into sw (1
 // without weights, 0 past N).  By the whole block.
-template <typename T, typename W>
+template <int ROWS, typename T, typename W>
 __device__ __forceinline__ void stage_value_rows(const W* __restrict__ w, const T* __restrict__ x,
                                                  int64_t N, int D, int64_t n0, T* raw, float* sw) {
-    const int rows = static_cast<int>(max(int64_t(0), min(static_cast<int64_t>(kValueRows), N - n0)));
+    const int rows = static_cast<int>(max(int64_t(0), min(static_cast<int64_t>(ROWS), N - n0)));
     const int nt = blockDim.x;
-    const T* src = x + n0 * D;          // n0 is a multiple of 128: 16-byte aligned
+    const T* src = x + n0 * D;          // n0 is a multiple of 32: 16-byte aligned
     const int n_el = rows * D, nvec = n_el / 8;
     for (int i = threadIdx.x; i < nvec; i += nt)
         reinterpret_cast<uint4*>(raw)[i] = reinterpret_cast<const uint4*>(src)[i];
     for (int i = nvec * 8 + threadIdx.x; i < n_el; i += nt) raw[i] = src[i];
-    for (int i = n_el + threadIdx.x; i < kValueRows * D; i += nt) raw[i] = from_f<T>(0.f);
-    for (int i = threadIdx.x; i < kValueRows; i += nt)
+    for (int i = n_el + threadIdx.x; i < ROWS * D; i += nt) raw[i] = from_f<T>(0.f);
+    for (int i = threadIdx.x; i < ROWS; i += nt)
         sw[i] = i < rows ? (w ? to_f(w[n0 + i]) : 1.f) : 0.f;
     __syncthreads();
 }
@@ -1834,11 +1841,11 @@ __device__ __forceinline__ void value_rows_max(const T* raw, const float* sw, co
 // The staged rows' scaled values into vt: item i is channel i mod Cp, keys
 // 16 (i / Cp) .. + 15 of the block.  (Npad is a multiple of 128, so the
 // block's keys are all inside.)
-template <typename T>
+template <int ROWS, typename T>
 __device__ __forceinline__ void value_rows_write(const T* raw, const float* sw, const float* mu, int D, int Cp,
                                                  const unsigned* vmax_bits, int64_t Npad, int64_t n0,
                                                  __half* __restrict__ vt) {
-    for (int i = threadIdx.x; i < Cp * (kValueRows / 16); i += blockDim.x) {
+    for (int i = threadIdx.x; i < Cp * (ROWS / 16); i += blockDim.x) {
         const int g = i / Cp, c = i - g * Cp;
         const float sc = c <= D ? pow2f(channel_exponent(vmax_bits[c])) : 0.f;
         const float m = c < D && mu ? mu[c] : 0.f;
@@ -1859,8 +1866,8 @@ __device__ __forceinline__ void value_rows_write(const T* raw, const float* sw, 
     }
 }
 
-template <typename T, typename W>
-__global__ void __launch_bounds__(kValueThreads)
+template <int ROWS, int THREADS, typename T, typename W>
+__global__ void __launch_bounds__(THREADS)
 point_value_max_kernel(const W* __restrict__ w, const T* __restrict__ x,
                        const float* __restrict__ mu, int64_t N, int D,
                        unsigned* __restrict__ vmax_bits) {
@@ -1868,19 +1875,19 @@ point_value_max_kernel(const W* __restrict__ w, const T* __restrict__ x,
     pdl_wait();
     extern __shared__ __align__(16) uint8_t value_smem[];
     T* raw = reinterpret_cast<T*>(value_smem);
-    __shared__ float sw[kValueRows];
+    __shared__ float sw[ROWS];
     __shared__ unsigned big[kOperandMaxCols + 1];
-    for (int i = threadIdx.x; i <= D; i += kValueThreads) big[i] = 0u;
-    const int64_t n0 = static_cast<int64_t>(blockIdx.x) * kValueRows;
-    stage_value_rows(w, x, N, D, n0, raw, sw);
-    value_rows_max(raw, sw, mu, static_cast<int>(min(static_cast<int64_t>(kValueRows), N - n0)), D, big);
+    for (int i = threadIdx.x; i <= D; i += THREADS) big[i] = 0u;
+    const int64_t n0 = static_cast<int64_t>(blockIdx.x) * ROWS;
+    stage_value_rows<ROWS>(w, x, N, D, n0, raw, sw);
+    value_rows_max(raw, sw, mu, static_cast<int>(min(static_cast<int64_t>(ROWS), N - n0)), D, big);
     __syncthreads();
-    for (int i = threadIdx.x; i <= D; i += kValueThreads)
+    for (int i = threadIdx.x; i <= D; i += THREADS)
         if (big[i] != 0u) atomicMax(&vmax_bits[i], big[i]);
 }
 
-template <typename T, typename W>
-__global__ void __launch_bounds__(kValueThreads)
+template <int ROWS, int THREADS, typename T, typename W>
+__global__ void __launch_bounds__(THREADS)
 point_value_prep_kernel(const W* __restrict__ w, const T* __restrict__ x,
                         const float* __restrict__ mu, int64_t N, int64_t Npad, int D, int Cp,
                         const unsigned* __restrict__ vmax_bits, __half* __restrict__ vt,
@@ -1889,12 +1896,12 @@ point_value_prep_kernel(const W* __restrict__ w, const T* __restrict__ x,
     pdl_wait();
     extern __shared__ __align__(16) uint8_t value_smem[];
     T* raw = reinterpret_cast<T*>(value_smem);
-    __shared__ float sw[kValueRows];
-    const int64_t n0 = static_cast<int64_t>(blockIdx.x) * kValueRows;
-    stage_value_rows(w, x, N, D, n0, raw, sw);
-    value_rows_write(raw, sw, mu, D, Cp, vmax_bits, Npad, n0, vt);
+    __shared__ float sw[ROWS];
+    const int64_t n0 = static_cast<int64_t>(blockIdx.x) * ROWS;
+    stage_value_rows<ROWS>(w, x, N, D, n0, raw, sw);
+    value_rows_write<ROWS>(raw, sw, mu, D, Cp, vmax_bits, Npad, n0, vt);
     if (blockIdx.x == 0)
-        for (int c = threadIdx.x; c < Cp; c += kValueThreads)
+        for (int c = threadIdx.x; c < Cp; c += THREADS)
             inv_scale[c] = c <= D ? pow2f(-channel_exponent(vmax_bits[c])) : 0.f;
 }
 
@@ -2051,21 +2058,27 @@ cudaError_t value_prep_typed(const void* w, const void* x, const float* mu, int6
         pdl_reset();   // the next kernel follows a memset
     }
     if (GRAD && Cw == 1 && ch0 == 0 && Cc == D + 1 && D >= 1 && N > 0) {
-        const size_t smem = static_cast<size_t>(kValueRows) * D * sizeof(T);
-        auto go = [&](auto kern, unsigned blocks, auto... args) {
+        auto go = [&](auto kern, int64_t blocks, int rows, int threads, auto... args) {
+            const size_t smem = static_cast<size_t>(rows) * D * sizeof(T);
             cudaError_t r = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                  static_cast<int>(smem));
             if (r != cudaSuccess) return r;
-            launch_kernel(kern, blocks, kValueThreads, smem, s, args...);
+            launch_kernel(kern, static_cast<unsigned>(blocks), threads, smem, s, args...);
             note_launches(1);
             return cudaGetLastError();
         };
-        e = go(point_value_max_kernel<T, W>, static_cast<unsigned>((N + kValueRows - 1) / kValueRows),
-               static_cast<const W*>(w), static_cast<const T*>(x), mu, N, D, vmax_bits);
-        if (e != cudaSuccess) return e;
-        return go(point_value_prep_kernel<T, W>, static_cast<unsigned>(Npad / kValueRows),
-                  static_cast<const W*>(w), static_cast<const T*>(x), mu, N, Npad, D, Cp,
-                  static_cast<const unsigned*>(vmax_bits), static_cast<__half*>(vt), inv_scale);
+        auto both = [&](auto rows_tag, auto threads_tag) {
+            constexpr int R = decltype(rows_tag)::value, TH = decltype(threads_tag)::value;
+            const cudaError_t r = go(point_value_max_kernel<R, TH, T, W>, (N + R - 1) / R, R, TH,
+                                     static_cast<const W*>(w), static_cast<const T*>(x), mu, N, D, vmax_bits);
+            if (r != cudaSuccess) return r;
+            return go(point_value_prep_kernel<R, TH, T, W>, Npad / R, R, TH, static_cast<const W*>(w),
+                      static_cast<const T*>(x), mu, N, Npad, D, Cp, static_cast<const unsigned*>(vmax_bits),
+                      static_cast<__half*>(vt), inv_scale);
+        };
+        if (Npad / kValueRows < kFewValueBlocks)
+            return both(std::integral_constant<int, kFewValueRows>(), std::integral_constant<int, kFewValueThreads>());
+        return both(std::integral_constant<int, kValueRows>(), std::integral_constant<int, kValueThreads>());
     }
     // 64 rows per block: several blocks per SM even for N of a few 10^4.
     const int64_t rows_per_block = 64;

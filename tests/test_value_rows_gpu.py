@@ -1,0 +1,28 @@
+"""Value channels of the gradient passes on both sides of the switch from blocks
+of 32 rows to blocks of 128 (304 of the larger), and at the edges of a block,
+against the float64 oracle with the suite's tolerances."""
+import numpy as np
+import pytest
+
+from tests.gpu_helpers import case, grad_check
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _gpu():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2609_04910_gb300.build import build_library
+    build_library()
+    torch.cuda.set_device(0)
+
+
+@pytest.mark.parametrize("dtype", ["fp16", "bf16"])
+@pytest.mark.parametrize("N,D", [(1, 3), (31, 64), (32, 17), (33, 1), (127, 100), (129, 8),
+                                 (38784, 5), (38785, 5), (38784, 64), (38785, 64), (40000, 33)])
+def test_rows(N, D, dtype):
+    M = 300
+    grad_check(case(M, N, D, 1, dtype), rows=np.arange(0, M, 7))
