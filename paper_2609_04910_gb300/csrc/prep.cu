@@ -2282,8 +2282,10 @@ mmd2_reduce_kernel(const float* __restrict__ s, const T* __restrict__ v, int64_t
 // time by 256 threads took 10 to 20 us more), and folded in
 // mmd2_reduce_kernel's order.  Whole calls, with the overlapped segments
 // before and after: 64 problems of 2000 points 70.0 -> 62.5 us, 16 of 4096
-// 82 -> 56, 8 of 8000 79.3 -> 73.5, one of 30000 105.3 -> 105.3 us.
+// 82 -> 56, 8 of 8000 79.3 -> 73.5, one of 30000 105.3 -> 105.3 us.  (bf16; one
+// of 5000 points, D = 64, with two slots' loads in flight 34.9, with six 33.5.)
 constexpr int kMmdThreads = 1024;
+constexpr int kMmdSlots = 6;
 
 template <typename T>
 __global__ void __launch_bounds__(kMmdThreads)
@@ -2316,14 +2318,19 @@ mmd2_slots_kernel(const float* __restrict__ part, int64_t Mpad, int64_t N, int r
         most = max(most, ns[i]);
         s[i] = 0.f;
     }
-#pragma unroll 2
-    for (int sl = 0; sl < most; ++sl) {
-        float x[PER];
+    // (Six slots' loads of the four points in flight together.)
+    for (int sl = 0; sl < most; sl += kMmdSlots) {
+        float x[kMmdSlots][PER];
 #pragma unroll
-        for (int i = 0; i < PER; ++i) x[i] = sl < ns[i] ? p[sl * step + i * kMmdThreads] : 0.f;
+        for (int u = 0; u < kMmdSlots; ++u)
 #pragma unroll
-        for (int i = 0; i < PER; ++i)
-            if (sl < ns[i]) s[i] += x[i];
+            for (int i = 0; i < PER; ++i)
+                x[u][i] = sl + u < ns[i] ? p[(sl + u) * step + i * kMmdThreads] : 0.f;
+#pragma unroll
+        for (int u = 0; u < kMmdSlots; ++u)
+#pragma unroll
+            for (int i = 0; i < PER; ++i)
+                if (sl + u < ns[i]) s[i] += x[u][i];
     }
 #pragma unroll
     for (int i = 0; i < PER; ++i) sums[t + i * kMmdThreads] = s[i];
