@@ -165,13 +165,15 @@ def _dtype_code(t):
 
 def _stream_ptr(stream):
     """The handle of ``stream`` or, by default, of the current device's current
-    stream.  The latter is read as a raw handle: making a torch.cuda.Stream of
-    it took 4.7 us of the 20 us that a small call spends outside the C ABI
-    (Grace host)."""
+    stream.  The latter is read as a raw handle where torch has one: making a
+    torch.cuda.Stream of it took 4.7 us of the 20 us that a small call spends
+    outside the C ABI (Grace host)."""
     if stream is None:
         import torch
-        if torch.cuda.is_initialized():
-            return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+        raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+        device = getattr(torch._C, "_cuda_getDevice", None)
+        if raw is not None and device is not None and torch.cuda.is_initialized():
+            return raw(device())
         stream = torch.cuda.current_stream()
     return stream.cuda_stream
 
