@@ -299,7 +299,10 @@ gs_status plan(const Call& c, int sms, bool* tensor, gs::TcPlan* tp, gs::SimtPla
         // go into the key operands and the key records keep the signs.  Not
         // for short segments (small problems), where the flag kernel and the
         // second pass of the fused kernel cost more than they save (B = 256
-        // problems of 1024 points: 0.135 -> 0.144 ms per call).
+        // problems of 1024 points: 0.135 -> 0.144 ms per call).  The upper
+        // triangle folds at any length, as it did before its short segments
+        // overlapped, so that MMD^2 keeps its bits (fp16, 64 problems of 2000
+        // points, D = 32 67 us; 61 unfolded, with other roundings).
         // The exponent scale c folds into the query rows with them (rn(c q^)
         // must stay a normal fp16 number for points of any spread: c <= 1/2,
         // and not far below it: c >= 2^-14).
@@ -459,7 +462,7 @@ gs_status run(Call c) {
                     static_cast<int>(c.D), tp.Dp, tp.mean_blocks, mu, half_c, ninf, c.stream, batch,
                     tp.vfold ? c.v : nullptr, (tp.vfold || tp.cfold) ? cexp : 0.f,
                     records_done ? &rec : nullptr,
-                    flags_done ? reinterpret_cast<float*>(ws + tp.off_rec) : nullptr, zero);
+                    flags_done ? reinterpret_cast<float*>(ws + tp.off_rec) : nullptr);
                 where = "preparation kernel";
             } else {
                 e = gs::launch_mean(t, c.q, c.k, c.M, c.N, static_cast<int>(c.D), tp.mean_blocks,
@@ -845,7 +848,8 @@ gs_status gauss_sum_mmd2(const void* x, const void* v, double tau, int64_t B, in
     if (status != GS_OK) return status;
     if (forced_alloc_failure()) return fail(GS_ERR_OUT_OF_MEMORY, "workspace allocation failed (test hook)");
     float* s_buf = nullptr;
-    // s (B x N float32), then the float64 chunk partials of the reduction.
+    // s (B x N float32; written only where the FMA kernel's partial sums are not
+    // reduced directly), then the float64 chunk partials of the reduction.
     const size_t s_bytes = (sizeof(float) * B * N + 255) & ~static_cast<size_t>(255);
     cudaError_t e = pool_alloc(reinterpret_cast<void**>(&s_buf),
                                     s_bytes + gs::mmd2_partial_bytes(B, N), st);

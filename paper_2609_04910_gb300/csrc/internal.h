@@ -205,8 +205,8 @@ struct ZeroWords {
     int n = 0;
 };
 // Common mean of q and k per problem.  With `rec`, the launch also writes
-// those key records where it can (the vectorised path); *rec_done says
-// whether it did.
+// those key records where it can (16-bit inputs); *rec_done says whether it
+// did.
 cudaError_t launch_mean(InType t, const void* q, const void* k, int64_t M, int64_t N, int D,
                         int blocks, float* partial, float* mu, cudaStream_t s, int batch = 1,
                         const RecordArgs* rec = nullptr, bool* rec_done = nullptr,
@@ -217,7 +217,7 @@ cudaError_t launch_mean(InType t, const void* q, const void* k, int64_t M, int64
 // then also computes where it can, *flags_done saying whether it did.)
 // Centred, rounded MMA operands of q (M rows, padded to Mpad) and, with
 // with_k, of k (N rows, padded to Npad), in one launch where the vector
-// path applies (16-bit inputs, D a multiple of 8).  aug: the augmented
+// path applies (D >= 1, fewer than 2^30 rows).  aug: the augmented
 // layout (Dp >= D + 2 aug_norm_terms(t)) into qh, and into qh_as_key (the
 // key layout of the same points, for q = k; may be null) and kh; plain:
 // x^ into qh / kh and the norm terms -(c/2)||x^||^2 into nrm_q / nrm_k
@@ -229,7 +229,8 @@ cudaError_t launch_operands(InType t, bool aug, const void* q, int64_t M, int64_
                             int batch = 1, const void* vw = nullptr, float cf = 0.f,
                             float* vf_rec = nullptr, bool* flags_done = nullptr);
 // Small 16-bit problems: the mean, operands, records and flags of the two
-// launches above in one, with the same results; see prep_cluster_kernel.
+// launches above in one, with the same results bit for bit; see
+// prep_cluster_kernel.
 // prep_cluster_fits says whether a call is one.
 constexpr int64_t kPrepMaxRows = 2048;       // M + N (M for q = k) per problem
 constexpr int64_t kPrepMaxElements = int64_t(1) << 17;   // (M + N) D
@@ -240,7 +241,7 @@ cudaError_t launch_prep_cluster(InType t, bool aug, const void* q, int64_t M, in
                                 void* qh_as_key, float* nrm_q, bool with_k, const void* k, int64_t N,
                                 int64_t Npad, void* kh, float* nrm_k, int D, int Dp, int blocks, float* mu,
                                 float half_c, float pad_value, cudaStream_t s, int batch, const void* vw,
-                                float cf, const RecordArgs* rec, float* vf_rec, ZeroWords zero);
+                                float cf, const RecordArgs* rec, float* vf_rec);
 // Transposed fp16 value operand of the two-MMA kernel for the channels
 // ch0 .. ch0 + Cc - 1 (Cp >= Cc rows of Npad keys), with per-channel
 // power-of-two scales.  Forward: channel ch of key n is w[n, ch] (w has the

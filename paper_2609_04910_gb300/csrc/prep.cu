@@ -187,6 +187,19 @@ __device__ __forceinline__ void write_key_record(const RecordJob<TV>& j, int64_t
     }
 }
 
+// Thread t of the blocks that write records instead of partial sums: key record
+// t, or the sign record of key t.
+template <typename TV>
+__device__ __forceinline__ void write_record(const RecordJob<TV>& rj, int64_t t, int problem) {
+    if (rj.signs) {
+        if constexpr (std::is_same<TV, __half>::value) {
+            if (t < 2 * rj.pairs) write_sign_record(rj.v, rj.N, rj.rec, t, problem, 2 * rj.pairs);
+        }
+    } else if (t < rj.pairs) {
+        write_key_record(rj, t, problem);
+    }
+}
+
 struct MeanShared {
     float sum[kMeanVecThreads][9];
     float max[kMeanVecThreads][9];
@@ -265,14 +278,7 @@ mean_partial_vec_kernel(const T* __restrict__ q, const T* __restrict__ k, int64_
     pdl_trigger();
     pdl_wait();
     if (static_cast<int>(blockIdx.x) >= G) {
-        const int64_t t = static_cast<int64_t>(blockIdx.x - G) * kMeanVecThreads + threadIdx.x;
-        if (rj.signs) {
-            if constexpr (std::is_same<TV, __half>::value) {
-                if (t < 2 * rj.pairs) write_sign_record(rj.v, rj.N, rj.rec, t, blockIdx.y, 2 * rj.pairs);
-            }
-        } else if (t < rj.pairs) {
-            write_key_record(rj, t, blockIdx.y);
-        }
+        write_record(rj, static_cast<int64_t>(blockIdx.x - G) * kMeanVecThreads + threadIdx.x, blockIdx.y);
         return;
     }
     // Problem blockIdx.y of a batch: its own points and partial rows.
@@ -406,14 +412,7 @@ mean_partial_rows_kernel(const T* __restrict__ q, const T* __restrict__ k, int64
     pdl_trigger();
     pdl_wait();
     if (static_cast<int>(blockIdx.x) >= mblocks) {
-        const int64_t t = static_cast<int64_t>(blockIdx.x - mblocks) * kMeanVecThreads + threadIdx.x;
-        if (rj.signs) {
-            if constexpr (std::is_same<TV, __half>::value) {
-                if (t < 2 * rj.pairs) write_sign_record(rj.v, rj.N, rj.rec, t, blockIdx.y, 2 * rj.pairs);
-            }
-        } else if (t < rj.pairs) {
-            write_key_record(rj, t, blockIdx.y);
-        }
+        write_record(rj, static_cast<int64_t>(blockIdx.x - mblocks) * kMeanVecThreads + threadIdx.x, blockIdx.y);
         return;
     }
     // Problem blockIdx.y of a batch: its own points and partial rows.
@@ -592,6 +591,8 @@ __device__ __forceinline__ float log_weight(const __half* vw) {
 constexpr int kRowsPerBlock = 32;
 constexpr int kOperandThreads = 128;
 constexpr int kOperandMaxCols = 256;
+
+// (The vector path below takes every call but those of D = 0 and of 2^30 rows.)
 
 template <typename T, bool AUG>
 __global__ void __launch_bounds__(kOperandThreads)
@@ -1910,7 +1911,7 @@ point_value_prep_kernel(const W* __restrict__ w, const T* __restrict__ x,
 // blocks: the partial sums of the mean (the blocks' shares of the split that
 // the separate kernels would use, so that the mean has the same bits), their
 // fold through distributed shared memory, the operand rows, and what rides
-// along: key or sign records, folded-value flags and cleared words.  The
+// along: key or sign records and folded-value flags.  The
 // smallest calls wait for the host, about 2 us per launch; this takes two
 // launches out.  Its own chain (loads, reduction, two cluster barriers, rows)
 // is longer than that of the three kernels it replaces once a block has more
@@ -1933,7 +1934,6 @@ struct PrepArgs {
     float total;
     int mant_bits, min_exp;
     float* mu;
-    ZeroWords zero;
     // Records (out null: none) and folded-value flags (vf_rec null: none).
     RecordArgs rec;
     float* vf_rec;
@@ -1980,8 +1980,6 @@ prep_cluster_kernel(const PrepArgs<T> a) {
             }
         }
     }
-    if (rank == 0 && b == 0)
-        for (int i = tid; i < a.zero.n; i += kOperandVecThreads) a.zero.p[i] = 0u;
 
     // Mean: this block's chunks of the split, then the fold over all of them.
     const T* q = a.q + static_cast<int64_t>(b) * a.M * D;
@@ -2167,47 +2165,31 @@ cudaError_t launch_mean(InType t, const void* q, const void* k, int64_t M, int64
     const MeanSplit sp = mean_split(t, M, N, D, blocks);
     const int G = sp.G, Gq = sp.Gq;
     const int64_t rpb = sp.rpb;
-    if (sp.vec) {
-        // Key records (see RecordJob) in blocks G .. G + rblocks - 1.
+    if (sp.vec || (t != InType::F32 && D >= 1 && D <= kMeanVecThreads)) {
+        // Key records (see RecordJob) in the blocks behind those of the mean, one
+        // thread per key pair, or per key for sign records.
         const int64_t pairs = rec ? rec->Npad / 2 : 0;
-        // One thread per key pair, or per key for sign records.
         const int64_t rthreads = rec && rec->signs ? 2 * pairs : pairs;
         const int rblocks = static_cast<int>((rthreads + kMeanVecThreads - 1) / kMeanVecThreads);
-        auto go = [&](auto tag, auto vtag) {
-            using T = decltype(tag);
-            using TV = decltype(vtag);
-            const RecordJob<TV> rj = {rec ? static_cast<const TV*>(rec->v) : nullptr, rec ? rec->N : 0,
-                                      pairs, rec ? rec->C : 0, rec ? rec->out : nullptr,
-                                      rec && rec->signs};
-            launch_kernel(mean_partial_vec_kernel<T, TV>, dim3(G + rblocks, batch), kMeanVecThreads, 0,
-                          s, static_cast<const T*>(q), static_cast<const T*>(k), M, N, D, rpb, Gq, G,
-                          partial, rj);
-        };
-        const bool vf = rec && rec->v_f32;
-        if (t == InType::F16) {
-            if (vf) go(__half(), float()); else go(__half(), __half());
-        } else {
-            if (vf) go(__nv_bfloat16(), float()); else go(__nv_bfloat16(), __nv_bfloat16());
-        }
-        if (rec_done) *rec_done = rec != nullptr;
-        note_launches(1);
-    } else if (t != InType::F32 && D >= 1 && D <= kMeanVecThreads) {
-        // As many chunks per block as leave about 300 blocks.
-        const int chunks = static_cast<int>(
-            std::min<int64_t>(kMeanVecThreads / D, std::max<int64_t>(1, static_cast<int64_t>(G) * batch / 304)));
+        // (Rows form: as many chunks per block as leave about 300 blocks.)
+        const int chunks = sp.vec ? 1 : static_cast<int>(std::min<int64_t>(
+            kMeanVecThreads / D, std::max<int64_t>(1, static_cast<int64_t>(G) * batch / 304)));
         const int mblocks = (G + chunks - 1) / chunks;
-        const int64_t pairs = rec ? rec->Npad / 2 : 0;
-        const int64_t rthreads = rec && rec->signs ? 2 * pairs : pairs;
-        const int rblocks = static_cast<int>((rthreads + kMeanVecThreads - 1) / kMeanVecThreads);
         auto go = [&](auto tag, auto vtag) {
             using T = decltype(tag);
             using TV = decltype(vtag);
             const RecordJob<TV> rj = {rec ? static_cast<const TV*>(rec->v) : nullptr, rec ? rec->N : 0,
                                       pairs, rec ? rec->C : 0, rec ? rec->out : nullptr,
                                       rec && rec->signs};
-            launch_kernel(mean_partial_rows_kernel<T, TV>, dim3(mblocks + rblocks, batch), kMeanVecThreads,
-                          0, s, static_cast<const T*>(q), static_cast<const T*>(k), M, N, D, rpb, G,
-                          chunks, mblocks, partial, rj);
+            const T* qt = static_cast<const T*>(q);
+            const T* kt = static_cast<const T*>(k);
+            const dim3 grid(mblocks + rblocks, batch);
+            if (sp.vec)
+                launch_kernel(mean_partial_vec_kernel<T, TV>, grid, kMeanVecThreads, 0, s, qt, kt, M, N, D, rpb, Gq,
+                              G, partial, rj);
+            else
+                launch_kernel(mean_partial_rows_kernel<T, TV>, grid, kMeanVecThreads, 0, s, qt, kt, M, N, D, rpb, G,
+                              chunks, mblocks, partial, rj);
         };
         const bool vf = rec && rec->v_f32;
         if (t == InType::F16) {
@@ -2511,7 +2493,7 @@ cudaError_t launch_prep_cluster(InType t, bool aug, const void* q, int64_t M, in
                                 void* qh_as_key, float* nrm_q, bool with_k, const void* k, int64_t N,
                                 int64_t Npad, void* kh, float* nrm_k, int D, int Dp, int blocks, float* mu,
                                 float half_c, float pad_value, cudaStream_t s, int batch, const void* vw,
-                                float cf, const RecordArgs* rec, float* vf_rec, ZeroWords zero) {
+                                float cf, const RecordArgs* rec, float* vf_rec) {
     auto fill = [&](auto tag) {
         using T = decltype(tag);
         PrepArgs<T> a = {};
@@ -2529,7 +2511,6 @@ cudaError_t launch_prep_cluster(InType t, bool aug, const void* q, int64_t M, in
         a.mant_bits = mean_mant_bits(t);
         a.min_exp = mean_min_exp(t);
         a.mu = mu;
-        a.zero = zero;
         if (rec) a.rec = *rec;
         a.vf_rec = vf_rec;
         a.vf_tiles = Npad / kRecTile;
