@@ -172,6 +172,29 @@ __device__ __forceinline__ bool warp_wait(uint64_t* bar, uint32_t parity, volati
     return __all_sync(0xffffffffu, ok);
 }
 
+// Lane number for the release of a stage whose records this warp has used, tied
+// to the sums that took them in: the release is an arrival of lane 0 that must
+// not happen before the last record load has been served.  Program order does
+// not see to that: a shared-memory load whose result is not needed yet may still
+// be on its way when the arrival is performed, and the stage is refilled by the
+// TMA engine, not by a later instruction of the same kind.  (With four channels
+// and segments that overlap, warps then added values of the next segment's
+// tile: 14005 x 3527, D = 48, one call in three.)  No sum is the word ~0: the
+// arithmetic produces no such NaN.
+template <int C>
+__device__ __forceinline__ uint32_t lane_after(const uint64_t (&a)[C], uint32_t lane, uint32_t all = ~0u) {
+#pragma unroll
+    for (int cc = 0; cc < C; ++cc) all &= static_cast<uint32_t>(a[cc]);
+    return all == ~0u ? 1u : lane;
+}
+template <int C>
+__device__ __forceinline__ uint32_t lane_after(const uint64_t (&a)[C], const uint64_t (&b)[C], uint32_t lane) {
+    uint32_t all = ~0u;
+#pragma unroll
+    for (int cc = 0; cc < C; ++cc) all &= static_cast<uint32_t>(b[cc]);
+    return lane_after(a, lane, all);
+}
+
 // One segment of a CTA's work: the pair of query tiles tile_m and T
 // consecutive key tiles from kt0, and the partial-sum slot it writes.
 struct Segment {
@@ -785,13 +808,12 @@ tc_gauss_fma_kernel(const __grid_constant__ CUtensorMap tm_q,
                         // values is scheduled above it (the loads land asynchronously).
                         // With two slots (q^ in shared memory) the S slot is handed
                         // back only after the exponent work of this tile (with the
-                        // stage, below), because releasing it right after the loads
-                        // let the next MMAs into the slot corrupt S values of this
-                        // tile in some warps when the MMAs were long (measured with
-                        // 3xTF32 operands and three or more stages, also with the
-                        // loads' registers named in the wait; the early release was
-                        // no faster on the 65536^2, D = 64 sum either: 0.6428
-                        // against 0.6418 ms).
+                        // stage, below): sums came out wrong now and then when it
+                        // went back right after the loads and the MMAs were long
+                        // (3xTF32 operands, three or more stages; perhaps for the
+                        // reason that lane_after mends, not tried again since), and
+                        // that was no faster on the 65536^2, D = 64 sum either
+                        // (0.6428 against 0.6418 ms).
                         tmem_wait_ld_regs(r0, r1);
                     } else if (!HALVES) {
                         // q^ in TMEM: one S tile per query tile, handed back as
@@ -959,7 +981,7 @@ tc_gauss_fma_kernel(const __grid_constant__ CUtensorMap tm_q,
                         half(r0, a2_0, acc0);
                         tc_fence_before();
                         __syncwarp();
-                        mbar_arrive_if_zero(&bars->s_free[0], lane);
+                        mbar_arrive_if_zero(&bars->s_free[0], lane_after(acc0, lane));
                         ok = warp_wait(&bars->s_full[1], sl.phase, abort_flag, p.status);
                         if (!ok) break;
                         tc_fence_after();
@@ -1008,9 +1030,10 @@ tc_gauss_fma_kernel(const __grid_constant__ CUtensorMap tm_q,
                     // Lane 0 hands back the slot (two-slot path) and the stage,
                     // predicated rather than branched: a divergent branch here
                     // cost 0.7 % of the kernel time.
-                    if (QSM) mbar_arrive2_if_zero(&bars->s_free[sl.idx], &bars->kv_empty[s], lane);
-                    else if (HALVES) mbar_arrive2_if_zero(&bars->s_free[1], &bars->kv_empty[s], lane);
-                    else mbar_arrive_if_zero(&bars->kv_empty[s], lane);
+                    const uint32_t after = lane_after(acc0, acc1, lane);
+                    if (QSM) mbar_arrive2_if_zero(&bars->s_free[sl.idx], &bars->kv_empty[s], after);
+                    else if (HALVES) mbar_arrive2_if_zero(&bars->s_free[1], &bars->kv_empty[s], after);
+                    else mbar_arrive_if_zero(&bars->kv_empty[s], after);
                 }
             };
             tile_loop(std::integral_constant<bool, VF == 1>{});
