@@ -784,6 +784,7 @@ tc_gauss_fma_kernel(const __grid_constant__ CUtensorMap tm_q,
             // fast one alone.)
             auto tile_loop = [&](auto fast_tag) {
                 constexpr bool FAST = decltype(fast_tag)::value;
+                int s_prev = 0;                   // stage of the previous tile
                 for (int j = 0; j < T; ++j, st.advance(p.stages), sl.advance(SL)) {
                     const int s = st.idx;
                     const uint32_t col0 = static_cast<uint32_t>(sl.idx * 2 * BN);
@@ -815,6 +816,12 @@ tc_gauss_fma_kernel(const __grid_constant__ CUtensorMap tm_q,
                         // that was no faster on the 65536^2, D = 64 sum either
                         // (0.6428 against 0.6418 ms).
                         tmem_wait_ld_regs(r0, r1);
+                        // The previous tile's stage goes back here (two stages at
+                        // least: this tile's loads did not wait for it) rather than
+                        // at that tile's end, where waiting for its last sums cost
+                        // 8 %: 50021^2, D = 50, signed values, 409 against 435 us,
+                        // 403 untied.
+                        if (!FAST && j > 0) mbar_arrive_if_zero(&bars->kv_empty[s_prev], lane_after(acc0, acc1, lane));
                     } else if (!HALVES) {
                         // q^ in TMEM: one S tile per query tile, handed back as
                         // soon as it is in registers, since the MMAs of the next
@@ -866,12 +873,14 @@ tc_gauss_fma_kernel(const __grid_constant__ CUtensorMap tm_q,
                                                              &bars->s_full[sl2.idx], sl2.phase);
                     }
                     const float* rec = rec_smem(s) + (cg * 16) * REC_PAIR;
+                    uint32_t sign_word = 0u;      // FAST: the only record word read
                     const uint64_t w2 = (TRI && j >= w_from) ? f32x2_pack(1.f, 1.f) : 0ull;
                     if constexpr (FAST) {
                         // Folded values, every group of this problem of one sign:
                         // P = Phi |v| 2^-16 from the MMA's exponent, times this
                         // column group's sign word +-2^16; no per-key records.
                         const float uw = rec_smem(s)[BN + cg];
+                        sign_word = __float_as_uint(uw);
                         const uint64_t u2 = f32x2_pack(uw, uw);
         #pragma unroll
                         for (int t = 0; t < 16; ++t) {
@@ -1030,11 +1039,20 @@ tc_gauss_fma_kernel(const __grid_constant__ CUtensorMap tm_q,
                     // Lane 0 hands back the slot (two-slot path) and the stage,
                     // predicated rather than branched: a divergent branch here
                     // cost 0.7 % of the kernel time.
-                    const uint32_t after = lane_after(acc0, acc1, lane);
-                    if (QSM) mbar_arrive2_if_zero(&bars->s_free[sl.idx], &bars->kv_empty[s], after);
-                    else if (HALVES) mbar_arrive2_if_zero(&bars->s_free[1], &bars->kv_empty[s], after);
-                    else mbar_arrive_if_zero(&bars->kv_empty[s], after);
+                    // (The S slot waits for its loads alone, which are complete; tied
+                    // to the sums as well it cost the 65536^2, D = 64 sum 8 %.)
+                    if (QSM) mbar_arrive_if_zero(&bars->s_free[sl.idx], lane);
+                    if (FAST) {
+                        mbar_arrive_if_zero(&bars->kv_empty[s], sign_word == ~0u ? 1u : static_cast<uint32_t>(lane));
+                    } else if (HALVES) {
+                        mbar_arrive2_if_zero(&bars->s_free[1], &bars->kv_empty[s], lane_after(acc0, acc1, lane));
+                    } else if (!QSM) {
+                        mbar_arrive_if_zero(&bars->kv_empty[s], lane_after(acc0, acc1, lane));
+                    }
+                    s_prev = s;
                 }
+                if (QSM && !FAST && ok && T > 0)
+                    mbar_arrive_if_zero(&bars->kv_empty[s_prev], lane_after(acc0, acc1, lane));
             };
             tile_loop(std::integral_constant<bool, VF == 1>{});
             if (HALVES) {
