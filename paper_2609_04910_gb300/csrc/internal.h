@@ -167,8 +167,8 @@ struct TcPlan {
 
 struct SimtPlan {
     int64_t M, N, D, Cv;
-    int dmax;          // register tile of the query row (forward: 4, 8, 16, 24, 32, 48, 64 or
-                       // 128 coordinates; gradient: 16, 32 or 64)
+    int dmax;          // register tile of the query row (forward: 4, 8, 16, 24, 32, 48, 56,
+                       // 64 or 128 coordinates; gradient: 16, 32 or 64)
     int cblk;          // channels per launch slice
     int threads;       // threads per block of the forward kernel
     int splits;

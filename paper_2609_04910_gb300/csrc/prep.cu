@@ -1550,15 +1550,20 @@ __global__ void finalize_kernel(const float* __restrict__ part, int splits,
 // of a 43 us call).  Here kFinalizeLanes threads share an output: thread y adds
 // splits y, y + kFinalizeLanes, ... in order, and thread 0 the sums in order.
 constexpr int kFinalizeLanes = 8;
-constexpr int kFinalizeManySplits = 16;
+
+// Whether an output's n partial sums are shared by several threads: 16 or more,
+// or four or more where one thread per output leaves SMs idle.
+__host__ __device__ inline bool many_partials(int n, int64_t outputs) {
+    return n >= 16 || (n >= 4 && outputs < 152 * 256);
+}
 
 // p[0], p[stride], .. (n of them) added up by the block's column of threads
-// threadIdx.x, into the return value of thread y = 0; fewer than
-// kFinalizeManySplits in order by that thread, as finalize_kernel adds them.
-// Every thread of the block calls this (n <= 0: none).
-__device__ __forceinline__ float sum_lanes(const float* __restrict__ p, int64_t stride, int n) {
+// threadIdx.x, into the return value of thread y = 0; a few (see many_partials)
+// in order by that thread, as finalize_kernel adds them.  Every thread of the
+// block calls this (n <= 0: none).
+__device__ __forceinline__ float sum_lanes(const float* __restrict__ p, int64_t stride, int n, int64_t outputs) {
     __shared__ float sums[kFinalizeLanes][32];
-    const int lanes = n < kFinalizeManySplits ? 1 : kFinalizeLanes;
+    const int lanes = many_partials(n, outputs) ? kFinalizeLanes : 1;
     float acc = 0.f;
     int s = static_cast<int>(threadIdx.y);
     if (s < lanes) {
@@ -1587,7 +1592,7 @@ finalize_many_kernel(const float* __restrict__ part, int splits, int64_t total, 
     pdl_trigger();
     pdl_wait();
     const int64_t idx = static_cast<int64_t>(blockIdx.x) * 32 + threadIdx.x;
-    const float sum = sum_lanes(part + idx, total, idx < total ? splits : 0);
+    const float sum = sum_lanes(part + idx, total, idx < total ? splits : 0, total);
     if (threadIdx.y == 0 && idx < total) out[idx] = sum;
 }
 
@@ -1616,7 +1621,7 @@ finalize_guarded_kernel(const float* __restrict__ part, int64_t Mpad, int64_t M,
             stride = Mpad * C;
         }
     }
-    const float sum = sum_lanes(p, stride, n);
+    const float sum = sum_lanes(p, stride, n, total);
     if (threadIdx.y == 0 && idx < total) out[idx] = sum;
 }
 
@@ -2655,7 +2660,7 @@ cudaError_t launch_finalize(const float* part, int splits, int64_t split_stride_
                             cudaStream_t s, int64_t main_rows) {
     const int64_t total = M * Cv;
     if (total == 0) return cudaSuccess;
-    if (splits >= kFinalizeManySplits && !inv_scale && main_rows == 0 && part_ld == Cv &&
+    if (many_partials(splits, total) && !inv_scale && main_rows == 0 && part_ld == Cv &&
         split_stride_rows == M) {
         launch_kernel(finalize_many_kernel, static_cast<unsigned>((total + 31) / 32), dim3(32, kFinalizeLanes), 0,
                       s, part, splits, total, out);

@@ -16,6 +16,7 @@
 // squared distance accumulates even and odd coordinates separately and
 // adds the two at the end).  Bound: the fp32 lanes, 2 D operations per pair.
 #include <algorithm>
+#include <cmath>
 
 #include "internal.h"
 #include "ptx.cuh"
@@ -88,22 +89,22 @@ simt_sum_kernel(const float* __restrict__ q, const float* __restrict__ k,
     const int64_t n_begin = static_cast<int64_t>(split) * keys_per_split;
     const int64_t n_end = min(N, n_begin + keys_per_split);
 
-    // Tile of KTF keys from t0 into buffer b; rows past n_end and the
-    // coordinates and channels past D and Cv are filled with zeros (nothing
-    // is read for them; their source address is v, which is never null here,
-    // as k may be when D = 0).
+    // Tile of up to KTF keys from t0 into buffer b; the coordinates and channels
+    // past D and Cv are filled with zeros (nothing is read for them; their
+    // source address is v, which is never null here, as k may be when D = 0).
+    // Rows past n_end are left as they are, and not used.
     auto load_tile = [&](int b, int64_t t0) {
         const int cnt = static_cast<int>(min(static_cast<int64_t>(KTF), n_end - t0));
         const float* kt = k + t0 * D;
-        for (int i = threadIdx.x; i < KTF * DMAX; i += nthreads) {
+        for (int i = threadIdx.x; i < cnt * DMAX; i += nthreads) {
             const int kk = i / DMAX, d = i - kk * DMAX;
-            const bool in = kk < cnt && d < D;
+            const bool in = d < D;
             cp_async4(&ks[b][kk][d], in ? kt + kk * D + d : v, in);
         }
         const float* vt = v + t0 * Cv + c0;
-        for (int i = threadIdx.x; i < KTF * CBLK; i += nthreads) {
+        for (int i = threadIdx.x; i < cnt * CBLK; i += nthreads) {
             const int kk = i / CBLK, j = i - kk * CBLK;
-            const bool in = kk < cnt && c0 + j < Cv;
+            const bool in = c0 + j < Cv;
             cp_async4(&vs[b][kk][j], in ? vt + static_cast<int64_t>(kk) * Cv + j : v, in);
         }
         cp_async_commit();
@@ -354,7 +355,7 @@ bool plan_simt(int64_t M, int64_t N, int64_t D, int64_t C, bool grad, int split_
     } else {
         // Register tiles of the query rows: the smallest that holds D.
         p->dmax = D <= 4 ? 4 : D <= 8 ? 8 : D <= 16 ? 16 : D <= 24 ? 24 : D <= 32 ? 32
-                : D <= 48 ? 48 : D <= 64 ? 64 : 128;
+                : D <= 48 ? 48 : D <= 56 ? 56 : D <= 64 ? 64 : 128;
         rows = THREADS / lanes_per_group(p->dmax) * ROWS;
         keys = key_tile(p->dmax);
     }
@@ -370,39 +371,47 @@ bool plan_simt(int64_t M, int64_t N, int64_t D, int64_t C, bool grad, int split_
                                  : std::max<int64_t>(4, ((N + splits - 1) / splits + 3) / 4 * 4);
     } else {
         // Threads per block and key splits by an estimate of the busiest SM's
-        // cycles, fitted to whole calls (one GB300, 216 shapes of 1 to 262144
-        // rows, 32 to 262144 keys, 4 to 100 coordinates, 1 and 4 channels,
-        // each with 33 choices; the estimate's choice is 2.8 % slower than the
-        // best one on average, at most 14 %).  A warp takes `key` issue cycles
-        // per key of its rows: coordinates, exponentials, values and its share
-        // of copying the key tile, which few threads per block make dear; an
-        // SMSP with fewer than two warps waits for latencies instead.  Each
-        // block costs a start, each split a partial sum to add.  Blocks of 128
-        // threads share the copies best; 64 and 32 (128 query rows up to 32
-        // coordinates) are for few rows, which full blocks would pad: 32 x
+        // time, fitted to whole calls (one GB300, 1800 shapes of 1 to 200000
+        // rows and keys, 1 to 128 coordinates, 1 to 16 channels, each with 30
+        // choices: the estimate's choice is 4 % slower than the best one on
+        // average).  A warp takes `key` issue cycles per key of its rows:
+        // coordinates, exponentials, values and its share of copying the key
+        // tile, which few threads per block make dear; an SMSP with fewer than
+        // about two warps waits for latencies instead.  Each block costs a
+        // start, each split a partial sum per output to write and add, and the
+        // blocks of a single wave wait at their barriers together.  Blocks
+        // of 128 threads share the copies best; 64 and 32 (128 query rows up to
+        // 32 coordinates) are for few rows, which full blocks would pad: 32 x
         // 65536, D = 64, 256 splits of 64-thread blocks 67 us, 608 of 32
         // threads 40.
         const int L = lanes_per_group(p->dmax);
-        const double issue = 2.8 * (p->dmax / L) + 10.0 + 1.6 * 4 * p->cblk / L + (L > 1 ? 6.0 : 0.0);
+        const double issue = 2.3 * (p->dmax / L) + 10.0 + 2.0 * p->cblk / L + (L > 1 ? 20.0 : 0.0);
+        const double few = L > 1 ? 1.5 : 2.1;                  // warps per SMSP
+        const double few4 = few * few * few * few;
         const int64_t smem = 2 * keys * (p->dmax + p->cblk) * 4 + 1024;
         double best = 1e300;
         for (int threads = THREADS; threads >= 32; threads /= 2) {
             const int64_t r = rows * threads / THREADS;
-            const double key = issue + 18.0 * (p->dmax + p->cblk) / threads;
+            const double key = issue + 20.0 * (p->dmax + p->cblk) / threads;
             const double warps = threads / 128.0;              // per SMSP and block
             const int64_t fit = std::min<int64_t>(228 * 1024 / smem, min_blocks(p->dmax, p->cblk) * THREADS / threads);
             blocks = (M + r - 1) / r * chunks;
-            for (int64_t per : {1, 2, 3, 4, 6, 8, 12, 16, 32}) {
+            int64_t tried = 0;
+            for (int64_t per : {1, 2, 3, 4, 6, 8, 12, 16, 24, 32}) {
                 const int64_t want = std::max<int64_t>(1, per * sms / blocks);
                 const int64_t kps = std::max<int64_t>(16, ((N + want - 1) / want + 3) / 4 * 4);
                 const int64_t n = (N + kps - 1) / kps;
+                if (n == tried) continue;
+                tried = n;
                 if (n > 1 && n * M * p->Cv > kMaxSplitFloats) break;
                 const int64_t per_sm = (blocks * n + sms - 1) / sms;
-                const int64_t conc = std::min(per_sm, fit), rounds = per_sm / conc, rem = per_sm % conc;
-                auto cycles = [&](int64_t nb) {
-                    return nb == 0 ? 0.0 : std::max(nb * warps, 2.0) * key * kps + 620.0 * (1.0 + 0.22 * nb * warps);
+                const int64_t conc = std::min(per_sm, fit), rounds = per_sm / conc, rem = per_sm - rounds * conc;
+                auto time = [&](int64_t nb) {
+                    const double w = nb * warps, w2 = w * w;
+                    return nb == 0 ? 0.0 : std::sqrt(std::sqrt(w2 * w2 + few4)) * key * kps + 200.0 + 60.0 * w;
                 };
-                const double cost = rounds * cycles(conc) + cycles(rem) + 6.3 * n;
+                const double cost = (rounds * time(conc) + time(rem)) * (1.0 + 0.07 * conc / per_sm) + 9.0 * n +
+                                    (n > 1 ? 0.2 * n * M * p->Cv / sms : 0.0);
                 if (cost < best * 0.995) {
                     best = cost;
                     p->keys_per_split = kps;
@@ -410,8 +419,8 @@ bool plan_simt(int64_t M, int64_t N, int64_t D, int64_t C, bool grad, int split_
                 }
             }
         }
-        // (Measured, D = 48 and 64: 630 to 830 of these cycles in a microsecond.)
-        p->micros = best / 720.0 + 5.0;
+        // (Measured, D = 33 to 64: 640 to 810 of these units in a microsecond.)
+        p->micros = best / 700.0 + 5.0;
     }
     p->splits = static_cast<int>((N + p->keys_per_split - 1) / p->keys_per_split);
     if (p->splits < 1) p->splits = 1;
@@ -438,6 +447,7 @@ cudaError_t launch_simt(const SimtPlan& p, bool grad, const float* q, const floa
         case 24: return launch_dmax<24>(p, q, k, v, half_c, part, s, guard);
         case 32: return launch_dmax<32>(p, q, k, v, half_c, part, s, guard);
         case 48: return launch_dmax<48>(p, q, k, v, half_c, part, s, guard);
+        case 56: return launch_dmax<56>(p, q, k, v, half_c, part, s, guard);
         case 64: return launch_dmax<64>(p, q, k, v, half_c, part, s, guard);
         default: return launch_dmax<128>(p, q, k, v, half_c, part, s, guard);
     }

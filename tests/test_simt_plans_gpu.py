@@ -37,12 +37,12 @@ def _check(M, N, D, C, **kw):
 
 @pytest.mark.parametrize("M,N", [(1, 65537), (31, 20001), (33, 70000), (129, 30000), (513, 8192),
                                  (3000, 3001), (70000, 33), (5, 7)])
-@pytest.mark.parametrize("D,C", [(3, 1), (16, 4), (32, 5), (33, 2), (64, 3), (100, 1), (128, 4)])
+@pytest.mark.parametrize("D,C", [(3, 1), (16, 4), (32, 5), (33, 2), (49, 1), (56, 4), (57, 2), (64, 3), (100, 1), (128, 4)])
 def test_shapes(M, N, D, C):
     _check(M, N, D, C)
 
 
-@pytest.mark.parametrize("splits", [1, 2, 15, 16, 17, 24, 63, 64, 65, 200])
+@pytest.mark.parametrize("splits", [1, 2, 3, 4, 5, 15, 16, 17, 24, 63, 64, 65, 200])
 @pytest.mark.parametrize("M,C", [(1, 1), (31, 3), (257, 4)])
 def test_splits(splits, M, C):
     _check(M, 6400, 20, C, split_n=splits)
