@@ -151,6 +151,16 @@ struct Call {
     bool rw_f32 = false;
     const void* kw = nullptr;
     bool kw_f32 = false;
+    // The plan of a batch's problems, worked out for the first of them.
+    struct Planned* planned = nullptr;
+};
+
+struct Planned {
+    bool valid = false;
+    bool tensor = false;
+    gs::TcPlan tp{};
+    gs::SimtPlan sp{};
+    size_t bytes = 0;
 };
 
 // Padded weight channels of a weighted pass (the kernel's instances).
@@ -370,8 +380,16 @@ gs_status run(Call c) {
     gs::TcPlan tp{};
     gs::SimtPlan sp{};
     size_t bytes = 0;
-    st = plan(c, g_sm_count[dev], &tensor, &tp, &sp, &bytes);
-    if (st != GS_OK) return st;
+    if (c.planned && c.planned->valid) {
+        tensor = c.planned->tensor;
+        tp = c.planned->tp;
+        sp = c.planned->sp;
+        bytes = c.planned->bytes;
+    } else {
+        st = plan(c, g_sm_count[dev], &tensor, &tp, &sp, &bytes);
+        if (st != GS_OK) return st;
+        if (c.planned) *c.planned = {true, tensor, tp, sp, bytes};
+    }
     if (tensor && g_is_sm103[dev] != 1)
         return fail(GS_ERR_UNSUPPORTED, "the tensor-core kernel needs an sm_103 (GB300) GPU");
     if (c.B > 1 && !(tensor && tp.fma)) {
@@ -380,9 +398,11 @@ gs_status run(Call c) {
         const int64_t es = c.dtype == GS_FP32 ? 4 : 2;
         const int64_t ws_ = c.w_f32 ? 4 : es, us = c.u_f32 ? 4 : es;
         const int64_t out_w1 = c.grad ? c.D : c.C;
+        Planned planned;
         for (int64_t b = 0; b < c.B; ++b) {
             Call cb = c;
             cb.B = 1;
+            cb.planned = &planned;
             cb.mmd_out = nullptr;
             cb.q = static_cast<const char*>(c.q) + b * c.M * c.D * es;
             cb.k = static_cast<const char*>(c.k) + b * c.N * c.D * es;
@@ -410,6 +430,7 @@ gs_status run(Call c) {
             // as in a caller's workspace too small for both.
             if (!forced) cudaGetLastError();
             c.opt.path = GS_PATH_SIMT;
+            c.planned = nullptr;
             return run(c);
         }
         if (forced) return fail(GS_ERR_OUT_OF_MEMORY, "workspace allocation failed (test hook)");
