@@ -1800,15 +1800,16 @@ finalize_point_quads_kernel(const float* __restrict__ part, int splits, int64_t 
 // per-channel maxima, or writes 16 keys of a channel per thread (two 16-byte
 // stores, whole sectors).  The element-wise kernels read 2 bytes at a time and
 // stored 4: 131072 keys, D = 32, ncu: 19.6 + 24.1 us, these 9.3 + 11.8.  Blocks
-// of 128 rows and 128 threads, or of 32 rows and 256 threads where the first
-// would leave SMs idle and each thread's chain of rows is what a call waits for
-// (whole calls, with blocks of 128 rows / of 32: gradient of 3000 points, D = 128
-// 57 / 39 us; vector-Jacobian product of 300 points, D = 64 78 / 56).
+// of 128 rows and 128 threads, or of 32 rows and 256 threads where each thread's
+// chain of rows is what a call waits for (whole calls, with blocks of 128 rows / of
+// 32: gradient of 3000 points, D = 128 57 / 39 us, of 601 points against 44831, D =
+// 64 72 / 53, of 131072 points, D = 32 2735 / 2707, of 300 against 200000, D = 64
+// 100 / 110; vector-Jacobian product of 300 points, D = 64 78 / 56).
 constexpr int kValueRows = 128;
 constexpr int kValueThreads = 128;
 constexpr int kFewValueRows = 32;
 constexpr int kFewValueThreads = 256;
-constexpr int64_t kFewValueBlocks = 304;     // (two per SM)
+constexpr int64_t kFewValueBlocks = 1280;    // of the larger blocks, 163840 keys
 
 // Rows [n0, n0 + ROWS) of x into raw (zeros past N); weights into sw (1
 // without weights, 0 past N).  By the whole block.
