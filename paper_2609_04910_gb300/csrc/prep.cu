@@ -1633,8 +1633,20 @@ constexpr int kFinalizeThreads = 256;
 // The sum over ns splits of one quad, added in split order.
 __device__ __forceinline__ float4 sum_splits4(const float* __restrict__ p, int64_t step, int ns) {
     float4 a = *reinterpret_cast<const float4*>(p);
-#pragma unroll 4
-    for (int s = 1; s < ns; ++s) {
+    int s = 1;
+    for (; s + 8 <= ns; s += 8) {     // (eight loads in flight)
+        float4 x[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) x[i] = *reinterpret_cast<const float4*>(p + (s + i) * step);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            a.x += x[i].x;
+            a.y += x[i].y;
+            a.z += x[i].z;
+            a.w += x[i].w;
+        }
+    }
+    for (; s < ns; ++s) {
         const float4 x = *reinterpret_cast<const float4*>(p + s * step);
         a.x += x.x;
         a.y += x.y;
@@ -1729,8 +1741,11 @@ __global__ void finalize_points_kernel(const float* __restrict__ part, int split
 // The same operations per output, in the same order.  (Bound: HBM and load
 // latency, about 4 (D + 16) bytes read and 4 D written per row; 131072 rows,
 // D = 32, ncu: one thread per output 56.5 us, quads 14.3.)
-template <typename T, typename U>
-__global__ void __launch_bounds__(kFinalizeThreads, 5)
+// IN_FLIGHT: splits loaded together.  Two cost the fewest registers, and most
+// rows have one split; few rows against many keys have up to 64 and wait for
+// them (gradient of 78 points against 61876, D = 32: two 72 us, eight 43 per call).
+template <typename T, typename U, int IN_FLIGHT>
+__global__ void __launch_bounds__(kFinalizeThreads, IN_FLIGHT > 2 ? 2 : 5)
 finalize_point_quads_kernel(const float* __restrict__ part, int splits, int64_t split_stride_rows,
                             int64_t M, int part_ld, const float* __restrict__ inv_scale,
                             const T* __restrict__ x, const float* __restrict__ mu, float tau, int D,
@@ -1766,9 +1781,26 @@ finalize_point_quads_kernel(const float* __restrict__ part, int splits, int64_t 
     for (int e = 0; e < 4; ++e) mf[e] = mu && d + e < D ? mu[d + e] : 0.f;
     float4 a = *reinterpret_cast<const float4*>(p + d);
     float ss = p[D];
-    // (Two at a time: more in flight cost registers, and most rows have one.)
+    int s = 1;
+    for (; IN_FLIGHT > 2 && s + IN_FLIGHT <= ns; s += IN_FLIGHT) {
+        float4 b[IN_FLIGHT];
+        float w1[IN_FLIGHT];
+#pragma unroll
+        for (int i = 0; i < IN_FLIGHT; ++i) {
+            b[i] = *reinterpret_cast<const float4*>(p + (s + i) * step + d);
+            w1[i] = p[(s + i) * step + D];
+        }
+#pragma unroll
+        for (int i = 0; i < IN_FLIGHT; ++i) {
+            ss += w1[i];
+            a.x += b[i].x;
+            a.y += b[i].y;
+            a.z += b[i].z;
+            a.w += b[i].w;
+        }
+    }
 #pragma unroll 2
-    for (int s = 1; s < ns; ++s) {
+    for (; s < ns; ++s) {
         const float4 b = *reinterpret_cast<const float4*>(p + s * step + d);
         ss += p[s * step + D];
         a.x += b.x;
@@ -2113,13 +2145,16 @@ cudaError_t finalize_points_typed(const float* part, int splits, int64_t stride_
     if (total == 0) return cudaSuccess;
     if constexpr (!DIRECT) {
         if (D >= 1 && Cw == 1 && ch0 == 0 && Cc == D + 1 && !accumulate && inv_scale && part_ld % 4 == 0) {
-            launch_kernel(finalize_point_quads_kernel<T, U>,
-                          static_cast<unsigned>((M * ((D + 3) / 4) + kFinalizeThreads - 1) / kFinalizeThreads),
-                          kFinalizeThreads, 0, s, part, splits, stride_rows, M, part_ld, inv_scale,
-                          static_cast<const T*>(x), mu, tau, D, static_cast<const U*>(u), out, s_out,
-                          main_rows);
-            note_launches(1);
-            return cudaGetLastError();
+            auto go = [&](auto kern) {
+                launch_kernel(kern,
+                              static_cast<unsigned>((M * ((D + 3) / 4) + kFinalizeThreads - 1) / kFinalizeThreads),
+                              kFinalizeThreads, 0, s, part, splits, stride_rows, M, part_ld, inv_scale,
+                              static_cast<const T*>(x), mu, tau, D, static_cast<const U*>(u), out, s_out,
+                              main_rows);
+                note_launches(1);
+                return cudaGetLastError();
+            };
+            return splits > 8 ? go(finalize_point_quads_kernel<T, U, 8>) : go(finalize_point_quads_kernel<T, U, 2>);
         }
     }
     const int threads = 256;

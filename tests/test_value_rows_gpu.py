@@ -27,3 +27,12 @@ def _gpu():
 def test_rows(N, D, dtype):
     M = 300
     grad_check(case(M, N, D, 1, dtype), rows=np.arange(0, M, 7))
+
+
+@pytest.mark.parametrize("dtype", ["fp16", "bf16"])
+@pytest.mark.parametrize("M,D", [(1, 3), (78, 32), (129, 64)])
+@pytest.mark.parametrize("splits", [1, 2, 8, 9, 10, 16, 17, 25, 33])
+def test_splits(splits, M, D, dtype):
+    """Both sides of eight splits, from where the contraction loads eight of a
+    row's partial sums together, with none to seven left over."""
+    grad_check(case(M, 40 * 128, D, 1, dtype), split_n=splits)
