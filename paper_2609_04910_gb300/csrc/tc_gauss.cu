@@ -918,11 +918,12 @@ bool plan_tensor(InType t, int64_t M, int64_t N, int64_t D, int64_t C, bool grad
     // key tiles take two stages instead of three, whose loads would delay the
     // first MMAs and q^ (three / two stages, whole calls, one GB300: 16384 x
     // 1000, D = 256 37.0 / 34.6 us, D = 208, C = 4 41 / 35; runs of 14 tiles, 1000 x
-    // 65536, D = 240 70 / 63, D = 256, C = 4 77.7 / 75.3, D = 144 48 / 49; runs of 54
-    // tiles, 16384^2, D = 160 84 / 93).
+    // 65536, D = 240 70 / 63, D = 256, C = 4 77.7 / 75.3, D = 144 48 / 49; runs of 23
+    // tiles, 9032 x 11983, D = 256 72.4 / 70.5; runs of 54 tiles, 16384^2, D = 160
+    // 84 / 93, D = 256 113 / 112, with C = 4 128 / 133).
     if (p->fma && !p->aug && !p->tf) {
         const int64_t seg = p->band_len > 0 ? p->band_len : std::min<int64_t>(key_tiles, p->unit_len);
-        if (seg <= 8 || (seg <= 16 && p->Dp > 192))
+        if (seg <= 8 || (seg <= 16 && p->Dp > 192) || (seg <= 40 && p->Dp > 240 && p->Cv <= 2))
             plan_fma_kernel(p->Dp, static_cast<int>(p->Cv), false, false, true, &nq, &p->stages, &p->smem_bytes);
     }
     // ~256 rows per block of the mean kernel, so that every SM has work.
