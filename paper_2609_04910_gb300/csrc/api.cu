@@ -218,8 +218,8 @@ gs::InType in_type(gs_dtype d) {
 // distances are cheap on the SIMT kernel (it works in register tiles of 4, 8,
 // 16, .. coordinates), from 2^26.  Measured on a GB300, C = 1, whole calls,
 // SIMT / tensor cores: 5800^2 pairs D = 4 24 / 35 us, 18684 x 2500, D = 7 37 /
-// 31 us, 5800^2, D = 16 50 / 37 us; 16384^2 pairs D = 4 113 / 70 us, D = 8
-// 172 / 70 us, D = 16 296 / 74 us.  One cloud against itself (q is k), whose
+// 31 us, 5800^2, D = 16 50 / 37 us; 16384^2 pairs D = 4 106 / 66 us, D = 8
+// 172 / 70 us, D = 16 281 / 71 us.  One cloud against itself (q is k), whose
 // operands are written once, from 3 x 2^24 pairs for D <= 4: MMD^2 of 8000
 // points, D = 3 41.5 / 39.2 us.
 // Batches keep 2^25 for every D: the tensor-core path runs them in one

@@ -43,8 +43,8 @@ constexpr int64_t kMaxSplitFloats = int64_t(1) << 22;
 // cp.async into two buffers, the next one under the arithmetic of the current
 // one.  Measured (one GB300, whole calls, C = 1, one row per thread in tiles
 // of 16, 32, 64 or 128 coordinates / this kernel): M = N = 16384, D = 4 435 /
-// 113 us, D = 16 435 / 296, D = 32 794 / 566, D = 48 1306 / 895, D = 64 1316
-// / 1144 (75 % of the lanes), D = 128 2919 / 2359; 4096^2, D = 16 39 / 27 us.
+// 106 us, D = 16 435 / 281, D = 32 794 / 524, D = 48 1306 / 824, D = 64 1316
+// / 1088 (78 % of the lanes), D = 128 2919 / 2291; 4096^2, D = 16 39 / 27 us.
 constexpr int ROWS = 4;
 __host__ __device__ constexpr int lanes_per_group(int dmax) { return dmax <= 32 ? 1 : dmax <= 64 ? 2 : 4; }
 __host__ __device__ constexpr int key_tile(int dmax) { return dmax <= 64 ? 64 : 32; }
@@ -383,7 +383,7 @@ bool plan_simt(int64_t M, int64_t N, int64_t D, int64_t C, bool grad, int split_
         // of 128 threads share the copies best; 64 and 32 (128 query rows up to
         // 32 coordinates) are for few rows, which full blocks would pad: 32 x
         // 65536, D = 64, 256 splits of 64-thread blocks 67 us, 608 of 32
-        // threads 40.
+        // threads 41.
         const int L = lanes_per_group(p->dmax);
         const double issue = 2.3 * (p->dmax / L) + 10.0 + 2.0 * p->cblk / L + (L > 1 ? 20.0 : 0.0);
         const double few = L > 1 ? 1.5 : 2.1;                  // warps per SMSP
