@@ -1835,13 +1835,16 @@ finalize_point_quads_kernel(const float* __restrict__ part, int splits, int64_t 
 // of 128 rows and 128 threads, or of 32 rows and 256 threads where each thread's
 // chain of rows is what a call waits for (whole calls, with blocks of 128 rows / of
 // 32: gradient of 3000 points, D = 128 57 / 39 us, of 601 points against 44831, D =
-// 64 72 / 53, of 131072 points, D = 32 2735 / 2707, of 300 against 200000, D = 64
-// 100 / 110; vector-Jacobian product of 300 points, D = 64 78 / 56).
+// 64 72 / 53; of 300 against 65536, D = 1 52 / 47, D = 12 49 / 44, D = 32 51 / 43, D
+// = 64 77 / 54; against 131072, D = 1 57 / 61, D = 12 55 / 57, D = 32 63 / 61, D =
+// 64 86 / 80; against 200000, D = 64 100 / 110; vector-Jacobian product of 300
+// points, D = 64 78 / 56).
 constexpr int kValueRows = 128;
 constexpr int kValueThreads = 128;
 constexpr int kFewValueRows = 32;
 constexpr int kFewValueThreads = 256;
-constexpr int64_t kFewValueBlocks = 1280;    // of the larger blocks, 163840 keys
+constexpr int64_t kFewValueBlocks = 1280;    // of the larger blocks, 163840 keys,
+constexpr int64_t kFewNarrowBlocks = 768;    // or 98304 of fewer than 32 coordinates
 
 // Rows [n0, n0 + ROWS) of x into raw (zeros past N); weights into sw (1
 // without weights, 0 past N).  By the whole block.
@@ -2112,7 +2115,7 @@ cudaError_t value_prep_typed(const void* w, const void* x, const float* mu, int6
                       static_cast<const T*>(x), mu, N, Npad, D, Cp, static_cast<const unsigned*>(vmax_bits),
                       static_cast<__half*>(vt), inv_scale);
         };
-        if (Npad / kValueRows < kFewValueBlocks)
+        if (Npad / kValueRows < (D < 32 ? kFewNarrowBlocks : kFewValueBlocks))
             return both(std::integral_constant<int, kFewValueRows>(), std::integral_constant<int, kFewValueThreads>());
         return both(std::integral_constant<int, kValueRows>(), std::integral_constant<int, kValueThreads>());
     }

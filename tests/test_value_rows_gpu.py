@@ -1,6 +1,6 @@
 """Value channels of the gradient passes on both sides of the switch from blocks
-of 32 rows to blocks of 128 (163840 keys), and at the edges of a block,
-against the float64 oracle with the suite's tolerances."""
+of 32 rows to blocks of 128 (163840 keys, 98304 below 32 coordinates), and at
+the edges of a block, against the float64 oracle with the suite's tolerances."""
 import numpy as np
 import pytest
 
@@ -22,8 +22,9 @@ def _gpu():
 
 @pytest.mark.parametrize("dtype", ["fp16", "bf16"])
 @pytest.mark.parametrize("N,D", [(1, 3), (31, 64), (32, 17), (33, 1), (127, 100), (129, 8),
-                                 (38785, 5), (40000, 33), (163712, 5), (163713, 5), (163712, 64),
-                                 (163713, 64)])
+                                 (38785, 5), (40000, 33), (98176, 5), (98177, 5), (98176, 31),
+                                 (98177, 31), (163712, 5), (163713, 5), (163712, 64), (163713, 64),
+                                 (163712, 32), (163713, 32)])
 def test_rows(N, D, dtype):
     M = 300
     grad_check(case(M, N, D, 1, dtype), rows=np.arange(0, M, 7))
