@@ -242,7 +242,7 @@ bool fp32_on_tensor_cores(const Call& c) {
 // the device decides whose sums count (see Guard in internal.h).  From 2^24
 // pairs, where its extra launches are repaid.
 // Measured on a GB300, whole calls, SIMT / guarded: 16384^2, D = 64, C = 1
-// 1145 / 150 us (the tensor cores' share of the work at three tf32 MMAs per
+// 1088 / 152 us (the tensor cores' share of the work at three tf32 MMAs per
 // product is 80 us), 8192^2, D = 50 289 / 64 us, 5800^2, D = 64 154 / 53 us.
 // Error against 64 bits at 8192^2, D = 33 to 64 (guarded / SIMT kernel): N(0, I)
 // points and values, relative 2-norm 1.0e-7 to 2.5e-7 / 1.3e-7 to 3.7e-7; two
